@@ -150,11 +150,12 @@ struct SelArgs {
     const float *cnrm_up;  // [L]
     float gamma2;          // 2 * gamma_d
     float gamma2_first;    // the same factor for the first-stage distances D
+    float gamma2_re;       // and for FP32 dot products summed across a warp (re_ops)
     int two_level;         // D is the BF16 tensor-core stage: recheck S in FP32
-    const int32_t *S;      // instead of D: per-row candidate lists of the fused
-    int s_stride;          // first stage ([n, lists...], n = -1: redo the row)
-    const int32_t *hard;   // the rows the fused first stage left undecided
-    const int *nhard;      // (their number, on the device)
+    const int32_t *hard;   // k_coarse_finish: the rows the fused first stage left
+    const int *nhard;      // undecided, those with a record from the front, those to
+    const int32_t *S;      // redo from the back (two counters, on the device), and
+    int s_cap;             // the first kind's records (room for s_cap): [n, lists...]
     int32_t *out;          // [m, P]
     uint32_t *err;
 };
@@ -183,6 +184,14 @@ __device__ __forceinline__ float bound_of(float Dt, float cnc, float cnrm, float
 }
 __device__ __forceinline__ float upper_of(float Dt, float E) { return __fadd_rn(Dt, E); }
 __device__ __forceinline__ float lower_of(float Dt, float E) { return __fsub_rn(Dt, E); }
+
+// Upper bound of ||x|| from an FP32 sum of squares of d values (any order:
+// relative error <= d u).  An FP64 sum and root here held the FP64 pipe for
+// most of a selection's time (rows of 128: 11 ns per row over the chip).
+__device__ __forceinline__ float norm_up(float ss, int d)
+{
+    return __fsqrt_ru(__fmul_ru(ss, 1.f + 4.f * (float)d * 5.9604645e-08f));
+}
 
 // block-wide helpers for SEL_NT threads
 __device__ float block_min(float v, float *red)
@@ -222,16 +231,10 @@ __global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
     __shared__ double sDx[SEL_SCAP];
     __shared__ int sSel[kMaxK];
 
-    // ||x|| upper bound from an FP64 sum
-    double part = 0.0;
-    for (int j = tid; j < a.d; j += SEL_NT) part += (double)xr[j] * (double)xr[j];
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    __shared__ double dred[SEL_NT / 32];
-    if ((tid & 31) == 0) dred[tid >> 5] = part;
-    __syncthreads();
-    double xs = 0.0;
-    for (int w = 0; w < SEL_NT / 32; ++w) xs += dred[w];
-    const float xn = __double2float_ru(sqrt(xs) * (1.0 + 1e-12));
+    // every warp sums the row's squares for itself
+    float part = 0.f;
+    for (int j = tid & 31; j < a.d; j += 32) part = fmaf(xr[j], xr[j], part);
+    const float xn = norm_up(warp_sum(part), a.d);
 
     // T = P-th smallest upper bound
     float T;
@@ -575,375 +578,459 @@ __global__ __launch_bounds__(CT_NT, 1) void k_coarse_tc(const float *__restrict_
 }
 
 // ------------------------------- fused BF16 first stage for assignment
-// P = 1, one CTA per 128 rows of x against ALL centroids, without writing
-// the distance matrix.  The BF16 centroids pass in chunks of CT_N = 256 rows
-// (TMA boxes of 64 columns x 256 rows, 128-byte swizzle, into two buffers),
-// one tcgen05.mma group per chunk into one of two 256-column TMEM buffers,
-// so that the MMA of the next step and the copy of the one after run under
-// each epilogue.  The chunks pass twice (recomputing a chunk's products
-// costs far less than keeping them):
-//   pass 1: per row Dmin = min_c Dt_c and A = max_c |Dt_c|.  With
-//           Ebig >= E_c for every c (the bound of the selection evaluated
-//           at max ||c||^2, A and max ||c||, rounded up), T = Dmin + Ebig
-//           (rounded up) is >= the smallest upper bound Dt_c + E_c;
-//   pass 2: the lists with lower bound Dt_c - E_c <= T, a superset of the
-//           selection's set S.  A list with Dt_c above thr = T + Ebig plus
-//           one unit in the last place of T (rounded up) cannot qualify and
-//           is rejected by one comparison; the rest take the exact test.
-// Pass 1 also keeps the row's second smallest Dt: when it is above thr only
-// the argmin can qualify, so the argmin is the answer; a tile whose rows
-// are all decided that way skips pass 2.
-// A row left with one list has its answer (S holds the nearest list): it
-// is written to `out1` directly.  Any other row is appended to `hard` and
-// leaves [n, list_0 .. list_{n-1}] for the finishing selection, n = -1 when
-// one of its four threads had more than CF_CAP lists (the row is then
-// redone from all lists).  ||x|| is bounded from the FP32 sum of squares
-// s of the tile's rows (relative error <= d u) as RU(sqrt(RU(s (1 + 4 d u)))).
-// One thread issues the copies and MMAs and waits for them; a block barrier
-// per step releases the others.
-constexpr int CF_CAP = 8;                   // lists per thread
+// P = 1 against ALL centroids, without writing the distance matrix.  One
+// persistent CTA per SM takes tiles of 128 rows of x; the BF16 centroids
+// pass once per tile in chunks of 128 (TMA boxes of 64 columns x 128 rows,
+// 128-byte swizzle), one tcgen05.mma group per chunk into one of four
+// 128-column TMEM buffers.  PARTS = 1: the single product, four chunk
+// buffers; PARTS = 2: the split (x hi c hi + x hi c lo + x lo c hi), two.
+// Warp 17 issues the copies and warp 16 the MMAs, so that a chunk is asked
+// for as soon as the MMAs have read the buffer it goes into (one thread for
+// both asks only when the next MMAs can be issued: 350 against 266 us for
+// the split over 200,000 rows and 2,048 lists).  Warps 0-15 (four threads per row, one
+// TMEM lane quarter and every fourth group of 16 columns each) hold the next
+// tile's rows in registers while they work on this one, and store them
+// (rounded, swizzled) as soon as the last chunk's MMAs have read the tile:
+// the next tile's first MMAs run under this tile's last epilogue.
+//
+// Per group of 16 lists a thread takes the smallest and second smallest Dt,
+// the list's place in the group carried in the key's low four mantissa bits
+// (a relative change below 2^-19 of Dt), and keeps the best three groups and
+// the fourth's minimum.  With Amax >= |Dt| (max ||c||^2 + 2.04 ||x|| max ||c||: the parts' roundings included),
+// Ebig >= E_c for every c (the bound of the selection evaluated at max
+// ||c||^2, Amax and max ||c||, rounded up) and delta >= the key error,
+// T = min key + delta + Ebig is >= the smallest upper bound Dt_c + E_c, and
+// a list can belong to the selection's set S only if its key is at most
+// thr = T + Ebig + delta plus one unit in the last place of T (rounded up).
+// A row whose second smallest key is above thr has its argmin as the answer.
+// Any other row is appended to `hard` with a record of the lists that can
+// qualify (a group's 16 lists when its second is within thr), or, when they
+// are more than CF_CAP, a thread's fourth group is within thr or the records
+// are full, to the rows to redo from all lists (hard's end, downwards).
+// ||x|| is bounded from the FP32 sum of squares s of the tile's rows
+// (relative error <= d u) as RU(sqrt(RU(s (1 + 4 d u)))).
+//
+// What bounds it: the epilogue's min/max and selects (4.6 half-rate
+// operations per list and row); a chunk's MMAs and its copy from L2 run
+// under it.  1,000,000 rows, 1,024 lists, d = 128: 560 us, 1,190 in launches
+// of one tile per CTA and two passes over the centroids; the split stage,
+// 200,000 rows: 142 us + 36 us to finish the undecided rows, 1,580 us when
+// the matrix of distances was written and read back.
+constexpr int CF_CAP = 32;                  // lists of one undecided row's record
 constexpr int CF_SUB = 4;                   // threads per row
-constexpr int CF_STRIDE = CF_SUB * CF_CAP + 1;  // ints per row of the output
-constexpr int CF_NT = 128 * CF_SUB;
+constexpr int CF_STRIDE = CF_CAP + 1;       // ints per record: n, lists
+constexpr int CF_EPI = 128 * CF_SUB;        // epilogue threads
+constexpr int CF_NT = CF_EPI + 64;          // + the MMA warp and the copy warp
+constexpr int CF_HDR = 4;                   // ints before the undecided rows: how many have
+                                            // a record, how many are to be redone
+constexpr int CF_CN = 128;                  // centroids of a chunk (and of a TMA box)
+constexpr int CF_TB = 4;                    // TMEM buffers
+constexpr int CF_LMIN = 16;                 // fewer lists take the matrix form
 
-__host__ __device__ inline size_t coarse_fused_smem(int d)
+constexpr int CW_LMAX = 4096;  // most lists of the fused stage and of one warp per row
+
+__host__ __device__ constexpr int cf_buffers(int parts) { return parts == 1 ? 4 : 2; }
+__host__ __device__ inline size_t coarse_fused_smem(int KC, int parts)
 {
-    const int KC = (d * 2 + 127) / 128;
-    return (size_t)KC * (CT_M + 2 * CT_N) * 128 + (size_t)CF_CAP * CF_NT * 4 + 1024;
+    // A (parts), the chunk buffers (parts each), ||c||^2
+    return (size_t)KC * parts * (CT_M + cf_buffers(parts) * CF_CN) * 128 + CW_LMAX * 4 + 1024;
 }
 
-template <int KC>
-__global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused1(
-    const __grid_constant__ CUtensorMap tmB, const float *__restrict__ x, int m, int d,
-    const float *__restrict__ cn, const float *__restrict__ cnrm_up, int L, float g1,
-    int32_t *__restrict__ out1, int32_t *__restrict__ outS, int32_t *__restrict__ hard,
-    int *nhard, uint32_t *err)
+__device__ __forceinline__ float min3f(float a, float b, float c)
+{
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+template <int KC, int PARTS>
+__global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
+    const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBlo,
+    const float *__restrict__ x, int m, int d, const float *__restrict__ cn,
+    const float *__restrict__ cnrm_up, int L, float g1, int32_t *__restrict__ out1,
+    int32_t *__restrict__ outS, int cap, int32_t *__restrict__ hard, int *nhard, uint32_t *err)
 {
     pdl_begin();
+    constexpr int CN = CF_CN, NB = cf_buffers(PARTS), TB = CF_TB;
+    constexpr uint32_t PBYTES = KC * CN * 128;    // one part of a chunk
+    constexpr uint32_t BBYTES = PARTS * PBYTES;
+    constexpr uint32_t ABYTES = KC * CT_M * 128;  // one part of the row tile
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-    __shared__ uint64_t fullb[2], mmab[2];
+    unsigned char *A = smem;                               // PARTS x KC x 128 rows x 128 B
+    unsigned char *B = smem + PARTS * ABYTES;              // NB x PARTS x KC x CN rows x 128 B
+    float *scn = reinterpret_cast<float *>(B + NB * BBYTES);
+    // chunk copied, chunk read (both per chunk buffer), products ready,
+    // products read (per TMEM buffer), row tile stored
+    __shared__ uint64_t fullb[NB], freeb[NB], mmab[TB], tempty[TB], afull;
     __shared__ uint32_t tmem_base;
-    __shared__ float sxn[CT_M], sMin[CF_SUB][CT_M], sSec[CF_SUB][CT_M], sMax[CF_SUB][CT_M];
-    __shared__ int sn[CF_SUB][CT_M], sArg[CF_SUB][CT_M];
+    __shared__ int s_abort_;
+    volatile int *s_abort = &s_abort_;
+    // by tile parity: the row's norm, and each thread's best key, its list,
+    // the best key of its other lists, and its candidate count
+    __shared__ float sxn[2][CT_M], sMin[2][CF_SUB][CT_M], sSec[2][CF_SUB][CT_M];
+    __shared__ int sArg[2][CF_SUB][CT_M], sn[CF_SUB][CT_M];
     __shared__ uint32_t smax[2];  // max ||c||^2, max ||c|| (bits of non-negative floats)
-    constexpr uint32_t BBYTES = KC * CT_N * 128;
-    unsigned char *A = smem;                                  // KC x 128 rows x 128 B
-    unsigned char *B = smem + (size_t)KC * CT_M * 128;        // 2 x KC x 256 rows x 128 B
-    int *rc = reinterpret_cast<int *>(B + 2 * BBYTES);        // [CF_CAP][CF_NT] lists
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q = warp & 3, sub = warp >> 2, rloc = q * 32 + lane;
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < NB; ++i) {
             mbar_init(&fullb[i], 1);
-            mbar_init(&mmab[i], 1);
+            mbar_init(&freeb[i], 1);
         }
+        for (int i = 0; i < TB; ++i) {
+            mbar_init(&mmab[i], 1);
+            mbar_init(&tempty[i], CF_EPI / 32);
+        }
+        mbar_init(&afull, CF_EPI / 32);
         fence_mbar_init();
         smax[0] = smax[1] = 0u;
+        s_abort_ = 0;
     }
-    if (warp == 0) tmem_alloc(&tmem_base, 2 * CT_N);
+    if (warp == CF_EPI / 32) tmem_alloc(&tmem_base, TB * CN);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    {
-        float a0 = 0.f, a1 = 0.f;
-        for (int c = tid; c < L; c += CF_NT) {
-            a0 = fmaxf(a0, __ldg(cn + c));
-            a1 = fmaxf(a1, __ldg(cnrm_up + c));
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            a0 = fmaxf(a0, __shfl_xor_sync(0xffffffffu, a0, o));
-            a1 = fmaxf(a1, __shfl_xor_sync(0xffffffffu, a1, o));
-        }
-        if (lane == 0) {
-            atomicMax(&smax[0], __float_as_uint(a0));
-            atomicMax(&smax[1], __float_as_uint(a1));
-        }
-    }
     const uint32_t tbase = tmem_base;
-    const uint32_t idesc = mma_idesc(1, 1, CT_M, CT_N);
-    const int nch = (L + CT_N - 1) / CT_N, nsteps = 2 * nch, ntiles = (m + CT_M - 1) / CT_M;
-    // thread 0's bookkeeping, bit b for buffer b: phases, and copies / MMAs
-    // issued but not waited for
-    uint32_t fph = 0u, mph = 0u, fpend = 0u, mpend = 0u;
-    bool ok = true;
+    const int nch = (L + CN - 1) / CN, ntiles = (m + CT_M - 1) / CT_M;
+    const uint32_t mine = (ntiles - 1 - blockIdx.x) / gridDim.x + 1;  // gridDim.x <= ntiles
 
-    auto load_b = [&](int j, int b) {  // chunk j -> B buffer b
-        mbar_arrive_expect_tx(&fullb[b], BBYTES);
+    if (warp == CF_EPI / 32 + 1) {
+        // ---- copies (one lane)
+        if (lane == 0) {
+            const uint32_t steps = mine * (uint32_t)nch;
+            uint32_t g = 0;
+            for (; g < steps; ++g) {
+                const uint32_t b = g % NB, u = g / NB;
+                if (u >= 1 && !mbar_wait_ab(&freeb[b], (u - 1) & 1, err, s_abort, kWaitNs)) break;
+                const int j = (int)(g % (uint32_t)nch);
+                mbar_arrive_expect_tx(&fullb[b], BBYTES);
 #pragma unroll
-        for (int kc = 0; kc < KC; ++kc)
-            tma_load_2d(B + (size_t)b * BBYTES + (size_t)kc * CT_N * 128, &tmB, kc * 64, j * CT_N,
-                        &fullb[b]);
-        fpend |= 1u << b;
-    };
-    auto wait_full = [&](int b) {
-        const bool g = mbar_wait_bounded(&fullb[b], (fph >> b) & 1u, err);
-        fph ^= 1u << b;
-        fpend &= ~(1u << b);
-        return g;
-    };
-    auto issue_mma = [&](int b) {  // B buffer b -> TMEM buffer b
-        const uint32_t abase = smem_u32(A), bbase = smem_u32(B + (size_t)b * BBYTES);
+                for (int pp = 0; pp < PARTS; ++pp)
 #pragma unroll
-        for (int kc = 0; kc < KC; ++kc)
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-                mma_bf16(tbase + b * CT_N, smem_desc_sw128(abase + kc * CT_M * 128 + ks * 32, 1024),
-                         smem_desc_sw128(bbase + kc * CT_N * 128 + ks * 32, 1024), idesc,
-                         (kc | ks) != 0);
-        mma_commit(&mmab[b]);
-        mpend |= 1u << b;
-    };
-    auto wait_mma = [&](int b) {
-        const bool g = mbar_wait_bounded(&mmab[b], (mph >> b) & 1u, err);
-        mph ^= 1u << b;
-        mpend &= ~(1u << b);
-        return g;
-    };
-
-    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const int row0 = tile * CT_M;
-        if (tid == 0) {
-            load_b(0, 0);
-            load_b(1 % nch, 1);
+                    for (int kc = 0; kc < KC; ++kc)
+                        tma_load_2d(B + b * BBYTES + pp * PBYTES + (size_t)kc * CN * 128,
+                                    pp ? &tmBlo : &tmB, kc * 64, j * CN, &fullb[b]);
+            }
+            // the copies issued last have landed before exit
+            for (uint32_t t = g > NB ? g - NB : 0; t < g; ++t)
+                mbar_wait_bounded(&fullb[t % NB], (t / NB) & 1, err);
         }
-        // A: the tile's rows rounded to BF16, zero past m or d.  The KC * 8
-        // chunks of a row sit in consecutive lanes: their sums of squares
-        // reduce by shuffles into the row's ||x|| bound
-        constexpr int nA = CT_M * KC * 8, W = KC * 8;
-        const float fx = 1.f + 4.f * (float)d * 5.9604645e-08f;
-        static_assert(nA % CF_NT == 0 || CF_NT % nA == 0, "whole warps per A pass");
-        for (int e0 = tid; e0 < nA; e0 += CF_NT * CT_AU) {
-            float4 f0[CT_AU], f1[CT_AU];
+        __syncwarp();
+    } else if (warp == CF_EPI / 32) {
+        // ---- MMAs (one lane)
+        if (lane == 0) {
+            const uint32_t steps = mine * (uint32_t)nch;
+            const uint32_t idesc = mma_idesc(1, 1, CT_M, CN);
+            const uint32_t abase = smem_u32(A);
+            uint32_t g = 0;
+            for (; g < steps; ++g) {
+                const uint32_t b = g % NB, tb = g % TB, ut = g / TB;
+                bool ok = mbar_wait_ab(&fullb[b], (g / NB) & 1, err, s_abort, kWaitNs);
+                if (ok && g % (uint32_t)nch == 0)  // the tile's rows are stored
+                    ok = mbar_wait_ab(&afull, (g / (uint32_t)nch) & 1, err, s_abort, kWaitNs);
+                if (ok && ut >= 1)  // this TMEM buffer has been read
+                    ok = mbar_wait_ab(&tempty[tb], (ut - 1) & 1, err, s_abort, kWaitNs);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t bbase = smem_u32(B + b * BBYTES);
+                // products: (x hi, c hi), then for the split (x hi, c lo), (x lo, c hi)
 #pragma unroll
-            for (int u = 0; u < CT_AU; ++u) {
-                const int e = e0 + u * CF_NT;
-                const int r = e / W, kc = (e >> 3) % KC, c = e & 7;
-                const int k0 = kc * 64 + c * 8;
+                for (int pr = 0; pr < (PARTS == 2 ? 3 : 1); ++pr) {
+                    const uint32_t ap = abase + (pr == 2 ? ABYTES : 0u);
+                    const uint32_t bp = bbase + (pr == 1 ? PBYTES : 0u);
+#pragma unroll
+                    for (int kc = 0; kc < KC; ++kc)
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_bf16(tbase + tb * CN,
+                                     smem_desc_sw128(ap + kc * CT_M * 128 + ks * 32, 1024),
+                                     smem_desc_sw128(bp + kc * CN * 128 + ks * 32, 1024), idesc,
+                                     (pr | kc | ks) != 0);
+                }
+                mma_commit(&freeb[b]);
+                mma_commit(&mmab[tb]);
+            }
+            // the last products are written before TMEM is released
+            if (g > 0) mbar_wait_bounded(&mmab[(g - 1) % TB], ((g - 1) / TB) & 1, err);
+        }
+        __syncwarp();
+    } else {
+        // ---- rows in, epilogue
+        const int q = warp & 3, sub = warp >> 2, rloc = q * 32 + lane;
+        constexpr int W = KC * 8;                  // 16-byte chunks of a row
+        constexpr int AU = CT_M * W / CF_EPI;      // chunks per thread: 2 KC
+        float4 f0[AU], f1[AU];
+        auto fetch = [&](int tile) {               // the tile's rows, zero past m or d
+#pragma unroll
+            for (int u = 0; u < AU; ++u) {
+                const int e = tid + u * CF_EPI, r = e / W, k0 = (e & (W - 1)) * 8;
+                const int row = tile * CT_M + r;
                 f0[u] = f1[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (e < nA && row0 + r < m && k0 < d) {
-                    const float4 *xr = reinterpret_cast<const float4 *>(x + (size_t)(row0 + r) * d + k0);
+                if (row < m && k0 < d) {
+                    const float4 *xr = reinterpret_cast<const float4 *>(x + (size_t)row * d + k0);
                     f0[u] = __ldg(xr);
                     f1[u] = __ldg(xr + 1);
                 }
             }
+        };
+        const float fx = 1.f + 4.f * (float)d * 5.9604645e-08f;
+        auto store = [&](int par) {                // rounded (and split) into A; the norms
 #pragma unroll
-            for (int u = 0; u < CT_AU; ++u) {
-                const int e = e0 + u * CF_NT;
-                if (e >= nA) break;  // warp-uniform: nA is a multiple of CF_NT / 2
-                const int r = e / W, kc = (e >> 3) % KC, c = e & 7;
+            for (int u = 0; u < AU; ++u) {
+                const int e = tid + u * CF_EPI, r = e / W, kc = (e >> 3) % KC, c = e & 7;
                 const float f[8] = {f0[u].x, f0[u].y, f0[u].z, f0[u].w,
                                     f1[u].x, f1[u].y, f1[u].z, f1[u].w};
-                uint32_t w[4];
+                uint32_t w[4], wl[4];
                 float sq = 0.f;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * t], f[2 * t + 1]);
                     w[t] = *reinterpret_cast<uint32_t *>(&h);
+                    if (PARTS == 2) {
+                        __nv_bfloat162 l = __floats2bfloat162_rn(f[2 * t] - __low2float(h),
+                                                                 f[2 * t + 1] - __high2float(h));
+                        wl[t] = *reinterpret_cast<uint32_t *>(&l);
+                    }
                     sq = fmaf(f[2 * t], f[2 * t], sq);
                     sq = fmaf(f[2 * t + 1], f[2 * t + 1], sq);
                 }
-                *reinterpret_cast<uint4 *>(A + (size_t)kc * CT_M * 128 + (size_t)(r >> 3) * 1024 +
-                                           (r & 7) * 128 + ((c ^ (r & 7)) << 4)) =
-                    make_uint4(w[0], w[1], w[2], w[3]);
+                unsigned char *o = A + (size_t)kc * CT_M * 128 + (size_t)(r >> 3) * 1024 +
+                                   (r & 7) * 128 + ((c ^ (r & 7)) << 4);
+                *reinterpret_cast<uint4 *>(o) = make_uint4(w[0], w[1], w[2], w[3]);
+                if (PARTS == 2)
+                    *reinterpret_cast<uint4 *>(o + ABYTES) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+                // the W chunks of a row sit in consecutive lanes
 #pragma unroll
-                for (int o = W >> 1; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-                if ((lane & (W - 1)) == 0) sxn[r] = __fsqrt_ru(__fmul_ru(sq, fx));
+                for (int s = W >> 1; s > 0; s >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, s);
+                if ((lane & (W - 1)) == 0) sxn[par][r] = __fsqrt_ru(__fmul_ru(sq, fx));
+            }
+            fence_proxy_async_smem();  // A (generic stores) is read by the MMAs
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&afull);
+        };
+        fetch((int)blockIdx.x);
+        store(0);
+        {  // ||c||^2 (lists past L far away) and the maxima
+            float a0 = 0.f, a1 = 0.f;
+            for (int c = tid; c < nch * CN; c += CF_EPI) {
+                const float v = c < L ? __ldg(cn + c) : 3.0e38f;
+                scn[c] = v;
+                if (c < L) {
+                    a0 = fmaxf(a0, v);
+                    a1 = fmaxf(a1, __ldg(cnrm_up + c));
+                }
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                a0 = fmaxf(a0, __shfl_xor_sync(0xffffffffu, a0, o));
+                a1 = fmaxf(a1, __shfl_xor_sync(0xffffffffu, a1, o));
+            }
+            if (lane == 0) {
+                atomicMax(&smax[0], __float_as_uint(a0));
+                atomicMax(&smax[1], __float_as_uint(a1));
             }
         }
-        fence_proxy_async_smem();  // A (generic stores) is read by the MMAs
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        bool got = true;  // thread 0: every wait so far succeeded
-        if (tid == 0) {
-            got = wait_full(0);
-            if (got) issue_mma(0);
-        }
-        const float xn = sxn[rloc];
-        // pass 1: smallest, second smallest and largest Dt, the smallest's list
-        float d1 = INFINITY, d2 = INFINITY, dmax = -INFINITY, T = INFINITY, thr = -INFINITY;
-        int c1 = -1, n = 0;
-        bool ovf = false, done = false;
-        for (int s = 0; s < nsteps; ++s) {
-            const int b = s & 1, j = s % nch;
-            if (tid == 0 && got) got = wait_mma(b);
-            // MMA s is done and every thread has finished epilogue s - 1
-            if (__syncthreads_or(!got)) {
-                ok = false;
+        named_bar_sync(1, CF_EPI);
+        const float cnmax = __uint_as_float(smax[0]), cmax = __uint_as_float(smax[1]);
+        uint32_t g = 0;
+        bool ok = true;
+        for (uint32_t t = 0; t < mine; ++t) {
+            const int tile = (int)(blockIdx.x + t * gridDim.x), row = tile * CT_M + rloc;
+            const int par = (int)(t & 1);
+            const bool more = t + 1 < mine;
+            if (more) fetch(tile + (int)gridDim.x);
+            // the best three groups (key, second key in it, group) and the
+            // best key of the others
+            float dg[3], sg[3], d4 = 3.3e38f;
+            int gi[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                dg[i] = sg[i] = 3.3e38f;
+                gi[i] = 0;
+            }
+            for (int j = 0; j < nch; ++j, ++g) {
+                const uint32_t b = g % TB;
+                ok = __all_sync(0xffffffffu, ok && mbar_wait_ab(&mmab[b], (g / TB) & 1, err, s_abort,
+                                                                kWaitNs));
+                tc_fence_after();
+                if (j == nch - 1 && more && ok) store(par ^ 1);  // this tile's MMAs are done
+                if (ok) {
+                    const uint32_t tad = tbase + b * CN + sub * 16 + ((uint32_t)(q * 32) << 16);
+                    float vv[2][16];
+                    tmem_ld16(tad, vv[0]);
+#pragma unroll
+                    for (int k = 0; k < CN / 64; ++k) {
+                        const int grp = j * (CN / 16) + sub + 4 * k;
+                        const float4 *cv4 = reinterpret_cast<const float4 *>(scn + grp * 16);
+                        float (&v)[16] = vv[k & 1];
+                        tmem_ld_wait(v);
+                        if (k + 1 < CN / 64)  // the next group's load runs under this one
+                            tmem_ld16(tad + (k + 1) * 64, vv[(k + 1) & 1]);
+                        float lo[8], hi[8];
+#pragma unroll
+                        for (int i4 = 0; i4 < 4; ++i4) {
+                            const float4 cv = cv4[i4];
+                            const float c4[4] = {cv.x, cv.y, cv.z, cv.w};
+                            float e[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const float Dt = fmaf(-2.f, v[4 * i4 + i], c4[i]);
+                                e[i] = __uint_as_float((__float_as_uint(Dt) & ~15u) |
+                                                       (uint32_t)(4 * i4 + i));
+                            }
+                            lo[2 * i4] = fminf(e[0], e[1]);
+                            hi[2 * i4] = fmaxf(e[0], e[1]);
+                            lo[2 * i4 + 1] = fminf(e[2], e[3]);
+                            hi[2 * i4 + 1] = fmaxf(e[2], e[3]);
+                        }
+#pragma unroll
+                        for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+                            for (int i = 0; i < w; ++i) {
+                                const float mx = fmaxf(lo[2 * i], lo[2 * i + 1]);
+                                hi[i] = min3f(hi[2 * i], hi[2 * i + 1], mx);
+                                lo[i] = fminf(lo[2 * i], lo[2 * i + 1]);
+                            }
+                        // insert the group into the sorted three
+                        float mv = lo[0], ms = hi[0];
+                        int mg = grp;
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) {
+                            const bool lt = mv < dg[i];
+                            const float td = dg[i], ts = sg[i];
+                            const int tg = gi[i];
+                            dg[i] = lt ? mv : td;
+                            sg[i] = lt ? ms : ts;
+                            gi[i] = lt ? mg : tg;
+                            mv = lt ? td : mv;
+                            ms = lt ? ts : ms;
+                            mg = lt ? tg : mg;
+                        }
+                        d4 = fminf(d4, mv);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tempty[b]);
+            }
+            const int c1 = gi[0] * 16 + (int)(__float_as_uint(dg[0]) & 15u);
+            sMin[par][sub][rloc] = dg[0];
+            sSec[par][sub][rloc] = fminf(sg[0], dg[1]);
+            sArg[par][sub][rloc] = c1;
+            ok = named_bar_and(1, CF_EPI, ok && !*s_abort);
+            if (!ok) {
+                // a wait ran out (the sticky error word is set): the rows left
+                // get list 0, so that nothing downstream reads garbage
+                for (uint32_t t2 = t; t2 < mine; ++t2) {
+                    const int r = (int)(blockIdx.x + t2 * gridDim.x) * CT_M + rloc;
+                    if (sub == 0 && r < m) out1[r] = 0;
+                }
                 break;
             }
-            tc_fence_after();
-            if (tid == 0) {
-                if (s + 1 < nsteps) {  // TMEM buffer b ^ 1 is free: MMA s + 1 under this epilogue
-                    got = wait_full(b ^ 1);
-                    if (got) issue_mma(b ^ 1);
-                }
-                if (got && s + 2 < nsteps) load_b((s + 2) % nch, b);  // MMA s has read buffer b
+            int kmin = 0;
+            float mn = sMin[par][0][rloc];
+#pragma unroll
+            for (int k = 1; k < CF_SUB; ++k) {
+                const float v = sMin[par][k][rloc];
+                if (v < mn) kmin = k;
+                mn = fminf(mn, v);
             }
-            for (int c16 = sub; c16 < CT_N / 16; c16 += CF_SUB) {  // warp-uniform
-                const int cb0 = j * CT_N + c16 * 16;
-                if (cb0 >= L) break;
-                const int nv = min(16, L - cb0);
-                float v[16], cv[16];
-                tmem_ld16(tbase + b * CT_N + c16 * 16 + ((uint32_t)(q * 32) << 16), v);
-                if (nv == 16) {
+            float second = sSec[par][kmin][rloc];
 #pragma unroll
-                    for (int i4 = 0; i4 < 4; ++i4) {
-                        const float4 t = __ldg(reinterpret_cast<const float4 *>(cn + cb0) + i4);
-                        cv[4 * i4] = t.x;
-                        cv[4 * i4 + 1] = t.y;
-                        cv[4 * i4 + 2] = t.z;
-                        cv[4 * i4 + 3] = t.w;
-                    }
-                } else {
+            for (int k = 0; k < CF_SUB; ++k)
+                if (k != kmin) second = fminf(second, sMin[par][k][rloc]);
+            // Ebig: the bound at the maxima, every step rounded up, times
+            // 1 + 2^-10 (covers the roundings of the bound itself)
+            const float xn = sxn[par][rloc];
+            const float ab = __fadd_ru(cnmax, __fmul_ru(__fmul_ru(2.04f, xn), cmax));
+            const float t1 = __fmul_ru(5.9604645e-08f, __fadd_ru(cnmax, ab));
+            const float t2 = __fmul_ru(__fmul_ru(g1, xn), cmax);
+            const float eb = __fadd_ru(
+                __fmul_ru(__fmul_ru(2.f, __fadd_ru(t1, t2)), 1.f + 1.f / 1024.f), 1e-30f);
+            const float delta = __fadd_ru(__fmul_ru(ab, 1.9073486e-06f), 1e-36f);  // 2^-19
+            const float T = __fadd_ru(__fadd_ru(mn, delta), eb);
+            // RN(Dt - E) <= T needs Dt < T + E + ulp(T) <= thr - delta
+            const float thr = __fadd_ru(__fadd_ru(__fadd_ru(T, eb), delta),
+                                        __fadd_ru(__fmul_ru(fabsf(T), 1.2e-7f), 1e-30f));
+            const bool decided = !(second <= thr) && mn <= thr;
+            if (decided && sub == 0 && row < m) out1[row] = sArg[par][kmin][rloc];
+            if (!named_bar_or(1, CF_EPI, !decided && row < m)) continue;
+            // undecided rows: each thread's lists that can qualify (a whole group
+            // may reach past L, whose lists never qualify)
+            int nl[3], nmine = 0;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) cv[i] = i < nv ? __ldg(cn + cb0 + i) : 0.f;
+            for (int i = 0; i < 3; ++i) {
+                nl[i] = !(dg[i] <= thr) ? 0 : sg[i] <= thr ? max(0, min(16, L - gi[i] * 16)) : 1;
+                nmine += nl[i];
+            }
+            sn[sub][rloc] = d4 <= thr ? -1 : nmine;
+            named_bar_sync(1, CF_EPI);
+            int h = -1, before = 0, total = 0;
+            if (!decided && row < m) {
+                bool redo = false;
+#pragma unroll
+                for (int k = 0; k < CF_SUB; ++k) {
+                    const int nk = sn[k][rloc];
+                    redo |= nk < 0;
+                    before += k < sub ? nk : 0;
+                    total += nk;
                 }
-                tmem_ld_wait(v);
-                if (s < nch) {
-                    auto see = [&](float Dt, int c) {
-                        const bool lt = Dt < d1;
-                        d2 = fminf(d2, lt ? d1 : Dt);
-                        c1 = lt ? c : c1;
-                        d1 = fminf(d1, Dt);
-                        dmax = fmaxf(dmax, Dt);
-                    };
-                    if (nv == 16) {
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) see(fmaf(-2.f, v[i], cv[i]), cb0 + i);
+                if (sub == 0) {
+                    redo |= total > CF_CAP;
+                    if (!redo) {
+                        h = atomicAdd(nhard, 1);
+                        redo = h >= cap;
+                        if (redo) h = -1;
+                    }
+                    if (redo) {
+                        hard[m - 1 - atomicAdd(nhard + 1, 1)] = row;
                     } else {
-#pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                            if (i < nv) see(fmaf(-2.f, v[i], cv[i]), cb0 + i);
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const float Dt = fmaf(-2.f, v[i], cv[i]);
-                        if (!(i < nv && Dt <= thr)) continue;
-                        const int c = cb0 + i;
-                        const float E = bound_of(Dt, cv[i], __ldg(cnrm_up + c), xn, g1);
-                        if (!(lower_of(Dt, E) <= T)) continue;
-                        if (n < CF_CAP) rc[n * CF_NT + tid] = c;
-                        else ovf = true;
-                        ++n;
+                        hard[h] = row;
+                        outS[(size_t)h * CF_STRIDE] = total;
                     }
                 }
             }
-            if (s == nch - 1) {  // end of pass 1: the row's T and quick-reject threshold
-                sMin[sub][rloc] = d1;
-                sSec[sub][rloc] = d2;
-                sMax[sub][rloc] = dmax;
-                sArg[sub][rloc] = c1;
-                __syncthreads();
-                int kmin = 0;
-                float mn = sMin[0][rloc], mx = sMax[0][rloc];
+            if (sub == 0) sArg[par][0][rloc] = h;  // the row's record, for its other threads
+            named_bar_sync(1, CF_EPI);
+            if (!decided && row < m) {
+                h = sArg[par][0][rloc];
+                if (h >= 0) {
+                    int32_t *o = outS + (size_t)h * CF_STRIDE + 1 + before;
 #pragma unroll
-                for (int k = 1; k < CF_SUB; ++k) {
-                    if (sMin[k][rloc] < mn) kmin = k;
-                    mn = fminf(mn, sMin[k][rloc]);
-                    mx = fmaxf(mx, sMax[k][rloc]);
-                }
-                float second = sSec[kmin][rloc];
-#pragma unroll
-                for (int k = 0; k < CF_SUB; ++k)
-                    if (k != kmin) second = fminf(second, sMin[k][rloc]);
-                const float ab = fmaxf(fabsf(mn), fabsf(mx));
-                // Ebig: the bound at the maxima, every step rounded up, times
-                // 1 + 2^-10 (covers the roundings of the bound itself)
-                const float t1 = __fmul_ru(5.9604645e-08f, __fadd_ru(__uint_as_float(smax[0]), ab));
-                const float t2 = __fmul_ru(__fmul_ru(g1, xn), __uint_as_float(smax[1]));
-                const float eb = __fadd_ru(
-                    __fmul_ru(__fmul_ru(2.f, __fadd_ru(t1, t2)), 1.f + 1.f / 1024.f), 1e-30f);
-                T = __fadd_ru(mn, eb);
-                // RN(Dt - E) <= T needs Dt < T + E + ulp(T) <= thr
-                thr = __fadd_ru(__fadd_ru(T, eb), __fadd_ru(__fmul_ru(fabsf(T), 1.2e-7f), 1e-30f));
-                // decided: no list but the argmin has Dt <= thr
-                const bool decided = !(second <= thr) && mn <= thr;
-                if (!__syncthreads_or(!decided && row0 + rloc < m)) {
-                    if (sub == 0 && row0 + rloc < m) out1[row0 + rloc] = sArg[kmin][rloc];
-                    if (tid == 0)  // the pass-2 copy and MMA already issued are waited for
-                        for (int i = 0; i < 2; ++i) {
-                            if ((fpend >> i) & 1u) got &= wait_full(i);
-                            if ((mpend >> i) & 1u) got &= wait_mma(i);
-                        }
-                    done = true;
-                    break;
+                    for (int i = 0; i < 3; ++i) {
+                        const bool whole = sg[i] <= thr;
+                        const int first = gi[i] * 16 + (whole ? 0 : (int)(__float_as_uint(dg[i]) & 15u));
+                        for (int k = 0; k < nl[i]; ++k) *o++ = min(first + k, L - 1);
+                    }
                 }
             }
-            tc_fence_before();
         }
-        if (!ok) break;
-        if (done) {
-            if (__syncthreads_or(!got)) ok = false;  // a drain wait ran out
-            continue;                                // sMin ... are rewritten after a barrier
-        }
-        sn[sub][rloc] = ovf ? -1 : n;
-        __syncthreads();
-        const int r = row0 + rloc;
-        if (r < m) {
-            int32_t *o = outS + (size_t)r * CF_STRIDE;
-            int before = 0, total = 0;
-            bool bad = false;
-#pragma unroll
-            for (int k = 0; k < CF_SUB; ++k) {
-                const int nk = sn[k][rloc];
-                bad |= nk < 0;
-                before += k < sub ? nk : 0;
-                total += nk;
-            }
-            if (!bad && total == 1) {
-                if (n == 1) out1[r] = rc[tid];
-            } else {
-                if (bad) {
-                    if (sub == 0) o[0] = -1;
-                } else {
-                    for (int k = 0; k < n; ++k) o[1 + before + k] = rc[k * CF_NT + tid];
-                    if (sub == 0) o[0] = total;
-                }
-                if (sub == 0) hard[atomicAdd(nhard, 1)] = r;
-            }
-        }
-        __syncthreads();  // sxn, sMin, sMax, sn, the lists and A are reused by the next tile
-    }
-    if (!ok) {
-        // a wait ran out: thread 0 waits (bounded) for its copies and MMAs
-        // still in flight; every row of this CTA's tiles goes to the full
-        // selection
-        if (tid == 0)
-            for (int i = 0; i < 2; ++i) {
-                if ((fpend >> i) & 1u) wait_full(i);
-                if ((mpend >> i) & 1u) wait_mma(i);
-            }
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-            for (int r = tile * CT_M + tid; r < min(m, tile * CT_M + CT_M); r += CF_NT) {
-                outS[(size_t)r * CF_STRIDE] = -1;
-                hard[atomicAdd(nhard, 1)] = r;
-            }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) tmem_dealloc(tbase, 2 * CT_N);
+    if (warp == CF_EPI / 32) tmem_dealloc(tbase, TB * CN);
 }
 
-// TMA descriptor of the BF16 centroids for the fused first stage: boxes of
-// 64 columns x CT_N rows, 128-byte swizzle; rows past nlist read as zero.
+// TMA descriptors of the BF16 centroids (and of their low parts) for the
+// fused first stage: boxes of 64 columns x CF_CN rows, 128-byte swizzle;
+// rows past nlist and columns past d read as zero.
 bool coarse_make_map(sivf_index *ix)
 {
     const int d = ix->d;
-    if (!ix->cent_bf16 || d < 64 || d > 128 || d % 16) return false;
+    if (!ix->cent_bf16 || !ix->cent_lo || d > 128 || d % 16) return false;
     auto enc = tmap_encode_fn();
     if (!enc) return false;
     cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)ix->nlist};
     cuuint64_t strides[1] = {(cuuint64_t)d * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)CT_N};
+    cuuint32_t box[2] = {64, (cuuint32_t)CF_CN};
     cuuint32_t es[2] = {1, 1};
-    return enc(reinterpret_cast<CUtensorMap *>(ix->tmap_cent), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-               ix->cent_bf16, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    auto make = [&](unsigned char *map, void *base) {
+        return enc(reinterpret_cast<CUtensorMap *>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base,
+                   dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    return make(ix->tmap_cent, ix->cent_bf16) && make(ix->tmap_cent_lo, ix->cent_lo);
 }
 
 // ----------------------------------------------- warp-per-row selection
@@ -952,17 +1039,14 @@ bool coarse_make_map(sivf_index *ix)
 // (sorted, in registers), the warp extracts the P-th smallest of their
 // union as T, then gathers S, tests the sure members and re-decides the
 // rest in FP64 exactly as above.  Rows whose S exceeds CW_SCAP take the
-// serial FP64 path.  FROM_S: the candidate set comes from the fused first
-// stage (a superset of S for its BF16 bound); a row it marked as overflowed
-// is selected from all lists with FP32 distances computed here.
+// serial FP64 path.
 constexpr int CW_ROWS = 4;     // rows (warps) per block
 constexpr int CW_PMAX = 8;
 constexpr int CW_SCAP = 128;
-constexpr int CW_LMAX = 4096;  // most lists for one warp per row
 constexpr int CW_RG = 4;       // FP32 rechecks in flight per warp
 
 // PM: length of each lane's sorted list (1 when P = 1, else CW_PMAX)
-template <int PM, bool FROM_S>
+template <int PM>
 __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_select_w(SelArgs a)
 {
     pdl_begin();
@@ -976,54 +1060,16 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_select_w(SelArgs a)
     __shared__ __align__(16) float sX[CW_ROWS][kMaxD];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int L = a.L, P = a.P;
-    const int nrows = FROM_S ? *a.nhard : a.m;
-    for (int it = blockIdx.x * CW_ROWS + w; it < nrows; it += gridDim.x * CW_ROWS) {  // whole warps
-        const int row = FROM_S ? a.hard[it] : it;
-        const float *Dr = FROM_S ? nullptr : a.D + (size_t)row * L;
+    for (int row = blockIdx.x * CW_ROWS + w; row < a.m; row += gridDim.x * CW_ROWS) {  // whole warps
+        const float *Dr = a.D + (size_t)row * L;
         const float *xr = a.x + (size_t)row * a.d;
-        int two_level = a.two_level;
-        float g1 = two_level ? a.gamma2_first : a.gamma2;
-
-        // ||x|| upper bound from an FP64 sum
-        double part = 0.0;
-        for (int j = lane; j < a.d; j += 32) part += (double)xr[j] * (double)xr[j];
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        const float xn = __double2float_ru(sqrt(part) * (1.0 + 1e-12));
-
-        // first-stage distance of list c: the approximate matrix, or for a row
-        // the fused first stage could not record, an FP32 dot product (one lane)
+        const int two_level = a.two_level;
+        const float g1 = two_level ? a.gamma2_first : a.gamma2;
+        float part = 0.f;
+        for (int j = lane; j < a.d; j += 32) part = fmaf(xr[j], xr[j], part);
+        const float xn = norm_up(warp_sum(part), a.d);
         int ns = 0;
-        bool have_s = false;
-        if (FROM_S) {
-            for (int j = lane; j < a.d; j += 32) sX[w][j] = xr[j];
-            const int32_t *Sr = a.S + (size_t)row * a.s_stride;
-            const int n0 = Sr[0];
-            if (n0 >= 0 && n0 <= CW_SCAP) {
-                for (int p = lane; p < n0; p += 32) sIdx[w][p] = Sr[1 + p];
-                ns = n0;
-                have_s = true;
-            } else {
-                two_level = 0;
-                g1 = a.gamma2;
-            }
-            __syncwarp();
-        }
-        auto dt_of = [&](int c) -> float {
-            if (!FROM_S) return __ldg(Dr + c);
-            const float4 *x4 = reinterpret_cast<const float4 *>(sX[w]);
-            const float4 *c4 = reinterpret_cast<const float4 *>(a.cent + (size_t)c * a.d);
-            float acc = 0.f;
-            for (int j4 = 0; j4 < (a.d >> 2); ++j4) {
-                const float4 xv = x4[j4], cv = __ldg(c4 + j4);
-                acc = fmaf(xv.x, cv.x, acc);
-                acc = fmaf(xv.y, cv.y, acc);
-                acc = fmaf(xv.z, cv.z, acc);
-                acc = fmaf(xv.w, cv.w, acc);
-            }
-            for (int j = a.d & ~3; j < a.d; ++j)
-                acc = fmaf(sX[w][j], __ldg(a.cent + (size_t)c * a.d + j), acc);
-            return fmaf(-2.f, acc, __ldg(a.cn + c));
-        };
+        auto dt_of = [&](int c) -> float { return __ldg(Dr + c); };
 
         // P-th smallest of the values v(i), i < n, each lane keeping its
         // CW_PMAX smallest in a sorted register list
@@ -1070,15 +1116,14 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_select_w(SelArgs a)
         };
 
         // T = P-th smallest upper bound over all lists
-        float T = INFINITY;
-        if (!have_s) T = pth_smallest([&](int c) {
+        float T = pth_smallest([&](int c) {
             const float Dt = dt_of(c);
             return upper_of(Dt, bound_of(Dt, __ldg(a.cn + c), __ldg(a.cnrm_up + c), xn, g1));
         }, L);
 
         // candidate set S = {c : lower bound <= T}
         constexpr int CU = 8;
-        for (int c00 = 0; c00 < (have_s ? 0 : L); c00 += 32 * CU) {
+        for (int c00 = 0; c00 < L; c00 += 32 * CU) {
             float lbv[CU], ubv[CU], dtv[CU];
 #pragma unroll
             for (int u = 0; u < CU; ++u) {
@@ -1154,7 +1199,7 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_select_w(SelArgs a)
                     const int c = sIdx[w][p];
                     const float cnc = __ldg(a.cn + c);
                     const float Dt = fmaf(-2.f, acc, cnc);
-                    const float E = bound_of(Dt, cnc, __ldg(a.cnrm_up + c), xn, a.gamma2);
+                    const float E = bound_of(Dt, cnc, __ldg(a.cnrm_up + c), xn, a.gamma2_re);
                     sLB[w][p] = lower_of(Dt, E);
                     sUB[w][p] = upper_of(Dt, E);
                     sDt[w][p] = Dt;
@@ -1296,6 +1341,208 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_select_w(SelArgs a)
             }
         }
         __syncwarp();  // the warp's shared rows are reused by its next row
+    }
+}
+
+// Roundings of a dot product of d values whose partial sums a warp holds
+// (float4s lane, lane + 32, ... accumulated by fused multiply-adds) and adds
+// by five shuffles: its error is at most gamma_n sum |x_j c_j| with n =
+// 4 ceil(d / 128) + 5, against n = d for one running sum.  At d = 128 that
+// leaves a fourteenth of the near-ties to the FP64 step, whose dependent
+// FP64 additions are what an undecided row costs most.
+__host__ __device__ constexpr int re_ops(int d) { return 4 * ((d + 127) / 128) + 5; }
+
+// Finishing selection of the rows the fused first stage left undecided (P =
+// 1).  With a record, one warp per row: the FP32 distance of each candidate
+// list (CW_RG at a time, lanes over the coordinates), one list per lane; the
+// lists whose lower bound is at most the smallest upper bound remain, and if
+// they are several, their FP64 distances decide (ties to the lower index).
+// A row to redo takes a block: its warps read all lists' rows, FN_RG in
+// flight each, into one table of distances (a warp alone, list after list,
+// took 1.2 ms at 2,048 lists, the tail of the launch).
+constexpr int FN_RG = 8;
+__global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_finish(SelArgs a)
+{
+    pdl_begin();
+    __shared__ __align__(16) float sX[CW_ROWS][kMaxD];
+    __shared__ float sD[CW_LMAX];
+    __shared__ float sT[CW_ROWS];
+    __shared__ double sB[CW_ROWS];
+    __shared__ int sC[CW_ROWS];
+    __shared__ int s_found, s_one;
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int L = a.L, d = a.d, n4 = d >> 2;
+    const int nrec = min(a.nhard[0], a.s_cap), nredo = a.nhard[1];
+    auto load_x = [&](const float *xr, float *to) {  // the row; its norm's bound
+        float part = 0.f;
+        for (int j = lane; j < d; j += 32) {
+            const float v = xr[j];
+            to[j] = v;
+            part = fmaf(v, v, part);
+        }
+        return norm_up(warp_sum(part), d);
+    };
+    // partial dot product of list c's row with the row x4, this lane's share
+    auto share = [&](const float4 *x4, int c) {
+        const float4 *c4 = reinterpret_cast<const float4 *>(a.cent + (size_t)c * d);
+        float s = 0.f;
+#pragma unroll
+        for (int u = 0; u < kMaxD / 128; ++u) {
+            const int j4 = lane + 32 * u;
+            if (j4 >= n4) break;
+            const float4 xv = x4[j4], cv = __ldg(c4 + j4);
+            s = fmaf(xv.x, cv.x, s);
+            s = fmaf(xv.y, cv.y, s);
+            s = fmaf(xv.z, cv.z, s);
+            s = fmaf(xv.w, cv.w, s);
+        }
+        return s;
+    };
+    auto bounds = [&](int c, float Dt, float xn, float &lb, float &ub) {
+        const float E = bound_of(Dt, __ldg(a.cn + c), __ldg(a.cnrm_up + c), xn, a.gamma2_re);
+        lb = lower_of(Dt, E);
+        ub = upper_of(Dt, E);
+    };
+    auto fmin_warp = [&](float v) {
+        for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+        return v;
+    };
+    double bd = INFINITY;  // the best of this thread's lists, by FP64 distance and index
+    int bc = 0x7fffffff;
+    auto better = [&](double D, int c) {
+        if (D < bd || (D == bd && c < bc)) {
+            bd = D;
+            bc = c;
+        }
+    };
+    auto best_warp = [&]() {
+        for (int o = 16; o > 0; o >>= 1) {
+            const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+            const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
+            better(od, oc);
+        }
+    };
+    auto write = [&](int row, int c) {
+        if (c < 0 || c >= L) {
+            atomicOr(a.err, ERR_SELECT);
+            c = -1;
+        }
+        a.out[row] = c;
+    };
+
+    for (int it = blockIdx.x * CW_ROWS + w; it < nrec; it += gridDim.x * CW_ROWS) {  // whole warps
+        const int row = a.hard[it];
+        const int32_t *Sr = a.S + (size_t)it * CF_STRIDE;
+        const int n0 = min(Sr[0], CF_CAP);
+        const int c = lane < n0 ? Sr[1 + lane] : 0;
+        const float *xr = a.x + (size_t)row * d;
+        __syncwarp();  // the warp's sX is still read for its last row
+        const float xn = load_x(xr, sX[w]);
+        __syncwarp();
+        const float4 *x4 = reinterpret_cast<const float4 *>(sX[w]);
+        float dot = 0.f;
+        for (int p0 = 0; p0 < n0; p0 += CW_RG) {
+            float s[CW_RG];
+#pragma unroll
+            for (int t = 0; t < CW_RG; ++t) {
+                const int ct = __shfl_sync(0xffffffffu, c, p0 + t);
+                s[t] = p0 + t < n0 ? share(x4, ct) : 0.f;  // warp-uniform
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int t = 0; t < CW_RG; ++t) s[t] += __shfl_xor_sync(0xffffffffu, s[t], o);
+#pragma unroll
+            for (int t = 0; t < CW_RG; ++t)
+                if (lane == p0 + t) dot = s[t];
+        }
+        float lb = INFINITY, ub = INFINITY;
+        if (lane < n0) bounds(c, fmaf(-2.f, dot, __ldg(a.cn + c)), xn, lb, ub);
+        const float T = fmin_warp(ub);
+        const bool in = lane < n0 && lb <= T;
+        const uint32_t mk = __ballot_sync(0xffffffffu, in);
+        int chosen = -1;
+        if (__popc(mk) == 1) {
+            chosen = __shfl_sync(0xffffffffu, c, __ffs(mk) - 1);
+        } else if (mk) {
+            bd = INFINITY;
+            bc = 0x7fffffff;
+            if (in) better(exact_dist(xr, a.cent + (size_t)c * d, d), c);
+            best_warp();
+            chosen = bc;
+        }
+        if (lane == 0) write(row, chosen);
+    }
+
+    for (int it = blockIdx.x; it < nredo; it += gridDim.x) {
+        const int row = a.hard[a.m - 1 - it];
+        const float *xr = a.x + (size_t)row * d;
+        __syncthreads();  // the tables are still read for the last row
+        const float xn = load_x(xr, sX[w]);
+        if (tid == 0) {
+            s_found = 0;
+            s_one = -1;
+        }
+        __syncwarp();
+        const float4 *x4 = reinterpret_cast<const float4 *>(sX[w]);
+        float T = INFINITY;
+        for (int c0 = w * FN_RG; c0 < L; c0 += CW_ROWS * FN_RG) {
+            float s[FN_RG];
+#pragma unroll
+            for (int t = 0; t < FN_RG; ++t) s[t] = share(x4, min(c0 + t, L - 1));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int t = 0; t < FN_RG; ++t) s[t] += __shfl_xor_sync(0xffffffffu, s[t], o);
+            float dot = s[0];
+#pragma unroll
+            for (int t = 1; t < FN_RG; ++t)
+                if (lane == t) dot = s[t];
+            const int c = c0 + lane;
+            if (lane < FN_RG && c < L) {
+                const float Dt = fmaf(-2.f, dot, __ldg(a.cn + c));
+                float lb, ub;
+                bounds(c, Dt, xn, lb, ub);
+                sD[c] = Dt;
+                T = fminf(T, ub);
+            }
+        }
+        T = fmin_warp(T);
+        if (lane == 0) sT[w] = T;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < CW_ROWS; ++k) T = fminf(T, sT[k]);
+        for (int c = tid; c < L; c += CW_ROWS * 32) {
+            float lb, ub;
+            bounds(c, sD[c], xn, lb, ub);
+            if (lb <= T) {
+                atomicAdd(&s_found, 1);
+                s_one = c;
+            }
+        }
+        __syncthreads();
+        const int found = s_found;
+        if (found <= 1) {
+            if (tid == 0) write(row, s_one);
+            continue;
+        }
+        bd = INFINITY;
+        bc = 0x7fffffff;
+        for (int c = tid; c < L; c += CW_ROWS * 32) {
+            float lb, ub;
+            bounds(c, sD[c], xn, lb, ub);
+            if (lb <= T) better(exact_dist(xr, a.cent + (size_t)c * d, d), c);
+        }
+        best_warp();
+        if (lane == 0) {
+            sB[w] = bd;
+            sC[w] = bc;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            for (int k = 1; k < CW_ROWS; ++k) better(sB[k], sC[k]);
+            write(row, bc);
+        }
     }
 }
 
@@ -1468,12 +1715,16 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
     const int split = first_stage_split(ix, P);
     const bool two = split != 0;
     const float gamma2_first = (float)(2.0 * first_stage_rel(d, split) * (1.0 + 1e-6));
-    // assignment with the single BF16 product: the fused first stage keeps
-    // only each row's candidate lists (needs CF_STRIDE ints per row of the
-    // distance buffer, and d <= 128 for its shared memory)
-    const bool fused = split == 1 && ix->tmap_cent_ok &&
-                       (size_t)32 + (size_t)rows_per_chunk * (CF_STRIDE + 1) <=
-                           (size_t)rows_per_chunk * L;
+    // assignment (d <= 128) takes the fused first stage, which keeps only the
+    // undecided rows and their candidate lists.  It needs far less room than
+    // the matrix: a launch takes as many rows as leave records for half of
+    // them (958,000 where the matrix of L = 1024 lists takes 16,384); among
+    // close centroids about a third are undecided
+    const int64_t room = rows_per_chunk * L;
+    const bool fused = P == 1 && two && ix->tmap_cent_ok && L >= CF_LMIN;
+    int64_t rows = rows_per_chunk;
+    if (fused)
+        rows = std::min<int64_t>(std::max<int64_t>((room - CF_HDR) * 2 / (2 + CF_STRIDE), 1), m);
     int nsm = 0;
     if (fused) {
         int dev = 0;
@@ -1481,31 +1732,39 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         nsm = std::max(nsm, 1);
     }
-    for (int64_t r0 = 0; r0 < m; r0 += rows_per_chunk) {
-        int mc = (int)std::min<int64_t>(rows_per_chunk, m - r0);
+    for (int64_t r0 = 0; r0 < m; r0 += rows) {
+        int mc = (int)std::min<int64_t>(rows, m - r0);
+        const int cap = fused ? (int)std::min<int64_t>((room - CF_HDR - mc) / CF_STRIDE, mc) : 0;
         const int tok = prof_begin(ix, PROF_COARSE, 2, st);
+        // the distance buffer of the fused stage: the number of undecided
+        // rows, those rows, the records
+        int32_t *nh = reinterpret_cast<int32_t *>(Dbuf), *rec = nh + CF_HDR + mc;
         if (fused) {
-            const size_t smem = coarse_fused_smem(d);
-            // the distance buffer holds the undecided-row count, the
-            // undecided rows and the candidate lists
-            int32_t *nh = reinterpret_cast<int32_t *>(Dbuf);
-            cudaMemsetAsync(nh, 0, sizeof(int32_t), st);
+            const int KC = d <= 64 ? 1 : 2, parts = split == 3 ? 2 : 1;
+            const size_t smem = coarse_fused_smem(KC, parts);
+            cudaMemsetAsync(nh, 0, 2 * sizeof(int32_t), st);
             const int nt = (mc + CT_M - 1) / CT_M;
             const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent);
-            // shared memory opted in once per instantiation (index KC - 1)
-            static size_t attr[2] = {0, 0};
-            auto go = [&](auto kern, int kc) {
-                if (smem > attr[kc - 1]) {
+            const CUtensorMap &tl = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent_lo);
+            // shared memory opted in once per instantiation
+            static bool attr[4] = {false, false, false, false};
+            auto go = [&](auto kern, int i) {
+                if (!attr[i]) {
                     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
-                    attr[kc - 1] = smem;
+                    attr[i] = true;
                 }
-                launch_pdl(kern, std::min(nt, nsm), CF_NT, smem, st, tm, x + r0 * d, mc, d,
-                           ix->cnorm, ix->cnrm_up, L, gamma2_first, out + r0, nh + 32 + mc, nh + 32,
+                launch_pdl(kern, std::min(nt, nsm), CF_NT, smem, st, tm, tl, x + r0 * d, mc, d,
+                           ix->cnorm, ix->cnrm_up, L, gamma2_first, out + r0, rec, cap, nh + CF_HDR,
                            nh, ix->err);
             };
-            if (d <= 64) go(k_coarse_fused1<1>, 1);
-            else go(k_coarse_fused1<2>, 2);
+            if (parts == 1) {
+                if (KC == 1) go(k_coarse_fused<1, 1>, 0);
+                else go(k_coarse_fused<2, 1>, 1);
+            } else {
+                if (KC == 1) go(k_coarse_fused<1, 2>, 2);
+                else go(k_coarse_fused<2, 2>, 3);
+            }
         } else if (two) {
             const size_t smem = coarse_tc_smem(d, split);
             dim3 g((mc + CT_M - 1) / CT_M, (L + CT_N - 1) / CT_N);
@@ -1535,10 +1794,10 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         }
         SelArgs a;
         a.D = fused ? nullptr : Dbuf;
-        a.S = fused ? reinterpret_cast<const int32_t *>(Dbuf) + 32 + mc : nullptr;
-        a.s_stride = CF_STRIDE;
-        a.hard = reinterpret_cast<const int32_t *>(Dbuf) + 32;
-        a.nhard = reinterpret_cast<const int *>(Dbuf);
+        a.hard = nh + CF_HDR;
+        a.nhard = nh;
+        a.S = rec;
+        a.s_cap = cap;
         a.m = mc;
         a.L = L;
         a.P = P;
@@ -1549,16 +1808,18 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         a.cnrm_up = ix->cnrm_up;
         a.gamma2 = (float)(2.0 * gd * (1.0 + 1e-6));
         a.gamma2_first = gamma2_first;
+        const double gr = re_ops(d) * u / (1.0 - re_ops(d) * u);
+        a.gamma2_re = (float)(2.0 * gr * (1.0 + 1e-6));
         a.two_level = two;
         a.out = out + r0 * P;
         a.err = ix->err;
         if (warp_rows) {
             const unsigned gw = (unsigned)((mc + CW_ROWS - 1) / CW_ROWS);
-            if (fused)  // loops over the undecided rows, usually none
-                launch_pdl(k_coarse_select_w<1, true>, std::min<unsigned>(gw, 2u * (unsigned)nsm),
-                           CW_ROWS * 32, 0, st, a);
-            else if (P == 1) launch_pdl(k_coarse_select_w<1, false>, gw, CW_ROWS * 32, 0, st, a);
-            else launch_pdl(k_coarse_select_w<CW_PMAX, false>, gw, CW_ROWS * 32, 0, st, a);
+            if (fused)  // loops over the undecided rows
+                launch_pdl(k_coarse_finish, std::min<unsigned>(gw, 10u * (unsigned)nsm), CW_ROWS * 32,
+                           0, st, a);
+            else if (P == 1) launch_pdl(k_coarse_select_w<1>, gw, CW_ROWS * 32, 0, st, a);
+            else launch_pdl(k_coarse_select_w<CW_PMAX>, gw, CW_ROWS * 32, 0, st, a);
         } else {
             launch_pdl(k_coarse_select, mc, SEL_NT, 0, st, a);
         }

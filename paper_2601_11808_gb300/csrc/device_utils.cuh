@@ -91,6 +91,26 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
+// mbarrier wait bounded in time (the index's wait limit) that also gives
+// up as soon as another role of the CTA has stopped (abort flag in shared
+// memory); a wait that runs out sets ERR_TIMEOUT and the abort flag.
+// Copies already in flight are drained by the producer with the default
+// limit before the CTA exits.
+__device__ __forceinline__ bool mbar_wait_ab(uint64_t *bar, uint32_t parity, uint32_t *err,
+                                             volatile int *abort_flag, uint64_t limit_ns)
+{
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t t0 = gtimer_ns();
+    for (uint32_t it = 1; it < (1u << 30); ++it) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((it & 63u) == 0u && *abort_flag) return false;
+        if (gtimer_ns() - t0 > limit_ns) break;
+    }
+    atomicOr(err, ERR_TIMEOUT);
+    *abort_flag = 1;
+    return false;
+}
+
 // One bulk copy global -> shared of `bytes` (multiple of 16, both addresses
 // 16-byte aligned) that completes transaction bytes on `bar`.
 __device__ __forceinline__ void bulk_g2s(void *dst_smem, const void *src_gmem,

@@ -453,52 +453,6 @@ __device__ __forceinline__ float fold_row(float *bd, int32_t *bs, int K, int Kw,
     return dmax;
 }
 
-// mbarrier wait bounded in time (the index's wait limit) that also gives
-// up as soon as another role of the CTA has stopped (abort flag in shared
-// memory); a wait that runs out sets ERR_TIMEOUT and the abort flag.
-// Copies already in flight are drained by the producer with the default
-// limit before the CTA exits.
-__device__ __forceinline__ bool mbar_wait_ab(uint64_t *bar, uint32_t parity, uint32_t *err,
-                                             volatile int *abort_flag, uint64_t limit_ns)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = gtimer_ns();
-    for (uint32_t it = 1; it < (1u << 30); ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 63u) == 0u && *abort_flag) return false;
-        if (gtimer_ns() - t0 > limit_ns) break;
-    }
-    atomicOr(err, ERR_TIMEOUT);
-    *abort_flag = 1;
-    return false;
-}
-
-// named barrier over `n` threads that also returns the AND of `pred`
-__device__ __forceinline__ bool named_bar_and(int id, int n, bool pred)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
-        " bar.red.and.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-        : "=r"(r)
-        : "r"((uint32_t)pred), "r"(id), "r"(n)
-        : "memory");
-    return r != 0;
-}
-
-// named barrier over `n` threads that also returns the OR of `pred`
-__device__ __forceinline__ bool named_bar_or(int id, int n, bool pred)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
-        " bar.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-        : "=r"(r)
-        : "r"((uint32_t)pred), "r"(id), "r"(n)
-        : "memory");
-    return r != 0;
-}
-
 // 16-byte asynchronous copy global -> shared; bytes past `src_bytes` (0 or
 // 16) are zero-filled
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, uint32_t src_bytes)

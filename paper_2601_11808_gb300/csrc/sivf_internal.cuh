@@ -139,8 +139,10 @@ struct sivf_index {
     // the same copies with boxes of min(C, 64) rows (query-row scan)
     alignas(64) unsigned char tmap_qt_bf16[128];
     alignas(64) unsigned char tmap_qt_fp8[128];
-    // the BF16 centroids in boxes of 64 x 256 (fused coarse first stage)
+    // the BF16 centroids and their low parts in boxes of 64 x 128 (fused
+    // coarse first stage)
     alignas(64) unsigned char tmap_cent[128];
+    alignas(64) unsigned char tmap_cent_lo[128];
     bool tmap_cent_ok;
     // nearest-list assignment takes the split-BF16 first stage (the single
     // BF16 product's bound is wide against the centroid spacing)

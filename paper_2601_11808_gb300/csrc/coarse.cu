@@ -40,33 +40,36 @@
 namespace sivf {
 
 // ------------------------------------------------------------ centroid prep
+// One warp per centroid, lanes over the coordinates (one thread per centroid
+// walked its row with dependent FP64 additions: 63 us for 1,024 x 128).
 __global__ void k_centroid_norms(const float *__restrict__ cent, int L, int d,
                                  float *__restrict__ cn, float *__restrict__ cnrm_up,
-                                 float *__restrict__ inv_scale8, uint16_t *__restrict__ cb,
-                                 uint16_t *__restrict__ clo)
+                                 uint16_t *__restrict__ cb, uint16_t *__restrict__ clo)
 {
     pdl_begin();
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (c >= L) return;
     const float *v = cent + (size_t)c * d;
-    double s = 0.0, mx = 0.0;
-    for (int j = 0; j < d; ++j) {
-        double t = (double)v[j];
+    double s = 0.0;
+    for (int j = lane; j < d; j += 32) {
+        const float f = v[j];
+        const double t = (double)f;
         s = __dadd_rn(s, __dmul_rn(t, t));
-        mx = fmax(mx, fabs(t));
-    }
-    cn[c] = __double2float_rn(s);
-    cnrm_up[c] = __double2float_ru(sqrt(s) * (1.0 + 1e-12));
-    if (cb)
-        for (int j = 0; j < d; ++j) {
-            const __nv_bfloat16 h = __float2bfloat16_rn(v[j]);
+        if (cb) {
+            const __nv_bfloat16 h = __float2bfloat16_rn(f);
             cb[(size_t)c * d + j] = *reinterpret_cast<const uint16_t *>(&h);
             if (clo) {
-                const __nv_bfloat16 l = __float2bfloat16_rn(v[j] - __bfloat162float(h));
+                const __nv_bfloat16 l = __float2bfloat16_rn(f - __bfloat162float(h));
                 clo[(size_t)c * d + j] = *reinterpret_cast<const uint16_t *>(&l);
             }
         }
-    (void)mx;
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+        cn[c] = __double2float_rn(s);
+        cnrm_up[c] = __double2float_ru(sqrt(s) * (1.0 + 1e-12));
+    }
 }
 
 // ----------------------------------------------------- FP32 tile GEMM (SIMT)
@@ -1589,8 +1592,8 @@ __global__ void k_fp8_scales(const float *__restrict__ cent, int L, int d,
 void centroid_prep(sivf_index *ix, cudaStream_t st)
 {
     ix->launches += 1;
-    launch_pdl(k_centroid_norms, (ix->nlist + 127) / 128, 128, 0, st, ix->cent, ix->nlist, ix->d,
-               ix->cnorm, ix->cnrm_up, ix->inv_scale8, ix->cent_bf16, ix->cent_lo);
+    launch_pdl(k_centroid_norms, (ix->nlist * 32 + 127) / 128, 128, 0, st, ix->cent, ix->nlist, ix->d,
+               ix->cnorm, ix->cnrm_up, ix->cent_bf16, ix->cent_lo);
     if (ix->x8) {
         ix->launches += 1;
         launch_pdl(k_fp8_scales, (ix->nlist * 32 + 127) / 128, 128, 0, st, ix->cent, ix->nlist,
@@ -1599,35 +1602,70 @@ void centroid_prep(sivf_index *ix, cudaStream_t st)
 }
 
 // Squared distance from each centroid to its nearest other centroid, FP32
-// (a statistic that picks the first stage, never a result).  One warp per
-// list, its lanes striding over the other centroids.
-__global__ void k_cent_gap(const float *__restrict__ cent, int L, int d,
-                           float *__restrict__ gap2)
+// (a statistic that picks the first stage, never a result).  A block takes
+// GAP_N centroids against every GAP_N-row tile of a share of the others,
+// both in shared memory (rows padded by one float4 against bank conflicts),
+// each thread 2 x 2 pairs; the shares meet by atomicMin (distances are not
+// negative, so their bits order as integers).  At L = 1,024, d = 128 the
+// arithmetic is 10 us; with one warp per centroid, every lane walking a row
+// of its own, the uncoalesced reads took 555 us.
+constexpr int GAP_N = 32;
+constexpr int GAP_NT = GAP_N * GAP_N / 4;
+__global__ __launch_bounds__(GAP_NT) void k_cent_gap(const float *__restrict__ cent, int L, int d,
+                                                     int *__restrict__ gap2)
 {
     pdl_begin();
-    const int lane = threadIdx.x & 31;
-    const int l = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (l >= L) return;
-    const float *cl = cent + (size_t)l * d;
-    float best = INFINITY;
-    for (int o = lane; o < L; o += 32) {
-        if (o == l) continue;
-        const float *co = cent + (size_t)o * d;
-        float s0 = 0.f, s1 = 0.f;
-        int j = 0;
-        for (; j + 1 < d; j += 2) {
-            const float t0 = cl[j] - co[j], t1 = cl[j + 1] - co[j + 1];
-            s0 = fmaf(t0, t0, s0);
-            s1 = fmaf(t1, t1, s1);
+    extern __shared__ __align__(16) float4 gsm[];
+    const int n4 = d >> 2, DP = n4 + 1, tid = threadIdx.x;
+    float4 *sa = gsm, *sb = gsm + GAP_N * DP;
+    const int a0 = blockIdx.x * GAP_N, ta = tid / (GAP_N / 2), tb = tid % (GAP_N / 2);
+    const float4 *c4 = reinterpret_cast<const float4 *>(cent);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto stage = [&](float4 *to, int r0) {
+        for (int e = tid; e < GAP_N * n4; e += GAP_NT) {
+            const int r = e / n4, j = e % n4;
+            to[r * DP + j] = r0 + r < L ? __ldg(c4 + (size_t)(r0 + r) * n4 + j) : zero;
         }
-        if (j < d) {
-            const float t0 = cl[j] - co[j];
-            s0 = fmaf(t0, t0, s0);
+    };
+    stage(sa, a0);
+    float best[2] = {INFINITY, INFINITY};
+    for (int b0 = blockIdx.y * GAP_N; b0 < L; b0 += gridDim.y * GAP_N) {
+        __syncthreads();
+        stage(sb, b0);
+        __syncthreads();
+        float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+        for (int j = 0; j < n4; ++j) {
+            const float4 u[2] = {sa[ta * DP + j], sa[(ta + GAP_N / 2) * DP + j]};
+            const float4 v[2] = {sb[tb * DP + j], sb[(tb + GAP_N / 2) * DP + j]};
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    float t = u[i].x - v[k].x;
+                    s[i][k] = fmaf(t, t, s[i][k]);
+                    t = u[i].y - v[k].y;
+                    s[i][k] = fmaf(t, t, s[i][k]);
+                    t = u[i].z - v[k].z;
+                    s[i][k] = fmaf(t, t, s[i][k]);
+                    t = u[i].w - v[k].w;
+                    s[i][k] = fmaf(t, t, s[i][k]);
+                }
         }
-        best = fminf(best, s0 + s1);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int a = a0 + ta + i * (GAP_N / 2), b = b0 + tb + k * (GAP_N / 2);
+                if (b < L && b != a) best[i] = fminf(best[i], s[i][k]);
+            }
     }
-    for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if (lane == 0) gap2[l] = best;
+    // the 16 threads of a row sit in one half warp
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        for (int o = 8; o > 0; o >>= 1) best[i] = fminf(best[i], __shfl_xor_sync(0xffffffffu, best[i], o));
+        const int a = a0 + ta + i * (GAP_N / 2);
+        if (tb == 0 && a < L) atomicMin(gap2 + a, __float_as_int(best[i]));
+    }
 }
 
 // relative error of the BF16 first stage's dot products, |acc - x.c| /
@@ -1666,7 +1704,12 @@ cudaError_t assign_stage_choose(sivf_index *ix, cudaStream_t st)
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&gap2), sizeof(float) * L, st);
     if (e != cudaSuccess) return e;
     ix->launches += 1;
-    launch_pdl(k_cent_gap, (L * 32 + 127) / 128, 128, 0, st, ix->cent, L, d, gap2);
+    // 0x7f7f7f7f: 3.4e38, no other centroid seen yet
+    cudaMemsetAsync(gap2, 0x7f, sizeof(float) * L, st);
+    const int na = (L + GAP_N - 1) / GAP_N;
+    const size_t gsmem = (size_t)2 * GAP_N * (d / 4 + 1) * 16;  // 33.8 KB at d = 128
+    launch_pdl(k_cent_gap, dim3(na, std::min(na, std::max(1, 152 * 4 / na))), GAP_NT, gsmem, st,
+               ix->cent, L, d, reinterpret_cast<int *>(gap2));
     std::vector<float> g((size_t)L), cn((size_t)L);
     e = cudaGetLastError();
     if (e == cudaSuccess)

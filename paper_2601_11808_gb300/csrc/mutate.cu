@@ -7,8 +7,9 @@
 // vectors of the same list (stable in batch order), the list's head slab
 // takes the first C - fill of them and fresh slabs popped from the free
 // stack take the rest.  Payload, id and address-table entry are written
-// first, then a device fence, then the validity bit (Theorem 1: the bit is
-// the publication point).  Kernels, in stream order:
+// by one kernel, the validity bits by the next (Theorem 1: the bit is the
+// publication point; the kernel boundary orders the two).  Kernels, in
+// stream order:
 //   claim     last occurrence of each id wins (atomicMax into claim[id])
 //   rank      per block of 1024 vectors: stable sort by list, local ranks,
 //             run counts per (list, block)
@@ -18,8 +19,9 @@
 //             ids that are live
 //   reclaim   lists that lost a slab: directory compaction, slab to the stack
 //   alloc     per touched list: fill the head, pop fresh slabs
-//   append    per vector: payload + copies + id + table, fence, bit
-//   cleanup   reset the per-batch bookkeeping
+//   append    per vector: payload + copies + id + table
+//   publish   per touched list: the validity bits of its new slots; reset
+//             the per-batch bookkeeping
 //
 // Delete.  Per id: table lookup, atomicAnd on the validity word; the thread
 // that takes the bit 1 -> 0 invalidates the table entry and decrements the
@@ -99,38 +101,62 @@ static IndexView view_of(sivf_index *ix)
          i += (int64_t)gridDim.x * blockDim.x)
 
 // ------------------------------------------------------------ delete core
-__device__ __forceinline__ void delete_one(const IndexView &V, int64_t id,
-                                           int32_t *affected, bool count)
+// Takes id's vector out; 1 if it was there.  The caller adds the removals
+// up (drop_total): a counter per vector on one address held a delete of
+// 1,000,000 ids for most of its 193 us.
+__device__ __forceinline__ int delete_one(const IndexView &V, int64_t id, int32_t *affected)
 {
     const int64_t coord = V.att[id];
-    if (coord < 0) return;
+    if (coord < 0) return 0;
     const int64_t s = coord >> 32;
     const int o = (int)(coord & 0xffffffff);
     if (s >= V.n_slabs || o >= V.C) {
         atomicOr(V.err, ERR_BAD_SLAB);
-        return;
+        return 0;
     }
+    const int l = V.meta[s].list;  // changes only where no delete runs
     const uint32_t m = 1u << (o & 31);
     const uint32_t old = atomicAnd(&V.bits[s * V.W + (o >> 5)], ~m);
-    if (!(old & m)) return;  // already cleared: a repeat of this id
+    if (!(old & m)) return 0;  // already cleared: a repeat of this id
     V.att[id] = -1;
-    atomicAdd(reinterpret_cast<unsigned long long *>(V.live_total),
-              (unsigned long long)(-1LL));
-    if (count) atomicAdd(reinterpret_cast<unsigned long long *>(&V.ctl->count), 1ull);
-    const int l = V.meta[s].list;
     if (l < 0 || l >= V.nlist) {
         atomicOr(V.err, ERR_BAD_SLAB);
-        return;
+        return 1;
     }
-    atomicSub(&V.list_live[l], 1);
+    // one subtraction per list among the warp's threads that got here
+    // (a skewed batch takes most of its vectors from a few lists)
+    const uint32_t peers = __match_any_sync(__activemask(), l);
+    if ((lanemask_lt() & peers) == 0u) atomicSub(&V.list_live[l], __popc(peers));
     if (atomicSub(&V.meta[s].live, 1) == 1) {
         if (atomicCAS(&V.aff_flag[l], 0, 1) == 0)
             affected[atomicAdd(&V.ctl->naffected, 1)] = l;
     }
+    return 1;
+}
+
+// a block's removals off the live total (and onto the batch's count)
+__device__ __forceinline__ void drop_total(const IndexView &V, int n, bool count)
+{
+    __shared__ int s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&s_n, n);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_n) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(V.live_total),
+                  (unsigned long long)(-(long long)s_n));
+        if (count)
+            atomicAdd(reinterpret_cast<unsigned long long *>(&V.ctl->count),
+                      (unsigned long long)s_n);
+    }
 }
 
 // one warp per list that lost a slab: stable compaction of the directory,
-// emptied slabs reset and pushed on the free stack
+// emptied slabs reset and pushed on the free stack.  RC_U x 32 entries and
+// their slabs' counts are in flight at once: a directory of 2,000 slabs
+// walked 32 at a time took 90 us, two dependent loads after each other.
+constexpr int RC_U = 8;
 __global__ void k_reclaim(IndexView V, const int32_t *__restrict__ affected)
 {
     pdl_begin();
@@ -148,25 +174,41 @@ __global__ void k_reclaim(IndexView V, const int32_t *__restrict__ affected)
         const int h = V.head[l];
         int kept = 0;
         bool hfree = false;
-        for (int base = 0; base < n; base += 32) {
-            const int i = base + lane;
-            const int s = i < n ? D[i] : -1;
-            const bool valid = s >= 0 && s < V.n_slabs;
-            if (i < n && !valid) atomicOr(V.err, ERR_BAD_SLAB);
-            const bool keep = valid && V.meta[s].live > 0;
-            const bool drop = valid && !keep;
-            const uint32_t km = __ballot_sync(0xffffffffu, keep);
-            __syncwarp();
-            if (keep) D[kept + __popc(km & lanemask_lt())] = s;
-            kept += __popc(km);
-            if (drop) {
-                V.meta[s].list = -1;
-                V.meta[s].fill = 0;
-                V.meta[s].live = 0;
-                const int t = atomicAdd(V.free_top, 1);
-                if (t >= V.n_slabs) atomicOr(V.err, ERR_STACK);
-                else V.free_list[t] = s;
-                if (s == h) hfree = true;
+        for (int base = 0; base < n; base += 32 * RC_U) {
+            int sv[RC_U], live[RC_U];
+#pragma unroll
+            for (int u = 0; u < RC_U; ++u) {
+                const int i = base + 32 * u + lane;
+                sv[u] = i < n ? D[i] : -1;
+                if (i < n && (sv[u] < 0 || sv[u] >= V.n_slabs)) {
+                    atomicOr(V.err, ERR_BAD_SLAB);
+                    sv[u] = -1;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < RC_U; ++u) live[u] = sv[u] >= 0 ? V.meta[sv[u]].live : 0;
+            __syncwarp();  // the entries are read before any is overwritten
+#pragma unroll
+            for (int u = 0; u < RC_U; ++u) {
+                if (base + 32 * u >= n) break;  // warp-uniform
+                const int s = sv[u];
+                const bool keep = s >= 0 && live[u] > 0, drop = s >= 0 && !keep;
+                const uint32_t km = __ballot_sync(0xffffffffu, keep);
+                const uint32_t dm = __ballot_sync(0xffffffffu, drop);
+                if (keep) D[kept + __popc(km & lanemask_lt())] = s;
+                kept += __popc(km);
+                if (dm == 0u) continue;
+                int t = 0;
+                if (lane == 0) t = atomicAdd(V.free_top, __popc(dm));
+                t = __shfl_sync(0xffffffffu, t, 0) + __popc(dm & lanemask_lt());
+                if (drop) {
+                    V.meta[s].list = -1;
+                    V.meta[s].fill = 0;
+                    V.meta[s].live = 0;
+                    if (t >= V.n_slabs) atomicOr(V.err, ERR_STACK);
+                    else V.free_list[t] = s;
+                    if (s == h) hfree = true;
+                }
             }
         }
         hfree = __any_sync(0xffffffffu, hfree);
@@ -194,7 +236,9 @@ __global__ void k_rm_phase1(IndexView V, const int64_t *__restrict__ ids, int64_
 {
     pdl_begin();
     if (V.ctl->flags & FLAG_BAD_ID) return;
-    GRID_STRIDE(i, n) delete_one(V, ids[i], affected, true);
+    int gone = 0;
+    GRID_STRIDE(i, n) gone += delete_one(V, ids[i], affected);
+    drop_total(V, gone, true);
 }
 
 // ------------------------------------------------------------- insert
@@ -336,64 +380,74 @@ __global__ void k_ins_overwrite(IndexView V, const int64_t *__restrict__ ids, in
         if (st != SIVF_OK) V.ctl->count = 0;
     }
     if (st != SIVF_OK) return;
+    int gone = 0;
     GRID_STRIDE(i, n)
     {
-        if (rloc[i] < 0) continue;
-        const int64_t id = ids[i];
-        if (V.att[id] >= 0) delete_one(V, id, affected, false);
+        if (rloc[i] >= 0) gone += delete_one(V, ids[i], affected);
     }
+    drop_total(V, gone, false);
 }
 
+// one warp per touched list: the head slab takes what fits, lanes over the
+// fresh slabs (one thread per list took 137 us where a list gets 2,000)
 __global__ void k_ins_alloc(IndexView V, const int32_t *__restrict__ touched,
                             const int32_t *__restrict__ bcnt, PlanEntry *__restrict__ plan)
 {
     pdl_begin();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (V.ctl->status != SIVF_OK || t >= V.ctl->ntouched) return;
+    const int lane = threadIdx.x & 31;
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (V.ctl->status != SIVF_OK || t >= V.ctl->ntouched) return;  // whole warps
     const int l = touched[t];
     const int cnt = bcnt[t];
     const int C = V.C;
     const int h = V.head[l];
+    const int pos0 = V.nslabs[l];
     const int fill = h >= 0 ? V.meta[h].fill : C;
     const int avail = C - fill;
     const int a = min(cnt, avail);
     const int need = cnt > avail ? (cnt - avail + C - 1) / C : 0;
-    const int pos0 = V.nslabs[l];
-    PlanEntry pe;
-    pe.head_old = h;
-    pe.fill_old = fill;
-    pe.into_head = a;
-    pe.dir_pos0 = pos0;
-    if (a > 0) {
-        V.meta[h].fill = fill + a;
-        V.meta[h].live += a;
+    __syncwarp();  // every lane has read the list's state before lane 0 changes it
+    int top = 0;
+    if (lane == 0) {
+        PlanEntry pe;
+        pe.head_old = h;
+        pe.fill_old = fill;
+        pe.into_head = a;
+        pe.dir_pos0 = pos0;
+        plan[t] = pe;
+        if (a > 0) {
+            V.meta[h].fill = fill + a;
+            V.meta[h].live += a;
+        }
+        if (need > 0) top = atomicSub(V.free_top, need);
     }
     if (need > 0) {
-        const int top = atomicSub(V.free_top, need);
+        top = __shfl_sync(0xffffffffu, top, 0);
         if (top - need < 0 || (int64_t)pos0 + need > V.dir_cap) {
-            atomicOr(V.err, ERR_STACK);
-            plan[t] = pe;
+            if (lane == 0) atomicOr(V.err, ERR_STACK);
             return;
         }
         const int rem = cnt - a;
-        int s = -1;
         // the reserved stack entries from the top down: on a fresh pool (slab
         // 0 on top) a list receives ascending consecutive slabs, which the
         // list scan fetches as one 128-row box
-        for (int j = 0; j < need; ++j) {
-            s = V.free_list[top - 1 - j];
+        for (int j = lane; j < need; j += 32) {
+            const int s = V.free_list[top - 1 - j];
             const int f = min(C, rem - j * C);
             V.meta[s].list = l;
             V.meta[s].fill = f;
             V.meta[s].live = f;
             V.dir[(size_t)l * V.dir_cap + pos0 + j] = s;
+            if (j == need - 1) {
+                V.nslabs[l] = pos0 + need;
+                V.head[l] = s;
+            }
         }
-        V.nslabs[l] = pos0 + need;
-        V.head[l] = s;
     }
-    atomicAdd(reinterpret_cast<unsigned long long *>(V.live_total), (unsigned long long)cnt);
-    V.list_live[l] += cnt;
-    plan[t] = pe;
+    if (lane == 0) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(V.live_total), (unsigned long long)cnt);
+        V.list_live[l] += cnt;
+    }
 }
 
 // sum over the 16 lanes of a half warp (every lane of the warp calls it)
@@ -403,8 +457,11 @@ __device__ __forceinline__ float half_sum(float v)
     return v;
 }
 
-// two kept vectors per warp, one per half (16 lanes of 16-byte chunks): a
-// batch of 10,000 takes one wave of resident warps instead of two
+// Two kept vectors per warp, one per half (16 lanes of 16-byte chunks): a
+// batch of 10,000 takes one wave of resident warps instead of two.  Bound
+// by HBM at large batches (read 4 d, write 4 d + copies) and by the chain of
+// five dependent loads to the slot at small ones, so the first two chunks
+// of the row are asked for before it.
 __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
                              const float *__restrict__ x, int64_t n,
                              const int32_t *__restrict__ lab, const int32_t *__restrict__ rloc,
@@ -424,6 +481,15 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
         int slot = 0;
         float ss = 0.f, rs = 0.f;
         if (on) {
+            constexpr int PRE = 2;
+            const float *xi = x + (size_t)i * d;
+            float4 pre[PRE];
+#pragma unroll
+            for (int u = 0; u < PRE; ++u) {
+                const int j = hl * 4 + 64 * u;
+                pre[u] = j < d ? __ldcs(reinterpret_cast<const float4 *>(xi + j))
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
             const int l = lab[i];
             const int r = V.runcnt[(size_t)l * V.nblk_max + (i >> 10)] + r0;
             const PlanEntry pe = plan[V.list_flag[l] - 1];
@@ -436,11 +502,9 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
                 slot = q % C;
             }
             const size_t row = (size_t)s * C + slot;
-            const float *xi = x + (size_t)i * d;
             const float inv = V.x8 ? V.inv_scale8[l] : 1.f;
             const float *cl = V.cent + (size_t)l * d;
-            for (int j = hl * 4; j < d; j += 64) {
-                const float4 v = *reinterpret_cast<const float4 *>(xi + j);
+            auto put = [&](int j, const float4 v) {
                 *reinterpret_cast<float4 *>(V.x32 + row * d + j) = v;
                 ss = fmaf(v.x, v.x, ss);
                 ss = fmaf(v.y, v.y, ss);
@@ -456,7 +520,7 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
                 }
                 if (V.x8) {
                     // residual r = fl32(x - c_l), code = E4M3(fl32(r * inv))
-                    const float4 c4 = *reinterpret_cast<const float4 *>(cl + j);
+                    const float4 c4 = __ldg(reinterpret_cast<const float4 *>(cl + j));
                     const float4 rv = make_float4(__fsub_rn(v.x, c4.x), __fsub_rn(v.y, c4.y),
                                                   __fsub_rn(v.z, c4.z), __fsub_rn(v.w, c4.w));
                     rs = fmaf(rv.x, rv.x, rs);
@@ -472,7 +536,12 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
                     *reinterpret_cast<uint32_t *>(V.x8 + row * d + j) =
                         (uint32_t)pa | ((uint32_t)pb << 16);
                 }
-            }
+            };
+#pragma unroll
+            for (int u = 0; u < PRE; ++u)
+                if (hl * 4 + 64 * u < d) put(hl * 4 + 64 * u, pre[u]);
+            for (int j = hl * 4 + 64 * PRE; j < d; j += 64)
+                put(j, __ldcs(reinterpret_cast<const float4 *>(xi + j)));
         }
         ss = half_sum(ss);
         if (V.x8) rs = half_sum(rs);
@@ -484,26 +553,54 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
             V.ids[row] = id;
             V.att[id] = (s << 32) | (int64_t)slot;
         }
-        // payload, id and table entry are visible before the bit (Theorem 1)
-        __threadfence();
-        __syncwarp();
-        if (on && hl == 0) {
-            __threadfence();
-            atomicOr(&V.bits[s * V.W + (slot >> 5)], 1u << (slot & 31));
-        }
     }
 }
 
-__global__ void k_ins_cleanup(IndexView V, const int64_t *__restrict__ ids, int64_t n, int nblk,
-                              const int32_t *__restrict__ touched)
+// The payload, ids and table entries of the batch are written (by the
+// kernel before): the validity bits of each touched list's new slots, a
+// warp per list (lanes over its slabs), whole words at a time.  Setting each
+// bit in the append kernel took two device fences per vector (510 us per
+// 1,000,000 vectors there).  Then the bookkeeping of the batch is reset.
+__global__ void k_ins_publish(IndexView V, const int64_t *__restrict__ ids, int64_t n, int nblk,
+                              const int32_t *__restrict__ touched,
+                              const int32_t *__restrict__ bcnt, const PlanEntry *__restrict__ plan)
 {
     pdl_begin();
+    const int nt = V.ctl->ntouched;
+    if (V.ctl->status == SIVF_OK) {
+        const int lane = threadIdx.x & 31, C = V.C, W = V.W;
+        const int nw = gridDim.x * blockDim.x / 32;
+        // bits [lo, hi) of a word whose first slot is w0
+        auto mask = [](int lo, int hi, int w0) {
+            const int a = max(lo - w0, 0), b = min(hi - w0, 32);
+            if (a >= b) return 0u;
+            return (b == 32 ? 0xffffffffu : (1u << b) - 1u) & ~((1u << a) - 1u);
+        };
+        for (int t = (blockIdx.x * blockDim.x + threadIdx.x) / 32; t < nt; t += nw) {
+            const int l = touched[t];
+            const PlanEntry pe = plan[t];
+            const int rem = bcnt[t] - pe.into_head;
+            if (pe.into_head > 0 && lane < W) {
+                const uint32_t m = mask(pe.fill_old, pe.fill_old + pe.into_head, lane * 32);
+                if (m) V.bits[(size_t)pe.head_old * W + lane] |= m;
+            }
+            const int need = (rem + C - 1) / C;
+            for (int e = lane; e < need * W; e += 32) {
+                const int j = e / W, w = e % W;
+                const int s = V.dir[(size_t)l * V.dir_cap + pe.dir_pos0 + j];
+                if (s < 0 || s >= V.n_slabs) {
+                    atomicOr(V.err, ERR_BAD_SLAB);
+                    continue;
+                }
+                V.bits[(size_t)s * W + w] = mask(0, min(C, rem - j * C), w * 32);
+            }
+        }
+    }
     GRID_STRIDE(i, n)
     {
         const int64_t id = ids[i];
         if (id >= 0 && id < V.n_max) V.claim[id] = -1;
     }
-    const int nt = V.ctl->ntouched;
     GRID_STRIDE(e, (int64_t)nt * nblk)
     {
         const int l = touched[e / nblk];
@@ -532,11 +629,13 @@ void insert_batch(sivf_index *ix, const int64_t *ids, const float *x, int64_t n,
                s.touched, s.bcnt);
     launch_pdl(k_ins_overwrite, grid_for(n, 256), 256, 0, st, V, ids, n, s.rloc, s.affected);
     launch_pdl(k_reclaim, grid_for((int64_t)tmax * 32, 256), 256, 0, st, V, s.affected);
-    launch_pdl(k_ins_alloc, (tmax + 127) / 128, 128, 0, st, V, s.touched, s.bcnt, s.plan);
+    launch_pdl(k_ins_alloc, (unsigned)(((int64_t)tmax * 32 + 127) / 128), 128, 0, st, V, s.touched,
+               s.bcnt, s.plan);
     launch_pdl(k_ins_append, grid_for(n * 16, 256), 256, 0, st, V, ids, x, n, s.lab, s.rloc,
                s.plan);
-    launch_pdl(k_ins_cleanup, grid_for(std::max<int64_t>(n, (int64_t)tmax * nblk), 256), 256, 0, st,
-               V, ids, n, nblk, s.touched);
+    launch_pdl(k_ins_publish,
+               grid_for(std::max({n, (int64_t)tmax * nblk, (int64_t)tmax * 32}), 256), 256, 0, st, V,
+               ids, n, nblk, s.touched, s.bcnt, s.plan);
     prof_end(ix, tok, st);
 }
 

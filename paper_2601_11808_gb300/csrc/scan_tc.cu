@@ -981,19 +981,87 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
 // (first run, runs)) by a radix select over the 64-bit (distance, slot)
 // keys of the valid entries, then sorted ascending, padded with (+inf, -1).
 constexpr int MT_NT = 128;
+// entries of the selection's shared buffer per warp (8 bytes each)
+__host__ __device__ constexpr int merge_cap(int E) { return 64 * E > 512 ? 64 * E : 512; }
 // The selection of one query (one warp): its best K' valid entries, unsorted,
-// into sd / ss (32 E entries of the warp's shared memory); returns their
-// number, min(valid entries, K').  hist: TC_HIST words of shared memory.
+// into sd / ss (merge_cap(E) entries of the warp's shared memory); returns
+// their number, min(valid entries, K').  hist: TC_HIST words of shared memory.
+// `bound` is the query's shared bound after the scan: at least K' entries
+// lie at or below it, so only those are gathered (four runs' entries in
+// flight at once) and the radix select works on shared memory.  Only when
+// more than the buffer holds are at or below the bound (ties) does it pass
+// over the runs in global memory, one run after the other, once per digit:
+// for a query with tens of runs that chain of loads took 130-180 us.
 template <int E>
 __device__ int merge_select(const int2 *__restrict__ qrun, int64_t nq, int64_t q, int nphase,
-                            int K, int RK, const int32_t *__restrict__ part_n,
+                            int K, int RK, float bound, const int32_t *__restrict__ part_n,
                             const float *__restrict__ part_d, const int64_t *__restrict__ part_i,
                             uint32_t *hist, float *sd, int32_t *ss, int lane)
 {
+    constexpr int CAP = merge_cap(E);
     const int2 r0 = qrun[q];
     const int2 r1 = nphase > 1 ? qrun[nq + q] : make_int2(0, 0);
     const int NR = r0.y + r1.y;
     auto run_of = [&](int t) -> int64_t { return t < r0.y ? r0.x + t : r1.x + (t - r0.y); };
+    int have = 0;
+    for (int t0 = 0; t0 < NR && have <= CAP; t0 += 32) {
+        const int cl = t0 + lane < NR ? min(part_n[run_of(t0 + lane)], RK) : 0;
+        for (int u = 0; u < 32 && t0 + u < NR && have <= CAP; u += 4) {
+            int c[4], cm = 0;
+            int64_t rb[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                c[r] = __shfl_sync(0xffffffffu, cl, u + r);
+                rb[r] = c[r] > 0 ? run_of(t0 + u + r) * RK + lane : 0;
+                cm = max(cm, c[r]);
+            }
+            for (int j0 = 0; j0 < cm; j0 += 64) {
+                float dv[8];
+                int32_t sv[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int r = e >> 1, j = j0 + 32 * (e & 1);
+                    const bool ok = j + lane < c[r];
+                    dv[e] = ok ? part_d[rb[r] + j] : INFINITY;
+                    sv[e] = ok ? (int32_t)part_i[rb[r] + j] : 0;
+                    if (!(dv[e] <= bound) || !ok) sv[e] = -1;
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t mk = __ballot_sync(0xffffffffu, sv[e] >= 0);
+                    const int p = have + __popc(mk & lanemask_lt());
+                    if (sv[e] >= 0 && p < CAP) {
+                        sd[p] = dv[e];
+                        ss[p] = sv[e];
+                    }
+                    have += __popc(mk);
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (have <= CAP) {
+        if (have <= K) return have;
+        uint64_t prefix, mask;
+        warp_radix_kth([&](int i) { return ds_key(sd[i], ss[i]); }, have, K, hist, lane, prefix, mask);
+        int w = 0;  // compaction in place (every write index <= its read index)
+        for (int i0 = 0; i0 < have; i0 += 32) {
+            const int i = i0 + lane;
+            const float dv = i < have ? sd[i] : INFINITY;
+            const int32_t sv = i < have ? ss[i] : 0;
+            const bool take = i < have && (ds_key(dv, sv) & mask) <= prefix;
+            const uint32_t mk = __ballot_sync(0xffffffffu, take);
+            __syncwarp();
+            if (take) {
+                const int p = w + __popc(mk & lanemask_lt());
+                sd[p] = dv;
+                ss[p] = sv;
+            }
+            w += __popc(mk);
+            __syncwarp();
+        }
+        return min(w, K);
+    }
     auto key_at = [&](int64_t e) -> uint64_t { return ds_key(part_d[e], (int32_t)part_i[e]); };
     // visit every valid entry: f(valid, index) for 32 entries at a time,
     // called by the whole warp (the loops are warp-uniform)
@@ -1106,6 +1174,7 @@ __device__ int merge_select(const int2 *__restrict__ qrun, int64_t nq, int64_t q
 template <int E>
 __global__ __launch_bounds__(MT_NT) void k_merge_tc(const int2 *__restrict__ qrun, int64_t nq,
                                                     int nphase, int K, int RK,
+                                                    const float *__restrict__ thr,
                                                     const int32_t *__restrict__ part_n,
                                                     const float *__restrict__ part_d,
                                                     const int64_t *__restrict__ part_i,
@@ -1115,13 +1184,13 @@ __global__ __launch_bounds__(MT_NT) void k_merge_tc(const int2 *__restrict__ qru
     pdl_begin();
     constexpr int NW = MT_NT / 32;
     __shared__ uint32_t hist_s[NW][TC_HIST];
-    __shared__ float sd[NW][32 * E];
-    __shared__ int32_t ss[NW][32 * E];
+    __shared__ float sd[NW][merge_cap(E)];
+    __shared__ int32_t ss[NW][merge_cap(E)];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t q = (blockIdx.x * (int64_t)MT_NT + threadIdx.x) >> 5;
     if (q >= nq) return;  // whole warps
     uint32_t *hist = hist_s[warp];
-    const int nk = merge_select<E>(qrun, nq, q, nphase, K, RK, part_n, part_d, part_i, hist,
+    const int nk = merge_select<E>(qrun, nq, q, nphase, K, RK, thr[q], part_n, part_d, part_i, hist,
                                    sd[warp], ss[warp], lane);
     float v[E];
     int32_t sv[E];
@@ -1148,7 +1217,7 @@ void merge_tc(sivf_index *ix, int64_t nq, int nphase, const SearchScratch &s, in
     const unsigned blocks = (unsigned)((nq * 32 + MT_NT - 1) / MT_NT);
     const int tok = prof_begin(ix, PROF_MERGE, 1, st);
 #define SIVF_MTC(E_)                                                                               \
-    launch_pdl(k_merge_tc<E_>, blocks, MT_NT, 0, st, s.qrun, nq, nphase, Kc, RK, s.part_n,         \
+    launch_pdl(k_merge_tc<E_>, blocks, MT_NT, 0, st, s.qrun, nq, nphase, Kc, RK, s.thr, s.part_n,  \
                s.part_d, s.part_i, out_d, out_s)
     if (Kc <= 32) SIVF_MTC(1);
     else if (Kc <= 64) SIVF_MTC(2);
@@ -1272,20 +1341,21 @@ constexpr int RR_UNR = 2;
 template <int E, int NQ>
 __global__ __launch_bounds__(MT_NT, NQ <= 4 ? 9 : 2) void k_merge_rerank(
     const int2 *__restrict__ qrun, int64_t nq, int nphase, int K, int RK,
-    const int32_t *__restrict__ part_n, const float *__restrict__ part_d,
-    const int64_t *__restrict__ part_i, const float *__restrict__ q, int d,
+    const float *__restrict__ thr, const int32_t *__restrict__ part_n,
+    const float *__restrict__ part_d, const int64_t *__restrict__ part_i,
+    const float *__restrict__ q, int d,
     const float *__restrict__ x32, const int64_t *__restrict__ ids, int k,
     float *__restrict__ dist, int64_t *__restrict__ labels)
 {
     pdl_begin();
     constexpr int NW = MT_NT / 32;
     __shared__ uint32_t hist_s[NW][TC_HIST];
-    __shared__ float sd[NW][32 * E];
-    __shared__ int32_t ss[NW][32 * E];
+    __shared__ float sd[NW][merge_cap(E)];
+    __shared__ int32_t ss[NW][merge_cap(E)];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 3, t = lane & 7;
     const int64_t qi = (blockIdx.x * (int64_t)MT_NT + threadIdx.x) >> 5;
     if (qi >= nq) return;  // whole warps
-    const int nk = merge_select<E>(qrun, nq, qi, nphase, K, RK, part_n, part_d, part_i,
+    const int nk = merge_select<E>(qrun, nq, qi, nphase, K, RK, thr[qi], part_n, part_d, part_i,
                                    hist_s[warp], sd[warp], ss[warp], lane);
     int64_t id[E];
 #pragma unroll
@@ -1841,7 +1911,7 @@ void merge_rerank(sivf_index *ix, const float *q, int64_t nq, int nphase,
     const unsigned blocks = (unsigned)((nq * 32 + MT_NT - 1) / MT_NT);
     const int tok = prof_begin(ix, PROF_RERANK, 1, st);
 #define SIVF_MRR(E_, NQ_)                                                                          \
-    launch_pdl(k_merge_rerank<E_, NQ_>, blocks, MT_NT, 0, st, s.qrun, nq, nphase, Kc, RK,          \
+    launch_pdl(k_merge_rerank<E_, NQ_>, blocks, MT_NT, 0, st, s.qrun, nq, nphase, Kc, RK, s.thr,   \
                s.part_n, s.part_d, s.part_i, q, ix->d, ix->x32, ix->ids, k, dist,                  \
                labels)
     const bool wide = ix->d > 128;

@@ -767,7 +767,7 @@ static sivf_status search_impl(sivf_index *ix, const float *q, int64_t nq, int k
         int32_t *probes = b.take<int32_t>((size_t)m * P);
         sc.lcnt = b.take<int32_t>(L);
         sc.loff = b.take<int32_t>(L + 1);
-        sc.ibase = b.take<int32_t>(L + 1);
+        sc.touched = b.take<int32_t>(L + 1);
         sc.nch = b.take<int32_t>(L);
         sc.prank = b.take<int32_t>((size_t)m * P);
         sc.qlist = b.take<int32_t>((size_t)m * P);

@@ -46,80 +46,142 @@ __global__ void k_srch_hist(const int32_t *__restrict__ probes, int64_t nq, int 
     }
 }
 
-// One block.  Chunking: a list is cut into slab chunks so that no work item
-// is longer than 1 / (ips * 152) of the launch's whole work W (query tiles x
-// slabs summed over the probed lists) and no chunk is shorter than `spc`
-// slabs, at most `chmax` chunks per list; a heavy list (a skewed
+// inclusive scans of two values over the 1,024 threads of a block; `sh` is
+// 64 ints of shared memory; *ta, *tb receive the totals
+__device__ __forceinline__ void block_scan2(int32_t &a, int32_t &b, int32_t *sh, int32_t *ta,
+                                            int32_t *tb)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t va = __shfl_up_sync(0xffffffffu, a, o), vb = __shfl_up_sync(0xffffffffu, b, o);
+        if (lane >= o) {
+            a += va;
+            b += vb;
+        }
+    }
+    __syncthreads();  // sh may still be read from an earlier scan
+    if (lane == 31) {
+        sh[w] = a;
+        sh[32 + w] = b;
+    }
+    __syncthreads();
+    if (w == 0) {
+        int32_t sa = sh[lane], sb = sh[32 + lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t va = __shfl_up_sync(0xffffffffu, sa, o),
+                          vb = __shfl_up_sync(0xffffffffu, sb, o);
+            if (lane >= o) {
+                sa += va;
+                sb += vb;
+            }
+        }
+        sh[lane] = sa;
+        sh[32 + lane] = sb;
+    }
+    __syncthreads();
+    if (w > 0) {
+        a += sh[w - 1];
+        b += sh[32 + w - 1];
+    }
+    *ta = sh[31];
+    *tb = sh[63];
+}
+
+// the launch's whole work, summed over a block of 1,024 threads
+__device__ __forceinline__ unsigned long long block_work(unsigned long long w,
+                                                         unsigned long long *sw)
+{
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = w;
+    __syncthreads();
+    unsigned long long W = 0;
+    for (int i = 0; i < 32; ++i) W += sw[i];
+    return W;
+}
+
+// Slabs a chunk has at least.  A list is cut into slab chunks so that no
+// work item is longer than 1 / (ips * 152) of the launch's whole work W
+// (query tiles x slabs summed over the probed lists) and no chunk is shorter
+// than `spc` slabs, at most `chmax` chunks per list; a heavy list (a skewed
 // distribution puts most vectors in a few lists) is spread over many SMs
 // instead of holding one SM for the length of the launch.  With
 // target = max(spc, ceil(W / (ips * 152))) the chunks beyond the first of
 // every list add at most ips * 152 items, and at most tq * ips * 152 output
-// runs, to one tile per pair: the scratch is sized from that bound.  Then
-// exclusive scans over the lists of the pair counts and of the work items.
+// runs, to one tile per pair: the scratch is sized from that bound.
+__device__ __forceinline__ int chunk_target(unsigned long long W, int spc, int ips)
+{
+    const unsigned long long slots = (unsigned long long)ips * 152;
+    return (int)min(max((unsigned long long)spc, (W + slots - 1) / slots), 1ull << 30);
+}
+
+// pairs scored and slab bytes streamed (per tile, and once per list)
+struct ScanCount {
+    unsigned long long pairs = 0, bytes = 0, ubytes = 0;
+    __device__ void list(int m, int nt, int ns, int live, int64_t slab_bytes)
+    {
+        pairs += (unsigned long long)m * (unsigned long long)max(live, 0);
+        bytes += (unsigned long long)nt * ns * slab_bytes;
+        ubytes += (unsigned long long)ns * slab_bytes;
+    }
+    __device__ void add_to(int64_t *stat) const  // whole warps
+    {
+        unsigned long long v[3] = {pairs, bytes, ubytes};
+        for (int i = 0; i < 3; ++i) {
+            for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+            if ((threadIdx.x & 31) == 0 && v[i])
+                atomicAdd(reinterpret_cast<unsigned long long *>(stat + 1 + i), v[i]);
+        }
+    }
+};
+
+// One block: the lists' chunks (chunk_target), then exclusive scans over the
+// lists of the pair counts and of the work items.  Thread t takes the lists
+// t, t + 1024, ... (their order in the groups and items is of no account), so
+// that its loads are coalesced and independent: contiguous lists per thread
+// took 50 us at 16,384 lists, a chain of strided loads.
 __global__ __launch_bounds__(1024) void k_srch_plan(const int32_t *__restrict__ lcnt,
                                                     const int32_t *__restrict__ nslabs,
                                                     const int32_t *__restrict__ list_live,
                                                     int L, int tq, int chmax, int spc, int ips,
                                                     int64_t item_cap, int64_t slab_bytes,
                                                     int32_t *__restrict__ loff,
-                                                    int32_t *__restrict__ ibase,
                                                     int32_t *__restrict__ nch,
                                                     int2 *__restrict__ items, Ctl *ctl,
                                                     int64_t *stat, uint32_t *err)
 {
     pdl_begin();
-    __shared__ int32_t sa[1024], sb[1024];
+    __shared__ int32_t sh[64];
     __shared__ unsigned long long sw[32];
     const int tid = threadIdx.x;
-    const int per = (L + 1023) / 1024;
-    const int b0 = tid * per, b1 = min(L, b0 + per);
     unsigned long long wsum = 0;
-    for (int l = b0; l < b1; ++l) {
+#pragma unroll 8
+    for (int l = tid; l < L; l += 1024) {
         const int m = lcnt[l], ns = nslabs[l];
         if (m > 0 && ns > 0) wsum += (unsigned long long)((m + tq - 1) / tq) * ns;
     }
-    for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
-    if ((tid & 31) == 0) sw[tid >> 5] = wsum;
-    __syncthreads();
-    unsigned long long W = 0;
-    for (int i = 0; i < 32; ++i) W += sw[i];
-    const unsigned long long slots = (unsigned long long)ips * 152;
-    const unsigned long long share = (W + slots - 1) / slots;
-    const int target = (int)min(max((unsigned long long)spc, share), 1ull << 30);
+    const int target = chunk_target(block_work(wsum, sw), spc, ips);
     int32_t ca = 0, cb = 0;
-    unsigned long long pairs = 0, bytes = 0, ubytes = 0;
-    for (int l = b0; l < b1; ++l) {
-        int m = lcnt[l], ns = nslabs[l];
-        int nt = (m + tq - 1) / tq;
-        int c = (m > 0 && ns > 0) ? min(chmax, max(1, (ns + target - 1) / target)) : 0;
-        c = min(c, ns);
+    ScanCount cnt;
+#pragma unroll 4
+    for (int l = tid; l < L; l += 1024) {
+        const int m = lcnt[l], ns = nslabs[l], live = list_live[l];
+        const int nt = (m + tq - 1) / tq;
+        const int c = (m > 0 && ns > 0) ? min(min(chmax, max(1, (ns + target - 1) / target)), ns) : 0;
         nch[l] = c;
         ca += m;
         cb += nt * c;
-        if (c) {
-            pairs += (unsigned long long)m * (unsigned long long)max(list_live[l], 0);
-            bytes += (unsigned long long)nt * ns * slab_bytes;
-            ubytes += (unsigned long long)ns * slab_bytes;
-        }
+        if (c) cnt.list(m, nt, ns, live, slab_bytes);
     }
-    if (stat && pairs) atomicAdd(reinterpret_cast<unsigned long long *>(stat + 1), pairs);
-    if (stat && bytes) atomicAdd(reinterpret_cast<unsigned long long *>(stat + 2), bytes);
-    if (stat && ubytes) atomicAdd(reinterpret_cast<unsigned long long *>(stat + 3), ubytes);
-    sa[tid] = ca;
-    sb[tid] = cb;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        int32_t va = tid >= o ? sa[tid - o] : 0, vb = tid >= o ? sb[tid - o] : 0;
-        __syncthreads();
-        sa[tid] += va;
-        sb[tid] += vb;
-        __syncthreads();
-    }
-    int32_t ea = sa[tid] - ca, eb = sb[tid] - cb;
-    for (int l = b0; l < b1; ++l) {
+    if (stat) cnt.add_to(stat);
+    int32_t ea = ca, eb = cb, ta, tb;
+    block_scan2(ea, eb, sh, &ta, &tb);
+    ea -= ca;
+    eb -= cb;
+#pragma unroll 4
+    for (int l = tid; l < L; l += 1024) {
         const int m = lcnt[l], c = nch[l], nt = (m + tq - 1) / tq;
         loff[l] = ea;
-        ibase[l] = eb;
         // work items of list l: (list, tile << 8 | chunk)
         for (int t = 0; t < nt * c; ++t) {
             if (eb + t < item_cap) items[eb + t] = make_int2(l, ((t / c) << 8) | (t % c));
@@ -127,13 +189,140 @@ __global__ __launch_bounds__(1024) void k_srch_plan(const int32_t *__restrict__ 
         ea += m;
         eb += nt * c;
     }
-    if (tid == 1023) {
-        loff[L] = sa[1023];
-        ibase[L] = sb[1023];
-        if (sb[1023] > item_cap) atomicOr(err, ERR_PLAN);
-        ctl->nitems = (int32_t)min((int64_t)sb[1023], item_cap);
-        ctl->nscan = sa[1023];
+    if (tid == 0) {
+        if (tb > item_cap) atomicOr(err, ERR_PLAN);
+        ctl->nitems = (int32_t)min((int64_t)tb, item_cap);
+        ctl->nscan = ta;
         ctl->next_item = 0;
+    }
+}
+
+// The whole grouping of a small launch (at most SG_PAIRS pairs) in one
+// block: count the pairs of each touched list, cut the lists into chunks,
+// lay out the groups, the items and the output runs.  Pairs are taken in
+// query order, eight consecutive ones per thread, so that a scan over them
+// gives every query one contiguous block of runs.  It replaces a memset and
+// three launches, and looks only at the lists the pairs touch, not at all L
+// (61 queries x 31 lists of 16,384: 64 us before, most of it in the plan).
+constexpr int SG_PER = 8;
+constexpr int SG_PAIRS = 1024 * SG_PER;
+__global__ __launch_bounds__(1024) void k_srch_small(
+    const int32_t *__restrict__ probes, int64_t nq, int P, int p0, int p1, int L, bool dedupe,
+    const int32_t *__restrict__ nslabs, const int32_t *__restrict__ list_live, int tq, int chmax,
+    int spc, int ips, int64_t item_cap, int64_t slab_bytes, int32_t *lcnt, int32_t *touched,
+    int32_t *loff, int32_t *nch, int2 *items, int32_t *qlist, int32_t *prun, int2 *qrun, Ctl *ctl,
+    int64_t run_cap, int64_t *stat, uint32_t *err)
+{
+    pdl_begin();
+    __shared__ int32_t sh[64];
+    __shared__ unsigned long long sw[32];
+    __shared__ int s_nt, s_base;
+    const int tid = threadIdx.x, np = p1 - p0, n = (int)nq * np;
+    const int per = (n + 1023) / 1024;  // <= SG_PER
+    int ev[SG_PER], lv[SG_PER], rk[SG_PER];  // n <= SG_PAIRS, P <= 1024: ev fits
+    if (tid == 0) s_nt = 0;
+#pragma unroll
+    for (int i = 0; i < SG_PER; ++i) {
+        const int t = tid * per + i;
+        ev[i] = i < per && t < n ? (t / np) * P + p0 + t % np : -1;
+        lv[i] = ev[i] >= 0 ? probes[ev[i]] : -1;
+        if (lv[i] >= L) lv[i] = -1;
+    }
+    if (dedupe)
+#pragma unroll
+        for (int i = 0; i < SG_PER; ++i) {
+            if (lv[i] < 0) continue;
+            for (int f = (ev[i] / P) * P; f < ev[i]; ++f)
+                if (probes[f] == lv[i]) {
+                    lv[i] = -1;
+                    break;
+                }
+        }
+#pragma unroll
+    for (int i = 0; i < SG_PER; ++i)
+        if (lv[i] >= 0) lcnt[lv[i]] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < SG_PER; ++i) {
+        rk[i] = lv[i] >= 0 ? atomicAdd(&lcnt[lv[i]], 1) : -1;
+        if (rk[i] == 0) touched[atomicAdd(&s_nt, 1)] = lv[i];
+    }
+    __syncthreads();
+    const int nt = s_nt;
+    // the touched lists: chunks, groups, items
+    unsigned long long wsum = 0;
+    for (int j = tid; j < nt; j += 1024) {
+        const int l = touched[j], m = __ldcg(lcnt + l), ns = nslabs[l];
+        if (ns > 0) wsum += (unsigned long long)((m + tq - 1) / tq) * ns;
+    }
+    const int target = chunk_target(block_work(wsum, sw), spc, ips);
+    int32_t ca = 0, cb = 0;
+    ScanCount cnt;
+    for (int j = tid; j < nt; j += 1024) {
+        const int l = touched[j], m = __ldcg(lcnt + l), ns = nslabs[l], k = (m + tq - 1) / tq;
+        const int c = ns > 0 ? min(min(chmax, max(1, (ns + target - 1) / target)), ns) : 0;
+        nch[l] = c;
+        ca += m;
+        cb += k * c;
+        if (c) cnt.list(m, k, ns, list_live[l], slab_bytes);
+    }
+    if (stat) cnt.add_to(stat);
+    int32_t ea = ca, eb = cb, ta, tb;
+    block_scan2(ea, eb, sh, &ta, &tb);
+    ea -= ca;
+    eb -= cb;
+    for (int j = tid; j < nt; j += 1024) {
+        const int l = touched[j], m = __ldcg(lcnt + l), c = nch[l], k = (m + tq - 1) / tq;
+        loff[l] = ea;
+        for (int t = 0; t < k * c; ++t)
+            if (eb + t < item_cap) items[eb + t] = make_int2(l, ((t / c) << 8) | (t % c));
+        ea += m;
+        eb += k * c;
+    }
+    if (tid == 0) {
+        if (tb > item_cap) atomicOr(err, ERR_PLAN);
+        ctl->nitems = (int32_t)min((int64_t)tb, item_cap);
+        ctl->nscan = ta;
+        ctl->next_item = 0;
+    }
+    __syncthreads();
+    // the pairs: their place in the list's group, their output runs
+    int cv[SG_PER], mine = 0;
+#pragma unroll
+    for (int i = 0; i < SG_PER; ++i) {
+        cv[i] = 0;
+        if (lv[i] < 0) continue;
+        qlist[loff[lv[i]] + rk[i]] = ev[i];
+        cv[i] = nch[lv[i]];
+        mine += cv[i];
+    }
+    int32_t run = mine, dummy = 0, total, td;
+    block_scan2(run, dummy, sh, &total, &td);
+    if (tid == 0) s_base = atomicAdd(&ctl->nruns, total);
+    __syncthreads();
+    const int base = s_base;
+    const bool fits = base >= 0 && (int64_t)base + total <= run_cap;
+    if (!fits && tid == 0) atomicOr(err, ERR_PLAN);
+    run += base - mine;
+    int2 *qr = qrun + (p0 > 0 ? nq : 0);
+    const int first = run;
+#pragma unroll
+    for (int i = 0; i < SG_PER; ++i) {
+        if (ev[i] < 0) continue;
+        prun[ev[i]] = cv[i] > 0 && fits ? run : -1;
+        if (ev[i] % P == p0) qr[ev[i] / P].x = fits ? run : 0;
+        run += cv[i];
+    }
+    __syncthreads();  // every query's first run is written
+    run = first;
+#pragma unroll
+    for (int i = 0; i < SG_PER; ++i) {
+        if (ev[i] < 0) continue;
+        run += cv[i];
+        if (ev[i] % P == p1 - 1) {
+            const int q = ev[i] / P;
+            qr[q].y = fits ? run - qr[q].x : 0;
+        }
     }
 }
 
@@ -264,7 +453,7 @@ struct ScanArgs {
     const float *q;
     int64_t nq;
     int P, K, M;
-    const int32_t *qlist, *loff, *lcnt, *ibase, *nch;
+    const int32_t *qlist, *loff, *lcnt, *nch;
     const int32_t *prun;  // first output run of each pair
     const int2 *items;
     float *part_d;
@@ -954,13 +1143,22 @@ void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_
                  cudaStream_t st, bool stats)
 {
     const int L = ix->nlist;
-    cudaMemsetAsync(s.lcnt, 0, sizeof(int32_t) * L, st);
     const int64_t n = nq * (p1 - p0);
+    if (n <= SG_PAIRS) {
+        const int tg = prof_begin(ix, PROF_GROUP, 1, st);
+        launch_pdl(k_srch_small, 1, 1024, 0, st, probes, nq, P, p0, p1, L, dedupe, ix->nslabs,
+                   ix->list_live, pl.tq, pl.ch, pl.slabs_per_chunk, pl.ips, pl.item_cap, slab_bytes,
+                   s.lcnt, s.touched, s.loff, s.nch, s.items, s.qlist, s.prun, s.qrun, ix->ctl,
+                   pl.run_cap, stats ? ix->stat : nullptr, ix->err);
+        prof_end(ix, tg, st);
+        return;
+    }
+    cudaMemsetAsync(s.lcnt, 0, sizeof(int32_t) * L, st);
     const int g = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
     const int tg = prof_begin(ix, PROF_GROUP, 3, st);
     launch_pdl(k_srch_hist, g, 256, 0, st, probes, nq, P, p0, p1, L, dedupe, s.lcnt, s.prank);
     launch_pdl(k_srch_plan, 1, 1024, 0, st, s.lcnt, ix->nslabs, ix->list_live, L, pl.tq, pl.ch,
-               pl.slabs_per_chunk, pl.ips, pl.item_cap, slab_bytes, s.loff, s.ibase, s.nch, s.items,
+               pl.slabs_per_chunk, pl.ips, pl.item_cap, slab_bytes, s.loff, s.nch, s.items,
                ix->ctl, stats ? ix->stat : nullptr, ix->err);
     if (p1 - p0 >= 8) {
         const int gs = (int)std::max<int64_t>(1, std::min<int64_t>((nq + SC_Q - 1) / SC_Q, 152 * 16));
@@ -992,7 +1190,6 @@ void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t
     a.qlist = s.qlist;
     a.loff = s.loff;
     a.lcnt = s.lcnt;
-    a.ibase = s.ibase;
     a.nch = s.nch;
     a.part_d = s.part_d;
     a.part_i = s.part_i;

@@ -70,7 +70,7 @@ struct TcArgs {
     const float *q;
     int64_t nq;
     int P, K, M;
-    const int32_t *qlist, *loff, *lcnt, *ibase, *nch;
+    const int32_t *qlist, *loff, *lcnt, *nch;
     const int32_t *prun;  // first output run of each pair (-1: not scanned)
     const int2 *items;
     const float *qn, *qsc;
@@ -1851,7 +1851,6 @@ void scan_lists_tc(sivf_index *ix, int dtype, const float *q, int64_t nq, int P,
     a.qlist = s.qlist;
     a.loff = s.loff;
     a.lcnt = s.lcnt;
-    a.ibase = s.ibase;
     a.nch = s.nch;
     a.part_d = s.part_d;
     a.part_i = s.part_i;

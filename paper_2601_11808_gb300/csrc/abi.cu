@@ -262,6 +262,7 @@ sivf_status sivf_create(const sivf_config *cfg, sivf_index **out)
     if (ix->dtypes & (1u << SIVF_FP8E4M3)) ALLOC(ix->x8, rows * d);
     if (ix->dtypes & (1u << SIVF_FP8E4M3)) ALLOC(ix->rnorm, rows);
     ALLOC(ix->inv_scale8, (size_t)L);
+    ALLOC(ix->lrad2, (size_t)L);
     ALLOC(ix->xnorm, rows);
     ALLOC(ix->ids, rows);
     ALLOC(ix->bits, S * ix->W);
@@ -285,6 +286,7 @@ sivf_status sivf_create(const sivf_config *cfg, sivf_index **out)
         cudaMemset(ix->head, 0xff, (size_t)L * 4) != cudaSuccess ||
         cudaMemset(ix->nslabs, 0, (size_t)L * 4) != cudaSuccess ||
         cudaMemset(ix->list_live, 0, (size_t)L * 4) != cudaSuccess ||
+        cudaMemset(ix->lrad2, 0, (size_t)L * 4) != cudaSuccess ||
         cudaMemset(ix->att, 0xff, (size_t)ix->n_max * 8) != cudaSuccess ||
         cudaMemset(ix->claim, 0xff, (size_t)ix->n_max * 4) != cudaSuccess ||
         cudaMemset(ix->list_flag, 0, (size_t)L * 4) != cudaSuccess ||
@@ -309,7 +311,7 @@ sivf_status sivf_destroy(sivf_index *ix)
     if (!ix) return SIVF_OK;
     cudaDeviceSynchronize();
     void *ptrs[] = {ix->cent, ix->cnorm, ix->cnrm_up, ix->cent_bf16, ix->cent_lo, ix->x32, ix->xb16,
-                    ix->x8, ix->rnorm, ix->inv_scale8, ix->xnorm, ix->ids, ix->bits, ix->meta,
+                    ix->x8, ix->rnorm, ix->inv_scale8, ix->lrad2, ix->xnorm, ix->ids, ix->bits, ix->meta,
                     ix->free_list, ix->free_top, ix->head, ix->nslabs, ix->list_live, ix->dir, ix->att,
                     ix->claim, ix->list_flag, ix->aff_flag, ix->runcnt, ix->err};
     for (void *p : ptrs)
@@ -346,6 +348,8 @@ sivf_status sivf_set_centroids(sivf_index *ix, const float *c, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     CUDA_TRY(ix, cudaMemcpyAsync(ix->cent, c, sizeof(float) * ix->nlist * ix->d,
                                  cudaMemcpyDeviceToDevice, s));
+    // no members: radii left by deleted ones belong to the old centroids
+    CUDA_TRY(ix, cudaMemsetAsync(ix->lrad2, 0, sizeof(float) * ix->nlist, s));
     centroid_prep(ix, s);
     CUDA_TRY(ix, cudaGetLastError());
     CUDA_TRY(ix, assign_stage_choose(ix, s));
@@ -404,6 +408,7 @@ sivf_status sivf_train(sivf_index *ix, const float *x, int64_t n, int iters, uin
     int64_t *rows_dev = b.take<int64_t>((size_t)L);
     CUDA_TRY(ix, cudaMemcpy(rows_dev, rows.data(), sizeof(int64_t) * L, cudaMemcpyHostToDevice));
     CUDA_TRY(ix, cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), s));
+    CUDA_TRY(ix, cudaMemsetAsync(ix->lrad2, 0, sizeof(float) * L, s));
     train_gather(ix, x, rows_dev, s);
     centroid_prep(ix, s);
     // the assignment's first stage is chosen on the initial centroids and
@@ -798,13 +803,16 @@ static sivf_status search_impl(sivf_index *ix, const float *q, int64_t nq, int k
             coarse_topP(ix, qq, m, P, probes, Dbuf, rows, s);
         if (!tc) {
             scan_lists(ix, qq, m, P, probes, probes_in != nullptr && !probes_unique, pl, sc, s);
-            merge_topk(ix, m, P, probes, pl, sc, k, dist + q0 * k, labels + q0 * k, s);
+            merge_topk(ix, m, P, pl, sc, k, dist + q0 * k, labels + q0 * k, s);
         } else {
             const int esz = dtype == SIVF_BF16 ? 2 : 1;
             // per slab: payload copy, ||x||^2 and the validity bitmap
             const int64_t sb = (int64_t)ix->C * (ix->d * esz + 4) + ix->C / 8;
             CUDA_TRY(ix, cudaMemsetAsync(sc.thr, 0x7f, sizeof(float) * m, s));
-            if (fp8) pair_prep(ix, qq, m, P, probes, sc.pqn, sc.pqsc, sc.qcast, s);
+            // split 1: the other lists' pairs are coded when they are grouped,
+            // unless the nearest list's bound prunes them
+            const bool later = P > 1 && pl.split == 1 && !pl.qt;
+            if (fp8) pair_prep(ix, qq, m, P, later ? 1 : P, probes, sc.pqn, sc.pqsc, sc.qcast, s);
             else query_prep(ix, qq, m, sc.qn, sc.qsc, sc.qcast, s);
             int nphase = 1;
             const bool dd = probes_in != nullptr && !probes_unique;  // repeated probes dropped
@@ -826,15 +834,18 @@ static sivf_status search_impl(sivf_index *ix, const float *q, int64_t nq, int k
             } else {
                 // vector-row scan.  With split == 1, phase 1: every query's
                 // nearest list alone sets a tight bound on its K'-th
-                // distance; phase 2 scans the other lists under it
+                // distance; phase 2 scans the other lists under it, those that
+                // can hold a vector within it (prune_pairs)
                 const int split = P > 1 && pl.split == 1 ? 1 : P;
-                group_pairs(ix, m, P, 0, split, probes, dd, pl, sc, sb, s);
+                group_pairs(ix, m, P, 0, split, probes, dd, split < P ? bound_plan(ix, pl) : pl, sc,
+                            sb, s);
                 scan_lists_tc(ix, dtype, qq, m, P, Kc, pl, sc, s);
                 if (split < P) {
                     SearchPlan pl2 = pl;  // the other lists: the plan's phase-2 tile
                     pl2.tq = pl.tq2;
                     pl2.M = pl.M2;
-                    group_pairs(ix, m, P, split, P, probes, dd, pl2, sc, sb, s);
+                    prune_pairs(ix, dtype, qq, m, P, probes, dd, sc, s);
+                    group_pairs(ix, m, P, split, P, probes, false, pl2, sc, sb, s, true, true);
                     scan_lists_tc(ix, dtype, qq, m, P, Kc, pl2, sc, s);
                 }
                 nphase = split < P ? 2 : 1;

@@ -181,6 +181,8 @@ sivf_status sivf_load(const char *path, sivf_index **out)
             return bad(SIVF_E_CUDA, "centroid preparation failed");
         ix->have_centroids = true;
     }
+    sivf::list_radii(ix, 0);
+    if (cudaDeviceSynchronize() != cudaSuccess) return bad(SIVF_E_CUDA, "list radii failed");
     if (cudaMemcpy(ix->inv_scale8, scales.data(), scales.size() * 4, cudaMemcpyHostToDevice) !=
         cudaSuccess)
         return bad(SIVF_E_CUDA, "device write failed");

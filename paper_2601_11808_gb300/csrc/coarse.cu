@@ -1674,7 +1674,7 @@ __global__ __launch_bounds__(GAP_NT) void k_cent_gap(const float *__restrict__ c
 // (single) or 3 d (split) terms.  Single: 2 ub + ub^2 (both roundings) plus
 // the accumulation; split: the dropped products xl cl, and the roundings of
 // xl and cl (each ub^2 relative), 3.1 ub^2 in all, plus the accumulation.
-static double first_stage_rel(int d, int split)
+double first_stage_rel(int d, int split)
 {
     const double ub = 1.0 / 256.0;
     const double gacc = (split == 3 ? 3.0 * d : (double)d) * std::ldexp(1.0, -22);

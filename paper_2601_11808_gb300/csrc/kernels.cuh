@@ -56,6 +56,8 @@ inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
 void centroid_prep(sivf_index *ix, cudaStream_t st);
 cudaError_t assign_stage_choose(sivf_index *ix, cudaStream_t st);
 int first_stage_split(const sivf_index *ix, int P);
+// relative error bound of the BF16 (split 1) or split BF16 (3) dot products
+double first_stage_rel(int d, int split);
 // exact top-P set of each row of x, in ascending list index; Dbuf holds
 // rows_per_chunk * nlist floats
 // rows of one coarse chunk and the scratch of a coarse selection of n rows
@@ -90,6 +92,8 @@ void insert_batch(sivf_index *ix, const int64_t *ids, const float *x, int64_t n,
                   const InsertScratch &s, cudaStream_t st);
 void remove_batch(sivf_index *ix, const int64_t *ids, int64_t n, int32_t *affected,
                   cudaStream_t st);
+// the lists' radii (lrad2) from the live rows of a loaded index
+void list_radii(sivf_index *ix, cudaStream_t st);
 
 // ---- search (scan.cu)
 struct SearchScratch {
@@ -155,21 +159,30 @@ void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t
                 bool dedupe, const SearchPlan &pl, const SearchScratch &s, cudaStream_t st);
 // group the pairs with probe rank in [p0, p1) by list and lay out the work
 // items and output runs; `stats` adds the scan's pairs and bytes to the
-// index's counters (off for the seed launch of the query-row scan)
+// index's counters (off for the seed launch of the query-row scan);
+// `flagged`: only the pairs prune_pairs left (prank >= 0) take part
 void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_t *probes,
                  bool dedupe, const SearchPlan &pl, const SearchScratch &s, int64_t slab_bytes,
-                 cudaStream_t st, bool stats = true);
-void merge_topk(sivf_index *ix, int64_t nq, int P, const int32_t *probes,
-                const SearchPlan &pl, const SearchScratch &s, int k, float *dist,
-                int64_t *labels, cudaStream_t st);
+                 cudaStream_t st, bool stats = true, bool flagged = false);
+// the pairs past each query's nearest list (p >= 1) that may hold a vector
+// within the bound the nearest list left: prank = 0, else -1; FP8 residual
+// codes of the pairs that stay
+void prune_pairs(sivf_index *ix, int dtype, const float *q, int64_t nq, int P,
+                 const int32_t *probes, bool dedupe, const SearchScratch &s, cudaStream_t st);
+// the plan of a launch over the nearest lists, whose chunks leave bounds
+SearchPlan bound_plan(const sivf_index *ix, SearchPlan pl);
+// FP32: the nearest lists are scanned first, in a launch of their own
+bool fp32_two_phase(int64_t nq, int P);
+void merge_topk(sivf_index *ix, int64_t nq, int P, const SearchPlan &pl,
+                const SearchScratch &s, int k, float *dist, int64_t *labels, cudaStream_t st);
 
 // ---- reduced-precision scan + re-rank (scan_tc.cu)
 bool tc_make_maps(sivf_index *ix);
 // BF16 form: ||q||^2, unit scale and the row rounded to BF16
 void query_prep(sivf_index *ix, const float *q, int64_t nq, float *qn, float *qsc,
                 unsigned char *qcast, cudaStream_t st);
-// FP8 residual scan: per (query, probe) pair ||q - c_l||^2, scale, E4M3 row
-void pair_prep(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t *probes,
+// FP8 residual scan: ||q - c_l||^2, scale, E4M3 row of each query's first p1 pairs
+void pair_prep(sivf_index *ix, const float *q, int64_t nq, int P, int p1, const int32_t *probes,
                float *qn, float *qsc, unsigned char *qcast, cudaStream_t st);
 bool tc_fits(const sivf_index *ix, int Kc);
 // buffer entries of 32-query tiles for K' > 128 with one tile of room and

@@ -49,7 +49,8 @@ struct IndexView {
     int32_t *free_list, *free_top;
     int32_t *head, *nslabs, *dir, *list_live;
     const float *inv_scale8;
-    const float *cent;  // [nlist, d] (FP8 residual codes)
+    const float *cent;  // [nlist, d]
+    float *lrad2;       // [nlist] bound of the members' ||x - c_l||^2
     float *rnorm;       // [S, C] ||x - c_l||^2 or null
     int64_t *att;
     int32_t *claim, *list_flag, *aff_flag, *runcnt;
@@ -84,6 +85,7 @@ static IndexView view_of(sivf_index *ix)
     v.list_live = ix->list_live;
     v.inv_scale8 = ix->inv_scale8;
     v.cent = ix->cent;
+    v.lrad2 = ix->lrad2;
     v.rnorm = ix->rnorm;
     v.att = ix->att;
     v.claim = ix->claim;
@@ -214,6 +216,7 @@ __global__ void k_reclaim(IndexView V, const int32_t *__restrict__ affected)
         hfree = __any_sync(0xffffffffu, hfree);
         if (lane == 0) {
             V.nslabs[l] = kept;
+            if (kept == 0) V.lrad2[l] = 0.f;
             if (hfree) V.head[l] = -1;
             V.aff_flag[l] = 0;
         }
@@ -457,6 +460,15 @@ __device__ __forceinline__ float half_sum(float v)
     return v;
 }
 
+// the list's bound takes in a member at FP32 ||x - c||^2 = rs (the sum's and
+// the differences' relative error is below (d + 4) u, doubled here)
+__device__ __forceinline__ void raise_radius(float *r2, float rs, int d)
+{
+    const float up = __fmul_ru(rs, 1.f + (2.f * d + 16.f) * 5.9604645e-08f);
+    // most members lie inside the bound: a load instead of an atomic
+    if (!(up <= __ldcg(r2))) atomicMax(reinterpret_cast<int *>(r2), __float_as_int(up));
+}
+
 // Two kept vectors per warp, one per half (16 lanes of 16-byte chunks): a
 // batch of 10,000 takes one wave of resident warps instead of two.  Bound
 // by HBM at large batches (read 4 d, write 4 d + copies) and by the chain of
@@ -518,15 +530,15 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
                     pk.y = *reinterpret_cast<uint32_t *>(&hi);
                     *reinterpret_cast<uint2 *>(V.xb16 + row * d + j) = pk;
                 }
+                const float4 c4 = __ldg(reinterpret_cast<const float4 *>(cl + j));
+                const float4 rv = make_float4(__fsub_rn(v.x, c4.x), __fsub_rn(v.y, c4.y),
+                                              __fsub_rn(v.z, c4.z), __fsub_rn(v.w, c4.w));
+                rs = fmaf(rv.x, rv.x, rs);
+                rs = fmaf(rv.y, rv.y, rs);
+                rs = fmaf(rv.z, rv.z, rs);
+                rs = fmaf(rv.w, rv.w, rs);
                 if (V.x8) {
                     // residual r = fl32(x - c_l), code = E4M3(fl32(r * inv))
-                    const float4 c4 = __ldg(reinterpret_cast<const float4 *>(cl + j));
-                    const float4 rv = make_float4(__fsub_rn(v.x, c4.x), __fsub_rn(v.y, c4.y),
-                                                  __fsub_rn(v.z, c4.z), __fsub_rn(v.w, c4.w));
-                    rs = fmaf(rv.x, rv.x, rs);
-                    rs = fmaf(rv.y, rv.y, rs);
-                    rs = fmaf(rv.z, rv.z, rs);
-                    rs = fmaf(rv.w, rv.w, rs);
                     float2 a = make_float2(__fmul_rn(rv.x, inv), __fmul_rn(rv.y, inv));
                     float2 b = make_float2(__fmul_rn(rv.z, inv), __fmul_rn(rv.w, inv));
                     __nv_fp8x2_storage_t pa =
@@ -544,8 +556,9 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
                 put(j, __ldcs(reinterpret_cast<const float4 *>(xi + j)));
         }
         ss = half_sum(ss);
-        if (V.x8) rs = half_sum(rs);
+        rs = half_sum(rs);
         if (on && hl == 0) {
+            raise_radius(V.lrad2 + lab[i], rs, d);
             const size_t row = (size_t)s * C + slot;
             const int64_t id = ids[i];
             V.xnorm[row] = ss;
@@ -609,7 +622,36 @@ __global__ void k_ins_publish(IndexView V, const int64_t *__restrict__ ids, int6
     }
 }
 
+// a warp per slab: its live rows' distances from their list's centroid
+__global__ void k_list_radii(IndexView V)
+{
+    pdl_begin();
+    const int lane = threadIdx.x & 31, d = V.d;
+    const int64_t nw = (int64_t)gridDim.x * blockDim.x / 32;
+    for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; s < V.n_slabs; s += nw) {
+        const int l = V.meta[s].list;
+        if (l < 0 || l >= V.nlist) continue;
+        for (int o = 0; o < V.C; ++o) {
+            if (!((V.bits[s * V.W + (o >> 5)] >> (o & 31)) & 1u)) continue;
+            const float *xr = V.x32 + ((size_t)s * V.C + o) * d, *cl = V.cent + (size_t)l * d;
+            float rs = 0.f;
+            for (int j = lane; j < d; j += 32) {
+                const float r = __fsub_rn(xr[j], cl[j]);
+                rs = fmaf(r, r, rs);
+            }
+            rs = warp_sum(rs);
+            if (lane == 0) raise_radius(V.lrad2 + l, rs, d);
+        }
+    }
+}
+
 // ---------------------------------------------------------------- drivers
+void list_radii(sivf_index *ix, cudaStream_t st)
+{
+    ix->launches += 1;
+    launch_pdl(k_list_radii, 152 * 8, 256, 0, st, view_of(ix));
+}
+
 static int grid_for(int64_t n, int per_block)
 {
     int64_t g = (n + per_block - 1) / per_block;

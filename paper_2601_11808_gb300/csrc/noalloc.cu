@@ -165,7 +165,7 @@ extern "C" sivf_status sivf_search_noalloc(sivf_index *ix, const float *q, int64
     }
     coarse_topP(ix, q, nq, P, probes, Dbuf, rows, s);
     scan_lists(ix, q, nq, P, probes, false, pl, sc, s);
-    merge_topk(ix, nq, P, probes, pl, sc, k, dist, labels, s);
+    merge_topk(ix, nq, P, pl, sc, k, dist, labels, s);
     ix->ctl = own;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(SIVF_E_CUDA, cudaGetErrorString(e));

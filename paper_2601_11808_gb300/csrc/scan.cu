@@ -23,8 +23,8 @@ namespace sivf {
 // ------------------------------------------------------ grouping by list
 // pairs (q, p) with p in [p0, p1): rank of each pair inside its list group
 __global__ void k_srch_hist(const int32_t *__restrict__ probes, int64_t nq, int P, int p0,
-                            int p1, int L, bool dedupe, int32_t *__restrict__ lcnt,
-                            int32_t *__restrict__ prank)
+                            int p1, int L, bool dedupe, bool flagged,
+                            int32_t *__restrict__ lcnt, int32_t *__restrict__ prank)
 {
     pdl_begin();
     const int np = p1 - p0;
@@ -33,7 +33,7 @@ __global__ void k_srch_hist(const int32_t *__restrict__ probes, int64_t nq, int 
          t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t e = (t / np) * P + p0 + t % np;
         const int l = probes[e];
-        bool ok = l >= 0 && l < L;
+        bool ok = l >= 0 && l < L && !(flagged && prank[e] < 0);
         if (ok && dedupe) {
             const int64_t q0 = (e / P) * P;
             for (int64_t f = q0; f < e; ++f)
@@ -208,7 +208,8 @@ constexpr int SG_PER = 8;
 constexpr int SG_PAIRS = 1024 * SG_PER;
 __global__ __launch_bounds__(1024) void k_srch_small(
     const int32_t *__restrict__ probes, int64_t nq, int P, int p0, int p1, int L, bool dedupe,
-    const int32_t *__restrict__ nslabs, const int32_t *__restrict__ list_live, int tq, int chmax,
+    const int32_t *__restrict__ flags, const int32_t *__restrict__ nslabs,
+    const int32_t *__restrict__ list_live, int tq, int chmax,
     int spc, int ips, int64_t item_cap, int64_t slab_bytes, int32_t *lcnt, int32_t *touched,
     int32_t *loff, int32_t *nch, int2 *items, int32_t *qlist, int32_t *prun, int2 *qrun, Ctl *ctl,
     int64_t run_cap, int64_t *stat, uint32_t *err)
@@ -226,7 +227,7 @@ __global__ __launch_bounds__(1024) void k_srch_small(
         const int t = tid * per + i;
         ev[i] = i < per && t < n ? (t / np) * P + p0 + t % np : -1;
         lv[i] = ev[i] >= 0 ? probes[ev[i]] : -1;
-        if (lv[i] >= L) lv[i] = -1;
+        if (lv[i] >= L || (flags && ev[i] >= 0 && flags[ev[i]] < 0)) lv[i] = -1;
     }
     if (dedupe)
 #pragma unroll
@@ -325,6 +326,205 @@ __global__ __launch_bounds__(1024) void k_srch_small(
         }
     }
 }
+
+// ------------------------------------------------------- pair pruning
+// Which of a query's farther lists (p >= 1) may hold a vector within the
+// bound t its nearest list left.  Every member x of list l lies within R_l
+// of the centroid, so ||q - x|| >= ||q - c_l|| - R_l (triangle inequality);
+// when the scan's own distance of every x is then provably above t, the pair
+// takes no part: none of its vectors could have been kept, so the results
+// are the same.  Where cells overlap (a query's neighbours in one cluster)
+// nothing is pruned and the kernel costs a read of each pair's centroid;
+// between separate clusters it removes the pair's whole scan: the 63 farther
+// lists of a Deep-like search (10,000 queries, 4,096 lists) took 2.4 of 5.4
+// ms.  Lower bounds of the scan's distance D, rq = ||q - c_l||, rounded
+// towards keeping the pair:
+//   FP32: D >= (rq - R)^2 up to the direct form's rounding;
+//   BF16: D >= (rq - R)^2 - 2 e ||q|| (||c|| + R), e the error of the BF16
+//     products (first_stage_rel, doubled), and the norms' roundings;
+//   FP8: D = rq^2 + rx^2 - 2 s q^.x^ with ||q^|| <= rq + eq and ||x^|| <= rx +
+//     ex (E4M3 rounds to 2^-4 relative, 2^-10 of a code unit below the
+//     smallest normal; saturation only shortens x^), least at rx = R.
+// One warp takes PR_P consecutive pairs of one query, their centroid rows in
+// flight together; a FP8 pair that stays gets its residual codes here.
+constexpr int PR_P = 4;
+struct PruneArgs {
+    const float *q;
+    int64_t nq;
+    int P, d, L;
+    const int32_t *probes;
+    bool dedupe;
+    const float *cent, *cnrm_up, *lrad2, *thr, *inv_scale8, *qn;
+    float e_bf16;
+    float *pqn, *pqsc;
+    unsigned char *qcast;
+    int32_t *prank;
+};
+
+template <int DT>  // sivf_scan_dtype
+__global__ __launch_bounds__(256) void k_pair_prune(PruneArgs a)
+{
+    pdl_begin();
+    constexpr int NV = kMaxD / 128;  // float4 of a row per lane
+    const int lane = threadIdx.x & 31, d = a.d, n4 = d >> 2;
+    const int np = a.P - 1, ng = (np + PR_P - 1) / PR_P;
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (t >= a.nq * ng) return;  // whole warps
+    const int64_t qi = t / ng;
+    const int pb = 1 + (int)(t % ng) * PR_P;
+    const float *qr = a.q + (size_t)qi * d;
+    int lv[PR_P];
+    float4 r[PR_P][NV];
+#pragma unroll
+    for (int k = 0; k < PR_P; ++k) {
+        const int64_t e = qi * a.P + pb + k;
+        lv[k] = pb + k < a.P ? a.probes[e] : -1;
+        if (lv[k] >= a.L) lv[k] = -1;
+    }
+#pragma unroll
+    for (int k = 0; k < PR_P; ++k)
+#pragma unroll
+        for (int u = 0; u < NV; ++u) {
+            const int j4 = lane + 32 * u;
+            r[k][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (lv[k] >= 0 && j4 < n4)
+                r[k][u] = __ldg(reinterpret_cast<const float4 *>(a.cent + (size_t)lv[k] * d) + j4);
+        }
+    float ss[PR_P], mx[PR_P];
+#pragma unroll
+    for (int k = 0; k < PR_P; ++k) ss[k] = mx[k] = 0.f;
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+        const int j4 = lane + 32 * u;
+        if (j4 >= n4) break;
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(qr) + j4);
+#pragma unroll
+        for (int k = 0; k < PR_P; ++k) {
+            const float4 c = r[k][u];
+            r[k][u] = make_float4(__fsub_rn(v.x, c.x), __fsub_rn(v.y, c.y), __fsub_rn(v.z, c.z),
+                                  __fsub_rn(v.w, c.w));
+            ss[k] = fmaf(r[k][u].x, r[k][u].x, ss[k]);
+            ss[k] = fmaf(r[k][u].y, r[k][u].y, ss[k]);
+            ss[k] = fmaf(r[k][u].z, r[k][u].z, ss[k]);
+            ss[k] = fmaf(r[k][u].w, r[k][u].w, ss[k]);
+            if (DT == SIVF_FP8E4M3)
+                mx[k] = fmaxf(mx[k], fmaxf(fmaxf(fabsf(r[k][u].x), fabsf(r[k][u].y)),
+                                           fmaxf(fabsf(r[k][u].z), fabsf(r[k][u].w))));
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < PR_P; ++k) ss[k] = warp_sum(ss[k]);
+    if (DT == SIVF_FP8E4M3)
+#pragma unroll
+        for (int k = 0; k < PR_P; ++k)
+            for (int o = 16; o > 0; o >>= 1) mx[k] = fmaxf(mx[k], __shfl_xor_sync(0xffffffffu, mx[k], o));
+    const float u32 = 5.9604645e-08f;                    // 2^-24
+    const float up = 1.f + (2.f * d + 32.f) * u32, dn = 1.f - (2.f * d + 32.f) * u32;
+    const float bound = __ldcg(a.thr + qi);
+#pragma unroll
+    for (int k = 0; k < PR_P; ++k) {
+        if (pb + k >= a.P) break;  // warp-uniform
+        const int64_t e = qi * a.P + pb + k;
+        bool keep = lv[k] >= 0;
+        if (keep && a.dedupe) {
+            bool dup = false;
+            for (int f = lane; f < pb + k; f += 32) dup |= a.probes[qi * a.P + f] == lv[k];
+            keep = !__any_sync(0xffffffffu, dup);
+        }
+        const float sc = mx[k] > 0.f ? 448.f / (2.f * mx[k]) : 1.f;
+        if (keep) {
+            const float R = __fsqrt_ru(__ldg(a.lrad2 + lv[k]));
+            const float rlo = __fsqrt_rd(__fmul_rd(ss[k], dn)), rhi = __fsqrt_ru(__fmul_ru(ss[k], up));
+            const float gap = __fsub_rd(rlo, R);
+            float lo = -INFINITY;  // lower bound of the scan's distances
+            if (gap > 0.f) {
+                if (DT == SIVF_FP32) {
+                    lo = __fmul_rd(__fmul_rd(gap, gap), dn);
+                } else if (DT == SIVF_BF16) {
+                    const float qn = __fsqrt_ru(__fmul_ru(__ldg(a.qn + qi), up));
+                    const float xn = __fadd_ru(__ldg(a.cnrm_up + lv[k]), R);
+                    const float n2 = __fadd_ru(__fmul_ru(qn, qn), __fmul_ru(xn, xn));
+                    const float err = __fadd_ru(__fmul_ru(__fmul_ru(a.e_bf16, qn), __fmul_ru(2.f, xn)),
+                                                __fmul_ru(n2, (2.f * d + 64.f) * u32));
+                    lo = __fsub_rd(__fmul_rd(gap, gap), err);
+                } else {
+                    const float sq = sqrtf((float)d) * 1.01f * 9.765625e-04f;  // 2^-10
+                    const float A = __fadd_ru(__fmul_ru(rhi, 1.0626f), __fdiv_ru(sq, sc));
+                    const float X = __fadd_ru(__fmul_ru(R, 1.0626f),
+                                              __fdiv_ru(sq, __ldg(a.inv_scale8 + lv[k])));
+                    // products' accumulation (4 d u) and the norms' roundings
+                    const float err = __fmul_ru(__fadd_ru(__fmul_ru(rhi, rhi), __fmul_ru(A, X)),
+                                                (16.f * d + 64.f) * u32);
+                    lo = __fsub_rd(__fsub_rd(__fadd_rd(__fmul_rd(rlo, rlo), __fmul_rd(__fmul_rd(R, R), dn)),
+                                             __fmul_ru(2.f, __fmul_ru(A, X))),
+                                   err);
+                }
+            }
+            keep = !(lo > bound);
+        }
+        if (lane == 0) a.prank[e] = keep ? 0 : -1;
+        if (DT == SIVF_FP8E4M3 && keep) {
+            if (lane == 0) {
+                a.pqn[e] = ss[k];
+                a.pqsc[e] = sc;
+            }
+#pragma unroll
+            for (int u = 0; u < NV; ++u) {
+                const int j4 = lane + 32 * u;
+                if (j4 >= n4) break;
+                const uint32_t lo8 = __nv_cvt_float2_to_fp8x2(
+                    make_float2(__fmul_rn(r[k][u].x, sc), __fmul_rn(r[k][u].y, sc)), __NV_SATFINITE, __NV_E4M3);
+                const uint32_t hi8 = __nv_cvt_float2_to_fp8x2(
+                    make_float2(__fmul_rn(r[k][u].z, sc), __fmul_rn(r[k][u].w, sc)), __NV_SATFINITE, __NV_E4M3);
+                reinterpret_cast<uint32_t *>(a.qcast + (size_t)e * d)[j4] = (lo8 & 0xffffu) | (hi8 << 16);
+            }
+        }
+    }
+}
+
+void prune_pairs(sivf_index *ix, int dtype, const float *q, int64_t nq, int P,
+                 const int32_t *probes, bool dedupe, const SearchScratch &s, cudaStream_t st)
+{
+    PruneArgs a;
+    a.q = q;
+    a.nq = nq;
+    a.P = P;
+    a.d = ix->d;
+    a.L = ix->nlist;
+    a.probes = probes;
+    a.dedupe = dedupe;
+    a.cent = ix->cent;
+    a.cnrm_up = ix->cnrm_up;
+    a.lrad2 = ix->lrad2;
+    a.thr = s.thr;
+    a.inv_scale8 = ix->inv_scale8;
+    a.qn = s.qn;
+    a.e_bf16 = (float)(2.0 * first_stage_rel(ix->d, 1) * (1.0 + 1e-6));
+    a.pqn = s.pqn;
+    a.pqsc = s.pqsc;
+    a.qcast = s.qcast;
+    a.prank = s.prank;
+    const int64_t warps = nq * ((P - 1 + PR_P - 1) / PR_P);
+    const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
+    const int tg = prof_begin(ix, PROF_GROUP, 1, st);
+    if (dtype == SIVF_FP32) launch_pdl(k_pair_prune<SIVF_FP32>, blocks, 256, 0, st, a);
+    else if (dtype == SIVF_BF16) launch_pdl(k_pair_prune<SIVF_BF16>, blocks, 256, 0, st, a);
+    else launch_pdl(k_pair_prune<SIVF_FP8E4M3>, blocks, 256, 0, st, a);
+    prof_end(ix, tg, st);
+}
+
+// Phase 1's plan: a chunk of the nearest list leaves a bound only when it
+// holds K vectors, so it gets twice that many slots
+SearchPlan bound_plan(const sivf_index *ix, SearchPlan pl)
+{
+    pl.slabs_per_chunk = std::max(pl.slabs_per_chunk, (2 * pl.K + ix->C - 1) / ix->C);
+    return pl;
+}
+
+// A launch of the nearest lists alone pays where the others have work to
+// save: its four extra launches cost about 12 us, a scan of 2,048 pairs more
+// than that; a handful of pairs is scanned at once
+bool fp32_two_phase(int64_t nq, int P) { return P > 1 && nq * P >= 2048; }
 
 // One thread per query, whole warps together: each pair goes to its list's
 // group (qlist), and the query's pairs of this phase reserve consecutive
@@ -915,25 +1115,83 @@ __global__ __launch_bounds__(SCAN_NT, 1) void k_scan(ScanArgs a)
 
 // ------------------------------------------------------- per-query merge
 constexpr int MERGE_NT = 128;
-constexpr int MERGE_RUNS_PER_LANE = 64;
+constexpr int MERGE_RUNS_PER_LANE = 64;  // both phases' runs: at most 2,048 per query
 
+// One warp per query.  A query's runs of one scan phase (K entries each,
+// sorted, padded with (+inf, -1)) are contiguous, and at least k entries lie
+// at or below its shared bound after the scan: the warp streams them, gathers
+// those (usually little more than k) and sorts them in registers.  Only when
+// there are more than 32 E (ties, or k near 32 E) does it walk all runs, a
+// cursor per run, one result after the other.
+template <int E>
 __global__ __launch_bounds__(MERGE_NT) void k_merge(const int2 *__restrict__ qrun, int64_t nq,
-                                                    int K, int k,
+                                                    int nphase, int K, int k,
+                                                    const float *__restrict__ thr,
                                                     const float *__restrict__ part_d,
                                                     const int64_t *__restrict__ part_i,
                                                     float *__restrict__ dist,
                                                     int64_t *__restrict__ labels)
 {
     pdl_begin();
-    const int lane = threadIdx.x & 31;
+    constexpr int MU = 8;  // loads in flight per lane
+    __shared__ float sd[MERGE_NT / 32][32 * E];
+    __shared__ int64_t si[MERGE_NT / 32][32 * E];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t q = (blockIdx.x * (int64_t)MERGE_NT + threadIdx.x) >> 5;
-    if (q >= nq) return;
-    // the query's runs (sorted, padded with (+inf, -1)) are contiguous:
-    // r = lane, lane + 32, ... of them, cursor per run kept in local memory
-    const int2 qr = qrun[q];
+    if (q >= nq) return;  // whole warps
+    const int2 r0 = qrun[q];
+    const int2 r1 = nphase > 1 ? qrun[nq + q] : make_int2(0, 0);
+    const float bound = thr[q];
+    int have = 0;
+    for (int ph = 0; ph < 2 && k <= 32 * E; ++ph) {
+        const int64_t b = (int64_t)(ph ? r1.x : r0.x) * K;
+        const int64_t n = (int64_t)(ph ? r1.y : r0.y) * K;
+        for (int64_t i0 = lane; i0 - lane < n && have <= 32 * E; i0 += 32 * MU) {
+            float v[MU];
+            bool in[MU];
+#pragma unroll
+            for (int u = 0; u < MU; ++u)
+                v[u] = i0 + 32 * u < n ? part_d[b + i0 + 32 * u] : INFINITY;
+#pragma unroll
+            for (int u = 0; u < MU; ++u) in[u] = v[u] <= bound;  // pads are +inf
+#pragma unroll
+            for (int u = 0; u < MU; ++u) {
+                const uint32_t mk = __ballot_sync(0xffffffffu, in[u]);
+                const int p = have + __popc(mk & lanemask_lt());
+                if (in[u] && p < 32 * E) {
+                    sd[w][p] = v[u];
+                    si[w][p] = part_i[b + i0 + 32 * u];
+                }
+                have += __popc(mk);
+            }
+        }
+    }
+    __syncwarp();
+    if (k <= 32 * E && have <= 32 * E) {
+        float v[E];
+        int64_t id[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = lane + 32 * e;
+            v[e] = i < have ? sd[w][i] : INFINITY;
+            id[e] = i < have ? si[w][i] : 0x7fffffffffffffffLL;
+        }
+        warp_bitonic_sort<E>(v, id, lane);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = lane + 32 * e;
+            if (i < k) {
+                dist[q * k + i] = i < have ? v[e] : INFINITY;
+                labels[q * k + i] = i < have ? id[e] : -1;
+            }
+        }
+        return;
+    }
+    // cursors: run r = lane + 32 j of both phases' runs
+    const int NR = r0.y + r1.y;
     int cur[MERGE_RUNS_PER_LANE];
     int nrun = 0;
-    for (int r = lane; r < qr.y && nrun < MERGE_RUNS_PER_LANE; r += 32) cur[nrun++] = 0;
+    for (int r = lane; r < NR && nrun < MERGE_RUNS_PER_LANE; r += 32) cur[nrun++] = 0;
     auto head = [&](int j, float &hd, int64_t &hi) {
         int r = lane + 32 * j;
         if (cur[j] >= K) {
@@ -941,7 +1199,7 @@ __global__ __launch_bounds__(MERGE_NT) void k_merge(const int2 *__restrict__ qru
             hi = -1;
             return;
         }
-        int64_t e = ((int64_t)qr.x + r) * K + cur[j];
+        const int64_t e = (int64_t)(r < r0.y ? r0.x + r : r1.x + (r - r0.y)) * K + cur[j];
         hd = part_d[e];
         hi = part_i[e];
         if (hi < 0) hd = INFINITY;
@@ -1140,14 +1398,14 @@ bool scan_fits(const sivf_index *ix, int K)
 
 void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_t *probes,
                  bool dedupe, const SearchPlan &pl, const SearchScratch &s, int64_t slab_bytes,
-                 cudaStream_t st, bool stats)
+                 cudaStream_t st, bool stats, bool flagged)
 {
     const int L = ix->nlist;
     const int64_t n = nq * (p1 - p0);
     if (n <= SG_PAIRS) {
         const int tg = prof_begin(ix, PROF_GROUP, 1, st);
-        launch_pdl(k_srch_small, 1, 1024, 0, st, probes, nq, P, p0, p1, L, dedupe, ix->nslabs,
-                   ix->list_live, pl.tq, pl.ch, pl.slabs_per_chunk, pl.ips, pl.item_cap, slab_bytes,
+        launch_pdl(k_srch_small, 1, 1024, 0, st, probes, nq, P, p0, p1, L, dedupe,
+                   flagged ? s.prank : nullptr, ix->nslabs, ix->list_live, pl.tq, pl.ch, pl.slabs_per_chunk, pl.ips, pl.item_cap, slab_bytes,
                    s.lcnt, s.touched, s.loff, s.nch, s.items, s.qlist, s.prun, s.qrun, ix->ctl,
                    pl.run_cap, stats ? ix->stat : nullptr, ix->err);
         prof_end(ix, tg, st);
@@ -1156,7 +1414,7 @@ void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_
     cudaMemsetAsync(s.lcnt, 0, sizeof(int32_t) * L, st);
     const int g = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
     const int tg = prof_begin(ix, PROF_GROUP, 3, st);
-    launch_pdl(k_srch_hist, g, 256, 0, st, probes, nq, P, p0, p1, L, dedupe, s.lcnt, s.prank);
+    launch_pdl(k_srch_hist, g, 256, 0, st, probes, nq, P, p0, p1, L, dedupe, flagged, s.lcnt, s.prank);
     launch_pdl(k_srch_plan, 1, 1024, 0, st, s.lcnt, ix->nslabs, ix->list_live, L, pl.tq, pl.ch,
                pl.slabs_per_chunk, pl.ips, pl.item_cap, slab_bytes, s.loff, s.nch, s.items,
                ix->ctl, stats ? ix->stat : nullptr, ix->err);
@@ -1172,13 +1430,24 @@ void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_
     prof_end(ix, tg, st);
 }
 
+static void scan_launch(sivf_index *ix, int tq, const ScanArgs &a, size_t smem, cudaStream_t st)
+{
+    const int grid = 152;  // persistent: one CTA per SM
+#define SIVF_SCAN_CASE(TQ_, C_) \
+    if (tq == TQ_ && ix->C == C_) return launch_scan<TQ_, C_>(ix, a, smem, grid, st);
+    SIVF_SCAN_CASE(8, 32) SIVF_SCAN_CASE(16, 32) SIVF_SCAN_CASE(32, 32) SIVF_SCAN_CASE(64, 32)
+    SIVF_SCAN_CASE(8, 64) SIVF_SCAN_CASE(16, 64) SIVF_SCAN_CASE(32, 64) SIVF_SCAN_CASE(64, 64)
+    SIVF_SCAN_CASE(8, 128) SIVF_SCAN_CASE(16, 128) SIVF_SCAN_CASE(32, 128)
+    SIVF_SCAN_CASE(64, 128)
+#undef SIVF_SCAN_CASE
+}
+
 void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t *probes,
                 bool dedupe, const SearchPlan &pl, const SearchScratch &s, cudaStream_t st)
 {
     const int L = ix->nlist;
     cudaMemsetAsync(s.thr, 0x7f, sizeof(float) * nq, st);  // 3.4e38: no bound yet
-    group_pairs(ix, nq, P, 0, P, probes, dedupe, pl, s,
-                (int64_t)ix->C * (ix->d * 4 + 8) + ix->C / 8, st);
+    const int64_t sb = (int64_t)ix->C * (ix->d * 4 + 8) + ix->C / 8;
 
     ScanArgs a;
     a.q = q;
@@ -1208,25 +1477,31 @@ void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t
     a.ctl = ix->ctl;
     a.err = ix->err;
     const size_t smem = scan_smem(pl.tq, ix->C, ix->d, a.M).total;
-    const int grid = 152;  // persistent: one CTA per SM
-#define SIVF_SCAN_CASE(TQ_, C_) \
-    if (pl.tq == TQ_ && ix->C == C_) return launch_scan<TQ_, C_>(ix, a, smem, grid, st);
-    SIVF_SCAN_CASE(8, 32) SIVF_SCAN_CASE(16, 32) SIVF_SCAN_CASE(32, 32) SIVF_SCAN_CASE(64, 32)
-    SIVF_SCAN_CASE(8, 64) SIVF_SCAN_CASE(16, 64) SIVF_SCAN_CASE(32, 64) SIVF_SCAN_CASE(64, 64)
-    SIVF_SCAN_CASE(8, 128) SIVF_SCAN_CASE(16, 128) SIVF_SCAN_CASE(32, 128)
-    SIVF_SCAN_CASE(64, 128)
-#undef SIVF_SCAN_CASE
+    // the nearest lists first: the others then meet a tight bound, which most
+    // of their vectors do not pass and whole lists may not (prune_pairs)
+    const int split = fp32_two_phase(nq, P) ? 1 : P;
+    group_pairs(ix, nq, P, 0, split, probes, dedupe, split < P ? bound_plan(ix, pl) : pl, s, sb, st);
+    scan_launch(ix, pl.tq, a, smem, st);
+    if (split < P) {
+        prune_pairs(ix, SIVF_FP32, q, nq, P, probes, dedupe, s, st);
+        group_pairs(ix, nq, P, split, P, probes, false, pl, s, sb, st, true, true);
+        scan_launch(ix, pl.tq, a, smem, st);
+    }
 }
 
-void merge_topk(sivf_index *ix, int64_t nq, int P, const int32_t *probes,
-                const SearchPlan &pl, const SearchScratch &s, int k, float *dist,
-                int64_t *labels, cudaStream_t st)
+void merge_topk(sivf_index *ix, int64_t nq, int P, const SearchPlan &pl,
+                const SearchScratch &s, int k, float *dist, int64_t *labels, cudaStream_t st)
 {
-    int64_t warps = nq;
-    int64_t blocks = (warps * 32 + MERGE_NT - 1) / MERGE_NT;
+    const unsigned blocks = (unsigned)((nq * 32 + MERGE_NT - 1) / MERGE_NT);
+    const int nphase = fp32_two_phase(nq, P) ? 2 : 1;
     const int tok = prof_begin(ix, PROF_MERGE, 1, st);
-    launch_pdl(k_merge, (unsigned)blocks, MERGE_NT, 0, st, s.qrun, nq, pl.K, k, s.part_d, s.part_i,
-               dist, labels);
+#define SIVF_MERGE(E_)                                                                            \
+    launch_pdl(k_merge<E_>, blocks, MERGE_NT, 0, st, s.qrun, nq, nphase, pl.K, k, s.thr, s.part_d, \
+               s.part_i, dist, labels)
+    if (k <= 24) SIVF_MERGE(2);
+    else if (k <= 72) SIVF_MERGE(4);
+    else SIVF_MERGE(8);
+#undef SIVF_MERGE
     prof_end(ix, tok, st);
 }
 

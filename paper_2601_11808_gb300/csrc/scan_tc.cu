@@ -1563,15 +1563,16 @@ void query_prep(sivf_index *ix, const float *q, int64_t nq, float *qn, float *qs
 // scale)) (round to nearest even, saturated).  One warp per pair; pairs with
 // no list are left untouched (they are never scanned).
 constexpr int PP_V4 = 2;  // float4 of the residual per lane (d <= 256)
-__global__ void k_pair_prep(const float *__restrict__ q, int64_t npairs, int P, int d, int L,
+__global__ void k_pair_prep(const float *__restrict__ q, int64_t npairs, int P, int p1, int d, int L,
                             const int32_t *__restrict__ probes, const float *__restrict__ cent,
                             float *__restrict__ qn, float *__restrict__ qsc,
                             unsigned char *__restrict__ qcast)
 {
     pdl_begin();
     const int lane = threadIdx.x & 31;
-    const int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (e >= npairs) return;
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (t >= npairs) return;
+    const int64_t e = (t / p1) * P + t % p1;
     const int l = probes[e];
     if (l < 0 || l >= L) return;
     const float *qr = q + (size_t)(e / P) * d;
@@ -1639,12 +1640,12 @@ __global__ void k_pair_prep(const float *__restrict__ q, int64_t npairs, int P, 
     }
 }
 
-void pair_prep(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t *probes,
+void pair_prep(sivf_index *ix, const float *q, int64_t nq, int P, int p1, const int32_t *probes,
                float *qn, float *qsc, unsigned char *qcast, cudaStream_t st)
 {
     ix->launches += 1;
-    const int64_t np = nq * P;
-    launch_pdl(k_pair_prep, (unsigned)((np * 32 + 255) / 256), 256, 0, st, q, np, P, ix->d,
+    const int64_t np = nq * p1;
+    launch_pdl(k_pair_prep, (unsigned)((np * 32 + 255) / 256), 256, 0, st, q, np, P, p1, ix->d,
                ix->nlist, probes, ix->cent, qn, qsc, qcast);
 }
 

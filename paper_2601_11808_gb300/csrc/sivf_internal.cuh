@@ -128,6 +128,8 @@ struct sivf_index {
     int32_t *list_live;            // [nlist] live vectors per list
     int32_t *dir;                  // [nlist, dir_cap] slabs of each list
     float *inv_scale8;             // [nlist] FP8 inverse scale
+    float *lrad2;                  // [nlist] at least the largest ||x - c_l||^2 of the list's
+                                   // members since it was last empty (pair pruning)
     // TMA descriptors (CUtensorMap, 128 bytes) of the BF16 / FP8 copies
     alignas(64) unsigned char tmap_bf16[128];
     alignas(64) unsigned char tmap_fp8[128];

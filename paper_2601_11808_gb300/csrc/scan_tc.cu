@@ -62,8 +62,10 @@ template <int TN> struct TcShape {
     static constexpr int EPI = EW * 32;                 // epilogue threads
     static constexpr int NT = 128 + EPI;                // + TMA, MMA, context, B warps
     static constexpr int KMAX = TN == 48 ? 64 : TN == 32 ? 128 : 512;  // deepest K'
-    // TMEM columns per accumulator buffer (power of two, >= 32)
+    // TMEM columns per accumulator buffer (power of two, >= 32), and buffers:
+    // all 512 columns, so that a list of 1,024 rows is looked at twice
     static constexpr int TB = TN <= 32 ? 32 : 64;
+    static constexpr int NACC = 512 / TB;
 };
 
 struct TcArgs {
@@ -127,7 +129,7 @@ __host__ __device__ inline TcSmem tc_smem(int KC, int M, int nst)
     s.ctx = s.bs + (size_t)TN * M * 4;
     s.hist = s.ctx + (size_t)TC_CTX * tc_ctx_bytes(TN);
     s.bars = s.hist + (size_t)S::EW * TC_HIST * 4;
-    s.total = s.bars + 48 * 8 + 1024;                    // + base alignment slack
+    s.total = s.bars + 64 * 8 + 1024;                    // + base alignment slack
     return s;
 }
 
@@ -453,6 +455,54 @@ __device__ __forceinline__ float fold_row(float *bd, int32_t *bs, int K, int Kw,
     return dmax;
 }
 
+// A value at least K of the n values val(i) (n a multiple of 128, +inf for
+// none) lie at or below, by a bisection on the order-preserving keys that
+// stops at K .. K + K / 8 of them; +inf when fewer than K are finite.
+template <class V>
+__device__ __forceinline__ float kth_bound(V val, int n, int K, int lane)
+{
+    constexpr int R = 12;  // values per lane held in registers (n <= 384)
+    uint32_t key[R];
+    const bool regs = n <= 32 * R;
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+    int fin = 0;
+    const uint32_t kinf = fkey(INFINITY);
+    auto see = [&](uint32_t k) {
+        kmin = min(kmin, k);
+        if (k < kinf) {
+            kmax = max(kmax, k);
+            ++fin;
+        }
+    };
+    if (regs) {
+#pragma unroll
+        for (int e = 0; e < R; ++e) {
+            key[e] = 32 * e < n ? fkey(val(32 * e + lane)) : 0xffffffffu;
+            see(key[e]);
+        }
+    } else {
+        for (int i = lane; i < n; i += 32) see(fkey(val(i)));
+    }
+    if (__reduce_add_sync(0xffffffffu, fin) < K) return INFINITY;
+    uint32_t lo = __reduce_min_sync(0xffffffffu, kmin), hi = __reduce_max_sync(0xffffffffu, kmax);
+    const int Kw = K + (K >> 3);
+    while (lo < hi) {  // invariant: #(key <= hi) >= K
+        const uint32_t mid = lo + ((hi - lo) >> 1);
+        int c = 0;
+        if (regs) {
+#pragma unroll
+            for (int e = 0; e < R; ++e) c += key[e] <= mid;
+        } else {
+            for (int i = lane; i < n; i += 32) c += fkey(val(i)) <= mid;
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (c >= K) hi = mid;
+        else lo = mid + 1;
+        if (c >= K && c <= Kw) break;
+    }
+    return fkey_inv(hi);
+}
+
 // 16-byte asynchronous copy global -> shared; bytes past `src_bytes` (0 or
 // 16) are zero-filled
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, uint32_t src_bytes)
@@ -479,7 +529,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
 {
     pdl_begin();
     using S = TcShape<TN>;
-    constexpr int EW = S::EW, EPI = S::EPI, TB = S::TB;
+    constexpr int EW = S::EW, EPI = S::EPI, TB = S::TB, NACC = S::NACC;
     constexpr int ESZ = DT == 0 ? 2 : 1;
     constexpr int EPC = 128 / ESZ;  // elements per 128-byte chunk
     extern __shared__ unsigned char smem_raw[];
@@ -494,11 +544,12 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
     unsigned char *CTX = smem + L.ctx;
     uint32_t *Hist = reinterpret_cast<uint32_t *>(smem + L.hist);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bars);
-    uint64_t *full = bars, *empty = bars + 4, *tfull = bars + 8, *tempty = bars + 10,
-             *cfull = bars + 28, *cempty = bars + 30,
-             *bfull = bars + 32, *bfree = bars + 34;
-    uint32_t *tmem_base = reinterpret_cast<uint32_t *>(bars + 40);
-    volatile int *s_abort = reinterpret_cast<volatile int *>(bars + 41);
+    static_assert(TC_MAXST <= 4 && NACC <= 16 && TC_CTX == 2, "barrier layout");
+    uint64_t *full = bars, *empty = bars + 4, *tfull = bars + 8, *tempty = bars + 24,
+             *cfull = bars + 40, *cempty = bars + 42,
+             *bfull = bars + 44, *bfree = bars + 46;
+    uint32_t *tmem_base = reinterpret_cast<uint32_t *>(bars + 48);
+    volatile int *s_abort = reinterpret_cast<volatile int *>(bars + 49);
     __shared__ int32_t s_cnt[TN], s_nb[TN];  // pending candidates, held best
     __shared__ float s_kd[TN];
     __shared__ __align__(16) float s_t[TN];   // kd - ||q||^2 of each row
@@ -524,9 +575,11 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < NACC; ++i) {
             mbar_init(&tfull[i], 1);
             mbar_init(&tempty[i], EW);
+        }
+        for (int i = 0; i < 2; ++i) {
             mbar_init(&bfull[i], 32);
             mbar_init(&bfree[i], 1);
         }
@@ -537,7 +590,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
         fence_mbar_init();
         *s_abort = 0;
     }
-    if (warp == 2) tmem_alloc(tmem_base, 2 * TB);
+    if (warp == 2) tmem_alloc(tmem_base, NACC * TB);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -750,7 +803,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                 const uint32_t bbase = smem_u32(B + (size_t)bb * KC * TN * 128);
                 bool ab = false;
                 for (int b = 0; b < nblk; ++b, ++g) {
-                    const uint32_t st = g % NST, u = g / NST, buf = g & 1, ub = g >> 1;
+                    const uint32_t st = g % NST, u = g / NST, buf = g % NACC, ub = g / NACC;
                     if (!mbar_wait_ab(&full[st], u & 1, a.err, s_abort, a.wait_ns)) {
                         ab = true;
                         break;
@@ -777,17 +830,29 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                 mma_commit(&bfree[bb]);
             }
             // the last accumulator is written before TMEM is released
-            if (g > 0) mbar_wait_bounded(&tfull[(g - 1) & 1], ((g - 1) >> 1) & 1, a.err);
+            if (g > 0) mbar_wait_bounded(&tfull[(g - 1) % NACC], ((g - 1) / NACC) & 1, a.err);
         }
         __syncwarp();
     } else if (warp >= 4) {
         // ---- epilogue
+        // An item of at most 16 live columns per warp block leaves the other
+        // blocks' warps without columns: TP sets of warps then take every
+        // TP-th tile instead.  A group is the NACC tiles whose accumulators
+        // TMEM holds.  When some row has no bound yet, the item's first group
+        // is looked at twice: first each thread keeps the smallest distance
+        // of its rows per column (in `nbank` banks of tiles), and the K'-th
+        // smallest of those minima is a bound of the row's K'-th distance at
+        // least as many rows lie within; little more than K' rows pass it
+        // (128 minima of 8 rows: 45 for K' = 40).  Without it the first rows
+        // all pass and are reduced by folds that hold up every warp: 186 us
+        // against 118 for 10,000 queries' nearest of 1,024 lists.
         const int ew = warp - 4;             // epilogue warp
         const int qt = ew & 3;               // its TMEM lane quarter (warp % 4)
-        const int c0 = (ew >> 2) * TC_NCOL;  // its first query column
         const int et = ew * 32 + lane;       // epilogue thread
         const int v = qt * 32 + lane;        // A row = vector of the tile
+        const uint32_t tlane = (uint32_t)(qt * 32) << 16;
         uint32_t *hist = Hist + ew * TC_HIST;
+        float *smin = BD;                    // the minima, while no candidate is held
         uint32_t g = 0;
         for (int it = 0;; ++it) {
             const int j = it % TC_CTX;
@@ -798,19 +863,24 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
             if (flags & CF_STOP) break;
             const int m = h[1], sns = h[3], nblk = h[4], ME = h[5], chunk = h[7];
             const float inv_l = __int_as_float(h[9]);
+            // columns and tiles of this warp
+            const int ncb = (m + TC_NCOL - 1) / TC_NCOL, TP = max(1, (EW / 4) / ncb);
+            const int set = (ew >> 2) / ncb, c0 = ((ew >> 2) % ncb) * TC_NCOL;
+            const bool act = set < TP;
             // a row holds [0, nb) (at most RK) and appends at RK; its pending
-            // candidates are folded once a tile leaves more than FT of them:
-            // FT plus one tile always fits.  A fold keeps K' .. Kw.  For
-            // K' <= 128, past 224 pending rows a fold costs more than the
-            // extra folds that a lower trigger brings (measured at K' = 40:
-            // 224 beats 256, 192 and 160); deeper sets fold only when the
-            // room is full (the held K' dominate a fold's cost)
+            // candidates are folded once a round of TP tiles leaves more than
+            // FT of them: FT plus one round always fits.  A fold keeps K' ..
+            // Kw.  For K' <= 128, more than 96 pending before a round cost
+            // more in a fold than the extra folds that a lower trigger brings
+            // (measured at K' = 40); deeper sets fold only when the room is
+            // full (the held K' dominate a fold's cost)
             const int RK = a.RK, Kw = K + ((RK - K) >> 1);
-            const int FT = min(ME - RK, K > 128 ? ME - RK : 224) - TC_M;
+            const int FT = K > 128 ? ME - RK - TP * TC_M : min(ME - RK - TP * TC_M, 96);
             const int32_t *qp = c_qpair(j);
             const float *cqn = c_qn(j), *cqsc = c_qsc(j), *ckd = c_kd0(j);
             const int32_t *sl = c_sl(j);
             const uint32_t *bt = c_bits(j);
+            bool unbound = false;
             if (flags & CF_FIRST) {
                 for (int r = et; r < TN; r += EPI) {
                     const bool on = r < m;
@@ -819,120 +889,215 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                     s_kd[r] = on ? ckd[r] : INFINITY;
                     s_t[r] = on ? ckd[r] - cqn[r] : -INFINITY;
                     s_sc[r] = DT == 0 ? 2.f : 2.f / (inv_l * cqsc[r]);
+                    unbound |= on && ckd[r] > 1e38f;
                 }
             }
-            named_bar_sync(1, EPI);
+            // the tiles of one column are worth a second look from two on
+            const bool look = named_bar_or(1, EPI, unbound && nblk > 1);
             bool run = true;
-            // this thread's row's slab in A tile bb of the item, and that
-            // row's ||x||^2 read one tile ahead (its L2 latency hides behind
-            // the tile before)
-            auto row_slab = [&](int bb) {
-                return v / C < min(SPB, sns - bb * SPB) ? sl[bb * SPB + v / C] : -1;
+            // the slab of this thread's row in A tile b (-1: none), its slot
+            const int slot = v % C, jr = v / C;
+            auto row_slab = [&](int b) {
+                return jr < min(SPB, sns - b * SPB) ? sl[b * SPB + jr] : -1;
             };
-            const int s_first = nblk > 0 ? row_slab(0) : -1;
-            float xn_next = s_first >= 0 ? __ldg(a.xnorm + (size_t)s_first * C + v % C) : 0.f;
-            for (int b = 0; b < nblk; ++b, ++g) {
-                const uint32_t buf = g & 1, ub = g >> 1;
-                // row of this thread in the tile
-                const int nsl = min(SPB, sns - b * SPB);
-                const int jr = v / C, slot = v % C, mi = b * SPB + jr;
-                const int s = jr < nsl ? sl[mi] : -1;
-                const bool live = s >= 0 && ((bt[mi * 4 + (slot >> 5)] >> (slot & 31)) & 1u);
-                const int32_t gslot = s * C + slot;
-                const float xn = xn_next;
-                if (b + 1 < nblk) {
-                    const int s2 = row_slab(b + 1);
-                    xn_next = s2 >= 0 ? __ldg(a.xnorm + (size_t)s2 * C + slot) : 0.f;
+            auto row_live = [&](int b, int sv) {
+                return sv >= 0 && ((bt[(b * SPB + jr) * 4 + (slot >> 5)] >> (slot & 31)) & 1u);
+            };
+            auto row_norm = [&](int sv) {
+                return sv >= 0 ? __ldg(a.xnorm + (size_t)sv * C + slot) : 0.f;
+            };
+            auto tile_wait = [&](int i) {  // accumulator of the group's tile i
+                const bool w = mbar_wait_ab(&tfull[(g + i) % NACC], ((g + i) / NACC) & 1, a.err, s_abort,
+                                            a.wait_ns);
+                return __all_sync(0xffffffffu, w);  // tcgen05.ld is warp-aligned
+            };
+            auto tile_load = [&](int i, float (&dv)[TC_NCOL]) {
+                tmem_ld16(tbase + ((g + i) % NACC) * TB + c0 + tlane, dv);
+                tmem_ld_wait(dv);
+            };
+            auto scales = [&](int i4, float (&sc)[4]) {
+                sc[0] = sc[1] = sc[2] = sc[3] = 2.f;
+                if (DT == 1) {
+                    const float4 sv = reinterpret_cast<const float4 *>(s_sc + c0)[i4];
+                    sc[0] = sv.x;
+                    sc[1] = sv.y;
+                    sc[2] = sv.z;
+                    sc[3] = sv.w;
                 }
-                bool wok = mbar_wait_ab(&tfull[buf], ub & 1, a.err, s_abort, a.wait_ns);
-                wok = __all_sync(0xffffffffu, wok);  // tcgen05.ld is warp-aligned
-                tc_fence_after();
-                const bool cols = c0 < m;           // warp-uniform
-                float dv[TC_NCOL];
-                if (wok && cols) {
-                    tmem_ld16(tbase + buf * TB + c0 + ((uint32_t)(qt * 32) << 16), dv);
-                    tmem_ld_wait();
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[buf]);
-
-                // a row passes for query n when -s q.x + ||x||^2 <= kd_n - ||q_n||^2:
-                // the 16 ballots first (independent), then, only if a row
-                // passed, lane i reserves column i's buffer positions with one
-                // shared atomic and the passing rows are written
-                bool need = false;
-                if (wok && cols) {
-                    uint32_t mk[TC_NCOL];
-                    const float4 *t4 = reinterpret_cast<const float4 *>(s_t + c0);
-                    const float4 *sc4 = reinterpret_cast<const float4 *>(s_sc + c0);
+            };
+            for (int gb = 0; gb < nblk && run; gb += NACC) {
+                const int ng = min(NACC, nblk - gb);
+                if (look && gb == 0) {
+                    const int nbs = max(1, ((5 * K + 255) / 256 + TP - 1) / TP);  // banks of a set
+                    const int per = ((ng + TP - 1) / TP + nbs - 1) / nbs;         // tiles of a bank
+                    bool wok = true;
+                    tc_fence_after();
+                    if (act) {
+                        float mn[TC_NCOL];
+                        int b = set;
+                        int s_next = b < ng ? row_slab(b) : -1;
+                        float x_next = row_norm(s_next);
+                        for (int bk = 0; bk < nbs; ++bk) {
 #pragma unroll
-                    for (int i4 = 0; i4 < TC_NCOL / 4; ++i4) {
-                        const float4 tv = t4[i4];
-                        const float tt[4] = {tv.x, tv.y, tv.z, tv.w};
-                        float sc[4] = {2.f, 2.f, 2.f, 2.f};
-                        if (DT == 1) {
-                            const float4 sv = sc4[i4];
-                            sc[0] = sv.x;
-                            sc[1] = sv.y;
-                            sc[2] = sv.z;
-                            sc[3] = sv.w;
-                        }
+                            for (int i = 0; i < TC_NCOL; ++i) mn[i] = INFINITY;
+                            for (int k = 0; k < per && b < ng; ++k, b += TP) {
+                                const bool live = row_live(b, s_next);
+                                const float xn = x_next;
+                                s_next = b + TP < ng ? row_slab(b + TP) : -1;
+                                x_next = row_norm(s_next);
+                                wok = wok && tile_wait(b);
+                                tc_fence_after();
+                                float dv[TC_NCOL];
+                                if (wok) {
+                                    tile_load(b, dv);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const int i = 4 * i4 + c;
-                            const float part = fmaf(-sc[c], dv[i], xn);
-                            mk[i] = __ballot_sync(0xffffffffu, live && c0 + i < m && part <= tt[c]);
-                        }
-                    }
-                    uint32_t any = 0u;
+                                    for (int i4 = 0; i4 < TC_NCOL / 4; ++i4) {
+                                        float sc[4];
+                                        scales(i4, sc);
 #pragma unroll
-                    for (int i = 0; i < TC_NCOL; ++i) any |= mk[i];
-                    if (any) {
-                        uint32_t my = 0u;
-#pragma unroll
-                        for (int i = 0; i < TC_NCOL; ++i)
-                            if (lane == i) my = mk[i];
-                        int mybase = 0;
-                        if (my) {
-                            mybase = atomicAdd(&s_cnt[c0 + lane], __popc(my));
-                            need = mybase + __popc(my) > FT;
-                        }
-#pragma unroll
-                        for (int i = 0; i < TC_NCOL; ++i) {
-                            if (!mk[i]) continue;
-                            const int n = c0 + i;
-                            const int base = __shfl_sync(0xffffffffu, mybase, i);
-                            if ((mk[i] >> lane) & 1u) {
-                                const int p = RK + base + __popc(mk[i] & lanemask_lt());
-                                BD[(size_t)n * ME + p] = fmaf(-s_sc[n], dv[i], cqn[n] + xn);
-                                BS[(size_t)n * ME + p] = gslot;
+                                        for (int c = 0; c < 4; ++c) {
+                                            const int i = 4 * i4 + c;
+                                            const float part = fmaf(-sc[c], dv[i], xn);
+                                            if (live) mn[i] = fminf(mn[i], part);
+                                        }
+                                    }
+                                }
                             }
+                            float *o = smin + (size_t)((set * nbs + bk) * ncb * TC_NCOL + c0) * TC_M + v;
+#pragma unroll
+                            for (int i = 0; i < TC_NCOL; ++i) o[i * TC_M] = mn[i];
                         }
                     }
-                }
-                if (named_bar_or(1, EPI, need || !wok || *s_abort)) {
+                    tc_fence_before();
                     run = named_bar_and(1, EPI, wok && !*s_abort);
                     if (!run) break;
-                    // fold the rows whose pending candidates passed FT
+                    const int nv = TP * nbs * TC_M;  // minima per column
                     for (int n = ew; n < m; n += EW) {
-                        const int cc = s_cnt[n];
-                        if (cc <= FT) continue;
-                        int nb = s_nb[n];
-                        const float kd = fold_row(BD + (size_t)n * ME, BS + (size_t)n * ME, K, Kw,
-                                                  RK, nb, cc, hist, lane);
-                        if (lane == 0) {
-                            s_nb[n] = nb;
-                            s_cnt[n] = 0;
+                        const float b = kth_bound(
+                            [&](int i) {
+                                return smin[((size_t)(i >> 7) * ncb * TC_NCOL + n) * TC_M + (i & 127)];
+                            },
+                            nv, K, lane);
+                        if (lane == 0 && b < INFINITY) {
+                            // room for the roundings of ||q||^2 + ||x||^2 - 2 s q.x, formed
+                            // in another order for the distances that are kept
+                            const float t = __fadd_ru(b, __fmul_ru(fabsf(b) + cqn[n], 4.8e-7f));
+                            const float kd = __fadd_ru(t, cqn[n]);
+                            if (t < s_t[n]) s_t[n] = t;
                             if (kd < s_kd[n]) {
                                 s_kd[n] = kd;
-                                s_t[n] = kd - cqn[n];
+                                if (kd >= 0.f)
+                                    atomicMin(reinterpret_cast<int *>(a.thr) + qp[n] / a.P,
+                                              __float_as_int(kd));
                             }
                         }
-                        __syncwarp();
+                    }
+                    named_bar_sync(1, EPI);
+                } else if (gb > 0) {
+                    // bounds other items of the queries have left meanwhile
+                    if (et < m) {
+                        const float kd = __ldcg(a.thr + qp[et] / a.P);
+                        if (kd < s_kd[et]) {
+                            s_kd[et] = kd;
+                            s_t[et] = fminf(s_t[et], kd - cqn[et]);
+                        }
                     }
                     named_bar_sync(1, EPI);
                 }
+                int s_next = act && set < ng ? row_slab(gb + set) : -1;
+                float x_next = row_norm(s_next);
+                for (int b0 = 0; b0 < ng; b0 += TP) {
+                    const int b = b0 + set;  // this warp's tile of the round
+                    const bool mine = act && b < ng;
+                    const int sv = s_next;
+                    const float xn = x_next;
+                    const bool live = mine && row_live(gb + b, sv);
+                    const int32_t gslot = sv * C + slot;
+                    bool wok = true;
+                    float dv[TC_NCOL];
+                    if (mine) {
+                        s_next = b + TP < ng ? row_slab(gb + b + TP) : -1;
+                        x_next = row_norm(s_next);
+                        wok = tile_wait(b);
+                        tc_fence_after();
+                        if (wok) tile_load(b, dv);
+                        tc_fence_before();
+                    }
+                    __syncwarp();
+                    if (lane == 0)
+                        for (int t = b0; t < min(ng, b0 + TP); ++t) mbar_arrive(&tempty[(g + t) % NACC]);
+
+                    // a row passes for query n when -s q.x + ||x||^2 <= kd_n - ||q_n||^2:
+                    // the 16 ballots first (independent), then, only if a row
+                    // passed, lane i reserves column i's buffer positions with one
+                    // shared atomic and the passing rows are written
+                    bool need = false;
+                    if (wok && mine) {
+                        uint32_t mk[TC_NCOL];
+                        const float4 *t4 = reinterpret_cast<const float4 *>(s_t + c0);
+#pragma unroll
+                        for (int i4 = 0; i4 < TC_NCOL / 4; ++i4) {
+                            const float4 tv = t4[i4];
+                            const float tt[4] = {tv.x, tv.y, tv.z, tv.w};
+                            float sc[4];
+                            scales(i4, sc);
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const int i = 4 * i4 + c;
+                                const float part = fmaf(-sc[c], dv[i], xn);
+                                mk[i] = __ballot_sync(0xffffffffu, live && c0 + i < m && part <= tt[c]);
+                            }
+                        }
+                        uint32_t any = 0u;
+#pragma unroll
+                        for (int i = 0; i < TC_NCOL; ++i) any |= mk[i];
+                        if (any) {
+                            uint32_t my = 0u;
+#pragma unroll
+                            for (int i = 0; i < TC_NCOL; ++i)
+                                if (lane == i) my = mk[i];
+                            int mybase = 0;
+                            if (my) {
+                                mybase = atomicAdd(&s_cnt[c0 + lane], __popc(my));
+                                need = mybase + __popc(my) > FT;
+                            }
+#pragma unroll
+                            for (int i = 0; i < TC_NCOL; ++i) {
+                                if (!mk[i]) continue;
+                                const int n = c0 + i;
+                                const int base = __shfl_sync(0xffffffffu, mybase, i);
+                                if ((mk[i] >> lane) & 1u) {
+                                    const int p = RK + base + __popc(mk[i] & lanemask_lt());
+                                    BD[(size_t)n * ME + p] = fmaf(-s_sc[n], dv[i], cqn[n] + xn);
+                                    BS[(size_t)n * ME + p] = gslot;
+                                }
+                            }
+                        }
+                    }
+                    if (named_bar_or(1, EPI, need || !wok || *s_abort)) {
+                        run = named_bar_and(1, EPI, wok && !*s_abort);
+                        if (!run) break;
+                        // fold the rows whose pending candidates passed FT
+                        for (int n = ew; n < m; n += EW) {
+                            const int cc = s_cnt[n];
+                            if (cc <= FT) continue;
+                            int nb = s_nb[n];
+                            const float kd = fold_row(BD + (size_t)n * ME, BS + (size_t)n * ME, K, Kw,
+                                                      RK, nb, cc, hist, lane);
+                            if (lane == 0) {
+                                s_nb[n] = nb;
+                                s_cnt[n] = 0;
+                                if (kd < s_kd[n]) {
+                                    s_kd[n] = kd;
+                                    s_t[n] = fminf(s_t[n], kd - cqn[n]);
+                                }
+                            }
+                            __syncwarp();
+                        }
+                        named_bar_sync(1, EPI);
+                    }
+                }
+                g += ng;
             }
             if (!run) {
                 if (et == 0) *s_abort = 1;
@@ -971,7 +1136,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 2) tmem_dealloc(tbase, 2 * TB);
+    if (warp == 2) tmem_dealloc(tbase, NACC * TB);
 }
 
 // ------------------------------------------------------- per-query merge

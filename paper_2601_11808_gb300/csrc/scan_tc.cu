@@ -1146,17 +1146,49 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
 // (first run, runs)) by a radix select over the 64-bit (distance, slot)
 // keys of the valid entries, then sorted ascending, padded with (+inf, -1).
 constexpr int MT_NT = 128;
+// The K smallest (distance, slot) entries of the warp's buffer sd / ss (n > K
+// distinct ones), in place and unsorted (every write index <= its read
+// index); returns the largest distance kept.
+__device__ __noinline__ float merge_reduce(float *sd, int32_t *ss, int n, int K, uint32_t *hist,
+                                           int lane)
+{
+    __syncwarp();
+    uint64_t prefix, mask;
+    warp_radix_kth([&](int i) { return ds_key(sd[i], ss[i]); }, n, K, hist, lane, prefix, mask);
+    int w = 0;
+    float top = -INFINITY;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const float dv = i < n ? sd[i] : INFINITY;
+        const int32_t sv = i < n ? ss[i] : 0;
+        const bool take = i < n && (ds_key(dv, sv) & mask) <= prefix;
+        const uint32_t mk = __ballot_sync(0xffffffffu, take);
+        __syncwarp();
+        if (take) {
+            const int p = w + __popc(mk & lanemask_lt());
+            sd[p] = dv;
+            ss[p] = sv;
+            top = fmaxf(top, dv);
+        }
+        w += __popc(mk);
+        __syncwarp();
+    }
+    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    return top;
+}
+
 // entries of the selection's shared buffer per warp (8 bytes each)
 __host__ __device__ constexpr int merge_cap(int E) { return 64 * E > 512 ? 64 * E : 512; }
 // The selection of one query (one warp): its best K' valid entries, unsorted,
 // into sd / ss (merge_cap(E) entries of the warp's shared memory); returns
 // their number, min(valid entries, K').  hist: TC_HIST words of shared memory.
 // `bound` is the query's shared bound after the scan: at least K' entries
-// lie at or below it, so only those are gathered (four runs' entries in
-// flight at once) and the radix select works on shared memory.  Only when
-// more than the buffer holds are at or below the bound (ties) does it pass
-// over the runs in global memory, one run after the other, once per digit:
-// for a query with tens of runs that chain of loads took 130-180 us.
+// lie at or below it, so only those are gathered, four runs' entries in
+// flight at once.  A list cut into many chunks leaves a loose bound (a K'-th
+// distance within one chunk), under which thousands of entries may lie:
+// whenever the buffer is nearly full it is reduced to its K' smallest (a
+// radix select on the 64-bit (distance, slot) keys) and the bound to the
+// largest of them.
 template <int E>
 __device__ int merge_select(const int2 *__restrict__ qrun, int64_t nq, int64_t q, int nphase,
                             int K, int RK, float bound, const int32_t *__restrict__ part_n,
@@ -1169,9 +1201,9 @@ __device__ int merge_select(const int2 *__restrict__ qrun, int64_t nq, int64_t q
     const int NR = r0.y + r1.y;
     auto run_of = [&](int t) -> int64_t { return t < r0.y ? r0.x + t : r1.x + (t - r0.y); };
     int have = 0;
-    for (int t0 = 0; t0 < NR && have <= CAP; t0 += 32) {
+    for (int t0 = 0; t0 < NR; t0 += 32) {
         const int cl = t0 + lane < NR ? min(part_n[run_of(t0 + lane)], RK) : 0;
-        for (int u = 0; u < 32 && t0 + u < NR && have <= CAP; u += 4) {
+        for (int u = 0; u < 32 && t0 + u < NR; u += 4) {
             int c[4], cm = 0;
             int64_t rb[4];
 #pragma unroll
@@ -1181,6 +1213,10 @@ __device__ int merge_select(const int2 *__restrict__ qrun, int64_t nq, int64_t q
                 cm = max(cm, c[r]);
             }
             for (int j0 = 0; j0 < cm; j0 += 64) {
+                if (have > CAP - 256) {  // warp-uniform; K <= CAP - 256
+                    bound = fminf(bound, merge_reduce(sd, ss, have, K, hist, lane));
+                    have = K;
+                }
                 float dv[8];
                 int32_t sv[8];
 #pragma unroll
@@ -1188,14 +1224,14 @@ __device__ int merge_select(const int2 *__restrict__ qrun, int64_t nq, int64_t q
                     const int r = e >> 1, j = j0 + 32 * (e & 1);
                     const bool ok = j + lane < c[r];
                     dv[e] = ok ? part_d[rb[r] + j] : INFINITY;
-                    sv[e] = ok ? (int32_t)part_i[rb[r] + j] : 0;
-                    if (!(dv[e] <= bound) || !ok) sv[e] = -1;
+                    sv[e] = ok ? (int32_t)part_i[rb[r] + j] : -1;
                 }
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    const uint32_t mk = __ballot_sync(0xffffffffu, sv[e] >= 0);
-                    const int p = have + __popc(mk & lanemask_lt());
-                    if (sv[e] >= 0 && p < CAP) {
+                    const bool in = sv[e] >= 0 && dv[e] <= bound;
+                    const uint32_t mk = __ballot_sync(0xffffffffu, in);
+                    if (in) {
+                        const int p = have + __popc(mk & lanemask_lt());
                         sd[p] = dv[e];
                         ss[p] = sv[e];
                     }
@@ -1204,136 +1240,12 @@ __device__ int merge_select(const int2 *__restrict__ qrun, int64_t nq, int64_t q
             }
         }
     }
-    __syncwarp();
-    if (have <= CAP) {
-        if (have <= K) return have;
-        uint64_t prefix, mask;
-        warp_radix_kth([&](int i) { return ds_key(sd[i], ss[i]); }, have, K, hist, lane, prefix, mask);
-        int w = 0;  // compaction in place (every write index <= its read index)
-        for (int i0 = 0; i0 < have; i0 += 32) {
-            const int i = i0 + lane;
-            const float dv = i < have ? sd[i] : INFINITY;
-            const int32_t sv = i < have ? ss[i] : 0;
-            const bool take = i < have && (ds_key(dv, sv) & mask) <= prefix;
-            const uint32_t mk = __ballot_sync(0xffffffffu, take);
-            __syncwarp();
-            if (take) {
-                const int p = w + __popc(mk & lanemask_lt());
-                sd[p] = dv;
-                ss[p] = sv;
-            }
-            w += __popc(mk);
-            __syncwarp();
-        }
-        return min(w, K);
+    if (have <= K) {
+        __syncwarp();
+        return have;
     }
-    auto key_at = [&](int64_t e) -> uint64_t { return ds_key(part_d[e], (int32_t)part_i[e]); };
-    // visit every valid entry: f(valid, index) for 32 entries at a time,
-    // called by the whole warp (the loops are warp-uniform)
-    auto each = [&](auto f) {
-        for (int t = 0; t < NR; ++t) {
-            const int64_t rb = run_of(t);
-            const int c = min(part_n[rb], RK);
-            for (int j0 = 0; j0 < c; j0 += 32) f(j0 + lane < c, rb * RK + j0 + lane);
-        }
-    };
-    int nv = 0;
-    for (int t = lane; t < NR; t += 32) nv += min(part_n[run_of(t)], RK);
-    for (int o = 16; o > 0; o >>= 1) nv += __shfl_xor_sync(0xffffffffu, nv, o);
-    uint64_t prefix = ~0ull, mask = 0ull;  // keep every valid entry
-    if (nv > K) {
-        // radix select: 8 bits per pass from the highest bit where the keys
-        // differ, stopping at the first pass whose chosen bin is taken whole
-        uint64_t kmin = ~0ull, kmax = 0ull;
-        each([&](bool ok, int64_t e) {
-            if (ok) {
-                const uint64_t k = key_at(e);
-                kmin = min(kmin, k);
-                kmax = max(kmax, k);
-            }
-        });
-        for (int o = 16; o > 0; o >>= 1) {
-            kmin = min(kmin, (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)kmin, o));
-            kmax = max(kmax, (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)kmax, o));
-        }
-        const uint64_t diff = kmin ^ kmax;
-        const int top = diff ? 63 - __clzll((long long)diff) : 0;
-        mask = top >= 63 ? 0ull : ~((2ull << top) - 1ull);
-        prefix = kmin & mask;
-        uint32_t need = (uint32_t)K;
-        for (int hi = top; hi >= 0; hi -= 8) {
-            const int shift = max(hi - 7, 0);
-            const uint32_t bmask = (1u << (hi - shift + 1)) - 1u;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) hist[lane * 8 + b] = 0u;
-            __syncwarp();
-            each([&](bool ok, int64_t e) {
-                if (ok) {
-                    const uint64_t k = key_at(e);
-                    if ((k & mask) == prefix) atomicAdd(&hist[(uint32_t)(k >> shift) & bmask], 1u);
-                }
-            });
-            __syncwarp();
-            uint32_t loc[8], sum = 0;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                loc[b] = hist[lane * 8 + b];
-                sum += loc[b];
-            }
-            uint32_t incl = sum;
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t tv = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += tv;
-            }
-            const uint32_t excl = incl - sum;
-            const bool mine = excl < need && incl >= need;
-            uint32_t bin = 0, below = 0, cnt = 0;
-            if (mine) {
-                uint32_t cum = excl;
-                for (int b = 0; b < 8; ++b) {
-                    if (cum + loc[b] >= need) {
-                        bin = (uint32_t)(lane * 8 + b);
-                        below = cum;
-                        cnt = loc[b];
-                        break;
-                    }
-                    cum += loc[b];
-                }
-            }
-            const uint32_t who = __ballot_sync(0xffffffffu, mine);
-            const int src = who ? __ffs(who) - 1 : 0;
-            bin = __shfl_sync(0xffffffffu, bin, src);
-            below = __shfl_sync(0xffffffffu, below, src);
-            cnt = __shfl_sync(0xffffffffu, cnt, src);
-            prefix |= (uint64_t)bin << shift;
-            mask |= (uint64_t)bmask << shift;
-            need -= below;
-            __syncwarp();
-            if (cnt == need) break;
-        }
-    }
-    int w = 0;
-    each([&](bool ok, int64_t e) {
-        bool take = false;
-        float dv = 0.f;
-        int32_t sv = 0;
-        if (ok) {
-            dv = part_d[e];
-            sv = (int32_t)part_i[e];
-            take = (ds_key(dv, sv) & mask) <= prefix;
-        }
-        const uint32_t mk = __ballot_sync(0xffffffffu, take);
-        if (take) {
-            const int p = w + __popc(mk & lanemask_lt());
-            if (p < 32 * E) {
-                sd[p] = dv;
-                ss[p] = sv;
-            }
-        }
-        w += __popc(mk);
-    });
-    __syncwarp();
-    return min(w, K);
+    merge_reduce(sd, ss, have, K, hist, lane);
+    return K;
 }
 
 template <int E>

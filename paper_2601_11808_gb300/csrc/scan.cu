@@ -140,6 +140,7 @@ struct ScanCount {
 // t, t + 1024, ... (their order in the groups and items is of no account), so
 // that its loads are coalesced and independent: contiguous lists per thread
 // took 50 us at 16,384 lists, a chain of strided loads.
+constexpr int PLAN_BIG = 256;  // heavy lists taken by the block
 __global__ __launch_bounds__(1024) void k_srch_plan(const int32_t *__restrict__ lcnt,
                                                     const int32_t *__restrict__ nslabs,
                                                     const int32_t *__restrict__ list_live,
@@ -178,16 +179,31 @@ __global__ __launch_bounds__(1024) void k_srch_plan(const int32_t *__restrict__ 
     block_scan2(ea, eb, sh, &ta, &tb);
     ea -= ca;
     eb -= cb;
+    // work items of list l: (list, tile << 8 | chunk); a heavy list's are
+    // written by the whole block (one thread took 35 us for 1,750)
+    __shared__ int s_big;
+    __shared__ int4 big[PLAN_BIG];
+    if (tid == 0) s_big = 0;
+    __syncthreads();
 #pragma unroll 4
     for (int l = tid; l < L; l += 1024) {
         const int m = lcnt[l], c = nch[l], nt = (m + tq - 1) / tq;
         loff[l] = ea;
-        // work items of list l: (list, tile << 8 | chunk)
-        for (int t = 0; t < nt * c; ++t) {
-            if (eb + t < item_cap) items[eb + t] = make_int2(l, ((t / c) << 8) | (t % c));
+        const int slot = nt * c > 16 ? atomicAdd(&s_big, 1) : PLAN_BIG;
+        if (slot < PLAN_BIG) {
+            big[slot] = make_int4(l, c, nt * c, eb);
+        } else {
+            for (int t = 0; t < nt * c; ++t)
+                if (eb + t < item_cap) items[eb + t] = make_int2(l, ((t / c) << 8) | (t % c));
         }
         ea += m;
         eb += nt * c;
+    }
+    __syncthreads();
+    for (int b = tid >> 5; b < min(s_big, PLAN_BIG); b += 32) {
+        const int4 w = big[b];
+        for (int t = tid & 31; t < w.z; t += 32)
+            if (w.w + t < item_cap) items[w.w + t] = make_int2(w.x, ((t / w.y) << 8) | (t % w.y));
     }
     if (tid == 0) {
         if (tb > item_cap) atomicOr(err, ERR_PLAN);
@@ -345,9 +361,11 @@ __global__ __launch_bounds__(1024) void k_srch_small(
 //   FP8: D = rq^2 + rx^2 - 2 s q^.x^ with ||q^|| <= rq + eq and ||x^|| <= rx +
 //     ex (E4M3 rounds to 2^-4 relative, 2^-10 of a code unit below the
 //     smallest normal; saturation only shortens x^), least at rx = R.
-// One warp takes PR_P consecutive pairs of one query, their centroid rows in
-// flight together; a FP8 pair that stays gets its residual codes here.
-constexpr int PR_P = 4;
+// One warp takes PR consecutive pairs of one query (8, or 4 for d > 128),
+// their centroid rows in flight together, and works out the bounds one pair
+// per lane (every lane for every pair: 324 against 82 us for 630,000 pairs);
+// a FP8 pair that stays gets its residual codes here.
+__host__ __device__ constexpr int prune_per(int NV) { return NV == 1 ? 8 : 4; }
 struct PruneArgs {
     const float *q;
     int64_t nq;
@@ -361,11 +379,11 @@ struct PruneArgs {
     int32_t *prank;
 };
 
-template <int DT>  // sivf_scan_dtype
+template <int DT, int NV>  // sivf_scan_dtype; float4 of a row per lane (d <= 128 NV)
 __global__ __launch_bounds__(256) void k_pair_prune(PruneArgs a)
 {
     pdl_begin();
-    constexpr int NV = kMaxD / 128;  // float4 of a row per lane
+    constexpr int PR_P = prune_per(NV);
     const int lane = threadIdx.x & 31, d = a.d, n4 = d >> 2;
     const int np = a.P - 1, ng = (np + PR_P - 1) / PR_P;
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -418,64 +436,83 @@ __global__ __launch_bounds__(256) void k_pair_prune(PruneArgs a)
 #pragma unroll
         for (int k = 0; k < PR_P; ++k)
             for (int o = 16; o > 0; o >>= 1) mx[k] = fmaxf(mx[k], __shfl_xor_sync(0xffffffffu, mx[k], o));
-    const float u32 = 5.9604645e-08f;                    // 2^-24
-    const float up = 1.f + (2.f * d + 32.f) * u32, dn = 1.f - (2.f * d + 32.f) * u32;
-    const float bound = __ldcg(a.thr + qi);
+    // lane k takes pair pb + k
+    const int np_here = min(PR_P, a.P - pb);
+    int l = -1;
+    float s2 = 0.f, mxl = 0.f;
 #pragma unroll
-    for (int k = 0; k < PR_P; ++k) {
-        if (pb + k >= a.P) break;  // warp-uniform
-        const int64_t e = qi * a.P + pb + k;
-        bool keep = lv[k] >= 0;
-        if (keep && a.dedupe) {
+    for (int k = 0; k < PR_P; ++k)
+        if (lane == k) {
+            l = lv[k];
+            s2 = ss[k];
+            mxl = mx[k];
+        }
+    bool keep = lane < np_here && l >= 0;
+    if (a.dedupe)
+        for (int k = 0; k < np_here; ++k) {
+            const int lk = __shfl_sync(0xffffffffu, l, k);
             bool dup = false;
-            for (int f = lane; f < pb + k; f += 32) dup |= a.probes[qi * a.P + f] == lv[k];
-            keep = !__any_sync(0xffffffffu, dup);
+            for (int f = lane; f < pb + k; f += 32) dup |= a.probes[qi * a.P + f] == lk;
+            dup = __any_sync(0xffffffffu, dup);
+            if (lane == k) keep &= !dup;
         }
-        const float sc = mx[k] > 0.f ? 448.f / (2.f * mx[k]) : 1.f;
-        if (keep) {
-            const float R = __fsqrt_ru(__ldg(a.lrad2 + lv[k]));
-            const float rlo = __fsqrt_rd(__fmul_rd(ss[k], dn)), rhi = __fsqrt_ru(__fmul_ru(ss[k], up));
-            const float gap = __fsub_rd(rlo, R);
-            float lo = -INFINITY;  // lower bound of the scan's distances
-            if (gap > 0.f) {
-                if (DT == SIVF_FP32) {
-                    lo = __fmul_rd(__fmul_rd(gap, gap), dn);
-                } else if (DT == SIVF_BF16) {
-                    const float qn = __fsqrt_ru(__fmul_ru(__ldg(a.qn + qi), up));
-                    const float xn = __fadd_ru(__ldg(a.cnrm_up + lv[k]), R);
-                    const float n2 = __fadd_ru(__fmul_ru(qn, qn), __fmul_ru(xn, xn));
-                    const float err = __fadd_ru(__fmul_ru(__fmul_ru(a.e_bf16, qn), __fmul_ru(2.f, xn)),
-                                                __fmul_ru(n2, (2.f * d + 64.f) * u32));
-                    lo = __fsub_rd(__fmul_rd(gap, gap), err);
-                } else {
-                    const float sq = sqrtf((float)d) * 1.01f * 9.765625e-04f;  // 2^-10
-                    const float A = __fadd_ru(__fmul_ru(rhi, 1.0626f), __fdiv_ru(sq, sc));
-                    const float X = __fadd_ru(__fmul_ru(R, 1.0626f),
-                                              __fdiv_ru(sq, __ldg(a.inv_scale8 + lv[k])));
-                    // products' accumulation (4 d u) and the norms' roundings
-                    const float err = __fmul_ru(__fadd_ru(__fmul_ru(rhi, rhi), __fmul_ru(A, X)),
-                                                (16.f * d + 64.f) * u32);
-                    lo = __fsub_rd(__fsub_rd(__fadd_rd(__fmul_rd(rlo, rlo), __fmul_rd(__fmul_rd(R, R), dn)),
-                                             __fmul_ru(2.f, __fmul_ru(A, X))),
-                                   err);
-                }
+    const float sc = mxl > 0.f ? 448.f / (2.f * mxl) : 1.f;
+    if (keep) {
+        const float u32 = 5.9604645e-08f;  // 2^-24
+        const float up = 1.f + (2.f * d + 32.f) * u32, dn = 1.f - (2.f * d + 32.f) * u32;
+        const float bound = __ldcg(a.thr + qi);
+        const float R = __fsqrt_ru(__ldg(a.lrad2 + l));
+        const float rlo = __fsqrt_rd(__fmul_rd(s2, dn)), rhi = __fsqrt_ru(__fmul_ru(s2, up));
+        const float gap = __fsub_rd(rlo, R);
+        float lo = -INFINITY;  // lower bound of the scan's distances
+        if (gap > 0.f) {
+            if (DT == SIVF_FP32) {
+                lo = __fmul_rd(__fmul_rd(gap, gap), dn);
+            } else if (DT == SIVF_BF16) {
+                const float qn = __fsqrt_ru(__fmul_ru(__ldg(a.qn + qi), up));
+                const float xn = __fadd_ru(__ldg(a.cnrm_up + l), R);
+                const float n2 = __fadd_ru(__fmul_ru(qn, qn), __fmul_ru(xn, xn));
+                const float err = __fadd_ru(__fmul_ru(__fmul_ru(a.e_bf16, qn), __fmul_ru(2.f, xn)),
+                                            __fmul_ru(n2, (2.f * d + 64.f) * u32));
+                lo = __fsub_rd(__fmul_rd(gap, gap), err);
+            } else {
+                const float sq = sqrtf((float)d) * 1.01f * 9.765625e-04f;  // 2^-10
+                const float A = __fadd_ru(__fmul_ru(rhi, 1.0626f), __fdiv_ru(sq, sc));
+                const float X = __fadd_ru(__fmul_ru(R, 1.0626f),
+                                          __fdiv_ru(sq, __ldg(a.inv_scale8 + l)));
+                // products' accumulation (4 d u) and the norms' roundings
+                const float err = __fmul_ru(__fadd_ru(__fmul_ru(rhi, rhi), __fmul_ru(A, X)),
+                                            (16.f * d + 64.f) * u32);
+                lo = __fsub_rd(__fsub_rd(__fadd_rd(__fmul_rd(rlo, rlo), __fmul_rd(__fmul_rd(R, R), dn)),
+                                         __fmul_ru(2.f, __fmul_ru(A, X))),
+                               err);
             }
-            keep = !(lo > bound);
         }
-        if (lane == 0) a.prank[e] = keep ? 0 : -1;
+        keep = !(lo > bound);
+    }
+    if (lane < np_here) {
+        const int64_t e = qi * a.P + pb + lane;
+        a.prank[e] = keep ? 0 : -1;
         if (DT == SIVF_FP8E4M3 && keep) {
-            if (lane == 0) {
-                a.pqn[e] = ss[k];
-                a.pqsc[e] = sc;
-            }
+            a.pqn[e] = s2;
+            a.pqsc[e] = sc;
+        }
+    }
+    const uint32_t stay = __ballot_sync(0xffffffffu, keep);
+    if (DT == SIVF_FP8E4M3 && stay) {
+#pragma unroll
+        for (int k = 0; k < PR_P; ++k) {
+            if (!((stay >> k) & 1u)) continue;  // warp-uniform
+            const int64_t e = qi * a.P + pb + k;
+            const float sk = __shfl_sync(0xffffffffu, sc, k);
 #pragma unroll
             for (int u = 0; u < NV; ++u) {
                 const int j4 = lane + 32 * u;
                 if (j4 >= n4) break;
                 const uint32_t lo8 = __nv_cvt_float2_to_fp8x2(
-                    make_float2(__fmul_rn(r[k][u].x, sc), __fmul_rn(r[k][u].y, sc)), __NV_SATFINITE, __NV_E4M3);
+                    make_float2(__fmul_rn(r[k][u].x, sk), __fmul_rn(r[k][u].y, sk)), __NV_SATFINITE, __NV_E4M3);
                 const uint32_t hi8 = __nv_cvt_float2_to_fp8x2(
-                    make_float2(__fmul_rn(r[k][u].z, sc), __fmul_rn(r[k][u].w, sc)), __NV_SATFINITE, __NV_E4M3);
+                    make_float2(__fmul_rn(r[k][u].z, sk), __fmul_rn(r[k][u].w, sk)), __NV_SATFINITE, __NV_E4M3);
                 reinterpret_cast<uint32_t *>(a.qcast + (size_t)e * d)[j4] = (lo8 & 0xffffu) | (hi8 << 16);
             }
         }
@@ -504,12 +541,14 @@ void prune_pairs(sivf_index *ix, int dtype, const float *q, int64_t nq, int P,
     a.pqsc = s.pqsc;
     a.qcast = s.qcast;
     a.prank = s.prank;
-    const int64_t warps = nq * ((P - 1 + PR_P - 1) / PR_P);
+    const int NV = ix->d <= 128 ? 1 : 2, per = prune_per(NV);
+    const int64_t warps = nq * ((P - 1 + per - 1) / per);
     const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
     const int tg = prof_begin(ix, PROF_GROUP, 1, st);
-    if (dtype == SIVF_FP32) launch_pdl(k_pair_prune<SIVF_FP32>, blocks, 256, 0, st, a);
-    else if (dtype == SIVF_BF16) launch_pdl(k_pair_prune<SIVF_BF16>, blocks, 256, 0, st, a);
-    else launch_pdl(k_pair_prune<SIVF_FP8E4M3>, blocks, 256, 0, st, a);
+    auto go = [&](auto one, auto two) { launch_pdl(NV == 1 ? one : two, blocks, 256, 0, st, a); };
+    if (dtype == SIVF_FP32) go(&k_pair_prune<SIVF_FP32, 1>, &k_pair_prune<SIVF_FP32, 2>);
+    else if (dtype == SIVF_BF16) go(&k_pair_prune<SIVF_BF16, 1>, &k_pair_prune<SIVF_BF16, 2>);
+    else go(&k_pair_prune<SIVF_FP8E4M3, 1>, &k_pair_prune<SIVF_FP8E4M3, 2>);
     prof_end(ix, tg, st);
 }
 
@@ -824,7 +863,7 @@ __device__ __forceinline__ void dist_tile(float (&acc)[RQ][RX], const float *__r
 }
 
 template <int TQ, int C>
-__global__ __launch_bounds__(SCAN_NT, 1) void k_scan(ScanArgs a)
+__global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(ScanArgs a)
 {
     pdl_begin();
     constexpr int QW = TQ >= 32 ? TQ / 32 : 1;
@@ -1260,8 +1299,19 @@ static void launch_scan(sivf_index *ix, const ScanArgs &a, size_t smem, int grid
                              (int)smem);
         attr = smem;
     }
+    // as many CTAs per SM as fit: the small tiles' shared memory leaves room
+    // for two or more, which hide each other's barriers and load latency
+    static size_t occ_smem = 0;
+    static int occ = 1;
+    if (smem != occ_smem) {
+        int n = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_scan<TQ, C>, SCAN_NT, smem) != cudaSuccess)
+            n = 1;
+        occ = std::max(1, n);
+        occ_smem = smem;
+    }
     const int tok = prof_begin(ix, PROF_SCAN, 1, st);
-    launch_pdl(k_scan<TQ, C>, grid, SCAN_NT, smem, st, a);
+    launch_pdl(k_scan<TQ, C>, grid * occ, SCAN_NT, smem, st, a);
     prof_end(ix, tok, st);
 }
 
@@ -1480,8 +1530,16 @@ void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t
     // the nearest lists first: the others then meet a tight bound, which most
     // of their vectors do not pass and whole lists may not (prune_pairs)
     const int split = fp32_two_phase(nq, P) ? 1 : P;
-    group_pairs(ix, nq, P, 0, split, probes, dedupe, split < P ? bound_plan(ix, pl) : pl, s, sb, st);
-    scan_launch(ix, pl.tq, a, smem, st);
+    SearchPlan pl1 = pl;
+    if (split < P) {
+        // one pair per query: a list gets nq / nlist of them, so the tile of
+        // the whole batch would stay mostly empty (64-query tiles for the 10
+        // of 10,000 queries over 1,024 lists: half the warps without a row)
+        pl1 = bound_plan(ix, pl);
+        pl1.tq = std::min(pl.tq, current_tile(ix, SIVF_FP32, nq, 1, pl.K).queries_per_tile);
+    }
+    group_pairs(ix, nq, P, 0, split, probes, dedupe, pl1, s, sb, st);
+    scan_launch(ix, pl1.tq, a, scan_smem(pl1.tq, ix->C, ix->d, a.M).total, st);
     if (split < P) {
         prune_pairs(ix, SIVF_FP32, q, nq, P, probes, dedupe, s, st);
         group_pairs(ix, nq, P, split, P, probes, false, pl, s, sb, st, true, true);

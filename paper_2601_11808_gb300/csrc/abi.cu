@@ -164,16 +164,18 @@ sivf_status read_status(sivf_index *ix, void *stream, int64_t *count)
 
 namespace sivf {
 
-int64_t coarse_rows(const sivf_index *ix, int64_t n)
+int64_t coarse_floats(const sivf_index *ix, int64_t n)
 {
-    // approximate-distance rows per chunk: at most 64 MB of scratch
-    int64_t r = ((int64_t)64 << 20) / (4 * (int64_t)ix->nlist);
-    return std::max<int64_t>(1, std::min<int64_t>(n, std::max<int64_t>(r, 128)));
+    // rows of approximate distances with their group minima, and a number per
+    // row: 64 MB of distances at most, 128 rows at least
+    const int64_t L = ix->nlist, r = ((int64_t)64 << 20) / (4 * L);
+    const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(n, std::max<int64_t>(r, 128)));
+    return rows * (1 + L + (L + 15) / 16) + 16;
 }
 
 size_t coarse_bytes(const sivf_index *ix, int64_t n)
 {
-    return (size_t)coarse_rows(ix, n) * ix->nlist * 4 + 256;
+    return (size_t)coarse_floats(ix, n) * 4 + 256;
 }
 
 int prof_begin(sivf_index *ix, int k, int n, cudaStream_t st)
@@ -253,6 +255,7 @@ sivf_status sivf_create(const sivf_config *cfg, sivf_index **out)
     ALLOC(ix->cent, (size_t)L * d);
     ALLOC(ix->cnorm, (size_t)L);
     ALLOC(ix->cnrm_up, (size_t)L);
+    ALLOC(ix->cmax, 2);
     // BF16 copy of the centroids for the tensor-core first stage of the
     // coarse selection (d % 16 == 0)
     if (d % 16 == 0 && d <= kMaxD) ALLOC(ix->cent_bf16, (size_t)L * d);
@@ -310,7 +313,7 @@ sivf_status sivf_destroy(sivf_index *ix)
 {
     if (!ix) return SIVF_OK;
     cudaDeviceSynchronize();
-    void *ptrs[] = {ix->cent, ix->cnorm, ix->cnrm_up, ix->cent_bf16, ix->cent_lo, ix->x32, ix->xb16,
+    void *ptrs[] = {ix->cent, ix->cnorm, ix->cnrm_up, ix->cmax, ix->cent_bf16, ix->cent_lo, ix->x32, ix->xb16,
                     ix->x8, ix->rnorm, ix->inv_scale8, ix->lrad2, ix->xnorm, ix->ids, ix->bits, ix->meta,
                     ix->free_list, ix->free_top, ix->head, ix->nslabs, ix->list_live, ix->dir, ix->att,
                     ix->claim, ix->list_flag, ix->aff_flag, ix->runcnt, ix->err};
@@ -395,14 +398,14 @@ sivf_status sivf_train(sivf_index *ix, const float *x, int64_t n, int iters, uin
             rows.push_back(r);
         }
     }
-    const int64_t crows = coarse_rows(ix, n);
+    const int64_t croom = coarse_floats(ix, n);
     const size_t need = coarse_bytes(ix, n) + (size_t)n * 4 + (size_t)L * d * 8 + (size_t)L * 4 +
                         (size_t)L * 8 + 5 * 256;
     Ctx *c;
     if ((st = get_ctx(ix, stream, need, &c))) return st;
     Bump b{c->scratch};
     int32_t *lab = b.take<int32_t>((size_t)n);
-    float *Dbuf = b.take<float>((size_t)crows * L);
+    float *Dbuf = b.take<float>((size_t)croom);
     double *sum = b.take<double>((size_t)L * d);
     int32_t *cnt = b.take<int32_t>((size_t)L);
     int64_t *rows_dev = b.take<int64_t>((size_t)L);
@@ -415,7 +418,7 @@ sivf_status sivf_train(sivf_index *ix, const float *x, int64_t n, int iters, uin
     // again on the trained ones
     CUDA_TRY(ix, assign_stage_choose(ix, s));
     for (int it = 0; it < iters; ++it) {
-        coarse_topP(ix, x, n, 1, lab, Dbuf, crows, s);
+        coarse_topP(ix, x, n, 1, lab, Dbuf, croom, s);
         train_step(ix, x, n, lab, sum, cnt, s);
         centroid_prep(ix, s);
     }
@@ -591,10 +594,10 @@ sivf_status sivf_add(sivf_index *ix, const int64_t *ids, const float *x, int64_t
     sc.bcnt = b.take<int32_t>(L);
     sc.plan = b.take<PlanEntry>(L);
     sc.affected = b.take<int32_t>(L);
-    const int64_t rows = coarse_rows(ix, n);
-    float *Dbuf = b.take<float>((size_t)rows * L);
+    const int64_t room = coarse_floats(ix, n);
+    float *Dbuf = b.take<float>((size_t)room);
     CUDA_TRY(ix, cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), s));
-    coarse_topP(ix, x, n, 1, sc.lab, Dbuf, rows, s);
+    coarse_topP(ix, x, n, 1, sc.lab, Dbuf, room, s);
     insert_batch(ix, ids, x, n, sc, s);
     CUDA_TRY(ix, cudaGetLastError());
     if (n_added) return read_status(ix, stream, n_added);
@@ -792,15 +795,15 @@ static sivf_status search_impl(sivf_index *ix, const float *q, int64_t nq, int k
         sc.pqsc = fp8 ? b.take<float>((size_t)m * P) : nullptr;
         float *cand_d = b.take<float>((size_t)m * pl.K);
         int64_t *cand_s = b.take<int64_t>((size_t)m * pl.K);
-        const int64_t rows = coarse_rows(ix, m);
-        float *Dbuf = b.take<float>((size_t)rows * L);
+        const int64_t room = coarse_floats(ix, m);
+        float *Dbuf = b.take<float>((size_t)room);
         CUDA_TRY(ix, cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), s));
         const float *qq = q + q0 * ix->d;
         if (probes_in)
             CUDA_TRY(ix, cudaMemcpyAsync(probes, probes_in + q0 * P, sizeof(int32_t) * m * P,
                                          cudaMemcpyDeviceToDevice, s));
         else
-            coarse_topP(ix, qq, m, P, probes, Dbuf, rows, s);
+            coarse_topP(ix, qq, m, P, probes, Dbuf, room, s);
         if (!tc) {
             scan_lists(ix, qq, m, P, probes, probes_in != nullptr && !probes_unique, pl, sc, s);
             merge_topk(ix, m, P, pl, sc, k, dist + q0 * k, labels + q0 * k, s);
@@ -910,9 +913,9 @@ static sivf_status coarse_only(sivf_index *ix, const float *x, int64_t n, int P,
     sivf_status st = get_ctx(ix, stream, coarse_bytes(ix, n), &c);
     if (st) return st;
     Bump b{c->scratch};
-    const int64_t rows = coarse_rows(ix, n);
-    float *Dbuf = b.take<float>((size_t)rows * ix->nlist);
-    coarse_topP(ix, x, n, P, out, Dbuf, rows, (cudaStream_t)stream);
+    const int64_t room = coarse_floats(ix, n);
+    float *Dbuf = b.take<float>((size_t)room);
+    coarse_topP(ix, x, n, P, out, Dbuf, room, (cudaStream_t)stream);
     CUDA_TRY(ix, cudaGetLastError());
     return SIVF_OK;
 }

@@ -44,7 +44,8 @@ namespace sivf {
 // walked its row with dependent FP64 additions: 63 us for 1,024 x 128).
 __global__ void k_centroid_norms(const float *__restrict__ cent, int L, int d,
                                  float *__restrict__ cn, float *__restrict__ cnrm_up,
-                                 uint16_t *__restrict__ cb, uint16_t *__restrict__ clo)
+                                 float *__restrict__ cmax, uint16_t *__restrict__ cb,
+                                 uint16_t *__restrict__ clo)
 {
     pdl_begin();
     const int lane = threadIdx.x & 31;
@@ -67,8 +68,12 @@ __global__ void k_centroid_norms(const float *__restrict__ cent, int L, int d,
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
-        cn[c] = __double2float_rn(s);
-        cnrm_up[c] = __double2float_ru(sqrt(s) * (1.0 + 1e-12));
+        const float n2 = __double2float_rn(s), nu = __double2float_ru(sqrt(s) * (1.0 + 1e-12));
+        cn[c] = n2;
+        cnrm_up[c] = nu;
+        // the largest of each (not negative, so their bits order as integers)
+        atomicMax(reinterpret_cast<int *>(cmax), __float_as_int(n2));
+        atomicMax(reinterpret_cast<int *>(cmax) + 1, __float_as_int(nu));
     }
 }
 
@@ -215,11 +220,9 @@ __device__ float block_min(float v, float *red)
     return r;
 }
 
-__global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
+// one row, by a block
+__device__ void select_row(const SelArgs &a, int row)
 {
-    pdl_begin();
-    const int row = blockIdx.x;
-    if (row >= a.m) return;
     const int tid = threadIdx.x;
     const float *Dr = a.D + (size_t)row * a.L;
     const float *xr = a.x + (size_t)row * a.d;
@@ -238,6 +241,8 @@ __global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
     float part = 0.f;
     for (int j = tid & 31; j < a.d; j += 32) part = fmaf(xr[j], xr[j], part);
     const float xn = norm_up(warp_sum(part), a.d);
+    const float gamma2 = a.two_level ? a.gamma2_first : a.gamma2;  // of the distances D
+    __syncthreads();  // shared memory may still be read for the block's last row
 
     // T = P-th smallest upper bound
     float T;
@@ -245,7 +250,7 @@ __global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
         float v = INFINITY;
         for (int c = tid; c < a.L; c += SEL_NT) {
             float Dt = Dr[c];
-            v = fminf(v, upper_of(Dt, bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, a.gamma2)));
+            v = fminf(v, upper_of(Dt, bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, gamma2)));
         }
         T = block_min(v, red);
     } else {
@@ -261,7 +266,7 @@ __global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
             const uint32_t prefix = s_prefix;
             for (int c = tid; c < a.L; c += SEL_NT) {
                 float Dt = Dr[c];
-                uint32_t k = fkey(upper_of(Dt, bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, a.gamma2)));
+                uint32_t k = fkey(upper_of(Dt, bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, gamma2)));
                 if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
             }
             __syncthreads();
@@ -305,7 +310,7 @@ __global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
     __syncthreads();
     for (int c = tid; c < a.L; c += SEL_NT) {
         float Dt = Dr[c];
-        float E = bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, a.gamma2);
+        float E = bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, gamma2);
         if (lower_of(Dt, E) <= T) {
             int p = atomicAdd(&s_ns, 1);
             if (p < SEL_SCAP) {
@@ -371,7 +376,7 @@ __global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
         int n = 0;
         for (int c = 0; c < a.L; ++c) {
             float Dt = Dr[c];
-            float E = bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, a.gamma2);
+            float E = bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, gamma2);
             if (lower_of(Dt, E) > T) continue;
             double Dc = exact_dist(xr, a.cent + (size_t)c * a.d, a.d);
             if (n == a.P && !(Dc < hd[n - 1])) continue;  // index order keeps ties
@@ -393,21 +398,40 @@ __global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
     // ties to the lower list index (the set itself is the exact one)
     const int nsel = min(s_nsel, a.P);
     if (s_nsel != a.P && tid == 0) atomicOr(a.err, ERR_SELECT);
+    for (int s = tid; s < nsel; s += SEL_NT) {  // their FP32 distances (P <= SEL_SCAP)
+        const int c = sSel[s];
+        float dc = Dr[c];
+        if (a.two_level) {
+            float dot = 0.f;
+            for (int j = 0; j < a.d; ++j) dot = fmaf(xr[j], __ldg(a.cent + (size_t)c * a.d + j), dot);
+            dc = fmaf(-2.f, dot, a.cn[c]);
+        }
+        sLB[s] = dc;
+    }
+    __syncthreads();
     for (int s = tid; s < a.P; s += SEL_NT) {
         if (s >= nsel) {
             outr[s] = -1;
             continue;
         }
         const int c = sSel[s];
-        const float dc = Dr[c];
+        const float dc = sLB[s];
         int pos = 0;
         for (int q = 0; q < nsel; ++q) {
             const int c2 = sSel[q];
-            const float d2 = Dr[c2];
+            const float d2 = sLB[q];
             pos += d2 < dc || (d2 == dc && c2 < c);
         }
         outr[pos] = c;
     }
+}
+
+__global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
+{
+    pdl_begin();
+    // all rows, a block each; or the rows k_coarse_pick left (usually none)
+    const int nrows = a.hard ? *a.nhard : a.m;
+    for (int it = blockIdx.x; it < nrows; it += gridDim.x) select_row(a, a.hard ? a.hard[it] : it);
 }
 
 // ------------------------------------------ BF16 tensor-core first stage
@@ -639,6 +663,20 @@ __host__ __device__ inline size_t coarse_fused_smem(int KC, int parts)
     return (size_t)KC * parts * (CT_M + cf_buffers(parts) * CF_CN) * 128 + CW_LMAX * 4 + 1024;
 }
 
+// Amax and Ebig: a bound of every |Dt| (the parts' roundings included), and
+// of every list's bound_of, evaluated at the maxima with every step rounded
+// up, times 1 + 2^-10 (covers the roundings of the bound itself)
+__device__ __forceinline__ float abs_max(float cnmax, float xn, float cmax)
+{
+    return __fadd_ru(cnmax, __fmul_ru(__fmul_ru(2.04f, xn), cmax));
+}
+__device__ __forceinline__ float bound_max(float cnmax, float ab, float xn, float cmax, float g1)
+{
+    const float t1 = __fmul_ru(5.9604645e-08f, __fadd_ru(cnmax, ab));
+    const float t2 = __fmul_ru(__fmul_ru(g1, xn), cmax);
+    return __fadd_ru(__fmul_ru(__fmul_ru(2.f, __fadd_ru(t1, t2)), 1.f + 1.f / 1024.f), 1e-30f);
+}
+
 __device__ __forceinline__ float min3f(float a, float b, float c)
 {
     float r;
@@ -646,11 +684,67 @@ __device__ __forceinline__ float min3f(float a, float b, float c)
     return r;
 }
 
+// A tile of 128 rows held in registers by CF_EPI threads: fetched as FP32
+// (zero past m or d), stored rounded to BF16 (and its low parts, abytes
+// further) in the swizzled operand layout; sxn receives the norms' bounds.
+template <int KC, int PARTS>
+struct RowTile {
+    static constexpr int W = KC * 8;              // 16-byte chunks of a row
+    static constexpr int AU = CT_M * W / CF_EPI;  // chunks per thread: 2 KC
+    float4 f0[AU], f1[AU];
+    __device__ __forceinline__ void fetch(const float *__restrict__ x, int row0, int m, int d, int tid)
+    {
+#pragma unroll
+        for (int u = 0; u < AU; ++u) {
+            const int e = tid + u * CF_EPI, row = row0 + e / W, k0 = (e & (W - 1)) * 8;
+            f0[u] = f1[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row < m && k0 < d) {
+                const float4 *xr = reinterpret_cast<const float4 *>(x + (size_t)row * d + k0);
+                f0[u] = __ldg(xr);
+                f1[u] = __ldg(xr + 1);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(unsigned char *A, uint32_t abytes, int d, int tid, float *sxn)
+    {
+        const float fx = 1.f + 4.f * (float)d * 5.9604645e-08f;
+#pragma unroll
+        for (int u = 0; u < AU; ++u) {
+            const int e = tid + u * CF_EPI, r = e / W, kc = (e >> 3) % KC, c = e & 7;
+            const float f[8] = {f0[u].x, f0[u].y, f0[u].z, f0[u].w,
+                                f1[u].x, f1[u].y, f1[u].z, f1[u].w};
+            uint32_t w[4], wl[4];
+            float sq = 0.f;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * t], f[2 * t + 1]);
+                w[t] = *reinterpret_cast<uint32_t *>(&h);
+                if (PARTS == 2) {
+                    __nv_bfloat162 l = __floats2bfloat162_rn(f[2 * t] - __low2float(h),
+                                                             f[2 * t + 1] - __high2float(h));
+                    wl[t] = *reinterpret_cast<uint32_t *>(&l);
+                }
+                sq = fmaf(f[2 * t], f[2 * t], sq);
+                sq = fmaf(f[2 * t + 1], f[2 * t + 1], sq);
+            }
+            unsigned char *o = A + (size_t)kc * CT_M * 128 + (size_t)(r >> 3) * 1024 + (r & 7) * 128 +
+                               ((c ^ (r & 7)) << 4);
+            *reinterpret_cast<uint4 *>(o) = make_uint4(w[0], w[1], w[2], w[3]);
+            if (PARTS == 2)
+                *reinterpret_cast<uint4 *>(o + abytes) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+            // the W chunks of a row sit in consecutive lanes
+#pragma unroll
+            for (int t = W >> 1; t > 0; t >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, t);
+            if ((tid & (W - 1)) == 0) sxn[r] = __fsqrt_ru(__fmul_ru(sq, fx));
+        }
+    }
+};
+
 template <int KC, int PARTS>
 __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
     const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBlo,
     const float *__restrict__ x, int m, int d, const float *__restrict__ cn,
-    const float *__restrict__ cnrm_up, int L, float g1, int32_t *__restrict__ out1,
+    const float *__restrict__ cmaxes, int L, float g1, int32_t *__restrict__ out1,
     int32_t *__restrict__ outS, int cap, int32_t *__restrict__ hard, int *nhard, uint32_t *err)
 {
     pdl_begin();
@@ -673,7 +767,6 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
     // the best key of its other lists, and its candidate count
     __shared__ float sxn[2][CT_M], sMin[2][CF_SUB][CT_M], sSec[2][CF_SUB][CT_M];
     __shared__ int sArg[2][CF_SUB][CT_M], sn[CF_SUB][CT_M];
-    __shared__ uint32_t smax[2];  // max ||c||^2, max ||c|| (bits of non-negative floats)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         for (int i = 0; i < NB; ++i) {
@@ -686,7 +779,6 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
         }
         mbar_init(&afull, CF_EPI / 32);
         fence_mbar_init();
-        smax[0] = smax[1] = 0u;
         s_abort_ = 0;
     }
     if (warp == CF_EPI / 32) tmem_alloc(&tmem_base, TB * CN);
@@ -760,80 +852,20 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
     } else {
         // ---- rows in, epilogue
         const int q = warp & 3, sub = warp >> 2, rloc = q * 32 + lane;
-        constexpr int W = KC * 8;                  // 16-byte chunks of a row
-        constexpr int AU = CT_M * W / CF_EPI;      // chunks per thread: 2 KC
-        float4 f0[AU], f1[AU];
-        auto fetch = [&](int tile) {               // the tile's rows, zero past m or d
-#pragma unroll
-            for (int u = 0; u < AU; ++u) {
-                const int e = tid + u * CF_EPI, r = e / W, k0 = (e & (W - 1)) * 8;
-                const int row = tile * CT_M + r;
-                f0[u] = f1[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (row < m && k0 < d) {
-                    const float4 *xr = reinterpret_cast<const float4 *>(x + (size_t)row * d + k0);
-                    f0[u] = __ldg(xr);
-                    f1[u] = __ldg(xr + 1);
-                }
-            }
-        };
-        const float fx = 1.f + 4.f * (float)d * 5.9604645e-08f;
-        auto store = [&](int par) {                // rounded (and split) into A; the norms
-#pragma unroll
-            for (int u = 0; u < AU; ++u) {
-                const int e = tid + u * CF_EPI, r = e / W, kc = (e >> 3) % KC, c = e & 7;
-                const float f[8] = {f0[u].x, f0[u].y, f0[u].z, f0[u].w,
-                                    f1[u].x, f1[u].y, f1[u].z, f1[u].w};
-                uint32_t w[4], wl[4];
-                float sq = 0.f;
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * t], f[2 * t + 1]);
-                    w[t] = *reinterpret_cast<uint32_t *>(&h);
-                    if (PARTS == 2) {
-                        __nv_bfloat162 l = __floats2bfloat162_rn(f[2 * t] - __low2float(h),
-                                                                 f[2 * t + 1] - __high2float(h));
-                        wl[t] = *reinterpret_cast<uint32_t *>(&l);
-                    }
-                    sq = fmaf(f[2 * t], f[2 * t], sq);
-                    sq = fmaf(f[2 * t + 1], f[2 * t + 1], sq);
-                }
-                unsigned char *o = A + (size_t)kc * CT_M * 128 + (size_t)(r >> 3) * 1024 +
-                                   (r & 7) * 128 + ((c ^ (r & 7)) << 4);
-                *reinterpret_cast<uint4 *>(o) = make_uint4(w[0], w[1], w[2], w[3]);
-                if (PARTS == 2)
-                    *reinterpret_cast<uint4 *>(o + ABYTES) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
-                // the W chunks of a row sit in consecutive lanes
-#pragma unroll
-                for (int s = W >> 1; s > 0; s >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, s);
-                if ((lane & (W - 1)) == 0) sxn[par][r] = __fsqrt_ru(__fmul_ru(sq, fx));
-            }
+        RowTile<KC, PARTS> rows;
+        auto fetch = [&](int tile) { rows.fetch(x, tile * CT_M, m, d, tid); };
+        auto store = [&](int par) {
+            rows.store(A, ABYTES, d, tid, sxn[par]);
             fence_proxy_async_smem();  // A (generic stores) is read by the MMAs
             __syncwarp();
             if (lane == 0) mbar_arrive(&afull);
         };
         fetch((int)blockIdx.x);
         store(0);
-        {  // ||c||^2 (lists past L far away) and the maxima
-            float a0 = 0.f, a1 = 0.f;
-            for (int c = tid; c < nch * CN; c += CF_EPI) {
-                const float v = c < L ? __ldg(cn + c) : 3.0e38f;
-                scn[c] = v;
-                if (c < L) {
-                    a0 = fmaxf(a0, v);
-                    a1 = fmaxf(a1, __ldg(cnrm_up + c));
-                }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                a0 = fmaxf(a0, __shfl_xor_sync(0xffffffffu, a0, o));
-                a1 = fmaxf(a1, __shfl_xor_sync(0xffffffffu, a1, o));
-            }
-            if (lane == 0) {
-                atomicMax(&smax[0], __float_as_uint(a0));
-                atomicMax(&smax[1], __float_as_uint(a1));
-            }
-        }
+        // ||c||^2, lists past L far away
+        for (int c = tid; c < nch * CN; c += CF_EPI) scn[c] = c < L ? __ldg(cn + c) : 3.0e38f;
         named_bar_sync(1, CF_EPI);
-        const float cnmax = __uint_as_float(smax[0]), cmax = __uint_as_float(smax[1]);
+        const float cnmax = __ldg(cmaxes), cmax = __ldg(cmaxes + 1);
         uint32_t g = 0;
         bool ok = true;
         for (uint32_t t = 0; t < mine; ++t) {
@@ -941,14 +973,8 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
 #pragma unroll
             for (int k = 0; k < CF_SUB; ++k)
                 if (k != kmin) second = fminf(second, sMin[par][k][rloc]);
-            // Ebig: the bound at the maxima, every step rounded up, times
-            // 1 + 2^-10 (covers the roundings of the bound itself)
             const float xn = sxn[par][rloc];
-            const float ab = __fadd_ru(cnmax, __fmul_ru(__fmul_ru(2.04f, xn), cmax));
-            const float t1 = __fmul_ru(5.9604645e-08f, __fadd_ru(cnmax, ab));
-            const float t2 = __fmul_ru(__fmul_ru(g1, xn), cmax);
-            const float eb = __fadd_ru(
-                __fmul_ru(__fmul_ru(2.f, __fadd_ru(t1, t2)), 1.f + 1.f / 1024.f), 1e-30f);
+            const float ab = abs_max(cnmax, xn, cmax), eb = bound_max(cnmax, ab, xn, cmax, g1);
             const float delta = __fadd_ru(__fmul_ru(ab, 1.9073486e-06f), 1e-36f);  // 2^-19
             const float T = __fadd_ru(__fadd_ru(mn, delta), eb);
             // RN(Dt - E) <= T needs Dt < T + E + ulp(T) <= thr - delta
@@ -1005,6 +1031,166 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
                         for (int k = 0; k < nl[i]; ++k) *o++ = min(first + k, L - 1);
                     }
                 }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == CF_EPI / 32) tmem_dealloc(tbase, TB * CN);
+}
+
+// ------------------------------------ split first stage for probe selection
+// Dt of a tile of 128 rows against a segment of the centroids' chunks, in the
+// split BF16 form, written to out[row][list], and the smallest Dt of each
+// group of 16 lists to gmin[row][group].  Roles and buffers as in
+// k_coarse_fused; grid (tiles, segments of `per` chunks), so that a few rows
+// over many lists fill the chip too.
+template <int KC>
+__global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
+    const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBlo,
+    const float *__restrict__ x, int m, int d, const float *__restrict__ cn, int L, int per,
+    float *__restrict__ out, float *__restrict__ gmin, uint32_t *err)
+{
+    pdl_begin();
+    constexpr int CN = CF_CN, NB = cf_buffers(2), TB = CF_TB;
+    constexpr uint32_t PBYTES = KC * CN * 128, BBYTES = 2 * PBYTES, ABYTES = KC * CT_M * 128;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+    unsigned char *A = smem, *B = smem + 2 * ABYTES;
+    __shared__ uint64_t fullb[NB], freeb[NB], mmab[TB], tempty[TB], afull;
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_abort_;
+    __shared__ float sxn[CT_M];
+    volatile int *s_abort = &s_abort_;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int i = 0; i < NB; ++i) {
+            mbar_init(&fullb[i], 1);
+            mbar_init(&freeb[i], 1);
+        }
+        for (int i = 0; i < TB; ++i) {
+            mbar_init(&mmab[i], 1);
+            mbar_init(&tempty[i], CF_EPI / 32);
+        }
+        mbar_init(&afull, CF_EPI / 32);
+        fence_mbar_init();
+        s_abort_ = 0;
+    }
+    if (warp == CF_EPI / 32) tmem_alloc(&tmem_base, TB * CN);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = tmem_base;
+    const int nch = (L + CN - 1) / CN, j0 = blockIdx.y * per;
+    const uint32_t steps = (uint32_t)max(0, min(per, nch - j0));
+    const int row0 = blockIdx.x * CT_M;
+
+    if (warp == CF_EPI / 32 + 1) {
+        if (lane == 0) {
+            uint32_t g = 0;
+            for (; g < steps; ++g) {
+                const uint32_t b = g % NB, u = g / NB;
+                if (u >= 1 && !mbar_wait_ab(&freeb[b], (u - 1) & 1, err, s_abort, kWaitNs)) break;
+                mbar_arrive_expect_tx(&fullb[b], BBYTES);
+#pragma unroll
+                for (int pp = 0; pp < 2; ++pp)
+#pragma unroll
+                    for (int kc = 0; kc < KC; ++kc)
+                        tma_load_2d(B + b * BBYTES + pp * PBYTES + (size_t)kc * CN * 128,
+                                    pp ? &tmBlo : &tmB, kc * 64, (j0 + (int)g) * CN, &fullb[b]);
+            }
+            // the copies issued last have landed before exit
+            for (uint32_t t = g > NB ? g - NB : 0; t < g; ++t)
+                mbar_wait_bounded(&fullb[t % NB], (t / NB) & 1, err);
+        }
+        __syncwarp();
+    } else if (warp == CF_EPI / 32) {
+        if (lane == 0) {
+            const uint32_t idesc = mma_idesc(1, 1, CT_M, CN), abase = smem_u32(A);
+            uint32_t g = 0;
+            bool ok = steps == 0 || mbar_wait_ab(&afull, 0, err, s_abort, kWaitNs);
+            for (; g < steps && ok; ++g) {
+                const uint32_t b = g % NB, tb = g % TB, ut = g / TB;
+                ok = mbar_wait_ab(&fullb[b], (g / NB) & 1, err, s_abort, kWaitNs);
+                if (ok && ut >= 1) ok = mbar_wait_ab(&tempty[tb], (ut - 1) & 1, err, s_abort, kWaitNs);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t bbase = smem_u32(B + b * BBYTES);
+#pragma unroll
+                for (int pr = 0; pr < 3; ++pr) {  // (x hi, c hi), (x hi, c lo), (x lo, c hi)
+                    const uint32_t ap = abase + (pr == 2 ? ABYTES : 0u);
+                    const uint32_t bp = bbase + (pr == 1 ? PBYTES : 0u);
+#pragma unroll
+                    for (int kc = 0; kc < KC; ++kc)
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_bf16(tbase + tb * CN,
+                                     smem_desc_sw128(ap + kc * CT_M * 128 + ks * 32, 1024),
+                                     smem_desc_sw128(bp + kc * CN * 128 + ks * 32, 1024), idesc,
+                                     (pr | kc | ks) != 0);
+                }
+                mma_commit(&freeb[b]);
+                mma_commit(&mmab[tb]);
+            }
+            // the last products are written before TMEM is released
+            if (g > 0) mbar_wait_bounded(&mmab[(g - 1) % TB], ((g - 1) / TB) & 1, err);
+        }
+        __syncwarp();
+    } else {
+        const int q = warp & 3, sub = warp >> 2, row = row0 + q * 32 + lane;
+        RowTile<KC, 2> rows;
+        rows.fetch(x, row0, m, d, tid);
+        rows.store(A, ABYTES, d, tid, sxn);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&afull);
+        const int G = (L + 15) / 16;
+        const bool vec = (L & 3) == 0;
+        bool ok = true;
+        for (uint32_t g = 0; g < steps; ++g) {
+            const uint32_t tb = g % TB;
+            ok = __all_sync(0xffffffffu, ok && mbar_wait_ab(&mmab[tb], (g / TB) & 1, err, s_abort, kWaitNs));
+            tc_fence_after();
+            float v[CN / 64][16];
+            if (ok) {
+#pragma unroll
+                for (int k = 0; k < CN / 64; ++k)
+                    tmem_ld16(tbase + tb * CN + (sub + 4 * k) * 16 + ((uint32_t)(q * 32) << 16), v[k]);
+#pragma unroll
+                for (int k = 0; k < CN / 64; ++k) tmem_ld_wait(v[k]);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty[tb]);
+            if (!ok) break;  // warp-uniform; no barrier follows before the last one
+            if (row >= m) continue;
+#pragma unroll
+            for (int k = 0; k < CN / 64; ++k) {
+                const int grp = (j0 + (int)g) * (CN / 16) + sub + 4 * k, c0 = grp * 16;
+                if (c0 >= L) break;
+                float *o = out + (size_t)row * L + c0;
+                float mn = INFINITY;
+                if (vec && c0 + 16 <= L) {
+#pragma unroll
+                    for (int i4 = 0; i4 < 4; ++i4) {
+                        const float4 c = __ldg(reinterpret_cast<const float4 *>(cn + c0) + i4);
+                        const float4 t = make_float4(
+                            fmaf(-2.f, v[k][4 * i4], c.x), fmaf(-2.f, v[k][4 * i4 + 1], c.y),
+                            fmaf(-2.f, v[k][4 * i4 + 2], c.z), fmaf(-2.f, v[k][4 * i4 + 3], c.w));
+                        reinterpret_cast<float4 *>(o)[i4] = t;
+                        mn = fminf(mn, fminf(fminf(t.x, t.y), fminf(t.z, t.w)));
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        if (c0 + i < L) {
+                            const float t = fmaf(-2.f, v[k][i], __ldg(cn + c0 + i));
+                            o[i] = t;
+                            mn = fminf(mn, t);
+                        }
+                }
+                gmin[(size_t)row * G + grp] = mn;
             }
         }
     }
@@ -1354,6 +1540,243 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_select_w(SelArgs a)
 // leaves a fourteenth of the near-ties to the FP64 step, whose dependent
 // FP64 additions are what an undecided row costs most.
 __host__ __device__ constexpr int re_ops(int d) { return 4 * ((d + 127) / 128) + 5; }
+// the same with eight lanes a row (float4s t, t + 8, ...) and three shuffles
+__host__ __device__ constexpr int pk_ops(int d) { return 4 * ((d + 31) / 32) + 3; }
+
+// ------------------------------------------ probe selection, P lists per row
+// One warp per row, from k_coarse_dist's distances and group minima.  The
+// P-th smallest group minimum b bounds the P-th smallest Dt (P groups each
+// hold a list at or below it), so only lists with Dt <= b + 2 Ebig can be
+// among the top P, and only groups whose minimum is within that are read: 75
+// of 4,096 lists for P = 64, where the block selection read every distance
+// six times.  Their distances are recomputed in FP32 (PK_RG at a time, eight
+// lanes each) and decided as in the other selections: sure members
+// by their FP32 intervals, the rest by FP64 distance.  A row with more
+// candidates than `cap` is left to k_coarse_select (its number in `hard`).
+// 10,000 rows of 4,096 lists, P = 64: 400 against 580 us (FP32 GEMM and
+// block selection); 61 rows of 16,384 lists, P = 32: 45 against 118 us.
+// Bound by the chain of one row (about 25 us at P = 64), not by throughput.
+constexpr int PK_RG = 16;      // FP32 rechecks in flight per warp
+constexpr int PK_PMAX = 128;   // most lists per row of this kernel
+__host__ __device__ constexpr int pk_cap(int P) { return (P + P / 2 + 64 + 31) / 32 * 32; }
+__host__ __device__ constexpr size_t pk_smem(int P)  // per warp: Dt, LB, UB, list, FP64, sure
+{
+    return (size_t)pk_cap(P) * (4 + 4 + 4 + 4 + 8 + 4) + kMaxD * 4;
+}
+
+__global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const float *__restrict__ gmin,
+                                                              const float *__restrict__ cmaxes,
+                                                              int32_t *hard, int *nhard)
+{
+    pdl_begin();
+    extern __shared__ __align__(16) unsigned char pk[];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row = blockIdx.x * CW_ROWS + w;
+    if (row >= a.m) return;  // whole warps
+    const int L = a.L, P = a.P, d = a.d, n4 = d >> 2, cap = pk_cap(P), G = (L + 15) / 16;
+    unsigned char *mem = pk + (size_t)w * pk_smem(P);
+    double *sDx = reinterpret_cast<double *>(mem);
+    float *sX = reinterpret_cast<float *>(sDx + cap), *sDt = sX + kMaxD, *sLB = sDt + cap, *sUB = sLB + cap;
+    int *sIdx = reinterpret_cast<int *>(sUB + cap), *sSure = sIdx + cap;
+    const float *Dr = a.D + (size_t)row * L, *gr = gmin + (size_t)row * G;
+    const float *xr = a.x + (size_t)row * d;
+    float part = 0.f;
+    for (int j = lane; j < d; j += 32) {
+        const float v = xr[j];
+        sX[j] = v;
+        part = fmaf(v, v, part);
+    }
+    const float xn = norm_up(warp_sum(part), d);
+    const float b = kth_bound<32>([&](int i) { return i < G ? __ldg(gr + i) : INFINITY; },
+                                  (G + 31) & ~31, P, lane);
+    const float cnmax = __ldg(cmaxes), cmax = __ldg(cmaxes + 1);
+    const float eb = bound_max(cnmax, abs_max(cnmax, xn, cmax), xn, cmax, a.gamma2_first);
+    // Dt - E <= T with T = b + Ebig needs Dt <= T + Ebig + its roundings
+    const float T0 = __fadd_ru(b, eb);
+    const float thr = __fadd_ru(__fadd_ru(T0, eb), __fadd_ru(__fmul_ru(fabsf(T0), 1.2e-7f), 1e-30f));
+    // the groups that can hold a candidate, then their lists: 4 lanes read a
+    // group, 32 groups in flight
+    int ng = 0, ns = 0;
+    int *sGrp = sSure;
+    for (int g0 = 0; g0 < G && ng <= cap; g0 += 128) {
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int gi = g0 + 32 * u + lane;
+            v[u] = gi < G ? __ldg(gr + gi) : INFINITY;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool in = g0 + 32 * u + lane < G && v[u] <= thr;
+            const uint32_t mk = __ballot_sync(0xffffffffu, in);
+            const int p = ng + __popc(mk & lanemask_lt());
+            if (in && p < cap) sGrp[p] = g0 + 32 * u + lane;
+            ng += __popc(mk);
+        }
+    }
+    __syncwarp();
+    const bool vec = (L & 3) == 0;
+    for (int t0 = 0; t0 < ng && ng <= cap && ns <= cap; t0 += 32) {
+        float v[4][4];
+        int cl[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = t0 + 8 * u + (lane >> 2);
+            cl[u] = t < ng ? sGrp[t] * 16 + (lane & 3) * 4 : L;
+            if (vec && cl[u] < L) {
+                const float4 f = __ldg(reinterpret_cast<const float4 *>(Dr + cl[u]));
+                v[u][0] = f.x;
+                v[u][1] = f.y;
+                v[u][2] = f.z;
+                v[u][3] = f.w;
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[u][k] = cl[u] + k < L ? __ldg(Dr + cl[u] + k) : INFINITY;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool ok = cl[u] + k < L && v[u][k] <= thr;
+                const uint32_t mk = __ballot_sync(0xffffffffu, ok);
+                const int p = ns + __popc(mk & lanemask_lt());
+                if (ok && p < cap) sIdx[p] = cl[u] + k;
+                ns += __popc(mk);
+            }
+    }
+    __syncwarp();
+    if (ng > cap || ns > cap || ns < P) {  // too many candidates (or no numbers): the block selection decides
+        if (lane == 0) hard[atomicAdd(nhard, 1)] = row;
+        return;
+    }
+    // FP32 distances and intervals: eight lanes a list, 16 lists in flight
+    for (int p = lane; p < ns; p += 32) {
+        sLB[p] = __ldg(a.cn + sIdx[p]);
+        sUB[p] = __ldg(a.cnrm_up + sIdx[p]);
+    }
+    __syncwarp();
+    {
+        const int g8 = lane >> 3, t8 = lane & 7;
+        const float4 *x4 = reinterpret_cast<const float4 *>(sX);
+        float4 xv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            xv[u] = t8 + 8 * u < n4 ? x4[t8 + 8 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int p0 = 0; p0 < ns; p0 += PK_RG) {
+            float4 cv[PK_RG / 4][4];
+#pragma unroll
+            for (int r = 0; r < PK_RG / 4; ++r) {
+                const float4 *c4 = reinterpret_cast<const float4 *>(
+                    a.cent + (size_t)sIdx[min(p0 + 4 * r + g8, ns - 1)] * d);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    cv[r][u] = t8 + 8 * u < n4 ? __ldg(c4 + t8 + 8 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int r = 0; r < PK_RG / 4; ++r) {
+                float dot = 0.f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    dot = fmaf(xv[u].x, cv[r][u].x, dot);
+                    dot = fmaf(xv[u].y, cv[r][u].y, dot);
+                    dot = fmaf(xv[u].z, cv[r][u].z, dot);
+                    dot = fmaf(xv[u].w, cv[r][u].w, dot);
+                }
+                dot += __shfl_xor_sync(0xffffffffu, dot, 4);
+                dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+                dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+                const int p = p0 + 4 * r + g8;
+                if (t8 == 0 && p < ns) {
+                    const float cnc = sLB[p], Dt = fmaf(-2.f, dot, cnc);
+                    const float E = bound_of(Dt, cnc, sUB[p], xn, a.gamma2_re);
+                    sDt[p] = Dt;
+                    sLB[p] = lower_of(Dt, E);
+                    sUB[p] = upper_of(Dt, E);
+                }
+            }
+        }
+    }
+    __syncwarp();
+    // T: at least P upper bounds lie at or below it
+    const float T = kth_bound<16>([&](int i) { return i < ns ? sUB[i] : INFINITY; }, (ns + 31) & ~31, P,
+                                  lane);
+    int nsure = 0, nmem = 0;
+    for (int p0 = 0; p0 < ns; p0 += 32) {
+        const int p = p0 + lane;
+        bool sure = false, mem_ = false;
+        if (p < ns) {
+            const float ub = sUB[p];
+            int cnt = 0;
+#pragma unroll 8
+            for (int k = 0; k < ns; ++k) cnt += sLB[k] <= ub;  // itself included
+            mem_ = sLB[p] <= T;
+            sure = mem_ && ub <= T && cnt <= P;
+            sSure[p] = sure ? 1 : mem_ ? 0 : -1;
+        }
+        nsure += __popc(__ballot_sync(0xffffffffu, sure));
+        nmem += __popc(__ballot_sync(0xffffffffu, mem_));
+    }
+    __syncwarp();
+    const int r = P - nsure, nb = nmem - nsure;
+    if (r > 0 && nb > r) {  // boundary members: FP64 distances, the best r of them
+        for (int p = lane; p < ns; p += 32)
+            if (sSure[p] == 0) sDx[p] = exact_dist(xr, a.cent + (size_t)sIdx[p] * d, d);
+        __syncwarp();
+    }
+    // the chosen to the front of sIdx / sDt, in place
+    int nsel = 0;
+    for (int p0 = 0; p0 < ns; p0 += 32) {
+        const int p = p0 + lane;
+        bool take = false;
+        if (p < ns) {
+            take = sSure[p] == 1;
+            if (sSure[p] == 0 && r > 0) {
+                take = true;
+                if (nb > r) {
+                    int rank = 0;
+                    for (int k = 0; k < ns; ++k)
+                        rank += sSure[k] == 0 &&
+                                (sDx[k] < sDx[p] || (sDx[k] == sDx[p] && sIdx[k] < sIdx[p]));
+                    take = rank < r;
+                }
+            }
+        }
+        sUB[p0 + lane] = take ? 1.f : 0.f;  // cap is a multiple of 32
+    }
+    __syncwarp();
+    for (int p0 = 0; p0 < ns; p0 += 32) {
+        const int p = p0 + lane;
+        const bool take = p < ns && sUB[p] > 0.f;
+        const float dt = p < ns ? sDt[p] : 0.f;
+        const int c = p < ns ? sIdx[p] : 0;
+        const uint32_t mk = __ballot_sync(0xffffffffu, take);
+        __syncwarp();
+        if (take) {  // write index <= read index
+            const int q = nsel + __popc(mk & lanemask_lt());
+            sDt[q] = dt;
+            sIdx[q] = c;
+        }
+        nsel += __popc(mk);
+        __syncwarp();
+    }
+    if (nsel != P && lane == 0) atomicOr(a.err, ERR_SELECT);
+    nsel = min(nsel, P);
+    // nearest first: ascending FP32 distance, ties to the lower list index
+    int32_t *outr = a.out + (size_t)row * P;
+    for (int s = lane; s < P; s += 32) {
+        if (s >= nsel) {
+            outr[s] = -1;
+            continue;
+        }
+        const int c = sIdx[s];
+        const float dc = sDt[s];
+        int pos = 0;
+#pragma unroll 8
+        for (int q = 0; q < nsel; ++q) pos += sDt[q] < dc || (sDt[q] == dc && sIdx[q] < c);
+        outr[pos] = c;
+    }
+}
 
 // Finishing selection of the rows the fused first stage left undecided (P =
 // 1).  With a record, one warp per row: the FP32 distance of each candidate
@@ -1362,16 +1785,18 @@ __host__ __device__ constexpr int re_ops(int d) { return 4 * ((d + 127) / 128) +
 // they are several, their FP64 distances decide (ties to the lower index).
 // A row to redo takes a block: its warps read all lists' rows, FN_RG in
 // flight each, into one table of distances (a warp alone, list after list,
-// took 1.2 ms at 2,048 lists, the tail of the launch).
-constexpr int FN_RG = 8;
-__global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_finish(SelArgs a)
+// took 1.2 ms at 2,048 lists, the tail of the launch; four warps with eight
+// in flight 0.23 ms).
+constexpr int FN_RG = 16;
+constexpr int FN_ROWS = 8;     // warps per block
+__global__ __launch_bounds__(FN_ROWS * 32) void k_coarse_finish(SelArgs a)
 {
     pdl_begin();
-    __shared__ __align__(16) float sX[CW_ROWS][kMaxD];
+    __shared__ __align__(16) float sX[FN_ROWS][kMaxD];
     __shared__ float sD[CW_LMAX];
-    __shared__ float sT[CW_ROWS];
-    __shared__ double sB[CW_ROWS];
-    __shared__ int sC[CW_ROWS];
+    __shared__ float sT[FN_ROWS];
+    __shared__ double sB[FN_ROWS];
+    __shared__ int sC[FN_ROWS];
     __shared__ int s_found, s_one;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const int L = a.L, d = a.d, n4 = d >> 2;
@@ -1433,7 +1858,7 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_finish(SelArgs a)
         a.out[row] = c;
     };
 
-    for (int it = blockIdx.x * CW_ROWS + w; it < nrec; it += gridDim.x * CW_ROWS) {  // whole warps
+    for (int it = blockIdx.x * FN_ROWS + w; it < nrec; it += gridDim.x * FN_ROWS) {  // whole warps
         const int row = a.hard[it];
         const int32_t *Sr = a.S + (size_t)it * CF_STRIDE;
         const int n0 = min(Sr[0], CF_CAP);
@@ -1489,7 +1914,7 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_finish(SelArgs a)
         __syncwarp();
         const float4 *x4 = reinterpret_cast<const float4 *>(sX[w]);
         float T = INFINITY;
-        for (int c0 = w * FN_RG; c0 < L; c0 += CW_ROWS * FN_RG) {
+        for (int c0 = w * FN_RG; c0 < L; c0 += FN_ROWS * FN_RG) {
             float s[FN_RG];
 #pragma unroll
             for (int t = 0; t < FN_RG; ++t) s[t] = share(x4, min(c0 + t, L - 1));
@@ -1514,8 +1939,8 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_finish(SelArgs a)
         if (lane == 0) sT[w] = T;
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < CW_ROWS; ++k) T = fminf(T, sT[k]);
-        for (int c = tid; c < L; c += CW_ROWS * 32) {
+        for (int k = 0; k < FN_ROWS; ++k) T = fminf(T, sT[k]);
+        for (int c = tid; c < L; c += FN_ROWS * 32) {
             float lb, ub;
             bounds(c, sD[c], xn, lb, ub);
             if (lb <= T) {
@@ -1531,7 +1956,7 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_finish(SelArgs a)
         }
         bd = INFINITY;
         bc = 0x7fffffff;
-        for (int c = tid; c < L; c += CW_ROWS * 32) {
+        for (int c = tid; c < L; c += FN_ROWS * 32) {
             float lb, ub;
             bounds(c, sD[c], xn, lb, ub);
             if (lb <= T) better(exact_dist(xr, a.cent + (size_t)c * d, d), c);
@@ -1543,7 +1968,7 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_finish(SelArgs a)
         }
         __syncthreads();
         if (tid == 0) {
-            for (int k = 1; k < CW_ROWS; ++k) better(sB[k], sC[k]);
+            for (int k = 1; k < FN_ROWS; ++k) better(sB[k], sC[k]);
             write(row, bc);
         }
     }
@@ -1592,8 +2017,9 @@ __global__ void k_fp8_scales(const float *__restrict__ cent, int L, int d,
 void centroid_prep(sivf_index *ix, cudaStream_t st)
 {
     ix->launches += 1;
+    cudaMemsetAsync(ix->cmax, 0, 2 * sizeof(float), st);
     launch_pdl(k_centroid_norms, (ix->nlist * 32 + 127) / 128, 128, 0, st, ix->cent, ix->nlist, ix->d,
-               ix->cnorm, ix->cnrm_up, ix->cent_bf16, ix->cent_lo);
+               ix->cnorm, ix->cnrm_up, ix->cmax, ix->cent_bf16, ix->cent_lo);
     if (ix->x8) {
         ix->launches += 1;
         launch_pdl(k_fp8_scales, (ix->nlist * 32 + 127) / 128, 128, 0, st, ix->cent, ix->nlist,
@@ -1746,16 +2172,44 @@ int first_stage_split(const sivf_index *ix, int P)
     return ix->cent_lo && d <= 128 ? 3 : 0;
 }
 
-// rows [0, m) of x -> out[m, P]; `Dbuf` holds at least rows_per_chunk * L
-// floats.
+// Probe selection by k_coarse_dist and k_coarse_pick: P lists need twice as
+// many groups of 16 for the group minima to bound them well (L >= 32 P); the
+// warp's candidate table holds P <= 128.
+static bool pick_rows(const sivf_index *ix, int P)
+{
+    return P >= 2 && P <= PK_PMAX && ix->tmap_cent_ok && (int64_t)ix->nlist >= 32 * (int64_t)P;
+}
+
+// Chunks per CTA of k_coarse_dist: the split of the lists that takes the
+// fewest steps, a CTA's start (its rows, the first chunk) counted as four
+static int dist_chunks(int tiles, int nch, int nsm)
+{
+    int best = nch;
+    int64_t cost = INT64_MAX;
+    for (int segs = 1; segs <= nch; ++segs) {
+        const int per = (nch + segs - 1) / segs;
+        const int64_t c = (((int64_t)tiles * ((nch + per - 1) / per) + nsm - 1) / nsm) * (per + 4);
+        if (c < cost) {
+            cost = c;
+            best = per;
+        }
+    }
+    return best;
+}
+
+// rows [0, m) of x -> out[m, P]; `Dbuf` holds at least `room` floats, L of
+// them at least.
 void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
-                 float *Dbuf, int64_t rows_per_chunk, cudaStream_t st)
+                 float *Dbuf, int64_t room, cudaStream_t st)
 {
     const int L = ix->nlist, d = ix->d;
     const double u = 5.9604644775390625e-08;
     const double gd = d * u / (1.0 - d * u);
     const bool warp_rows = P <= CW_PMAX && L <= CW_LMAX;
-    const int split = first_stage_split(ix, P);
+    // row numbers, distances and group minima of at least one row
+    const int64_t pick_row = 1 + L + (L + 15) / 16;
+    const bool pick = pick_rows(ix, P) && room >= CF_HDR + pick_row;
+    const int split = pick ? 3 : first_stage_split(ix, P);
     const bool two = split != 0;
     const float gamma2_first = (float)(2.0 * first_stage_rel(d, split) * (1.0 + 1e-6));
     // assignment (d <= 128) takes the fused first stage, which keeps only the
@@ -1763,13 +2217,14 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
     // the matrix: a launch takes as many rows as leave records for half of
     // them (958,000 where the matrix of L = 1024 lists takes 16,384); among
     // close centroids about a third are undecided
-    const int64_t room = rows_per_chunk * L;
     const bool fused = P == 1 && two && ix->tmap_cent_ok && L >= CF_LMIN;
-    int64_t rows = rows_per_chunk;
+    int64_t rows = std::min<int64_t>(std::max<int64_t>(room / L, 1), m);
     if (fused)
         rows = std::min<int64_t>(std::max<int64_t>((room - CF_HDR) * 2 / (2 + CF_STRIDE), 1), m);
+    else if (pick)
+        rows = std::min<int64_t>((room - CF_HDR) / pick_row, m);
     int nsm = 0;
-    if (fused) {
+    if (fused || pick) {
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1778,11 +2233,34 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
     for (int64_t r0 = 0; r0 < m; r0 += rows) {
         int mc = (int)std::min<int64_t>(rows, m - r0);
         const int cap = fused ? (int)std::min<int64_t>((room - CF_HDR - mc) / CF_STRIDE, mc) : 0;
-        const int tok = prof_begin(ix, PROF_COARSE, 2, st);
+        const int tok = prof_begin(ix, PROF_COARSE, pick ? 3 : 2, st);
         // the distance buffer of the fused stage: the number of undecided
-        // rows, those rows, the records
+        // rows, those rows, the records; of the pick: the number of rows left
+        // to the block selection, the distances, the group minima, those rows
         int32_t *nh = reinterpret_cast<int32_t *>(Dbuf), *rec = nh + CF_HDR + mc;
-        if (fused) {
+        float *Dm = pick ? Dbuf + CF_HDR : Dbuf, *gm = Dm + (size_t)mc * L;
+        int32_t *left = reinterpret_cast<int32_t *>(gm + (size_t)mc * ((L + 15) / 16));
+        if (pick) {
+            const int KC = d <= 64 ? 1 : 2;
+            const size_t smem = coarse_fused_smem(KC, 2);
+            cudaMemsetAsync(nh, 0, sizeof(int32_t), st);
+            const int nt = (mc + CT_M - 1) / CT_M, nch = (L + CF_CN - 1) / CF_CN;
+            const int per = dist_chunks(nt, nch, nsm);
+            const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent);
+            const CUtensorMap &tl = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent_lo);
+            static bool attr[2] = {false, false};
+            auto go = [&](auto kern, int i) {
+                if (!attr[i]) {
+                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+                    attr[i] = true;
+                }
+                launch_pdl(kern, dim3(nt, (nch + per - 1) / per), CF_NT, smem, st, tm, tl, x + r0 * d,
+                           mc, d, ix->cnorm, L, per, Dm, gm, ix->err);
+            };
+            if (KC == 1) go(k_coarse_dist<1>, 0);
+            else go(k_coarse_dist<2>, 1);
+        } else if (fused) {
             const int KC = d <= 64 ? 1 : 2, parts = split == 3 ? 2 : 1;
             const size_t smem = coarse_fused_smem(KC, parts);
             cudaMemsetAsync(nh, 0, 2 * sizeof(int32_t), st);
@@ -1798,7 +2276,7 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
                     attr[i] = true;
                 }
                 launch_pdl(kern, std::min(nt, nsm), CF_NT, smem, st, tm, tl, x + r0 * d, mc, d,
-                           ix->cnorm, ix->cnrm_up, L, gamma2_first, out + r0, rec, cap, nh + CF_HDR,
+                           ix->cnorm, ix->cmax, L, gamma2_first, out + r0, rec, cap, nh + CF_HDR,
                            nh, ix->err);
             };
             if (parts == 1) {
@@ -1836,8 +2314,8 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
                        Dbuf);
         }
         SelArgs a;
-        a.D = fused ? nullptr : Dbuf;
-        a.hard = nh + CF_HDR;
+        a.D = fused ? nullptr : Dm;
+        a.hard = fused ? nh + CF_HDR : pick ? left : nullptr;
         a.nhard = nh;
         a.S = rec;
         a.s_cap = cap;
@@ -1851,16 +2329,23 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         a.cnrm_up = ix->cnrm_up;
         a.gamma2 = (float)(2.0 * gd * (1.0 + 1e-6));
         a.gamma2_first = gamma2_first;
-        const double gr = re_ops(d) * u / (1.0 - re_ops(d) * u);
+        const int ro = pick ? pk_ops(d) : re_ops(d);
+        const double gr = ro * u / (1.0 - ro * u);
         a.gamma2_re = (float)(2.0 * gr * (1.0 + 1e-6));
         a.two_level = two;
         a.out = out + r0 * P;
         a.err = ix->err;
-        if (warp_rows) {
+        if (pick) {
+            const size_t smem = CW_ROWS * pk_smem(P);  // 32 KB at P = 128
+            launch_pdl(k_coarse_pick, (unsigned)((mc + CW_ROWS - 1) / CW_ROWS), CW_ROWS * 32, smem, st,
+                       a, gm, ix->cmax, left, nh);
+            launch_pdl(k_coarse_select, std::min(mc, nsm), SEL_NT, 0, st, a);
+        } else if (warp_rows) {
             const unsigned gw = (unsigned)((mc + CW_ROWS - 1) / CW_ROWS);
             if (fused)  // loops over the undecided rows
-                launch_pdl(k_coarse_finish, std::min<unsigned>(gw, 10u * (unsigned)nsm), CW_ROWS * 32,
-                           0, st, a);
+                launch_pdl(k_coarse_finish,
+                           std::min<unsigned>((unsigned)((mc + FN_ROWS - 1) / FN_ROWS), 5u * (unsigned)nsm),
+                           FN_ROWS * 32, 0, st, a);
             else if (P == 1) launch_pdl(k_coarse_select_w<1>, gw, CW_ROWS * 32, 0, st, a);
             else launch_pdl(k_coarse_select_w<CW_PMAX>, gw, CW_ROWS * 32, 0, st, a);
         } else {

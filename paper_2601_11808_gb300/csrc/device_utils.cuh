@@ -157,6 +157,56 @@ __device__ __forceinline__ float fkey_inv(uint32_t k)
     return __uint_as_float(u);
 }
 
+// A value at least K of the n values val(i) (n a multiple of 32, +inf for
+// none) lie at or below, by a bisection on the order-preserving keys that
+// stops at K .. K + K / 8 of them; +inf when fewer than K are finite.
+template <int R, class V>  // R: values per lane held in registers (n <= 32 R)
+__device__ __forceinline__ float kth_bound(V val, int n, int K, int lane)
+{
+    uint32_t key[R];
+    const bool regs = n <= 32 * R;
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+    int fin = 0;
+    const uint32_t kinf = fkey(INFINITY);
+    auto see = [&](uint32_t k) {
+        kmin = min(kmin, k);
+        if (k < kinf) {
+            kmax = max(kmax, k);
+            ++fin;
+        }
+    };
+    if (regs) {
+#pragma unroll
+        for (int e = 0; e < R; ++e) {
+            key[e] = 32 * e < n ? fkey(val(32 * e + lane)) : 0xffffffffu;
+            see(key[e]);
+        }
+    } else {
+        for (int i = lane; i < n; i += 32) see(fkey(val(i)));
+    }
+    if (__reduce_add_sync(0xffffffffu, fin) < K) return INFINITY;
+    uint32_t lo = __reduce_min_sync(0xffffffffu, kmin), hi = __reduce_max_sync(0xffffffffu, kmax);
+    const int Kw = K + (K >> 3);
+    for (int t = 0; lo < hi; ++t) {  // invariant: #(key <= hi) >= K
+        // halves of the value range first (about ten, where the keys' range
+        // spends its halvings on the exponents around zero), then of the keys
+        uint32_t mid = lo + ((hi - lo) >> 1);
+        if (t < 12) mid = min(max(fkey(0.5f * fkey_inv(lo) + 0.5f * fkey_inv(hi)), lo), hi - 1u);
+        int c = 0;
+        if (regs) {
+#pragma unroll
+            for (int e = 0; e < R; ++e) c += key[e] <= mid;
+        } else {
+            for (int i = lane; i < n; i += 32) c += fkey(val(i)) <= mid;
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (c >= K) hi = mid;
+        else lo = mid + 1;
+        if (c >= K && c <= Kw) break;
+    }
+    return fkey_inv(hi);
+}
+
 // Ascending (distance, id) bitonic sort of 32*E elements held E per lane
 // (element i = lane + 32 e); pads are (+inf, -1).
 template <int E>

@@ -206,7 +206,7 @@ sivf_status sivf_exec_create(sivf_index *ix, const sivf_op *ops, int nops, sivf_
         for (int i = 0; i < nops; ++i) {
             const sivf_op &op = e->ops[i];
             if (op.kind != SIVF_OP_SEARCH) continue;
-            coarse_topP(ix, op.x, op.n, op.nprobe, e->probes[i], e->cbuf, coarse_rows(ix, op.n),
+            coarse_topP(ix, op.x, op.n, op.nprobe, e->probes[i], e->cbuf, coarse_floats(ix, op.n),
                         e->side);
             cudaEventRecord(e->evs[i], e->side);
         }

@@ -58,18 +58,17 @@ cudaError_t assign_stage_choose(sivf_index *ix, cudaStream_t st);
 int first_stage_split(const sivf_index *ix, int P);
 // relative error bound of the BF16 (split 1) or split BF16 (3) dot products
 double first_stage_rel(int d, int split);
-// exact top-P set of each row of x, in ascending list index; Dbuf holds
-// rows_per_chunk * nlist floats
-// rows of one coarse chunk and the scratch of a coarse selection of n rows
-int64_t coarse_rows(const sivf_index *ix, int64_t n);
+// the scratch of a coarse selection of n rows, in floats and bytes
+int64_t coarse_floats(const sivf_index *ix, int64_t n);
 size_t coarse_bytes(const sivf_index *ix, int64_t n);
 // the search of sivf_search_with_probes for probes the library selected
 // itself (distinct per query, so not de-duplicated)
 sivf_status search_probed(sivf_index *ix, const float *q, int64_t nq, int k, int nprobe,
                           const int32_t *probes, sivf_scan_dtype dtype, float *dist,
                           int64_t *labels, void *stream);
+// exact top-P set of each row of x, nearest first; Dbuf holds `room` floats
 void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
-                 float *Dbuf, int64_t rows_per_chunk, cudaStream_t st);
+                 float *Dbuf, int64_t room, cudaStream_t st);
 
 // ---- quantizer training (train.cu)
 // centroids := the given training rows (device, nlist of them)

@@ -163,7 +163,7 @@ extern "C" sivf_status sivf_search_noalloc(sivf_index *ix, const float *q, int64
         ix->ctl = own;
         return fail(SIVF_E_CUDA, "cudaMemsetAsync failed");
     }
-    coarse_topP(ix, q, nq, P, probes, Dbuf, rows, s);
+    coarse_topP(ix, q, nq, P, probes, Dbuf, rows * L, s);
     scan_lists(ix, q, nq, P, probes, false, pl, sc, s);
     merge_topk(ix, nq, P, pl, sc, k, dist, labels, s);
     ix->ctl = own;

@@ -455,54 +455,6 @@ __device__ __forceinline__ float fold_row(float *bd, int32_t *bs, int K, int Kw,
     return dmax;
 }
 
-// A value at least K of the n values val(i) (n a multiple of 128, +inf for
-// none) lie at or below, by a bisection on the order-preserving keys that
-// stops at K .. K + K / 8 of them; +inf when fewer than K are finite.
-template <class V>
-__device__ __forceinline__ float kth_bound(V val, int n, int K, int lane)
-{
-    constexpr int R = 12;  // values per lane held in registers (n <= 384)
-    uint32_t key[R];
-    const bool regs = n <= 32 * R;
-    uint32_t kmin = 0xffffffffu, kmax = 0u;
-    int fin = 0;
-    const uint32_t kinf = fkey(INFINITY);
-    auto see = [&](uint32_t k) {
-        kmin = min(kmin, k);
-        if (k < kinf) {
-            kmax = max(kmax, k);
-            ++fin;
-        }
-    };
-    if (regs) {
-#pragma unroll
-        for (int e = 0; e < R; ++e) {
-            key[e] = 32 * e < n ? fkey(val(32 * e + lane)) : 0xffffffffu;
-            see(key[e]);
-        }
-    } else {
-        for (int i = lane; i < n; i += 32) see(fkey(val(i)));
-    }
-    if (__reduce_add_sync(0xffffffffu, fin) < K) return INFINITY;
-    uint32_t lo = __reduce_min_sync(0xffffffffu, kmin), hi = __reduce_max_sync(0xffffffffu, kmax);
-    const int Kw = K + (K >> 3);
-    while (lo < hi) {  // invariant: #(key <= hi) >= K
-        const uint32_t mid = lo + ((hi - lo) >> 1);
-        int c = 0;
-        if (regs) {
-#pragma unroll
-            for (int e = 0; e < R; ++e) c += key[e] <= mid;
-        } else {
-            for (int i = lane; i < n; i += 32) c += fkey(val(i)) <= mid;
-        }
-        c = __reduce_add_sync(0xffffffffu, c);
-        if (c >= K) hi = mid;
-        else lo = mid + 1;
-        if (c >= K && c <= Kw) break;
-    }
-    return fkey_inv(hi);
-}
-
 // 16-byte asynchronous copy global -> shared; bytes past `src_bytes` (0 or
 // 16) are zero-filled
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, uint32_t src_bytes)
@@ -973,7 +925,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                     if (!run) break;
                     const int nv = TP * nbs * TC_M;  // minima per column
                     for (int n = ew; n < m; n += EW) {
-                        const float b = kth_bound(
+                        const float b = kth_bound<12>(
                             [&](int i) {
                                 return smin[((size_t)(i >> 7) * ncb * TC_NCOL + n) * TC_M + (i & 127)];
                             },

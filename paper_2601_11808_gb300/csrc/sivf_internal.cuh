@@ -107,6 +107,7 @@ struct sivf_index {
     float *cent;                   // [nlist, d]
     float *cnorm;                  // [nlist] fl32(||c||^2), from an FP64 sum
     float *cnrm_up;                // [nlist] upper bound of ||c||
+    float *cmax;                   // [2] the largest cnorm, the largest cnrm_up
     uint16_t *cent_bf16;           // [nlist, d] bf16(c) (tensor-core coarse stage)
     uint16_t *cent_lo;             // [nlist, d] bf16(c - bf16(c)) (split stage)
 

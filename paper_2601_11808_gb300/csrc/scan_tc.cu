@@ -820,14 +820,18 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
             const int set = (ew >> 2) / ncb, c0 = ((ew >> 2) % ncb) * TC_NCOL;
             const bool act = set < TP;
             // a row holds [0, nb) (at most RK) and appends at RK; its pending
-            // candidates are folded once a round of TP tiles leaves more than
-            // FT of them: FT plus one round always fits.  A fold keeps K' ..
-            // Kw.  For K' <= 128, more than 96 pending before a round cost
+            // candidates are folded once a step leaves more than FT of them:
+            // FT plus one step always fits.  A step is a round of TP tiles, or,
+            // where a thin item's long buffers have room for it, a whole group:
+            // its warps then meet no barrier from tile to tile.  A fold keeps
+            // K' .. Kw.  For K' <= 128, more than 96 pending before a step cost
             // more in a fold than the extra folds that a lower trigger brings
             // (measured at K' = 40); deeper sets fold only when the room is
             // full (the held K' dominate a fold's cost)
             const int RK = a.RK, Kw = K + ((RK - K) >> 1);
-            const int FT = K > 128 ? ME - RK - TP * TC_M : min(ME - RK - TP * TC_M, 96);
+            const bool freely = ME - RK >= NACC * TC_M + 96;
+            const int step = freely ? NACC * TC_M : TP * TC_M;
+            const int FT = K > 128 ? ME - RK - step : min(ME - RK - step, 96);
             const int32_t *qp = c_qpair(j);
             const float *cqn = c_qn(j), *cqsc = c_qsc(j), *ckd = c_kd0(j);
             const int32_t *sl = c_sl(j);
@@ -958,19 +962,17 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                 }
                 int s_next = act && set < ng ? row_slab(gb + set) : -1;
                 float x_next = row_norm(s_next);
+                bool need = false, wok = true;
                 for (int b0 = 0; b0 < ng; b0 += TP) {
                     const int b = b0 + set;  // this warp's tile of the round
                     const bool mine = act && b < ng;
                     const int sv = s_next;
                     const float xn = x_next;
-                    const bool live = mine && row_live(gb + b, sv);
-                    const int32_t gslot = sv * C + slot;
-                    bool wok = true;
                     float dv[TC_NCOL];
                     if (mine) {
                         s_next = b + TP < ng ? row_slab(gb + b + TP) : -1;
                         x_next = row_norm(s_next);
-                        wok = tile_wait(b);
+                        wok = wok && tile_wait(b);
                         tc_fence_after();
                         if (wok) tile_load(b, dv);
                         tc_fence_before();
@@ -979,13 +981,13 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                     if (lane == 0)
                         for (int t = b0; t < min(ng, b0 + TP); ++t) mbar_arrive(&tempty[(g + t) % NACC]);
 
-                    // a row passes for query n when -s q.x + ||x||^2 <= kd_n - ||q_n||^2:
-                    // the 16 ballots first (independent), then, only if a row
-                    // passed, lane i reserves column i's buffer positions with one
-                    // shared atomic and the passing rows are written
-                    bool need = false;
+                    // the row passes for query n when -s q.x + ||x||^2 <= kd_n -
+                    // ||q_n||^2: one bit per column, then each lane takes its
+                    // passing columns one after the other (one lane in three has
+                    // any where a bound holds), a place in the column's buffer
+                    // by a shared atomic each
                     if (wok && mine) {
-                        uint32_t mk[TC_NCOL];
+                        uint32_t pm = 0u;
                         const float4 *t4 = reinterpret_cast<const float4 *>(s_t + c0);
 #pragma unroll
                         for (int i4 = 0; i4 < TC_NCOL / 4; ++i4) {
@@ -994,45 +996,40 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                             float sc[4];
                             scales(i4, sc);
 #pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                const int i = 4 * i4 + c;
-                                const float part = fmaf(-sc[c], dv[i], xn);
-                                mk[i] = __ballot_sync(0xffffffffu, live && c0 + i < m && part <= tt[c]);
-                            }
+                            for (int c = 0; c < 4; ++c)
+                                if (fmaf(-sc[c], dv[4 * i4 + c], xn) <= tt[c]) pm |= 1u << (4 * i4 + c);
                         }
-                        uint32_t any = 0u;
+                        // columns past m hold what an earlier item left there
+                        if (m - c0 < TC_NCOL) pm &= (1u << (m - c0)) - 1u;
+                        if (!row_live(gb + b, sv)) pm = 0u;
+                        const int32_t gslot = sv * C + slot;
+                        while (pm) {
+                            const int i = __ffs(pm) - 1, n = c0 + i;
+                            pm &= pm - 1;
+                            float x8[8], x4[4];
 #pragma unroll
-                        for (int i = 0; i < TC_NCOL; ++i) any |= mk[i];
-                        if (any) {
-                            uint32_t my = 0u;
+                            for (int k = 0; k < 8; ++k) x8[k] = i & 8 ? dv[k + 8] : dv[k];
 #pragma unroll
-                            for (int i = 0; i < TC_NCOL; ++i)
-                                if (lane == i) my = mk[i];
-                            int mybase = 0;
-                            if (my) {
-                                mybase = atomicAdd(&s_cnt[c0 + lane], __popc(my));
-                                need = mybase + __popc(my) > FT;
-                            }
-#pragma unroll
-                            for (int i = 0; i < TC_NCOL; ++i) {
-                                if (!mk[i]) continue;
-                                const int n = c0 + i;
-                                const int base = __shfl_sync(0xffffffffu, mybase, i);
-                                if ((mk[i] >> lane) & 1u) {
-                                    const int p = RK + base + __popc(mk[i] & lanemask_lt());
-                                    BD[(size_t)n * ME + p] = fmaf(-s_sc[n], dv[i], cqn[n] + xn);
-                                    BS[(size_t)n * ME + p] = gslot;
-                                }
-                            }
+                            for (int k = 0; k < 4; ++k) x4[k] = i & 4 ? x8[k + 4] : x8[k];
+                            const float xa = i & 2 ? x4[2] : x4[0], xb = i & 2 ? x4[3] : x4[1];
+                            const int p = atomicAdd(&s_cnt[n], 1);
+                            BD[n * ME + RK + p] = fmaf(-s_sc[n], i & 1 ? xb : xa, cqn[n] + xn);
+                            BS[n * ME + RK + p] = gslot;
+                            need |= p >= FT;
                         }
+                        __syncwarp();
                     }
+                    if (freely && b0 + TP < ng) continue;
                     if (named_bar_or(1, EPI, need || !wok || *s_abort)) {
                         run = named_bar_and(1, EPI, wok && !*s_abort);
                         if (!run) break;
-                        // fold the rows whose pending candidates passed FT
+                        need = false;
+                        // fold the rows with pending candidates of about this
+                        // many together: one row's fold holds every warp up, so
+                        // rows that would follow in the next tiles go with it
                         for (int n = ew; n < m; n += EW) {
                             const int cc = s_cnt[n];
-                            if (cc <= FT) continue;
+                            if (cc <= (K > 128 ? FT : FT >> 2)) continue;
                             int nb = s_nb[n];
                             const float kd = fold_row(BD + (size_t)n * ME, BS + (size_t)n * ME, K, Kw,
                                                       RK, nb, cc, hist, lane);
@@ -1042,6 +1039,10 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                                 if (kd < s_kd[n]) {
                                     s_kd[n] = kd;
                                     s_t[n] = fminf(s_t[n], kd - cqn[n]);
+                                    // items over other chunks of the list read it
+                                    if (kd >= 0.f)
+                                        atomicMin(reinterpret_cast<int *>(a.thr) + qp[n] / a.P,
+                                                  __float_as_int(kd));
                                 }
                             }
                             __syncwarp();

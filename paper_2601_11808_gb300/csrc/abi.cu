@@ -469,8 +469,7 @@ static size_t search_bytes(const sivf_index *ix, int64_t nq, int k, int P, Searc
     if (plo) *plo = pl;
     size_t parts = (size_t)pl.run_cap * pl.K;
     return coarse_bytes(ix, nq) + (size_t)nq * P * 4 * 4 + (size_t)(L + 1) * 4 * 4 +
-           parts * 12 + (size_t)nq * 4 * 3 + (size_t)nq * 16 + (size_t)nq * pl.K * 12 +
-           (size_t)pl.item_cap * 8 + 19 * 256;
+           parts * 12 + (size_t)nq * 4 * 3 + (size_t)nq * 16 + (size_t)pl.item_cap * 8 + 19 * 256;
 }
 
 // plan of the reduced-precision scan for K' candidates (the batch's tile)
@@ -489,7 +488,7 @@ static size_t chunk_need(const sivf_index *ix, int64_t m, int P, int Kc, int dty
     *plo = pl;
     return coarse_bytes(ix, m) + (size_t)m * P * 4 * 4 + (size_t)(L + 1) * 4 * 4 +
            (size_t)pl.run_cap * (pl.RK * 12 + 4) + (size_t)m * 4 * 3 + (size_t)m * 16 +
-           (size_t)m * pl.K * 12 + (size_t)pl.item_cap * 8 + (size_t)m * ix->d * 2 +
+           (size_t)pl.item_cap * 8 + (size_t)m * ix->d * 2 +
            (dtype == SIVF_FP8E4M3 ? (size_t)m * P * (ix->d + 8) : 0) + 23 * 256;
 }
 
@@ -793,8 +792,6 @@ static sivf_status search_impl(sivf_index *ix, const float *q, int64_t nq, int k
                       : nullptr;
         sc.pqn = fp8 ? b.take<float>((size_t)m * P) : nullptr;
         sc.pqsc = fp8 ? b.take<float>((size_t)m * P) : nullptr;
-        float *cand_d = b.take<float>((size_t)m * pl.K);
-        int64_t *cand_s = b.take<int64_t>((size_t)m * pl.K);
         const int64_t room = coarse_floats(ix, m);
         float *Dbuf = b.take<float>((size_t)room);
         CUDA_TRY(ix, cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), s));
@@ -857,8 +854,7 @@ static sivf_status search_impl(sivf_index *ix, const float *q, int64_t nq, int k
                 merge_tc(ix, m, nphase, sc, Kc, pl.RK, dist + q0 * k, labels + q0 * k, s);
                 slots_to_ids(ix, labels + q0 * k, m * k, s);
             } else {
-                merge_rerank(ix, qq, m, nphase, sc, Kc, pl.RK, k, cand_d, cand_s, dist + q0 * k,
-                             labels + q0 * k, s);
+                merge_rerank(ix, qq, m, nphase, sc, Kc, pl.RK, k, dist + q0 * k, labels + q0 * k, s);
             }
         }
         CUDA_TRY(ix, cudaGetLastError());

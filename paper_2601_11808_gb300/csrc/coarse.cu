@@ -1773,7 +1773,7 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
         const float dc = sDt[s];
         int pos = 0;
 #pragma unroll 8
-        for (int q = 0; q < nsel; ++q) pos += sDt[q] < dc || (sDt[q] == dc && sIdx[q] < c);
+        for (int q = 0; q < nsel; ++q) pos += (sDt[q] < dc) | ((sDt[q] == dc) & (sIdx[q] < c));  // no branches
         outr[pos] = c;
     }
 }

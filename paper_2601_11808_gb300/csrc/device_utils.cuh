@@ -159,7 +159,7 @@ __device__ __forceinline__ float fkey_inv(uint32_t k)
 
 // A value at least K of the n values val(i) (n a multiple of 32, +inf for
 // none) lie at or below, by a bisection on the order-preserving keys that
-// stops at K .. K + K / 8 of them; +inf when fewer than K are finite.
+// stops at about K + K / 8 of them; +inf when fewer than K are finite.
 template <int R, class V>  // R: values per lane held in registers (n <= 32 R)
 __device__ __forceinline__ float kth_bound(V val, int n, int K, int lane)
 {
@@ -186,7 +186,7 @@ __device__ __forceinline__ float kth_bound(V val, int n, int K, int lane)
     }
     if (__reduce_add_sync(0xffffffffu, fin) < K) return INFINITY;
     uint32_t lo = __reduce_min_sync(0xffffffffu, kmin), hi = __reduce_max_sync(0xffffffffu, kmax);
-    const int Kw = K + (K >> 3);
+    const int Kw = K + (K > 128 ? K >> 5 : K >> 3) + 1;
     for (int t = 0; lo < hi; ++t) {  // invariant: #(key <= hi) >= K
         // halves of the value range first (about ten, where the keys' range
         // spends its halvings on the exponents around zero), then of the keys

@@ -58,7 +58,10 @@ constexpr int TC_PF_BYTES = 192 * 1024;  // L2 prefetch distance per CTA
 // quarter, 16 query columns each.
 template <int TN> struct TcShape {
     static constexpr int N = TN;                        // queries per tile (MMA N)
-    static constexpr int EW = 4 * (TN / TC_NCOL);       // epilogue warps
+    // epilogue warps: three per TMEM lane quarter, also where TN has fewer
+    // blocks of 16 columns (they then share the tiles); FW of them fold
+    static constexpr int EW = 12;
+    static constexpr int FW = 4 * (TN / TC_NCOL);
     static constexpr int EPI = EW * 32;                 // epilogue threads
     static constexpr int NT = 128 + EPI;                // + TMA, MMA, context, B warps
     static constexpr int KMAX = TN == 48 ? 64 : TN == 32 ? 128 : 512;  // deepest K'
@@ -128,7 +131,7 @@ __host__ __device__ inline TcSmem tc_smem(int KC, int M, int nst)
     s.bs = s.bd + (size_t)TN * M * 4;
     s.ctx = s.bs + (size_t)TN * M * 4;
     s.hist = s.ctx + (size_t)TC_CTX * tc_ctx_bytes(TN);
-    s.bars = s.hist + (size_t)S::EW * TC_HIST * 4;
+    s.bars = s.hist + (size_t)S::FW * TC_HIST * 4;
     s.total = s.bars + 64 * 8 + 1024;                    // + base alignment slack
     return s;
 }
@@ -455,6 +458,96 @@ __device__ __forceinline__ float fold_row(float *bd, int32_t *bs, int K, int Kw,
     return dmax;
 }
 
+// As kth_bound (device_utils.cuh) for more values than registers hold, by
+// histograms of TC_HIST equal steps of the value range: of all values, then
+// of the step the K-th falls into, until little more than K lie within.
+// 2,304 values: about 5 passes over them where the bisection took 18.
+template <class V>
+__device__ float kth_bound_hist(V val, int n, int K, uint32_t *hist, int lane)
+{
+    const int Kw = K + (K >> 5) + 1;
+    float lo = INFINITY, hi = -INFINITY;
+    int fin = 0;
+#pragma unroll 8
+    for (int i = lane; i < n; i += 32) {
+        const float v = val(i);
+        if (v < INFINITY) {
+            lo = fminf(lo, v);
+            hi = fmaxf(hi, v);
+            ++fin;
+        }
+    }
+    if (__reduce_add_sync(0xffffffffu, fin) < K) return INFINITY;
+    int below = 0;  // values under lo
+    for (int round = 0; round < 4; ++round) {
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        const float scale = (float)TC_HIST / (hi - lo);
+        if (!(scale < INFINITY) || !(hi > lo)) break;
+        // the same rounding in every pass: monotone in v
+        auto bin = [&](float v) { return min(TC_HIST - 1, (int)__fmul_rn(__fsub_rn(v, lo), scale)); };
+#pragma unroll
+        for (int b = 0; b < TC_HIST / 32; ++b) hist[lane * (TC_HIST / 32) + b] = 0u;
+        __syncwarp();
+#pragma unroll 8
+        for (int i = lane; i < n; i += 32) {
+            const float v = val(i);
+            if (v >= lo && v <= hi) atomicAdd(&hist[bin(v)], 1u);
+        }
+        __syncwarp();
+        uint32_t loc[TC_HIST / 32], sum = 0;
+#pragma unroll
+        for (int b = 0; b < TC_HIST / 32; ++b) {
+            loc[b] = hist[lane * (TC_HIST / 32) + b];
+            sum += loc[b];
+        }
+        uint32_t incl = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const uint32_t need = (uint32_t)(K - below);
+        uint32_t cum = incl - sum;
+        const bool mine = cum < need && incl >= need;
+        int at = 0;
+        uint32_t under = 0, upto = 0;
+        if (mine)
+            for (int b = 0; b < TC_HIST / 32; ++b) {
+                if (cum + loc[b] >= need) {
+                    at = lane * (TC_HIST / 32) + b;
+                    under = cum;
+                    upto = cum + loc[b];
+                    break;
+                }
+                cum += loc[b];
+            }
+        const uint32_t who = __ballot_sync(0xffffffffu, mine);
+        const int src = who ? __ffs(who) - 1 : 0;
+        at = __shfl_sync(0xffffffffu, at, src);
+        under = __shfl_sync(0xffffffffu, under, src);
+        upto = __shfl_sync(0xffffffffu, upto, src);
+        __syncwarp();
+        // the step's own range; its largest value bounds the K-th
+        float l2 = INFINITY, h2 = -INFINITY;
+#pragma unroll 8
+        for (int i = lane; i < n; i += 32) {
+            const float v = val(i);
+            if (v >= lo && v <= hi && bin(v) == at) {
+                l2 = fminf(l2, v);
+                h2 = fmaxf(h2, v);
+            }
+        }
+        lo = l2;
+        hi = h2;
+        if (below + (int)upto <= Kw) break;
+        below += (int)under;
+    }
+    for (int o = 16; o > 0; o >>= 1) hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    return hi;
+}
+
 // 16-byte asynchronous copy global -> shared; bytes past `src_bytes` (0 or
 // 16) are zero-filled
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, uint32_t src_bytes)
@@ -481,7 +574,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
 {
     pdl_begin();
     using S = TcShape<TN>;
-    constexpr int EW = S::EW, EPI = S::EPI, TB = S::TB, NACC = S::NACC;
+    constexpr int EW = S::EW, FW = S::FW, EPI = S::EPI, TB = S::TB, NACC = S::NACC;
     constexpr int ESZ = DT == 0 ? 2 : 1;
     constexpr int EPC = 128 / ESZ;  // elements per 128-byte chunk
     extern __shared__ unsigned char smem_raw[];
@@ -803,7 +896,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
         const int et = ew * 32 + lane;       // epilogue thread
         const int v = qt * 32 + lane;        // A row = vector of the tile
         const uint32_t tlane = (uint32_t)(qt * 32) << 16;
-        uint32_t *hist = Hist + ew * TC_HIST;
+        uint32_t *hist = Hist + min(ew, FW - 1) * TC_HIST;
         float *smin = BD;                    // the minima, while no candidate is held
         uint32_t g = 0;
         for (int it = 0;; ++it) {
@@ -816,7 +909,10 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
             const int m = h[1], sns = h[3], nblk = h[4], ME = h[5], chunk = h[7];
             const float inv_l = __int_as_float(h[9]);
             // columns and tiles of this warp
-            const int ncb = (m + TC_NCOL - 1) / TC_NCOL, TP = max(1, (EW / 4) / ncb);
+            // (no more sets than a row's buffer has room for, twice over where a
+            // fold is dear)
+            const int ncb = (m + TC_NCOL - 1) / TC_NCOL;
+            const int TP = max(1, min((EW / 4) / ncb, (ME - a.RK) / (K > 128 ? 2 * TC_M : TC_M)));
             const int set = (ew >> 2) / ncb, c0 = ((ew >> 2) % ncb) * TC_NCOL;
             const bool act = set < TP;
             // a row holds [0, nb) (at most RK) and appends at RK; its pending
@@ -884,8 +980,13 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
             for (int gb = 0; gb < nblk && run; gb += NACC) {
                 const int ng = min(NACC, nblk - gb);
                 if (look && gb == 0) {
-                    const int nbs = max(1, ((5 * K + 255) / 256 + TP - 1) / TP);  // banks of a set
-                    const int per = ((ng + TP - 1) / TP + nbs - 1) / nbs;         // tiles of a bank
+                    // banks of a set: 2.5 K' minima per column at least; a bank per
+                    // tile for deep sets where they fit (every row its own minimum:
+                    // 412 of K' = 400's bound pass, else a quarter more than fit a run)
+                    const int tset = (ng + TP - 1) / TP;
+                    int nbs = max(1, ((5 * K + 255) / 256 + TP - 1) / TP);
+                    if (K > 128) nbs = max(nbs, min(tset, (TN * M * 8) / (TP * m * TC_M * 4)));
+                    const int per = (tset + nbs - 1) / nbs;                       // tiles of a bank
                     bool wok = true;
                     tc_fence_after();
                     if (act) {
@@ -919,21 +1020,23 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                                     }
                                 }
                             }
-                            float *o = smin + (size_t)((set * nbs + bk) * ncb * TC_NCOL + c0) * TC_M + v;
+                            float *o = smin + (size_t)((set * nbs + bk) * m + c0) * TC_M + v;
 #pragma unroll
-                            for (int i = 0; i < TC_NCOL; ++i) o[i * TC_M] = mn[i];
+                            for (int i = 0; i < TC_NCOL; ++i)
+                                if (c0 + i < m) o[i * TC_M] = mn[i];
                         }
                     }
                     tc_fence_before();
                     run = named_bar_and(1, EPI, wok && !*s_abort);
                     if (!run) break;
                     const int nv = TP * nbs * TC_M;  // minima per column
-                    for (int n = ew; n < m; n += EW) {
-                        const float b = kth_bound<12>(
-                            [&](int i) {
-                                return smin[((size_t)(i >> 7) * ncb * TC_NCOL + n) * TC_M + (i & 127)];
-                            },
-                            nv, K, lane);
+                    const bool many = nv > 32 * 12;  // past a warp's registers
+                    for (int n = many && ew >= FW ? m : ew; n < m; n += many ? FW : EW) {
+                        auto val = [&](int i) {
+                            return smin[((size_t)(i >> 7) * m + n) * TC_M + (i & 127)];
+                        };
+                        const float b = many ? kth_bound_hist(val, nv, K, hist, lane)
+                                             : kth_bound<12>(val, nv, K, lane);
                         if (lane == 0 && b < INFINITY) {
                             // room for the roundings of ||q||^2 + ||x||^2 - 2 s q.x, formed
                             // in another order for the distances that are kept
@@ -1027,7 +1130,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                         // fold the rows with pending candidates of about this
                         // many together: one row's fold holds every warp up, so
                         // rows that would follow in the next tiles go with it
-                        for (int n = ew; n < m; n += EW) {
+                        for (int n = ew < FW ? ew : m; n < m; n += FW) {
                             const int cc = s_cnt[n];
                             if (cc <= (K > 128 ? FT : FT >> 2)) continue;
                             int nb = s_nb[n];
@@ -1063,7 +1166,7 @@ __global__ __launch_bounds__(TcShape<TN>::NT, 1) void k_scan_tc(
                 // a bound on its K'-th distance becomes a bound of the query
                 // for the items that follow
                 named_bar_sync(1, EPI);
-                for (int n = ew; n < m; n += EW) {
+                for (int n = ew < FW ? ew : m; n < m; n += FW) {
                     const int cc = s_cnt[n];
                     int nb = s_nb[n];
                     float *bd = BD + (size_t)n * ME;
@@ -1259,103 +1362,6 @@ void merge_tc(sivf_index *ix, int64_t nq, int nphase, const SearchScratch &s, in
 }
 
 // ---------------------------------------------------------------- re-rank
-// One warp per query: exact FP32 direct-form distances of the K' merged
-// candidates (global slots) from the FP32 payload, then the best k by
-// (distance, id).  Eight lanes share a candidate row: lane t of a group
-// holds query chunks t, t + 8, ... (16 bytes each) in registers and reads
-// the same chunks of the row, so one load instruction of the warp covers
-// four whole 128-byte lines; RK_UNR rounds of four candidates are loaded
-// before any is reduced (the group's partial sums meet by shuffles).  The
-// candidates' slots are staged in shared memory first; their ids are read
-// into the owning lanes' registers then and used only by the sort.
-constexpr int RK_NT = 128;
-constexpr int RK_UNR = 4;  // measured best of 2, 4, 5, 8 and 10
-template <int E, int NQ>  // E: candidates per lane in the sort; NQ: chunks per lane (d <= 32 NQ)
-__global__ __launch_bounds__(RK_NT) void k_rerank(const float *__restrict__ q, int64_t nq, int d,
-                                                int Kc, const float *__restrict__ cand_d,
-                                                const int64_t *__restrict__ cand_s,
-                                                const float *__restrict__ x32,
-                                                const int64_t *__restrict__ ids, int k,
-                                                float *__restrict__ dist, int64_t *__restrict__ labels)
-{
-    pdl_begin();
-    __shared__ int64_t sgs[RK_NT / 32][32 * E];
-    __shared__ float sd[RK_NT / 32][32 * E];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 3, t = lane & 7;
-    const int64_t qi = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (qi >= nq) return;  // whole warps
-    const int n4 = d >> 2;
-    // candidate slots (-1: none); ids into registers, read by the sort
-    int64_t id[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int c = lane + 32 * e;
-        int64_t gs = -1;
-        if (c < Kc) {
-            gs = cand_s[qi * Kc + c];
-            if (!(cand_d[qi * Kc + c] < INFINITY)) gs = -1;
-        }
-        sgs[w][c] = gs;
-        id[e] = gs >= 0 ? __ldg(ids + gs) : -1;
-    }
-    const float4 *q4 = reinterpret_cast<const float4 *>(q + (size_t)qi * d);
-    float4 qv[NQ];
-#pragma unroll
-    for (int u = 0; u < NQ; ++u)
-        qv[u] = t + 8 * u < n4 ? __ldg(q4 + t + 8 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncwarp();
-    const float4 *x4 = reinterpret_cast<const float4 *>(x32);
-    for (int c0 = 0; c0 < Kc; c0 += 4 * RK_UNR) {
-        float4 xv[RK_UNR][NQ];
-        int64_t gs[RK_UNR];
-#pragma unroll
-        for (int r = 0; r < RK_UNR; ++r) {
-            const int c = c0 + 4 * r + g;
-            gs[r] = c < Kc ? sgs[w][c] : -1;
-#pragma unroll
-            for (int u = 0; u < NQ; ++u)
-                xv[r][u] = gs[r] >= 0 && t + 8 * u < n4 ? __ldg(x4 + gs[r] * n4 + t + 8 * u)
-                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int r = 0; r < RK_UNR; ++r) {
-            float acc = 0.f;
-#pragma unroll
-            for (int u = 0; u < NQ; ++u) {
-                float dd = qv[u].x - xv[r][u].x;
-                acc = fmaf(dd, dd, acc);
-                dd = qv[u].y - xv[r][u].y;
-                acc = fmaf(dd, dd, acc);
-                dd = qv[u].z - xv[r][u].z;
-                acc = fmaf(dd, dd, acc);
-                dd = qv[u].w - xv[r][u].w;
-                acc = fmaf(dd, dd, acc);
-            }
-            acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-            acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-            const int c = c0 + 4 * r + g;
-            if (t == 0 && c < Kc) sd[w][c] = gs[r] >= 0 ? acc : INFINITY;
-        }
-    }
-    __syncwarp();
-    float v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int c = lane + 32 * e;
-        v[e] = c < Kc && id[e] >= 0 ? sd[w][c] : INFINITY;
-    }
-    warp_bitonic_sort<E>(v, id, lane);
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = lane + 32 * e;
-        if (i < k) {
-            dist[qi * k + i] = id[e] >= 0 ? v[e] : INFINITY;
-            labels[qi * k + i] = id[e];
-        }
-    }
-}
-
 // The per-query merge and the re-rank in one warp per query (K' <= 128):
 // merge_select leaves the query's best K' (distance, slot) entries in shared
 // memory, and the warp re-ranks those slots exactly as k_rerank does (eight
@@ -1452,41 +1458,215 @@ __global__ __launch_bounds__(MT_NT, NQ <= 4 ? 9 : 2) void k_merge_rerank(
     }
 }
 
-// Deep re-rank (K' up to 512): one block per query; its warps compute the
-// candidates' exact FP32 direct-form distances into shared memory (eight
-// lanes per candidate row with 16-byte loads, RR_UNR rounds of four rows
-// per warp loaded before they are reduced, the query in registers), then
-// the block sorts them by (distance, id) with a bitonic network and writes
-// the best k.  Two rounds per batch keep the registers low enough for four
-// blocks per SM: the gather is bound by loads in flight, i.e. by resident
-// warps.
+// Merge and re-rank with one block per query (K' <= 512; deep sets, and few
+// queries).  The entries of the query's runs at or below its bound are
+// gathered into shared memory (four runs at a time or more) and reduced to the best K' by a block-wide radix
+// select on the 64-bit (distance, slot) keys, also whenever the buffer could
+// overflow; then the block's warps compute the candidates' exact FP32
+// direct-form distances (eight lanes per candidate row with 16-byte loads,
+// RR_UNR rounds of four rows per warp loaded before they are reduced, the
+// query in registers), and the block sorts them by (distance, id) with a
+// bitonic network and writes the best k.  Two rounds per batch keep the
+// registers low enough for four blocks per SM: the gather is bound by loads
+// in flight, i.e. by resident warps.  A warp per query for the merge, its
+// sorted candidates through global memory, took 301 + 582 us for 10,000
+// queries at K' = 400; fused 571 us (the rows alone: 230 us of HBM).
 constexpr int RR_NT = 256;
 constexpr int RR_MAX = 512;
+constexpr int RR_CAP = 2048;  // gathered entries: at most 4 RR_NT more than K' at once
+
+// the K smallest of the n > K entries sd / ss, in place and unsorted (whole
+// block; n <= RR_CAP); returns the largest distance kept
+__device__ float block_reduce_k(float *sd, int32_t *ss, int n, int K, uint32_t *hist)
+{
+    constexpr int PT = RR_CAP / RR_NT;
+    __shared__ unsigned long long s_min, s_max, s_prefix;
+    __shared__ uint32_t s_need, s_cnt;
+    __shared__ int s_n, s_top;
+    const int tid = threadIdx.x, lane = tid & 31;
+    uint64_t key[PT];
+    uint64_t kmin = ~0ull, kmax = 0ull;
+#pragma unroll
+    for (int e = 0; e < PT; ++e) {
+        const int i = tid + e * RR_NT;
+        key[e] = i < n ? ds_key(sd[i], ss[i]) : ~0ull;
+        if (i < n) {
+            kmin = min(kmin, key[e]);
+            kmax = max(kmax, key[e]);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        kmin = min(kmin, (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)kmin, o));
+        kmax = max(kmax, (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)kmax, o));
+    }
+    if (tid == 0) {
+        s_min = ~0ull;
+        s_max = 0ull;
+        s_n = 0;
+        s_top = 0;
+    }
+    __syncthreads();
+    if (lane == 0) {
+        atomicMin(&s_min, (unsigned long long)kmin);
+        atomicMax(&s_max, (unsigned long long)kmax);
+    }
+    __syncthreads();
+    const uint64_t diff = s_min ^ s_max;
+    const int top = diff ? 63 - __clzll((long long)diff) : 0;
+    uint64_t mask = top >= 63 ? 0ull : ~((2ull << top) - 1ull), prefix = s_min & mask;
+    uint32_t need = (uint32_t)K;
+    for (int hi = top; hi >= 0; hi -= 8) {
+        const int shift = max(hi - 7, 0);
+        const uint32_t bmask = (1u << (hi - shift + 1)) - 1u;
+        hist[tid] = 0u;  // RR_NT bins
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < PT; ++e)
+            if (tid + e * RR_NT < n && (key[e] & mask) == prefix)
+                atomicAdd(&hist[(uint32_t)(key[e] >> shift) & bmask], 1u);
+        __syncthreads();
+        if (tid < 32) {
+            uint32_t loc[8], sum = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                loc[k] = hist[lane * 8 + k];
+                sum += loc[k];
+            }
+            uint32_t incl = sum;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            uint32_t cum = incl - sum;
+            if (cum < need && incl >= need)
+                for (int k = 0; k < 8; ++k) {
+                    if (cum + loc[k] >= need) {
+                        s_prefix = prefix | ((uint64_t)(lane * 8 + k) << shift);
+                        s_need = need - cum;
+                        s_cnt = loc[k];
+                        break;
+                    }
+                    cum += loc[k];
+                }
+        }
+        __syncthreads();
+        prefix = s_prefix;
+        need = s_need;
+        mask |= (uint64_t)bmask << shift;
+        if (s_cnt == need) break;
+    }
+    // every entry is in registers: the kept ones go back to the front
+    uint32_t kk = 0u;
+#pragma unroll
+    for (int e = 0; e < PT; ++e) {
+        const bool take = tid + e * RR_NT < n && (key[e] & mask) <= prefix;
+        const uint32_t mk = __ballot_sync(0xffffffffu, take);
+        int base = 0;
+        if (lane == 0 && mk) base = atomicAdd(&s_n, __popc(mk));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (take) {
+            const int p = base + __popc(mk & lanemask_lt());
+            sd[p] = fkey_inv((uint32_t)(key[e] >> 32));
+            ss[p] = (int32_t)(uint32_t)key[e];
+            kk = max(kk, (uint32_t)(key[e] >> 32));
+        }
+    }
+    kk = __reduce_max_sync(0xffffffffu, kk);
+    if (lane == 0) atomicMax(reinterpret_cast<uint32_t *>(&s_top), kk);
+    __syncthreads();
+    return fkey_inv((uint32_t)s_top);
+}
+
 template <int NQ>  // 16-byte chunks of the row per lane (d <= 32 NQ)
-__global__ __launch_bounds__(RR_NT, NQ <= 4 ? 4 : 1) void k_rerank_wide(const float *__restrict__ q, int64_t nq,
-                                                       int d, int Kc,
-                                                       const float *__restrict__ cand_d,
-                                                       const int64_t *__restrict__ cand_s,
-                                                       const float *__restrict__ x32,
-                                                       const int64_t *__restrict__ ids, int k,
-                                                       float *__restrict__ dist,
-                                                       int64_t *__restrict__ labels)
+__global__ __launch_bounds__(RR_NT, NQ <= 4 ? 4 : 1) void k_merge_rerank_wide(
+    const int2 *__restrict__ qrun, int64_t nq, int nphase, int K, int RK, int tpr,
+    const float *__restrict__ thr, const int32_t *__restrict__ part_n,
+    const float *__restrict__ part_d, const int64_t *__restrict__ part_i,
+    const float *__restrict__ q, int d, const float *__restrict__ x32,
+    const int64_t *__restrict__ ids, int k, float *__restrict__ dist, int64_t *__restrict__ labels)
 {
     pdl_begin();
-    __shared__ float sd[RR_MAX];
+    __shared__ __align__(16) float sd[RR_CAP];
+    __shared__ int32_t ss[RR_CAP];
     __shared__ int64_t si[RR_MAX];
+    __shared__ uint32_t hist[RR_NT];
+    __shared__ int s_have;
     const int64_t qi = blockIdx.x;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 3, t = lane & 7;
     const int64_t PAD = 0x7fffffffffffffffLL;  // pads sort after every id
-    int N = 32;
-    while (N < Kc) N <<= 1;
     const int n4 = d >> 2;
     const float4 *q4 = reinterpret_cast<const float4 *>(q + (size_t)qi * d);
     const float4 *x4 = reinterpret_cast<const float4 *>(x32);
+    const int2 r0 = qrun[qi];
+    const int2 r1 = nphase > 1 ? qrun[nq + qi] : make_int2(0, 0);
+    const int NR = r0.y + r1.y;
+    auto run_of = [&](int r) -> int64_t { return r < r0.y ? r0.x + r : r1.x + (r - r0.y); };
+    float bound = thr[qi];
+    if (tid == 0) s_have = 0;
+    __syncthreads();
+    int have = 0;  // uniform over the block
+    // tpr threads read a run, 4 RR_NT / tpr runs at a time; the next ones'
+    // counts are read meanwhile
+    const int rw = RR_NT / tpr, j = tid % tpr, rj = tid / tpr;
+    int cn[4];
+    auto counts = [&](int rb) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            cn[r] = rb + r * rw + rj < NR ? min(part_n[run_of(rb + r * rw + rj)], RK) : 0;
+    };
+    counts(0);
+    for (int rb = 0; rb < NR; rb += 4 * rw) {
+        int c[4];
+        int64_t base[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            c[r] = cn[r];
+            base[r] = c[r] > 0 ? run_of(rb + r * rw + rj) * RK : 0;
+        }
+        counts(rb + 4 * rw);
+        for (int j0 = 0; j0 < RK; j0 += tpr) {
+            if (have > RR_CAP - 4 * RR_NT) {
+                bound = fminf(bound, block_reduce_k(sd, ss, have, K, hist));
+                have = K;
+                if (tid == 0) s_have = K;
+                __syncthreads();
+            }
+            float dv[4];
+            int32_t sv[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const bool ok = j0 + j < c[r];
+                dv[r] = ok ? part_d[base[r] + j0 + j] : INFINITY;
+                sv[r] = ok ? (int32_t)part_i[base[r] + j0 + j] : -1;
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const bool in = sv[r] >= 0 && dv[r] <= bound;
+                const uint32_t mk = __ballot_sync(0xffffffffu, in);
+                int b = 0;
+                if (lane == 0 && mk) b = atomicAdd(&s_have, __popc(mk));
+                b = __shfl_sync(0xffffffffu, b, 0);
+                if (in) {
+                    const int p = b + __popc(mk & lanemask_lt());
+                    sd[p] = dv[r];
+                    ss[p] = sv[r];
+                }
+            }
+            __syncthreads();
+            have = s_have;
+            __syncthreads();  // every thread has read it before it grows again
+        }
+    }
+    if (have > K) {
+        block_reduce_k(sd, ss, have, K, hist);
+        have = K;
+    }
     float4 qv[NQ];
 #pragma unroll
     for (int u = 0; u < NQ; ++u)
         qv[u] = t + 8 * u < n4 ? __ldg(q4 + t + 8 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+    int N = 32;
+    while (N < have) N <<= 1;  // <= RR_MAX
     constexpr int CPW = 4 * RR_UNR;  // candidates per warp and batch
     for (int c0 = warp * CPW; c0 < N; c0 += (RR_NT / 32) * CPW) {
         float4 xv[RR_UNR][NQ];
@@ -1494,11 +1674,7 @@ __global__ __launch_bounds__(RR_NT, NQ <= 4 ? 4 : 1) void k_rerank_wide(const fl
 #pragma unroll
         for (int r = 0; r < RR_UNR; ++r) {
             const int c = c0 + 4 * r + g;
-            gs[r] = -1;
-            if (c < Kc) {
-                const int64_t s0 = cand_s[qi * Kc + c];
-                if (s0 >= 0 && cand_d[qi * Kc + c] < INFINITY) gs[r] = s0;
-            }
+            gs[r] = c < have ? (int64_t)ss[c] : -1;
 #pragma unroll
             for (int u = 0; u < NQ; ++u)
                 xv[r][u] = gs[r] >= 0 && t + 8 * u < n4 ? __ldg(x4 + gs[r] * n4 + t + 8 * u)
@@ -1523,33 +1699,81 @@ __global__ __launch_bounds__(RR_NT, NQ <= 4 ? 4 : 1) void k_rerank_wide(const fl
             acc += __shfl_xor_sync(0xffffffffu, acc, 1);
             const int c = c0 + 4 * r + g;
             if (t == 0 && c < N) {
-                sd[c] = gs[r] >= 0 ? acc : INFINITY;
+                sd[c] = gs[r] >= 0 ? acc : INFINITY;  // the approximate one is no longer needed
                 si[c] = gs[r] >= 0 ? __ldg(ids + gs[r]) : PAD;
             }
         }
     }
     __syncthreads();
+    // sort by exact distance: 64-bit keys (distance, place), two per thread,
+    // exchanged by shuffles within a warp and through shared memory beyond
+    // (every stage through shared memory with the ids took as long as the rows'
+    // gather); equal distances are ranked by id below
+    uint64_t ky[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int i = tid + e * RR_NT;
+        ky[e] = i < N && si[i] != PAD ? ((uint64_t)fkey(sd[i]) << 32) | (uint32_t)i : ~0ull;
+    }
+    __syncthreads();
+    uint64_t *xk = reinterpret_cast<uint64_t *>(sd);  // RR_MAX keys
     for (int size = 2; size <= N; size <<= 1)
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = tid; t < N / 2; t += RR_NT) {
-                const int i = 2 * t - (t & (stride - 1)), j = i + stride;
-                const bool up = (i & size) == 0;
-                const bool lt = dk_less(sd[j], si[j], sd[i], si[i]);
-                if (lt == up) {
-                    const float td = sd[i];
-                    sd[i] = sd[j];
-                    sd[j] = td;
-                    const int64_t ti = si[i];
-                    si[i] = si[j];
-                    si[j] = ti;
-                }
+            if (stride == RR_NT) {  // size = 512: ascending
+                const uint64_t a = min(ky[0], ky[1]), b = max(ky[0], ky[1]);
+                ky[0] = a;
+                ky[1] = b;
+                continue;
             }
-            __syncthreads();
+            uint64_t o[2];
+            if (stride >= 32) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) xk[tid + e * RR_NT] = ky[e];
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < 2; ++e) o[e] = xk[(tid ^ stride) + e * RR_NT];
+                __syncthreads();
+            } else {
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    o[e] = __shfl_xor_sync(0xffffffffu, (unsigned long long)ky[e], stride);
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool up = ((tid + e * RR_NT) & size) == 0, lower = (tid & stride) == 0;
+                ky[e] = lower == up ? min(ky[e], o[e]) : max(ky[e], o[e]);
+            }
         }
-    for (int i = tid; i < k; i += RR_NT) {
-        const bool ok = i < N && si[i] != PAD;
-        dist[qi * k + i] = ok ? sd[i] : INFINITY;
-        labels[qi * k + i] = ok ? si[i] : -1;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) xk[tid + e * RR_NT] = ky[e];
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int i = tid + e * RR_NT;
+        if (i >= N) continue;
+        const uint64_t me = ky[e];
+        if (me == ~0ull) {
+            if (i < k) {
+                dist[qi * k + i] = INFINITY;
+                labels[qi * k + i] = -1;
+            }
+            continue;
+        }
+        const uint32_t dk = (uint32_t)(me >> 32);
+        const int64_t id = si[(uint32_t)me];
+        int pos = i;  // among equal distances: by id
+        for (int j = i - 1; j >= 0 && (uint32_t)(xk[j] >> 32) == dk; --j)
+            pos -= si[(uint32_t)xk[j]] > id;
+        for (int j = i + 1; j < N && (uint32_t)(xk[j] >> 32) == dk && xk[j] != ~0ull; ++j)
+            pos += si[(uint32_t)xk[j]] < id;
+        if (pos < k) {
+            dist[qi * k + pos] = fkey_inv(dk);
+            labels[qi * k + pos] = id;
+        }
+    }
+    for (int i = N + tid; i < k; i += RR_NT) {  // fewer candidates than k
+        dist[qi * k + i] = INFINITY;
+        labels[qi * k + i] = -1;
     }
 }
 
@@ -1927,15 +2151,24 @@ void scan_lists_tc(sivf_index *ix, int dtype, const float *q, int64_t nq, int P,
     prof_end(ix, tok, st);
 }
 
-// merge and re-rank of a search: fused for K' <= 128 (d <= 256), else the
-// merge into cand_d / cand_s followed by the wide re-rank
+// merge and re-rank of a search: a block per query for K' > 128 and for few
+// queries (one wave of blocks: a warp's chain of loads over the chunked lists'
+// runs takes 40 us however few the queries are, a block's 24; 1,000 queries
+// 41 against 46 us), else a warp each
 void merge_rerank(sivf_index *ix, const float *q, int64_t nq, int nphase,
-                  const SearchScratch &s, int Kc, int RK, int k, float *cand_d,
-                  int64_t *cand_s, float *dist, int64_t *labels, cudaStream_t st)
+                  const SearchScratch &s, int Kc, int RK, int k, float *dist, int64_t *labels,
+                  cudaStream_t st)
 {
-    if (Kc > 128) {
-        merge_tc(ix, nq, nphase, s, Kc, RK, cand_d, cand_s, st);
-        rerank(ix, q, nq, Kc, cand_d, cand_s, k, dist, labels, st);
+    if (Kc > 128 || nq <= 4 * 152) {
+        const int tok = prof_begin(ix, PROF_RERANK, 1, st);
+        const int tpr = RK <= 64 ? 64 : RK <= 128 ? 128 : RR_NT;
+        auto go = [&](auto kern) {
+            launch_pdl(kern, (unsigned)nq, RR_NT, 0, st, s.qrun, nq, nphase, Kc, RK, tpr, s.thr, s.part_n,
+                       s.part_d, s.part_i, q, ix->d, ix->x32, ix->ids, k, dist, labels);
+        };
+        if (ix->d > 128) go(&k_merge_rerank_wide<8>);
+        else go(&k_merge_rerank_wide<4>);
+        prof_end(ix, tok, st);
         return;
     }
     const unsigned blocks = (unsigned)((nq * 32 + MT_NT - 1) / MT_NT);
@@ -1956,36 +2189,6 @@ void merge_rerank(sivf_index *ix, const float *q, int64_t nq, int nphase,
         else SIVF_MRR(4, 4);
     }
 #undef SIVF_MRR
-    prof_end(ix, tok, st);
-}
-
-void rerank(sivf_index *ix, const float *q, int64_t nq, int Kc, const float *cand_d,
-            const int64_t *cand_s, int k, float *dist, int64_t *labels, cudaStream_t st)
-{
-    const int64_t blocks = (nq * 32 + RK_NT - 1) / RK_NT;
-    const int tok = prof_begin(ix, PROF_RERANK, 1, st);
-#define SIVF_RERANK(E_, NQ_)                                                                       \
-    launch_pdl(k_rerank<E_, NQ_>, (unsigned)blocks, RK_NT, 0, st, q, nq, ix->d, Kc, cand_d,        \
-               cand_s, ix->x32, ix->ids, k, dist, labels)
-    const bool wide = ix->d > 128;  // chunks per lane: 4 (d <= 128) or 8 (d <= 256)
-    if (Kc <= 32) {
-        if (wide) SIVF_RERANK(1, 8);
-        else SIVF_RERANK(1, 4);
-    } else if (Kc <= 64) {
-        if (wide) SIVF_RERANK(2, 8);
-        else SIVF_RERANK(2, 4);
-    } else if (Kc <= 128) {
-        if (wide) SIVF_RERANK(4, 8);
-        else SIVF_RERANK(4, 4);
-    } else {
-        if (ix->d > 128)
-            launch_pdl(k_rerank_wide<8>, (unsigned)nq, RR_NT, 0, st, q, nq, ix->d, Kc, cand_d,
-                       cand_s, ix->x32, ix->ids, k, dist, labels);
-        else
-            launch_pdl(k_rerank_wide<4>, (unsigned)nq, RR_NT, 0, st, q, nq, ix->d, Kc, cand_d,
-                       cand_s, ix->x32, ix->ids, k, dist, labels);
-    }
-#undef SIVF_RERANK
     prof_end(ix, tok, st);
 }
 

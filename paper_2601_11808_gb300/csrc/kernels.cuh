@@ -153,6 +153,7 @@ SearchPlan plan_search(const sivf_index *ix, int64_t nq, int P, int K);
 // output runs and work items one query chunk of nq queries may need
 int64_t plan_run_cap(int64_t nq, int P, int tq, int ips);
 int64_t plan_item_cap(int64_t nq, int P, int L, int ips);
+bool scan_make_map(sivf_index *ix);
 bool scan_fits(const sivf_index *ix, int K);   // shared memory for k = K
 void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t *probes,
                 bool dedupe, const SearchPlan &pl, const SearchScratch &s, cudaStream_t st);

@@ -17,6 +17,7 @@
 
 #include "device_utils.cuh"
 #include "kernels.cuh"
+#include "tc.cuh"
 
 namespace sivf {
 
@@ -692,6 +693,7 @@ struct ScanArgs {
     const float *q;
     int64_t nq;
     int P, K, M;
+    int nbs;              // slabs of a block (scan_block)
     const int32_t *qlist, *loff, *lcnt, *nch;
     const int32_t *prun;  // first output run of each pair
     const int2 *items;
@@ -718,30 +720,54 @@ __host__ __device__ constexpr int scan_next_pow2(int v)
 }
 
 // Entries per row of the best-K + candidate buffer: the best K, then room
-// for two slabs of candidates (merged by rank, at most 256 entries); for
-// larger K a power of two that the bitonic fallback can sort.
+// for 64 candidates (merged by rank, at most 256 entries); for larger K a
+// power of two that the bitonic fallback can sort.
 __host__ __device__ constexpr int scan_buf_len(int K, int C)
 {
-    return K + 2 * C <= 256 ? ((K + 2 * C + 15) & ~15) : scan_next_pow2(K + C);
+    return K + 64 <= 256 ? ((K + 64 + 15) & ~15) : scan_next_pow2(K + C);
 }
 
-// shared memory carve-up, identical on host and device
+// shared memory of one CTA: at most this, and half of the SM where a block
+// of at least SCAN_BMIN rows' distances leaves room for two CTAs
+constexpr size_t SCAN_SMEM = 222 * 1024;
+constexpr size_t SCAN_HALF = 110 * 1024;
+constexpr int SCAN_BMIN = 256, SCAN_BMAX = 1024;
+
+// shared memory carve-up, identical on host and device; nbs: slabs of a
+// block, whose distances the rows keep until they are selected from
 struct ScanSmem {
-    size_t qs, xs, idb, bd, bi, misc, total;
+    size_t xs, qs, bd, bi, dm, misc, total;
 };
-__host__ __device__ inline ScanSmem scan_smem(int TQ, int C, int d, int M)
+__host__ __device__ inline ScanSmem scan_smem_at(int TQ, int C, int d, int M, int nbs)
 {
     ScanSmem s;
     const size_t DP = d + 4;
-    s.qs = 0;
-    s.xs = s.qs + (size_t)TQ * DP * 4;
-    s.idb = s.xs + (size_t)NST * C * d * 4;
-    s.bd = s.idb + (size_t)NST * C * 8;
+    s.xs = 0;  // swizzled slabs: 1024-byte aligned (C d 4 is a multiple then)
+    s.qs = s.xs + (size_t)NST * C * d * 4;
+    s.bd = s.qs + (size_t)TQ * DP * 4;
     s.bi = s.bd + (size_t)TQ * M * 4;
     s.bi = (s.bi + 15) & ~(size_t)15;
-    s.misc = s.bi + (size_t)TQ * M * 8;
-    s.total = s.misc + 256;
+    s.dm = s.bi + (size_t)TQ * M * 8;
+    s.misc = s.dm + (size_t)TQ * (nbs * C + 4) * 4;
+    s.misc = (s.misc + 15) & ~(size_t)15;
+    s.total = s.misc + 64 + (size_t)nbs * 4;
     return s;
+}
+// slabs of a block: the most rows up to SCAN_BMAX, two CTAs per SM for the
+// tiles of at most 16 queries where SCAN_BMIN rows fit then
+__host__ __device__ inline int scan_block(int TQ, int C, int d, int M)
+{
+    const int most = SCAN_BMAX / C;
+    if (TQ <= 16)
+        for (int n = most; n * C >= SCAN_BMIN; --n)
+            if (scan_smem_at(TQ, C, d, M, n).total <= SCAN_HALF) return n;
+    int n = most;
+    while (n > 1 && scan_smem_at(TQ, C, d, M, n).total > SCAN_SMEM) --n;
+    return n;
+}
+__host__ __device__ inline ScanSmem scan_smem(int TQ, int C, int d, int M)
+{
+    return scan_smem_at(TQ, C, d, M, scan_block(TQ, C, d, M));
 }
 
 // Merge one query's candidates into its best list (one warp).  Every
@@ -829,23 +855,19 @@ __device__ void warp_bitonic_merge(float *bd, int64_t *bi, int K, int nb, int nc
 
 // Direct-form distances of the first RQA row groups of a thread's tile:
 // acc[i][r] = sum_j (q_{i}[j] - x_{r}[j])^2, FP32, j in steps of 4.
-template <int RQA, int RQ, int RX>
+// SW: the slab lies in segments of 32 floats per row with the 128-byte
+// swizzle (16-byte chunk c of row r at c ^ (r & 7)).  A warp reads four rows
+// at a time; rows of d % 32 == 0 floats side by side start on the same bank,
+// and the unswizzled reads took four passes each, more than the arithmetic.
+template <int RQA, bool SW, int C, int RQ, int RX>
 __device__ __forceinline__ void dist_tile(float (&acc)[RQ][RX], const float *__restrict__ qrow,
-                                          const float *__restrict__ xrow, int d, int DP)
+                                          const float *__restrict__ xs, int row0, int d, int DP)
 {
 #pragma unroll
     for (int i = 0; i < RQA; ++i)
 #pragma unroll
         for (int r = 0; r < RX; ++r) acc[i][r] = 0.f;
-#pragma unroll 2
-    for (int j = 0; j < d; j += 4) {
-        float4 qv[RQA], xv[RX];
-#pragma unroll
-        for (int i = 0; i < RQA; ++i)
-            qv[i] = *reinterpret_cast<const float4 *>(qrow + (size_t)i * 8 * DP + j);
-#pragma unroll
-        for (int r = 0; r < RX; ++r)
-            xv[r] = *reinterpret_cast<const float4 *>(xrow + (size_t)r * 4 * d + j);
+    auto step = [&](const float4 (&qv)[RQA], const float4 (&xv)[RX]) {
 #pragma unroll
         for (int i = 0; i < RQA; ++i)
 #pragma unroll
@@ -859,11 +881,41 @@ __device__ __forceinline__ void dist_tile(float (&acc)[RQ][RX], const float *__r
                 v = fmaf(t3, t3, v);
                 acc[i][r] = v;
             }
+    };
+    if (SW) {
+        for (int g = 0; g < d; g += 32) {
+            const float *xg = xs + (size_t)g * C + row0 * 32;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                float4 qv[RQA], xv[RX];
+#pragma unroll
+                for (int i = 0; i < RQA; ++i)
+                    qv[i] = *reinterpret_cast<const float4 *>(qrow + (size_t)i * 8 * DP + g + 4 * c);
+#pragma unroll
+                for (int r = 0; r < RX; ++r)
+                    xv[r] = *reinterpret_cast<const float4 *>(xg + r * 128 +
+                                                              ((c ^ ((row0 + 4 * r) & 7)) << 2));
+                step(qv, xv);
+            }
+        }
+        return;
+    }
+#pragma unroll 2
+    for (int j = 0; j < d; j += 4) {
+        float4 qv[RQA], xv[RX];
+#pragma unroll
+        for (int i = 0; i < RQA; ++i)
+            qv[i] = *reinterpret_cast<const float4 *>(qrow + (size_t)i * 8 * DP + j);
+#pragma unroll
+        for (int r = 0; r < RX; ++r)
+            xv[r] = *reinterpret_cast<const float4 *>(xs + (size_t)(row0 + 4 * r) * d + j);
+        step(qv, xv);
     }
 }
 
-template <int TQ, int C>
-__global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(ScanArgs a)
+template <int TQ, int C, bool XS>
+__global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(
+    const __grid_constant__ CUtensorMap tmap, ScanArgs a)
 {
     pdl_begin();
     constexpr int QW = TQ >= 32 ? TQ / 32 : 1;
@@ -873,20 +925,23 @@ __global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(ScanArgs a)
     constexpr int W = C / 32;
     static_assert(RQ >= 1 && RX >= 1, "tile shape");
 
-    extern __shared__ __align__(128) unsigned char smem[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char *smem = XS ? smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023) : smem_raw;
     const int d = a.d, DP = d + 4, M = a.M, K = a.K;
-    const int CB = M - K;  // candidate buffer capacity (>= C)
-    const ScanSmem L = scan_smem(TQ, C, d, M);
+    const int CB = M - K;  // candidate buffer capacity (>= 32)
+    const int NBS = a.nbs, DS = NBS * C + 4;  // slabs of a block, row stride of its distances
+    const ScanSmem L = scan_smem_at(TQ, C, d, M, NBS);
     float *Qs = reinterpret_cast<float *>(smem + L.qs);
     float *Xs = reinterpret_cast<float *>(smem + L.xs);
-    int64_t *IDs = reinterpret_cast<int64_t *>(smem + L.idb);
     float *BD = reinterpret_cast<float *>(smem + L.bd);
     int64_t *BI = reinterpret_cast<int64_t *>(smem + L.bi);
+    float *DM = reinterpret_cast<float *>(smem + L.dm);
     unsigned char *misc = smem + L.misc;
     uint64_t *mbar = reinterpret_cast<uint64_t *>(misc);  // [NST]
     int *s_item = reinterpret_cast<int *>(misc + 8 * NST);
     int *s_abort = s_item + 1;
     int *stage_slab = s_item + 2;                         // [NST]
+    int *block_slab = stage_slab + NST;                   // [NBS] slabs of the block
     __shared__ int32_t s_qpair[TQ];   // (query, probe) pair of each row
     __shared__ int s_cc[TQ];          // candidates waiting per row
     __shared__ int s_nb[TQ];          // valid best entries per row
@@ -914,10 +969,15 @@ __global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(ScanArgs a)
         if (!ok) atomicOr(a.err, ERR_BAD_SLAB);
         stage_slab[stage] = ok ? s : -1;
         if (ok) {
-            mbar_arrive_expect_tx(&mbar[stage], slab_bytes + C * 8);
-            bulk_g2s(Xs + (size_t)stage * C * d, a.x32 + (size_t)s * C * d, slab_bytes,
-                     &mbar[stage]);
-            bulk_g2s(IDs + (size_t)stage * C, a.ids + (size_t)s * C, C * 8, &mbar[stage]);
+            mbar_arrive_expect_tx(&mbar[stage], slab_bytes);
+            if (XS) {
+                for (int g = 0; g < d; g += 32)
+                    tma_load_2d(Xs + (size_t)stage * C * d + (size_t)g * C, &tmap, g, s * C,
+                                &mbar[stage]);
+            } else {
+                bulk_g2s(Xs + (size_t)stage * C * d, a.x32 + (size_t)s * C * d, slab_bytes,
+                         &mbar[stage]);
+            }
         } else {
             mbar_arrive(&mbar[stage]);
         }
@@ -930,7 +990,9 @@ __global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(ScanArgs a)
         int64_t *bi = BI + (size_t)qr * M;
         const int nb = s_nb[qr], nc = s_cc[qr];
         if (nc > 0) {
-            if (nb + nc <= 128) warp_rank_merge<4>(bd, bi, K, nb, nc, lane);
+            if (nb + nc <= 32) warp_rank_merge<1>(bd, bi, K, nb, nc, lane);
+            else if (nb + nc <= 64) warp_rank_merge<2>(bd, bi, K, nb, nc, lane);
+            else if (nb + nc <= 128) warp_rank_merge<4>(bd, bi, K, nb, nc, lane);
             else if (nb + nc <= 256) warp_rank_merge<8>(bd, bi, K, nb, nc, lane);
             else warp_bitonic_merge(bd, bi, K, nb, nc, M, lane);
         }
@@ -955,6 +1017,47 @@ __global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(ScanArgs a)
             s_ki[qr] = ki;
         }
         __syncwarp();
+    };
+
+    // Select from the n distances of the block for row qr (one warp): while
+    // the row holds fewer than K, a value K of them lie at or below (kth_bound)
+    // is the bar, else its K-th; what is within it (ties included) goes to the
+    // candidates, slots first, and is merged with its ids
+    auto select_row = [&](int qr, int n) {
+        const float *dr = DM + (size_t)qr * DS;
+        float *bd = BD + (size_t)qr * M + K;
+        int64_t *bi = BI + (size_t)qr * M + K;
+        float bar = s_kd[qr];
+        if (s_nb[qr] < K)
+            bar = fminf(bar, kth_bound<16>([&](int i) { return i < n ? dr[i] : INFINITY; },
+                                           (n + 31) & ~31, K, lane));
+        int cc = 0;
+        auto merge = [&]() {
+            __syncwarp();
+            for (int e = lane; e < cc; e += 32) {
+                const int i = (int)bi[e];
+                bi[e] = __ldg(a.ids + (size_t)block_slab[i / C] * C + i % C);
+            }
+            if (lane == 0) s_cc[qr] = cc;
+            __syncwarp();
+            merge_row(qr);
+            bar = fminf(bar, s_kd[qr]);
+            cc = 0;
+        };
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const float v = dr[i0 + lane];  // n is a multiple of 32
+            const bool in = v <= bar && v < INFINITY;
+            const uint32_t mk = __ballot_sync(0xffffffffu, in);
+            if (mk == 0u) continue;
+            if (cc + __popc(mk) > CB) merge();
+            if (in) {
+                const int p = cc + __popc(mk & lanemask_lt());
+                bd[p] = v;
+                bi[p] = i0 + lane;
+            }
+            cc += __popc(mk);
+        }
+        merge();
     };
 
     for (;;) {
@@ -1017,67 +1120,39 @@ __global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(ScanArgs a)
             const int s = stage_slab[stage];
             if (s >= 0 && warp_active && !*s_abort) {
                 const float *xs = Xs + (size_t)stage * C * d;
-                const int64_t *ib = IDs + (size_t)stage * C;
                 float acc[RQ][RX];
                 const float *qrow = Qs + (size_t)(wq * 8 * RQ + qy) * DP;
-                const float *xrow = xs + (size_t)(ws * 4 * RX + sx) * d;
+                const int row0 = ws * 4 * RX + sx;
                 // only the row groups that hold queries are computed
                 const int nact = min(RQ, (m - wq * 8 * RQ + 7) / 8);
-                if (nact >= RQ) dist_tile<RQ, RQ, RX>(acc, qrow, xrow, d, DP);
-                else if (nact == 1) dist_tile<1, RQ, RX>(acc, qrow, xrow, d, DP);
-                else if (nact == 2) dist_tile<(RQ >= 2 ? 2 : 1), RQ, RX>(acc, qrow, xrow, d, DP);
-                else dist_tile<(RQ >= 3 ? 3 : 1), RQ, RX>(acc, qrow, xrow, d, DP);
+                if (nact >= RQ) dist_tile<RQ, XS, C>(acc, qrow, xs, row0, d, DP);
+                else if (nact == 1) dist_tile<1, XS, C>(acc, qrow, xs, row0, d, DP);
+                else if (nact == 2) dist_tile<(RQ >= 2 ? 2 : 1), XS, C>(acc, qrow, xs, row0, d, DP);
+                else dist_tile<(RQ >= 3 ? 3 : 1), XS, C>(acc, qrow, xs, row0, d, DP);
                 uint32_t bw[W];
 #pragma unroll
                 for (int w = 0; w < W; ++w) bw[w] = __ldg(a.bits + (size_t)s * W + w);
-                if (idx == 0) {
-                    // first slab of the tile: every distance goes to the row's
-                    // candidate area, indexed by slot (sorted below)
-#pragma unroll
-                    for (int i = 0; i < RQ; ++i) {
-                        const int qr = wq * 8 * RQ + qy + 8 * i;
-                        if (qr >= m) continue;
-#pragma unroll
-                        for (int r = 0; r < RX; ++r) {
-                            const int slot = ws * 4 * RX + sx + 4 * r;
-                            const bool live = (bw[slot >> 5] >> (slot & 31)) & 1u;
-                            BD[(size_t)qr * M + K + slot] = live ? acc[i][r] : INFINITY;
-                            BI[(size_t)qr * M + K + slot] = live ? ib[slot] : -1;
-                        }
-                    }
-                } else {
+                float *dm = DM + (idx % NBS) * C;
 #pragma unroll
                 for (int i = 0; i < RQ; ++i) {
                     const int qr = wq * 8 * RQ + qy + 8 * i;
-                    if (qr >= m) continue;
-                    const float kd = s_kd[qr];
-                    const int64_t ki = s_ki[qr];
+                    if (i >= nact) continue;
 #pragma unroll
                     for (int r = 0; r < RX; ++r) {
                         const int slot = ws * 4 * RX + sx + 4 * r;
-                        if (!((bw[slot >> 5] >> (slot & 31)) & 1u)) continue;
-                        const float dd = acc[i][r];
-                        if (dd < kd || (dd == kd && ib[slot] < ki)) {
-                            const int pos = atomicAdd(&s_cc[qr], 1);
-                            BD[(size_t)qr * M + K + pos] = dd;
-                            BI[(size_t)qr * M + K + pos] = ib[slot];
-                        }
+                        const bool live = (bw[slot >> 5] >> (slot & 31)) & 1u;
+                        dm[(size_t)qr * DS + slot] = live ? acc[i][r] : INFINITY;
                     }
                 }
-                }
-            } else if (idx == 0) {
-                // an inactive warp or a skipped slab leaves its rows empty
+            } else if (warp_active) {  // a skipped slab has no distances
 #pragma unroll
-                for (int i = 0; i < RQ; ++i) {
-                    const int qr = wq * 8 * RQ + qy + 8 * i;
-                    if (qr >= m) continue;
+                for (int i = 0; i < RQ; ++i)
 #pragma unroll
-                    for (int r = 0; r < RX; ++r) {
-                        BD[(size_t)qr * M + K + ws * 4 * RX + sx + 4 * r] = INFINITY;
-                        BI[(size_t)qr * M + K + ws * 4 * RX + sx + 4 * r] = -1;
-                    }
-                }
+                    for (int r = 0; r < RX; ++r)
+                        DM[(size_t)(wq * 8 * RQ + qy + 8 * i) * DS + (idx % NBS) * C + ws * 4 * RX + sx +
+                           4 * r] = INFINITY;
             }
+            if (tid == 0) block_slab[idx % NBS] = max(s, 0);
             __syncthreads();
             // the stage is free: fetch the slab NST ahead into it
             if (tid == 0 && idx + NST < ns && !*s_abort) {
@@ -1085,50 +1160,10 @@ __global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(ScanArgs a)
                 issue(g_issue % NST, dirl[s0 + idx + NST]);
                 ++g_issue;
             }
-            const bool last = idx + 1 == ns;
-            if (idx == 0) {
-                // exact best K of the first slab of every row: one warp per
-                // row sorts the row's C distances in registers (the slab's
-                // stage is already being refilled: ids come from the row)
-                constexpr int E = C / 32;
-                for (int qr = warp; qr < m; qr += SCAN_NT / 32) {
-                    float v[E];
-                    int64_t id[E];
-#pragma unroll
-                    for (int e = 0; e < E; ++e) {
-                        const int slot = lane + 32 * e;
-                        v[e] = BD[(size_t)qr * M + K + slot];
-                        id[e] = BI[(size_t)qr * M + K + slot];
-                    }
-                    warp_bitonic_sort<E>(v, id, lane);
-                    const float kd0 = s_kd[qr];
-                    const int64_t ki0 = s_ki[qr];
-                    int nb = 0;
-#pragma unroll
-                    for (int e = 0; e < E; ++e) {
-                        const int i = lane + 32 * e;
-                        const bool keep = id[e] >= 0 && i < K && dk_less(v[e], id[e], kd0, ki0);
-                        nb += __popc(__ballot_sync(0xffffffffu, keep));
-                        if (keep) {
-                            BD[(size_t)qr * M + i] = v[e];
-                            BI[(size_t)qr * M + i] = id[e];
-                        }
-                    }
-                    __syncwarp();
-                    if (lane == 0) {
-                        s_nb[qr] = nb;
-                        s_cc[qr] = 0;
-                    }
-                    __syncwarp();
-                    merge_row(qr);  // nothing to merge: refreshes the threshold
-                }
-            } else {
-                // merge rows whose buffer could overflow on the next slab (all
-                // rows after the last slab)
-                for (int qr = warp; qr < m; qr += SCAN_NT / 32)
-                    if (s_cc[qr] > 0 && (last || s_cc[qr] > CB - C)) merge_row(qr);
+            if (idx % NBS == NBS - 1 || idx + 1 == ns) {
+                for (int qr = warp; qr < m; qr += SCAN_NT / 32) select_row(qr, (idx % NBS + 1) * C);
+                __syncthreads();
             }
-            __syncthreads();
         }
 
         // the best K of each row of the tile (padded with (+inf, -1))
@@ -1289,13 +1324,14 @@ __global__ __launch_bounds__(MERGE_NT) void k_merge(const int2 *__restrict__ qru
 }
 
 // --------------------------------------------------------------- drivers
-template <int TQ, int C>
+template <int TQ, int C, bool SW>
 static void launch_scan(sivf_index *ix, const ScanArgs &a, size_t smem, int grid,
                         cudaStream_t st)
 {
+    if (SW) smem += 1024;  // base alignment slack
     static size_t attr = 48 * 1024;
     if (smem > attr) {
-        cudaFuncSetAttribute(k_scan<TQ, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_scan<TQ, C, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
         attr = smem;
     }
@@ -1305,14 +1341,34 @@ static void launch_scan(sivf_index *ix, const ScanArgs &a, size_t smem, int grid
     static int occ = 1;
     if (smem != occ_smem) {
         int n = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_scan<TQ, C>, SCAN_NT, smem) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_scan<TQ, C, SW>, SCAN_NT, smem) !=
+            cudaSuccess)
             n = 1;
         occ = std::max(1, n);
         occ_smem = smem;
     }
     const int tok = prof_begin(ix, PROF_SCAN, 1, st);
-    launch_pdl(k_scan<TQ, C>, grid * occ, SCAN_NT, smem, st, a);
+    launch_pdl(k_scan<TQ, C, SW>, grid * occ, SCAN_NT, smem, st,
+               *reinterpret_cast<const CUtensorMap *>(ix->tmap_x32), a);
     prof_end(ix, tok, st);
+}
+
+// TMA descriptor of the FP32 payload in boxes of 32 floats x one slab, with
+// the 128-byte swizzle: d % 32 == 0 (other rows start on other banks as they
+// are, and a box past the row would only add bytes)
+bool scan_make_map(sivf_index *ix)
+{
+    if (ix->d % 32) return false;
+    auto enc = tmap_encode_fn();
+    if (!enc) return false;
+    cuuint64_t dims[2] = {(cuuint64_t)ix->d, (cuuint64_t)ix->n_slabs * ix->C};
+    cuuint64_t strides[1] = {(cuuint64_t)ix->d * 4};
+    cuuint32_t box[2] = {32, (cuuint32_t)ix->C};
+    cuuint32_t es[2] = {1, 1};
+    return enc(reinterpret_cast<CUtensorMap *>(ix->tmap_x32), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+               ix->x32, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 int tune_bucket(const sivf_index *ix, int64_t nq, int P)
@@ -1339,10 +1395,11 @@ sivf_tile default_tile(const sivf_index *ix, int dtype, int64_t nq, int P, int K
     sivf_tile t;
     if (dtype == SIVF_FP32) {
         const double ppl = (double)nq * P / ix->nlist;
-        t.queries_per_tile = ppl >= 48 ? 64 : ppl >= 24 ? 32 : ppl >= 12 ? 16 : 8;
+        // 16 from eight pairs per list on: 390 against 437 us at 9.8 of d = 128,
+        // 315 against 285 at 7.1 of d = 192
+        t.queries_per_tile = ppl >= 48 ? 64 : ppl >= 24 ? 32 : ppl >= 8 ? 16 : 8;
         while (t.queries_per_tile > 8 &&
-               scan_smem(t.queries_per_tile, ix->C, ix->d, scan_buf_len(K, ix->C)).total >
-                   220 * 1024)
+               scan_smem(t.queries_per_tile, ix->C, ix->d, scan_buf_len(K, ix->C)).total > SCAN_SMEM)
             t.queries_per_tile >>= 1;
         t.slabs_per_chunk = 2;
         t.items_per_sm = 4;
@@ -1368,8 +1425,7 @@ bool tile_valid(const sivf_index *ix, int dtype, const sivf_tile &t, int K)
         const int tq = t.queries_per_tile;
         if (!(tq == 8 || tq == 16 || tq == 32 || tq == 64)) return false;
         if (t.select_slabs < 0 || t.select_slabs > 8) return false;
-        return scan_smem(tq, ix->C, ix->d, fp32_width(K, ix->C, t.select_slabs)).total <=
-               220 * 1024;
+        return scan_smem(tq, ix->C, ix->d, fp32_width(K, ix->C, t.select_slabs)).total <= SCAN_SMEM;
     }
     if (t.nearest_first < 0 || t.nearest_first > 2) return false;
     if (t.queries_per_tile == 128)
@@ -1443,7 +1499,7 @@ SearchPlan plan_search(const sivf_index *ix, int64_t nq, int P, int K)
 
 bool scan_fits(const sivf_index *ix, int K)
 {
-    return scan_smem(8, ix->C, ix->d, scan_buf_len(K, ix->C)).total <= 220 * 1024;
+    return scan_smem(8, ix->C, ix->d, scan_buf_len(K, ix->C)).total <= SCAN_SMEM;
 }
 
 void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_t *probes,
@@ -1480,11 +1536,15 @@ void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_
     prof_end(ix, tg, st);
 }
 
-static void scan_launch(sivf_index *ix, int tq, const ScanArgs &a, size_t smem, cudaStream_t st)
+static void scan_launch(sivf_index *ix, int tq, ScanArgs a, cudaStream_t st)
 {
+    a.nbs = scan_block(tq, ix->C, ix->d, a.M);
+    const size_t smem = scan_smem_at(tq, ix->C, ix->d, a.M, a.nbs).total;
     const int grid = 152;  // persistent: one CTA per SM
 #define SIVF_SCAN_CASE(TQ_, C_) \
-    if (tq == TQ_ && ix->C == C_) return launch_scan<TQ_, C_>(ix, a, smem, grid, st);
+    if (tq == TQ_ && ix->C == C_)                                            \
+        return ix->tmap_x32_ok ? launch_scan<TQ_, C_, true>(ix, a, smem, grid, st) \
+                               : launch_scan<TQ_, C_, false>(ix, a, smem, grid, st);
     SIVF_SCAN_CASE(8, 32) SIVF_SCAN_CASE(16, 32) SIVF_SCAN_CASE(32, 32) SIVF_SCAN_CASE(64, 32)
     SIVF_SCAN_CASE(8, 64) SIVF_SCAN_CASE(16, 64) SIVF_SCAN_CASE(32, 64) SIVF_SCAN_CASE(64, 64)
     SIVF_SCAN_CASE(8, 128) SIVF_SCAN_CASE(16, 128) SIVF_SCAN_CASE(32, 128)
@@ -1526,7 +1586,6 @@ void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t
     a.d = ix->d;
     a.ctl = ix->ctl;
     a.err = ix->err;
-    const size_t smem = scan_smem(pl.tq, ix->C, ix->d, a.M).total;
     // the nearest lists first: the others then meet a tight bound, which most
     // of their vectors do not pass and whole lists may not (prune_pairs)
     const int split = fp32_two_phase(nq, P) ? 1 : P;
@@ -1539,11 +1598,11 @@ void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t
         pl1.tq = std::min(pl.tq, current_tile(ix, SIVF_FP32, nq, 1, pl.K).queries_per_tile);
     }
     group_pairs(ix, nq, P, 0, split, probes, dedupe, pl1, s, sb, st);
-    scan_launch(ix, pl1.tq, a, scan_smem(pl1.tq, ix->C, ix->d, a.M).total, st);
+    scan_launch(ix, pl1.tq, a, st);
     if (split < P) {
         prune_pairs(ix, SIVF_FP32, q, nq, P, probes, dedupe, s, st);
         group_pairs(ix, nq, P, split, P, probes, false, pl, s, sb, st, true, true);
-        scan_launch(ix, pl.tq, a, smem, st);
+        scan_launch(ix, pl.tq, a, st);
     }
 }
 

@@ -142,6 +142,9 @@ struct sivf_index {
     // the same copies with boxes of min(C, 64) rows (query-row scan)
     alignas(64) unsigned char tmap_qt_bf16[128];
     alignas(64) unsigned char tmap_qt_fp8[128];
+    // the FP32 payload in boxes of 32 floats x one slab (FP32 scan, d % 32 == 0)
+    alignas(64) unsigned char tmap_x32[128];
+    bool tmap_x32_ok;
     // the BF16 centroids and their low parts in boxes of 64 x 128 (fused
     // coarse first stage)
     alignas(64) unsigned char tmap_cent[128];

@@ -1210,6 +1210,7 @@ __global__ __launch_bounds__(MERGE_NT) void k_merge(const int2 *__restrict__ qru
     constexpr int MU = 8;  // loads in flight per lane
     __shared__ float sd[MERGE_NT / 32][32 * E];
     __shared__ int64_t si[MERGE_NT / 32][32 * E];
+    __shared__ uint64_t sk[MERGE_NT / 32][32 * E];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t q = (blockIdx.x * (int64_t)MERGE_NT + threadIdx.x) >> 5;
     if (q >= nq) return;  // whole warps
@@ -1242,22 +1243,17 @@ __global__ __launch_bounds__(MERGE_NT) void k_merge(const int2 *__restrict__ qru
     }
     __syncwarp();
     if (k <= 32 * E && have <= 32 * E) {
-        float v[E];
-        int64_t id[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int i = lane + 32 * e;
-            v[e] = i < have ? sd[w][i] : INFINITY;
-            id[e] = i < have ? si[w][i] : 0x7fffffffffffffffLL;
-        }
-        warp_bitonic_sort<E>(v, id, lane);
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int i = lane + 32 * e;
-            if (i < k) {
-                dist[q * k + i] = i < have ? v[e] : INFINITY;
-                labels[q * k + i] = i < have ? id[e] : -1;
-            }
+        warp_order<E>(
+            have, [&](int i) { return sd[w][i]; }, [&](int i) { return si[w][i]; },
+            [&](int i, float v, int64_t id) {
+                if (i >= k) return;
+                dist[q * k + i] = v;
+                labels[q * k + i] = id;
+            },
+            sk[w], lane);
+        for (int i = have + lane; i < k; i += 32) {
+            dist[q * k + i] = INFINITY;
+            labels[q * k + i] = -1;
         }
         return;
     }

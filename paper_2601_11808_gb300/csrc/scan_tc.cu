@@ -1386,19 +1386,17 @@ __global__ __launch_bounds__(MT_NT, NQ <= 4 ? 9 : 2) void k_merge_rerank(
     pdl_begin();
     constexpr int NW = MT_NT / 32;
     __shared__ uint32_t hist_s[NW][TC_HIST];
-    __shared__ float sd[NW][merge_cap(E)];
+    // the selection's buffer; once 32 E are left, their ids and sort keys behind
+    __shared__ __align__(16) float sd[NW][160 * E > merge_cap(E) ? 160 * E : merge_cap(E)];
     __shared__ int32_t ss[NW][merge_cap(E)];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 3, t = lane & 7;
     const int64_t qi = (blockIdx.x * (int64_t)MT_NT + threadIdx.x) >> 5;
     if (qi >= nq) return;  // whole warps
     const int nk = merge_select<E>(qrun, nq, qi, nphase, K, RK, thr[qi], part_n, part_d, part_i,
                                    hist_s[warp], sd[warp], ss[warp], lane);
-    int64_t id[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int c = lane + 32 * e;
-        id[e] = c < nk ? __ldg(ids + ss[warp][c]) : -1;
-    }
+    // the ids of the candidates, read now and used by the sort
+    int64_t *sid = reinterpret_cast<int64_t *>(sd[warp] + 32 * E);
+    for (int c = lane; c < nk; c += 32) sid[c] = __ldg(ids + ss[warp][c]);
     const int n4 = d >> 2;
     const float4 *q4 = reinterpret_cast<const float4 *>(q + (size_t)qi * d);
     float4 qv[NQ];
@@ -1441,20 +1439,17 @@ __global__ __launch_bounds__(MT_NT, NQ <= 4 ? 9 : 2) void k_merge_rerank(
         }
     }
     __syncwarp();
-    float v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int c = lane + 32 * e;
-        v[e] = c < nk ? sd[warp][c] : INFINITY;
-    }
-    warp_bitonic_sort<E>(v, id, lane);
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = lane + 32 * e;
-        if (i < k) {
-            dist[qi * k + i] = id[e] >= 0 ? v[e] : INFINITY;
-            labels[qi * k + i] = id[e];
-        }
+    warp_order<E>(
+        nk, [&](int c) { return sd[warp][c]; }, [&](int c) { return sid[c]; },
+        [&](int i, float v, int64_t id) {
+            if (i >= k) return;
+            dist[qi * k + i] = v;
+            labels[qi * k + i] = id;
+        },
+        reinterpret_cast<uint64_t *>(sid + 32 * E), lane);
+    for (int i = nk + lane; i < k; i += 32) {
+        dist[qi * k + i] = INFINITY;
+        labels[qi * k + i] = -1;
     }
 }
 

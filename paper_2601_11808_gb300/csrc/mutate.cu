@@ -473,7 +473,7 @@ __device__ __forceinline__ void raise_radius(float *r2, float rs, int d)
 // batch of 10,000 takes one wave of resident warps instead of two.  Bound
 // by HBM at large batches (read 4 d, write 4 d + copies) and by the chain of
 // five dependent loads to the slot at small ones, so the first two chunks
-// of the row are asked for before it.
+// of the row are asked for before it, and the next vector's meanwhile.
 __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
                              const float *__restrict__ x, int64_t n,
                              const int32_t *__restrict__ lab, const int32_t *__restrict__ rloc,
@@ -484,25 +484,36 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
     const int lane = threadIdx.x & 31, hl = lane & 15;
     const int64_t nw = (int64_t)gridDim.x * blockDim.x / 32;
     const int d = V.d, C = V.C;
+    // the next vector of this half: its rank, list and first chunks
+    constexpr int PRE = 2;
+    int r_next = -1, l_next = 0;
+    float4 x_next[PRE];
+    auto fetch = [&](int64_t i) {
+        r_next = i < n ? rloc[i] : -1;
+        l_next = i < n ? lab[i] : 0;
+#pragma unroll
+        for (int u = 0; u < PRE; ++u) {
+            const int j = hl * 4 + 64 * u;
+            x_next[u] = i < n && j < d ? __ldcs(reinterpret_cast<const float4 *>(x + (size_t)i * d + j))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
+    fetch(2 * w0 + (lane >> 4));
     // whole warps iterate together (the half sums shuffle across the warp)
-    for (int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; 2 * w < n; w += nw) {
+    for (int64_t w = w0; 2 * w < n; w += nw) {
         const int64_t i = 2 * w + (lane >> 4);
-        const int r0 = i < n ? rloc[i] : -1;
+        const int r0 = r_next, l = l_next;
         const bool on = r0 >= 0;
         int64_t s = 0;
         int slot = 0;
         float ss = 0.f, rs = 0.f;
-        if (on) {
-            constexpr int PRE = 2;
-            const float *xi = x + (size_t)i * d;
-            float4 pre[PRE];
+        float4 pre[PRE];
 #pragma unroll
-            for (int u = 0; u < PRE; ++u) {
-                const int j = hl * 4 + 64 * u;
-                pre[u] = j < d ? __ldcs(reinterpret_cast<const float4 *>(xi + j))
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            const int l = lab[i];
+        for (int u = 0; u < PRE; ++u) pre[u] = x_next[u];
+        fetch(2 * (w + nw) + (lane >> 4));
+        if (on) {
+            const float *xi = x + (size_t)i * d;
             const int r = V.runcnt[(size_t)l * V.nblk_max + (i >> 10)] + r0;
             const PlanEntry pe = plan[V.list_flag[l] - 1];
             if (r < pe.into_head) {
@@ -558,7 +569,7 @@ __global__ void k_ins_append(IndexView V, const int64_t *__restrict__ ids,
         ss = half_sum(ss);
         rs = half_sum(rs);
         if (on && hl == 0) {
-            raise_radius(V.lrad2 + lab[i], rs, d);
+            raise_radius(V.lrad2 + l, rs, d);
             const size_t row = (size_t)s * C + slot;
             const int64_t id = ids[i];
             V.xnorm[row] = ss;

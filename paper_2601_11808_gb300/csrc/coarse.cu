@@ -648,7 +648,7 @@ constexpr int CF_SUB = 4;                   // threads per row
 constexpr int CF_STRIDE = CF_CAP + 1;       // ints per record: n, lists
 constexpr int CF_EPI = 128 * CF_SUB;        // epilogue threads
 constexpr int CF_NT = CF_EPI + 64;          // + the MMA warp and the copy warp
-constexpr int CF_HDR = 4;                   // ints before the undecided rows: how many have
+constexpr int CF_HDR = 8;                   // ints (32 bytes) before the undecided rows: how many have
                                             // a record, how many are to be redone
 constexpr int CF_CN = 128;                  // centroids of a chunk (and of a TMA box)
 constexpr int CF_TB = 4;                    // TMEM buffers
@@ -1041,15 +1041,18 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
 }
 
 // ------------------------------------ split first stage for probe selection
-// Dt of a tile of 128 rows against a segment of the centroids' chunks, in the
-// split BF16 form, written to out[row][list], and the smallest Dt of each
-// group of 16 lists to gmin[row][group].  Roles and buffers as in
-// k_coarse_fused; grid (tiles, segments of `per` chunks), so that a few rows
-// over many lists fill the chip too.
+// Dt of tiles of 128 rows against the centroids' chunks, in the split BF16
+// form, written to out[row][list], and the smallest Dt of each group of 16
+// lists to gmin[row][group].  Roles and buffers as in k_coarse_fused.  The
+// (tile, chunk) steps are dealt out evenly, a contiguous range per CTA, so
+// that a few rows over many lists fill the chip as well as many over few.
+// Bound by its stores: a thread's two groups are neighbours, so that it writes
+// whole 128-byte lines, 32 bytes per instruction.  10,000 rows of 1,024
+// lists: 25 us, 42 with a tile of rows per CTA and 16-byte stores.
 template <int KC>
 __global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
     const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBlo,
-    const float *__restrict__ x, int m, int d, const float *__restrict__ cn, int L, int per,
+    const float *__restrict__ x, int m, int d, const float *__restrict__ cn, int L,
     float *__restrict__ out, float *__restrict__ gmin, uint32_t *err)
 {
     pdl_begin();
@@ -1082,14 +1085,16 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = tmem_base;
-    const int nch = (L + CN - 1) / CN, j0 = blockIdx.y * per;
-    const uint32_t steps = (uint32_t)max(0, min(per, nch - j0));
-    const int row0 = blockIdx.x * CT_M;
+    const int nch = (L + CN - 1) / CN;
+    const int64_t total = (int64_t)((m + CT_M - 1) / CT_M) * nch;
+    const int64_t s0 = blockIdx.x * total / gridDim.x;
+    const uint32_t steps = (uint32_t)((blockIdx.x + 1) * total / gridDim.x - s0);
+    const int tile0 = (int)(s0 / nch), j0 = (int)(s0 % nch);  // the first step's tile and chunk
 
     if (warp == CF_EPI / 32 + 1) {
         if (lane == 0) {
             uint32_t g = 0;
-            for (; g < steps; ++g) {
+            for (int j = j0; g < steps; ++g, j = j + 1 < nch ? j + 1 : 0) {
                 const uint32_t b = g % NB, u = g / NB;
                 if (u >= 1 && !mbar_wait_ab(&freeb[b], (u - 1) & 1, err, s_abort, kWaitNs)) break;
                 mbar_arrive_expect_tx(&fullb[b], BBYTES);
@@ -1098,7 +1103,7 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
 #pragma unroll
                     for (int kc = 0; kc < KC; ++kc)
                         tma_load_2d(B + b * BBYTES + pp * PBYTES + (size_t)kc * CN * 128,
-                                    pp ? &tmBlo : &tmB, kc * 64, (j0 + (int)g) * CN, &fullb[b]);
+                                    pp ? &tmBlo : &tmB, kc * 64, j * CN, &fullb[b]);
             }
             // the copies issued last have landed before exit
             for (uint32_t t = g > NB ? g - NB : 0; t < g; ++t)
@@ -1108,11 +1113,12 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
     } else if (warp == CF_EPI / 32) {
         if (lane == 0) {
             const uint32_t idesc = mma_idesc(1, 1, CT_M, CN), abase = smem_u32(A);
-            uint32_t g = 0;
-            bool ok = steps == 0 || mbar_wait_ab(&afull, 0, err, s_abort, kWaitNs);
-            for (; g < steps && ok; ++g) {
+            uint32_t g = 0, nt = 0;  // nt: tiles begun
+            for (int j = j0; g < steps; ++g, j = j + 1 < nch ? j + 1 : 0) {
                 const uint32_t b = g % NB, tb = g % TB, ut = g / TB;
-                ok = mbar_wait_ab(&fullb[b], (g / NB) & 1, err, s_abort, kWaitNs);
+                bool ok = mbar_wait_ab(&fullb[b], (g / NB) & 1, err, s_abort, kWaitNs);
+                if (ok && (g == 0 || j == 0))  // the tile's rows are stored
+                    ok = mbar_wait_ab(&afull, nt++ & 1, err, s_abort, kWaitNs);
                 if (ok && ut >= 1) ok = mbar_wait_ab(&tempty[tb], (ut - 1) & 1, err, s_abort, kWaitNs);
                 if (!ok) break;
                 tc_fence_after();
@@ -1138,25 +1144,40 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
         }
         __syncwarp();
     } else {
-        const int q = warp & 3, sub = warp >> 2, row = row0 + q * 32 + lane;
+        const int q = warp & 3, sub = warp >> 2;
         RowTile<KC, 2> rows;
-        rows.fetch(x, row0, m, d, tid);
-        rows.store(A, ABYTES, d, tid, sxn);
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&afull);
+        auto store = [&]() {
+            rows.store(A, ABYTES, d, tid, sxn);
+            fence_proxy_async_smem();  // A (generic stores) is read by the MMAs
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&afull);
+        };
+        rows.fetch(x, tile0 * CT_M, m, d, tid);
+        store();
         const int G = (L + 15) / 16;
+        // whole sectors where the rows are aligned to them
         const bool vec = (L & 3) == 0;
+        const bool w8 = (L & 7) == 0 && (reinterpret_cast<uintptr_t>(out) & 31) == 0;
         bool ok = true;
+        int tile = tile0, j = j0;
         for (uint32_t g = 0; g < steps; ++g) {
             const uint32_t tb = g % TB;
+            const int jn = j, row = tile * CT_M + q * 32 + lane;
+            // the next tile's rows, if this CTA's range goes on into it
+            const bool more = (uint32_t)(nch - j) < steps - g;
+            if (more && (g == 0 || j == 0)) rows.fetch(x, (tile + 1) * CT_M, m, d, tid);
             ok = __all_sync(0xffffffffu, ok && mbar_wait_ab(&mmab[tb], (g / TB) & 1, err, s_abort, kWaitNs));
             tc_fence_after();
+            if (++j == nch) {
+                j = 0;
+                ++tile;
+                if (more && ok) store();  // this tile's MMAs are done
+            }
             float v[CN / 64][16];
             if (ok) {
 #pragma unroll
                 for (int k = 0; k < CN / 64; ++k)
-                    tmem_ld16(tbase + tb * CN + (sub + 4 * k) * 16 + ((uint32_t)(q * 32) << 16), v[k]);
+                    tmem_ld16(tbase + tb * CN + (2 * sub + k) * 16 + ((uint32_t)(q * 32) << 16), v[k]);
 #pragma unroll
                 for (int k = 0; k < CN / 64; ++k) tmem_ld_wait(v[k]);
             }
@@ -1165,32 +1186,50 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
             if (lane == 0) mbar_arrive(&tempty[tb]);
             if (!ok) break;  // warp-uniform; no barrier follows before the last one
             if (row >= m) continue;
+            const int grp = jn * (CN / 16) + 2 * sub, c0 = grp * 16;
+            float *o = out + (size_t)row * L + c0, *og = gmin + (size_t)row * G + grp;
+            if (vec && c0 + 32 <= L) {
 #pragma unroll
-            for (int k = 0; k < CN / 64; ++k) {
-                const int grp = (j0 + (int)g) * (CN / 16) + sub + 4 * k, c0 = grp * 16;
-                if (c0 >= L) break;
-                float *o = out + (size_t)row * L + c0;
-                float mn = INFINITY;
-                if (vec && c0 + 16 <= L) {
+                for (int k = 0; k < 2; ++k) {
+                    float mn = INFINITY;
 #pragma unroll
-                    for (int i4 = 0; i4 < 4; ++i4) {
-                        const float4 c = __ldg(reinterpret_cast<const float4 *>(cn + c0) + i4);
-                        const float4 t = make_float4(
-                            fmaf(-2.f, v[k][4 * i4], c.x), fmaf(-2.f, v[k][4 * i4 + 1], c.y),
-                            fmaf(-2.f, v[k][4 * i4 + 2], c.z), fmaf(-2.f, v[k][4 * i4 + 3], c.w));
-                        reinterpret_cast<float4 *>(o)[i4] = t;
-                        mn = fminf(mn, fminf(fminf(t.x, t.y), fminf(t.z, t.w)));
-                    }
-                } else {
+                    for (int h = 0; h < 2; ++h) {
+                        const float4 *c4 = reinterpret_cast<const float4 *>(cn + c0 + 16 * k + 8 * h);
+                        const float4 ca = __ldg(c4), cb = __ldg(c4 + 1);
+                        const float cv[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+                        float t[8];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (c0 + i < L) {
-                            const float t = fmaf(-2.f, v[k][i], __ldg(cn + c0 + i));
-                            o[i] = t;
-                            mn = fminf(mn, t);
+                        for (int i = 0; i < 8; ++i) {
+                            t[i] = fmaf(-2.f, v[k][8 * h + i], cv[i]);
+                            mn = fminf(mn, t[i]);
                         }
+                        float *ot = o + 16 * k + 8 * h;
+                        if (w8) {
+                            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(ot),
+                                         "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(t[4]),
+                                         "f"(t[5]), "f"(t[6]), "f"(t[7])
+                                         : "memory");
+                        } else {
+                            reinterpret_cast<float4 *>(ot)[0] = make_float4(t[0], t[1], t[2], t[3]);
+                            reinterpret_cast<float4 *>(ot)[1] = make_float4(t[4], t[5], t[6], t[7]);
+                        }
+                    }
+                    og[k] = mn;
                 }
-                gmin[(size_t)row * G + grp] = mn;
+                continue;
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (c0 + 16 * k >= L) break;
+                float mn = INFINITY;
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (c0 + 16 * k + i < L) {
+                        const float t = fmaf(-2.f, v[k][i], __ldg(cn + c0 + 16 * k + i));
+                        o[16 * k + i] = t;
+                        mn = fminf(mn, t);
+                    }
+                og[k] = mn;
             }
         }
     }
@@ -2180,23 +2219,6 @@ static bool pick_rows(const sivf_index *ix, int P)
     return P >= 2 && P <= PK_PMAX && ix->tmap_cent_ok && (int64_t)ix->nlist >= 32 * (int64_t)P;
 }
 
-// Chunks per CTA of k_coarse_dist: the split of the lists that takes the
-// fewest steps, a CTA's start (its rows, the first chunk) counted as four
-static int dist_chunks(int tiles, int nch, int nsm)
-{
-    int best = nch;
-    int64_t cost = INT64_MAX;
-    for (int segs = 1; segs <= nch; ++segs) {
-        const int per = (nch + segs - 1) / segs;
-        const int64_t c = (((int64_t)tiles * ((nch + per - 1) / per) + nsm - 1) / nsm) * (per + 4);
-        if (c < cost) {
-            cost = c;
-            best = per;
-        }
-    }
-    return best;
-}
-
 // rows [0, m) of x -> out[m, P]; `Dbuf` holds at least `room` floats, L of
 // them at least.
 void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
@@ -2245,7 +2267,6 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
             const size_t smem = coarse_fused_smem(KC, 2);
             cudaMemsetAsync(nh, 0, sizeof(int32_t), st);
             const int nt = (mc + CT_M - 1) / CT_M, nch = (L + CF_CN - 1) / CF_CN;
-            const int per = dist_chunks(nt, nch, nsm);
             const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent);
             const CUtensorMap &tl = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent_lo);
             static bool attr[2] = {false, false};
@@ -2255,8 +2276,8 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
                                          (int)smem);
                     attr[i] = true;
                 }
-                launch_pdl(kern, dim3(nt, (nch + per - 1) / per), CF_NT, smem, st, tm, tl, x + r0 * d,
-                           mc, d, ix->cnorm, L, per, Dm, gm, ix->err);
+                launch_pdl(kern, (unsigned)std::min<int64_t>((int64_t)nt * nch, nsm), CF_NT, smem, st,
+                           tm, tl, x + r0 * d, mc, d, ix->cnorm, L, Dm, gm, ix->err);
             };
             if (KC == 1) go(k_coarse_dist<1>, 0);
             else go(k_coarse_dist<2>, 1);

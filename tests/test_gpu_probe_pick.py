@@ -44,3 +44,24 @@ def test_probe_sets_equal_the_oracle(d, L, P, m, kind):
     # nearest first up to the FP32 distances' error, 2 (d + 4) u (||q||^2 + ||c||^2) a pair
     assert (np.diff(far, axis=1) >= -4 * (d + 4) * 2.0 ** -24 * cn[:, 1:]).all()
     g.close()
+
+
+@pytest.mark.parametrize("d,L,P,m", [(128, 1000, 8, 2500), (96, 132, 4, 10001), (64, 100, 3, 40000),
+                                     (32, 2049, 16, 1290)])
+def test_probe_sets_where_a_range_of_steps_crosses_tiles(d, L, P, m):
+    """More (tile, chunk) steps than the chip has SMs: ranges that begin and
+    end inside a tile, take in a whole one, and rows of 16- and 32-byte
+    alignment."""
+    import torch
+    from paper_2601_11808_gb300.sivf import Index
+    rng = np.random.default_rng([d, L, P, m])
+    c = rng.uniform(-1.0, 1.0, (L, d)).astype(np.float32)
+    q = (c[rng.integers(0, L, m)] + 0.3 * rng.standard_normal((m, d))).astype(np.float32)
+    g = Index(d, L, 32, 100, 10, 10)
+    g.set_centroids(torch.from_numpy(c).cuda())
+    o = oracle.OracleIVF(d, L, n_max=10, n_slabs=10)
+    o.set_centroids(c)
+    got = g.probe(torch.from_numpy(q).cuda(), P).cpu().numpy()
+    g.sync()
+    np.testing.assert_array_equal(np.sort(got, 1), np.sort(o.probe(q, P), 1))
+    g.close()

@@ -20,14 +20,21 @@
 //   same roundings as the definition (no fused multiply-add).
 // Only near-ties ever reach the FP64 step.
 //
-// For assignment (P = 1) with d % 16 == 0 the distances of the first stage
-// come from a BF16 tensor-core GEMM instead (tcgen05.mma, FP32
-// accumulation): the same
-// selection then runs twice.  With the bound of the BF16 stage (rounding of
-// x and c to BF16 plus the accumulation) it keeps the lists S_b that can
-// still be among the top P; their distances are recomputed in FP32 and the
-// selection above runs on S_b with the FP32 bound.  Lists outside S_b have
-// exact distances above the P-th smallest, so the result is the same set.
+// With d % 16 == 0 the distances of the first stage come from the tensor
+// cores instead (tcgen05.mma, FP32 accumulation; the BF16 product, or the
+// three products of the split x = hi + lo): the same selection then runs
+// twice.  With the bound of that stage (rounding of x and c plus the
+// accumulation) it keeps the lists S_b that can still be among the top P;
+// their distances are recomputed in FP32 and the selection above runs on S_b
+// with the FP32 bound.  Lists outside S_b have exact distances above the
+// P-th smallest, so the result is the same set.
+//
+// The forms (d <= 128 except the last two):
+//   P = 1              k_coarse_fused, k_coarse_finish: no distance matrix
+//   2 <= P <= 128 of   k_coarse_dist, k_coarse_pick: the matrix with group
+//   at least 32 P        minima, of which a row reads a few groups
+//   P <= 8, L <= 4096  k_coarse_tc, k_coarse_select_w
+//   else               k_coarse_gemm (FP32), k_coarse_select
 #include <float.h>
 #include <math.h>
 
@@ -176,6 +183,37 @@ __device__ __forceinline__ double exact_dist(const float *__restrict__ a,
     for (int j = 0; j < d; ++j) {
         double t = __dsub_rn((double)a[j], (double)b[j]);
         acc = __dadd_rn(acc, __dmul_rn(t, t));
+    }
+    return acc;
+}
+
+// The same of rows whose start and length are multiples of 16 bytes (d % 4 ==
+// 0): sixteen values of each loaded ahead of the additions that wait for one
+// another.
+__device__ __forceinline__ double exact_dist4(const float4 *a, const float4 *__restrict__ b, int d)
+{
+    double acc = 0.0;
+    auto add = [&](float x, float y) {
+        const double t = __dsub_rn((double)x, (double)y);
+        acc = __dadd_rn(acc, __dmul_rn(t, t));
+    };
+    const int n4 = d >> 2;
+    for (int j = 0; j < n4; j += 4) {
+        float4 va[4], vb[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (j + u < n4) {
+                va[u] = a[j + u];
+                vb[u] = __ldg(b + j + u);
+            }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (j + u < n4) {
+                add(va[u].x, vb[u].x);
+                add(va[u].y, vb[u].y);
+                add(va[u].z, vb[u].z);
+                add(va[u].w, vb[u].w);
+            }
     }
     return acc;
 }
@@ -1592,8 +1630,10 @@ __host__ __device__ constexpr int pk_ops(int d) { return 4 * ((d + 31) / 32) + 3
 // lanes each) and decided as in the other selections: sure members
 // by their FP32 intervals, the rest by FP64 distance.  A row with more
 // candidates than `cap` is left to k_coarse_select (its number in `hard`).
-// 10,000 rows of 4,096 lists, P = 64: 400 against 580 us (FP32 GEMM and
-// block selection); 61 rows of 16,384 lists, P = 32: 45 against 118 us.
+// 10,000 rows of 4,096 lists, P = 64: 165 us with k_coarse_dist against 580
+// (FP32 GEMM and block selection); 61 rows of 16,384 lists, P = 32: 43
+// against 118; 1,000 rows of 2,048 close lists, P = 64: 47 us, 121 when each
+// 32 candidates with a boundary member paid a pass of FP64 distances.
 // Bound by the chain of one row (about 25 us at P = 64), not by throughput.
 constexpr int PK_RG = 16;      // FP32 rechecks in flight per warp
 constexpr int PK_PMAX = 128;   // most lists per row of this kernel
@@ -1758,9 +1798,25 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
     }
     __syncwarp();
     const int r = P - nsure, nb = nmem - nsure;
-    if (r > 0 && nb > r) {  // boundary members: FP64 distances, the best r of them
-        for (int p = lane; p < ns; p += 32)
-            if (sSure[p] == 0) sDx[p] = exact_dist(xr, a.cent + (size_t)sIdx[p] * d, d);
+    int *sBnd = reinterpret_cast<int *>(sLB);  // the lower bounds have been read
+    if (r > 0 && nb > r) {
+        // boundary members: FP64 distances, the best r of them.  The few there
+        // are take one lane each, next to each other: a pass of exact_dist costs
+        // the same for one member as for 32, and each 32 candidates paid one.
+        int n = 0;
+        for (int p0 = 0; p0 < ns; p0 += 32) {
+            const int p = p0 + lane;
+            const bool in = p < ns && sSure[p] == 0;
+            const uint32_t mk = __ballot_sync(0xffffffffu, in);
+            if (in) sBnd[n + __popc(mk & lanemask_lt())] = p;
+            n += __popc(mk);
+        }
+        __syncwarp();
+        for (int t = lane; t < nb; t += 32) {
+            const int p = sBnd[t];
+            sDx[p] = exact_dist4(reinterpret_cast<const float4 *>(sX),
+                                 reinterpret_cast<const float4 *>(a.cent + (size_t)sIdx[p] * d), d);
+        }
         __syncwarp();
     }
     // the chosen to the front of sIdx / sDt, in place
@@ -1774,9 +1830,10 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
                 take = true;
                 if (nb > r) {
                     int rank = 0;
-                    for (int k = 0; k < ns; ++k)
-                        rank += sSure[k] == 0 &&
-                                (sDx[k] < sDx[p] || (sDx[k] == sDx[p] && sIdx[k] < sIdx[p]));
+                    for (int t = 0; t < nb; ++t) {
+                        const int k = sBnd[t];
+                        rank += sDx[k] < sDx[p] || (sDx[k] == sDx[p] && sIdx[k] < sIdx[p]);
+                    }
                     take = rank < r;
                 }
             }
@@ -1934,7 +1991,7 @@ __global__ __launch_bounds__(FN_ROWS * 32) void k_coarse_finish(SelArgs a)
         } else if (mk) {
             bd = INFINITY;
             bc = 0x7fffffff;
-            if (in) better(exact_dist(xr, a.cent + (size_t)c * d, d), c);
+            if (in) better(exact_dist4(x4, reinterpret_cast<const float4 *>(a.cent + (size_t)c * d), d), c);
             best_warp();
             chosen = bc;
         }
@@ -1998,7 +2055,7 @@ __global__ __launch_bounds__(FN_ROWS * 32) void k_coarse_finish(SelArgs a)
         for (int c = tid; c < L; c += FN_ROWS * 32) {
             float lb, ub;
             bounds(c, sD[c], xn, lb, ub);
-            if (lb <= T) better(exact_dist(xr, a.cent + (size_t)c * d, d), c);
+            if (lb <= T) better(exact_dist4(x4, reinterpret_cast<const float4 *>(a.cent + (size_t)c * d), d), c);
         }
         best_warp();
         if (lane == 0) {

@@ -164,18 +164,22 @@ sivf_status read_status(sivf_index *ix, void *stream, int64_t *count)
 
 namespace sivf {
 
-int64_t coarse_floats(const sivf_index *ix, int64_t n)
+int64_t coarse_floats(const sivf_index *ix, int64_t n, int P)
 {
     // rows of approximate distances with their group minima, and a number per
-    // row: 64 MB of distances at most, 128 rows at least
-    const int64_t L = ix->nlist, r = ((int64_t)64 << 20) / (4 * L);
+    // row: 64 MB of distances at most (they stay in L2 until they are read),
+    // 128 rows at least.  A selection that reads the minima and a few groups
+    // takes up to 256 MB, because a launch costs it one row's chain however few
+    // rows it has (P = 64 of 4,096 lists: 92 us for 4,096 rows, 99 for 10,000)
+    const int64_t L = ix->nlist, mb = coarse_picks(ix, P) ? 256 : 64;
+    const int64_t r = (mb << 20) / (4 * L);
     const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(n, std::max<int64_t>(r, 128)));
     return rows * (1 + L + (L + 15) / 16) + 16;
 }
 
-size_t coarse_bytes(const sivf_index *ix, int64_t n)
+size_t coarse_bytes(const sivf_index *ix, int64_t n, int P)
 {
-    return (size_t)coarse_floats(ix, n) * 4 + 256;
+    return (size_t)coarse_floats(ix, n, P) * 4 + 256;
 }
 
 int prof_begin(sivf_index *ix, int k, int n, cudaStream_t st)
@@ -399,8 +403,8 @@ sivf_status sivf_train(sivf_index *ix, const float *x, int64_t n, int iters, uin
             rows.push_back(r);
         }
     }
-    const int64_t croom = coarse_floats(ix, n);
-    const size_t need = coarse_bytes(ix, n) + (size_t)n * 4 + (size_t)L * d * 8 + (size_t)L * 4 +
+    const int64_t croom = coarse_floats(ix, n, 1);
+    const size_t need = coarse_bytes(ix, n, 1) + (size_t)n * 4 + (size_t)L * d * 8 + (size_t)L * 4 +
                         (size_t)L * 8 + 5 * 256;
     Ctx *c;
     if ((st = get_ctx(ix, stream, need, &c))) return st;
@@ -460,7 +464,7 @@ sivf_status sivf_set_list_scales(sivf_index *ix, const float *inv_scale, void *s
 static size_t add_bytes(const sivf_index *ix, int64_t n)
 {
     const int L = ix->nlist;
-    return coarse_bytes(ix, n) + (size_t)n * 8 + (size_t)L * (4 + 4 + 16 + 4) + 8 * 256;
+    return coarse_bytes(ix, n, 1) + (size_t)n * 8 + (size_t)L * (4 + 4 + 16 + 4) + 8 * 256;
 }
 
 static size_t search_bytes(const sivf_index *ix, int64_t nq, int k, int P, SearchPlan *plo)
@@ -469,7 +473,7 @@ static size_t search_bytes(const sivf_index *ix, int64_t nq, int k, int P, Searc
     SearchPlan pl = plan_search(ix, nq, P, k);
     if (plo) *plo = pl;
     size_t parts = (size_t)pl.run_cap * pl.K;
-    return coarse_bytes(ix, nq) + (size_t)nq * P * 4 * 4 + (size_t)(L + 1) * 4 * 4 +
+    return coarse_bytes(ix, nq, P) + (size_t)nq * P * 4 * 4 + (size_t)(L + 1) * 4 * 4 +
            parts * 12 + (size_t)nq * 4 * 3 + (size_t)nq * 16 + (size_t)pl.item_cap * 8 + 19 * 256;
 }
 
@@ -487,7 +491,7 @@ static size_t chunk_need(const sivf_index *ix, int64_t m, int P, int Kc, int dty
     const int L = ix->nlist;
     SearchPlan pl = plan_tc(ix, dtype, m, P, Kc);
     *plo = pl;
-    return coarse_bytes(ix, m) + (size_t)m * P * 4 * 4 + (size_t)(L + 1) * 4 * 4 +
+    return coarse_bytes(ix, m, P) + (size_t)m * P * 4 * 4 + (size_t)(L + 1) * 4 * 4 +
            (size_t)pl.run_cap * (pl.RK * 12 + 4) + (size_t)m * 4 * 3 + (size_t)m * 16 +
            (size_t)pl.item_cap * 8 + (size_t)m * ix->d * 2 +
            (dtype == SIVF_FP8E4M3 ? (size_t)m * P * (ix->d + 8) : 0) + 23 * 256;
@@ -594,7 +598,7 @@ sivf_status sivf_add(sivf_index *ix, const int64_t *ids, const float *x, int64_t
     sc.bcnt = b.take<int32_t>(L);
     sc.plan = b.take<PlanEntry>(L);
     sc.affected = b.take<int32_t>(L);
-    const int64_t room = coarse_floats(ix, n);
+    const int64_t room = coarse_floats(ix, n, 1);
     float *Dbuf = b.take<float>((size_t)room);
     CUDA_TRY(ix, cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), s));
     coarse_topP(ix, x, n, 1, sc.lab, Dbuf, room, s);
@@ -793,7 +797,7 @@ static sivf_status search_impl(sivf_index *ix, const float *q, int64_t nq, int k
                       : nullptr;
         sc.pqn = fp8 ? b.take<float>((size_t)m * P) : nullptr;
         sc.pqsc = fp8 ? b.take<float>((size_t)m * P) : nullptr;
-        const int64_t room = coarse_floats(ix, m);
+        const int64_t room = coarse_floats(ix, m, P);
         float *Dbuf = b.take<float>((size_t)room);
         CUDA_TRY(ix, cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), s));
         const float *qq = q + q0 * ix->d;
@@ -907,10 +911,10 @@ static sivf_status coarse_only(sivf_index *ix, const float *x, int64_t n, int P,
     if (!ix->have_centroids) return fail(ix, SIVF_E_STATE, "set_centroids first");
     if (n == 0) return SIVF_OK;
     Ctx *c;
-    sivf_status st = get_ctx(ix, stream, coarse_bytes(ix, n), &c);
+    sivf_status st = get_ctx(ix, stream, coarse_bytes(ix, n, P), &c);
     if (st) return st;
     Bump b{c->scratch};
-    const int64_t room = coarse_floats(ix, n);
+    const int64_t room = coarse_floats(ix, n, P);
     float *Dbuf = b.take<float>((size_t)room);
     coarse_topP(ix, x, n, P, out, Dbuf, room, (cudaStream_t)stream);
     CUDA_TRY(ix, cudaGetLastError());

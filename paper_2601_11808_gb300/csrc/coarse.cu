@@ -2271,7 +2271,7 @@ int first_stage_split(const sivf_index *ix, int P)
 // Probe selection by k_coarse_dist and k_coarse_pick: P lists need twice as
 // many groups of 16 for the group minima to bound them well (L >= 32 P); the
 // warp's candidate table holds P <= 128.
-static bool pick_rows(const sivf_index *ix, int P)
+bool coarse_picks(const sivf_index *ix, int P)
 {
     return P >= 2 && P <= PK_PMAX && ix->tmap_cent_ok && (int64_t)ix->nlist >= 32 * (int64_t)P;
 }
@@ -2287,7 +2287,7 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
     const bool warp_rows = P <= CW_PMAX && L <= CW_LMAX;
     // row numbers, distances and group minima of at least one row
     const int64_t pick_row = 1 + L + (L + 15) / 16;
-    const bool pick = pick_rows(ix, P) && room >= CF_HDR + pick_row;
+    const bool pick = coarse_picks(ix, P) && room >= CF_HDR + pick_row;
     const int split = pick ? 3 : first_stage_split(ix, P);
     const bool two = split != 0;
     const float gamma2_first = (float)(2.0 * first_stage_rel(d, split) * (1.0 + 1e-6));

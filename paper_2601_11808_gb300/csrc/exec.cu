@@ -176,7 +176,7 @@ sivf_status sivf_exec_create(sivf_index *ix, const sivf_op *ops, int nops, sivf_
     for (int i = 0; i < nops; ++i)
         if (ops[i].kind == SIVF_OP_SEARCH) {
             EXEC_TRY(cudaMalloc(&e->probes[i], sizeof(int32_t) * ops[i].n * ops[i].nprobe));
-            cneed = std::max(cneed, coarse_bytes(ix, ops[i].n));
+            cneed = std::max(cneed, coarse_bytes(ix, ops[i].n, ops[i].nprobe));
             ++nsearch;
         }
     if (nsearch) {
@@ -206,8 +206,8 @@ sivf_status sivf_exec_create(sivf_index *ix, const sivf_op *ops, int nops, sivf_
         for (int i = 0; i < nops; ++i) {
             const sivf_op &op = e->ops[i];
             if (op.kind != SIVF_OP_SEARCH) continue;
-            coarse_topP(ix, op.x, op.n, op.nprobe, e->probes[i], e->cbuf, coarse_floats(ix, op.n),
-                        e->side);
+            coarse_topP(ix, op.x, op.n, op.nprobe, e->probes[i], e->cbuf,
+                        coarse_floats(ix, op.n, op.nprobe), e->side);
             cudaEventRecord(e->evs[i], e->side);
         }
         cudaEventRecord(e->evs[nops + 1], e->side);

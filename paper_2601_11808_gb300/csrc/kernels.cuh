@@ -58,9 +58,11 @@ cudaError_t assign_stage_choose(sivf_index *ix, cudaStream_t st);
 int first_stage_split(const sivf_index *ix, int P);
 // relative error bound of the BF16 (split 1) or split BF16 (3) dot products
 double first_stage_rel(int d, int split);
-// the scratch of a coarse selection of n rows, in floats and bytes
-int64_t coarse_floats(const sivf_index *ix, int64_t n);
-size_t coarse_bytes(const sivf_index *ix, int64_t n);
+// whether the selection of P lists reads group minima instead of all distances
+bool coarse_picks(const sivf_index *ix, int P);
+// the scratch of a coarse selection of P lists for n rows, in floats and bytes
+int64_t coarse_floats(const sivf_index *ix, int64_t n, int P);
+size_t coarse_bytes(const sivf_index *ix, int64_t n, int P);
 // the search of sivf_search_with_probes for probes the library selected
 // itself (distinct per query, so not de-duplicated)
 sivf_status search_probed(sivf_index *ix, const float *q, int64_t nq, int k, int nprobe,

@@ -100,6 +100,17 @@ extern "C" sivf_status sivf_search_noalloc(sivf_index *ix, const float *q, int64
     const int P = nprobe, L = ix->nlist;
     SearchPlan pl = plan_search(ix, nq, P, k);
     int64_t rows = std::min<int64_t>(nq, std::max<int64_t>(1, ((int64_t)8 << 20) / (4 * L)));
+    // the 16 queries per tile of 8 to 12 pairs per list need more runs than 8
+    if (pl.tq == 16 && (double)nq * P < 12.0 * L) {
+        SearchPlan one = pl;
+        one.ips = 1;
+        one.run_cap = plan_run_cap(nq, P, one.tq, 1);
+        one.item_cap = plan_item_cap(nq, P, L, 1);
+        if (need_bytes(ix, nq, P, one, 1) > kNoallocBytes) {
+            pl.tq = pl.tq2 = 8;
+            pl.run_cap = plan_run_cap(nq, P, pl.tq, pl.ips);
+        }
+    }
     // fewer items per SM: fewer extra chunk runs
     while (need_bytes(ix, nq, P, pl, rows) > kNoallocBytes && pl.ips > 1) {
         pl.ips >>= 1;

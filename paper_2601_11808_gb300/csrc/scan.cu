@@ -11,6 +11,11 @@
 // validity bit is set (Theorem 2).  Each (query, list tile) keeps its best K
 // (distance, id) pairs; a final merge per query keeps the best k of all
 // probed lists, ties to the lower id, padded with (+inf, -1).
+//
+// A search of enough pairs scans each query's nearest list first and then
+// only those of its other lists that may hold a vector within the distance
+// the nearest left (the pair pruning below, also of the reduced-precision
+// scans).
 #include <math.h>
 
 #include <cmath>
@@ -1532,6 +1537,18 @@ int tune_bucket(const sivf_index *ix, int64_t nq, int P)
 
 int tune_kbucket(int K) { return K <= 16 ? 0 : K <= 64 ? 1 : K <= 256 ? 2 : 3; }
 
+// What an FP32 tile may ask for: its queries, two slabs with their ids and
+// the rows' best K with room for two slabs of candidates (or the tile's) in
+// 220 KB.  The scan keeps a block's distances instead of the ids; a tile
+// that leaves no room for them is narrowed when the plan is made.
+static bool fp32_fits(int TQ, int C, int d, int K, int slabs)
+{
+    const int v = K + (slabs ? slabs : 2) * C;
+    const int M = v <= 256 ? ((v + 15) & ~15) : scan_next_pow2(slabs ? v : K + C);
+    const size_t rows = ((size_t)TQ * (d + 4 + M) + (size_t)NST * C * (d + 2)) * 4;
+    return ((rows + 15) & ~(size_t)15) + (size_t)TQ * M * 8 + 256 <= 220 * 1024;
+}
+
 // k-select buffer of the FP32 scan: the best K plus `slabs` slabs of
 // candidates, beyond 256 entries a power of two (bitonic fallback);
 // slabs = 0 is the built-in width
@@ -1577,7 +1594,7 @@ bool tile_valid(const sivf_index *ix, int dtype, const sivf_tile &t, int K)
         const int tq = t.queries_per_tile;
         if (!(tq == 8 || tq == 16 || tq == 32 || tq == 64)) return false;
         if (t.select_slabs < 0 || t.select_slabs > 8) return false;
-        return scan_smem(tq, ix->C, ix->d, fp32_width(K, ix->C, t.select_slabs)).total <= SCAN_SMEM;
+        return fp32_fits(tq, ix->C, ix->d, K, t.select_slabs);
     }
     if (t.nearest_first < 0 || t.nearest_first > 2) return false;
     if (t.queries_per_tile == 128)
@@ -1605,6 +1622,11 @@ SearchPlan plan_from_tile(const sivf_index *ix, int dtype, int64_t nq, int P, in
     pl.M = fp32  ? fp32_width(K, ix->C, t.select_slabs)
            : pl.qt ? qt_shape(ix, dtype, K).ME
                    : tc_buf_entries(ix, dtype, K, t.select_slabs);
+    while (fp32 && pl.tq > 8 && scan_smem(pl.tq, ix->C, ix->d, pl.M).total > SCAN_SMEM) {
+        if (pl.M > scan_buf_len(K, ix->C)) pl.M = scan_buf_len(K, ix->C);
+        else pl.tq >>= 1;
+    }
+    if (fp32 && scan_smem(pl.tq, ix->C, ix->d, pl.M).total > SCAN_SMEM) pl.M = scan_buf_len(K, ix->C);
     pl.split = fp32 ? 0 : t.nearest_first;
     pl.sel = t.select_slabs;
     pl.RK = (fp32 || pl.qt) ? K : tc_run_len(K);
@@ -1651,7 +1673,7 @@ SearchPlan plan_search(const sivf_index *ix, int64_t nq, int P, int K)
 
 bool scan_fits(const sivf_index *ix, int K)
 {
-    return scan_smem(8, ix->C, ix->d, scan_buf_len(K, ix->C)).total <= SCAN_SMEM;
+    return fp32_fits(8, ix->C, ix->d, K, 0);
 }
 
 void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_t *probes,

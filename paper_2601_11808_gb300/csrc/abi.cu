@@ -473,7 +473,7 @@ static size_t search_bytes(const sivf_index *ix, int64_t nq, int k, int P, Searc
     SearchPlan pl = plan_search(ix, nq, P, k);
     if (plo) *plo = pl;
     size_t parts = (size_t)pl.run_cap * pl.K;
-    return coarse_bytes(ix, nq, P) + (size_t)nq * P * 4 * 4 + (size_t)(L + 1) * 4 * 4 +
+    return coarse_bytes(ix, nq, P) + (size_t)nq * P * 4 * 4 + (size_t)(L + 1) * 4 * 3 +
            parts * 12 + (size_t)nq * 4 * 3 + (size_t)nq * 16 + (size_t)pl.item_cap * 8 + 19 * 256;
 }
 
@@ -491,7 +491,7 @@ static size_t chunk_need(const sivf_index *ix, int64_t m, int P, int Kc, int dty
     const int L = ix->nlist;
     SearchPlan pl = plan_tc(ix, dtype, m, P, Kc);
     *plo = pl;
-    return coarse_bytes(ix, m, P) + (size_t)m * P * 4 * 4 + (size_t)(L + 1) * 4 * 4 +
+    return coarse_bytes(ix, m, P) + (size_t)m * P * 4 * 4 + (size_t)(L + 1) * 4 * 3 +
            (size_t)pl.run_cap * (pl.RK * 12 + 4) + (size_t)m * 4 * 3 + (size_t)m * 16 +
            (size_t)pl.item_cap * 8 + (size_t)m * ix->d * 2 +
            (dtype == SIVF_FP8E4M3 ? (size_t)m * P * (ix->d + 8) : 0) + 23 * 256;
@@ -779,7 +779,6 @@ static sivf_status search_impl(sivf_index *ix, const float *q, int64_t nq, int k
         int32_t *probes = b.take<int32_t>((size_t)m * P);
         sc.lcnt = b.take<int32_t>(L);
         sc.loff = b.take<int32_t>(L + 1);
-        sc.touched = b.take<int32_t>(L + 1);
         sc.nch = b.take<int32_t>(L);
         sc.prank = b.take<int32_t>((size_t)m * P);
         sc.qlist = b.take<int32_t>((size_t)m * P);

@@ -100,7 +100,6 @@ void list_radii(sivf_index *ix, cudaStream_t st);
 struct SearchScratch {
     int32_t *lcnt;       // [nlist] (query, list) pairs per list
     int32_t *loff;       // [nlist + 1]
-    int32_t *touched;    // [nlist + 1] lists some pair probes (small launches)
     int32_t *nch;        // [nlist] slab chunks of each list
     int32_t *prank;      // [nq * P] rank of the pair inside its list group
     int32_t *qlist;      // [nq * P] pairs grouped by list (q * P + p)

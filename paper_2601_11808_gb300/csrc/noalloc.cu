@@ -61,7 +61,7 @@ size_t need_bytes(const sivf_index *ix, int64_t nq, int P, const sivf::SearchPla
     add((size_t)nq * P * 4);          // probes
     add(L * 4);                       // lcnt
     add((L + 1) * 4);                 // loff
-    add((L + 1) * 4);                 // touched
+    add((L + 1) * 4);                 // not used: batches are refused from the same size on
     add(L * 4);                       // nch
     add((size_t)nq * P * 4);          // prank
     add((size_t)nq * P * 4);          // qlist
@@ -151,7 +151,6 @@ extern "C" sivf_status sivf_search_noalloc(sivf_index *ix, const float *q, int64
     SearchScratch sc{};
     sc.lcnt = c.take<int32_t>(L);
     sc.loff = c.take<int32_t>(L + 1);
-    sc.touched = c.take<int32_t>(L + 1);
     sc.nch = c.take<int32_t>(L);
     sc.prank = c.take<int32_t>((size_t)nq * P);
     sc.qlist = c.take<int32_t>((size_t)nq * P);

@@ -219,140 +219,15 @@ __global__ __launch_bounds__(1024) void k_srch_plan(const int32_t *__restrict__ 
     }
 }
 
-// The whole grouping of a small launch (at most SG_PAIRS pairs) in one
-// block: count the pairs of each touched list, cut the lists into chunks,
-// lay out the groups, the items and the output runs.  Pairs are taken in
-// query order, eight consecutive ones per thread, so that a scan over them
-// gives every query one contiguous block of runs.  It replaces a memset and
-// three launches, and looks only at the lists the pairs touch, not at all L
-// (61 queries x 31 lists of 16,384: 64 us before, most of it in the plan).
-constexpr int SG_PER = 8;
-constexpr int SG_PAIRS = 1024 * SG_PER;
-__global__ __launch_bounds__(1024) void k_srch_small(
-    const int32_t *__restrict__ probes, int64_t nq, int P, int p0, int p1, int L, bool dedupe,
-    const int32_t *__restrict__ flags, const int32_t *__restrict__ nslabs,
-    const int32_t *__restrict__ list_live, int tq, int chmax,
-    int spc, int ips, int64_t item_cap, int64_t slab_bytes, int32_t *lcnt, int32_t *touched,
-    int32_t *loff, int32_t *nch, int2 *items, int32_t *qlist, int32_t *prun, int2 *qrun, Ctl *ctl,
-    int64_t run_cap, int64_t *stat, uint32_t *err)
-{
-    pdl_begin();
-    __shared__ int32_t sh[64];
-    __shared__ unsigned long long sw[32];
-    __shared__ int s_nt, s_base;
-    const int tid = threadIdx.x, np = p1 - p0, n = (int)nq * np;
-    const int per = (n + 1023) / 1024;  // <= SG_PER
-    int ev[SG_PER], lv[SG_PER], rk[SG_PER];  // n <= SG_PAIRS, P <= 1024: ev fits
-    if (tid == 0) s_nt = 0;
-#pragma unroll
-    for (int i = 0; i < SG_PER; ++i) {
-        const int t = tid * per + i;
-        ev[i] = i < per && t < n ? (t / np) * P + p0 + t % np : -1;
-        lv[i] = ev[i] >= 0 ? probes[ev[i]] : -1;
-        if (lv[i] >= L || (flags && ev[i] >= 0 && flags[ev[i]] < 0)) lv[i] = -1;
-    }
-    if (dedupe)
-#pragma unroll
-        for (int i = 0; i < SG_PER; ++i) {
-            if (lv[i] < 0) continue;
-            for (int f = (ev[i] / P) * P; f < ev[i]; ++f)
-                if (probes[f] == lv[i]) {
-                    lv[i] = -1;
-                    break;
-                }
-        }
-#pragma unroll
-    for (int i = 0; i < SG_PER; ++i)
-        if (lv[i] >= 0) lcnt[lv[i]] = 0;
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < SG_PER; ++i) {
-        rk[i] = lv[i] >= 0 ? atomicAdd(&lcnt[lv[i]], 1) : -1;
-        if (rk[i] == 0) touched[atomicAdd(&s_nt, 1)] = lv[i];
-    }
-    __syncthreads();
-    const int nt = s_nt;
-    // the touched lists: chunks, groups, items
-    unsigned long long wsum = 0;
-    for (int j = tid; j < nt; j += 1024) {
-        const int l = touched[j], m = __ldcg(lcnt + l), ns = nslabs[l];
-        if (ns > 0) wsum += (unsigned long long)((m + tq - 1) / tq) * ns;
-    }
-    const int target = chunk_target(block_work(wsum, sw), spc, ips);
-    int32_t ca = 0, cb = 0;
-    ScanCount cnt;
-    for (int j = tid; j < nt; j += 1024) {
-        const int l = touched[j], m = __ldcg(lcnt + l), ns = nslabs[l], k = (m + tq - 1) / tq;
-        const int c = ns > 0 ? min(min(chmax, max(1, (ns + target - 1) / target)), ns) : 0;
-        nch[l] = c;
-        ca += m;
-        cb += k * c;
-        if (c) cnt.list(m, k, ns, list_live[l], slab_bytes);
-    }
-    if (stat) cnt.add_to(stat);
-    int32_t ea = ca, eb = cb, ta, tb;
-    block_scan2(ea, eb, sh, &ta, &tb);
-    ea -= ca;
-    eb -= cb;
-    for (int j = tid; j < nt; j += 1024) {
-        const int l = touched[j], m = __ldcg(lcnt + l), c = nch[l], k = (m + tq - 1) / tq;
-        loff[l] = ea;
-        for (int t = 0; t < k * c; ++t)
-            if (eb + t < item_cap) items[eb + t] = make_int2(l, ((t / c) << 8) | (t % c));
-        ea += m;
-        eb += k * c;
-    }
-    if (tid == 0) {
-        if (tb > item_cap) atomicOr(err, ERR_PLAN);
-        ctl->nitems = (int32_t)min((int64_t)tb, item_cap);
-        ctl->nscan = ta;
-        ctl->next_item = 0;
-    }
-    __syncthreads();
-    // the pairs: their place in the list's group, their output runs
-    int cv[SG_PER], mine = 0;
-#pragma unroll
-    for (int i = 0; i < SG_PER; ++i) {
-        cv[i] = 0;
-        if (lv[i] < 0) continue;
-        qlist[loff[lv[i]] + rk[i]] = ev[i];
-        cv[i] = nch[lv[i]];
-        mine += cv[i];
-    }
-    int32_t run = mine, dummy = 0, total, td;
-    block_scan2(run, dummy, sh, &total, &td);
-    if (tid == 0) s_base = atomicAdd(&ctl->nruns, total);
-    __syncthreads();
-    const int base = s_base;
-    const bool fits = base >= 0 && (int64_t)base + total <= run_cap;
-    if (!fits && tid == 0) atomicOr(err, ERR_PLAN);
-    run += base - mine;
-    int2 *qr = qrun + (p0 > 0 ? nq : 0);
-    const int first = run;
-#pragma unroll
-    for (int i = 0; i < SG_PER; ++i) {
-        if (ev[i] < 0) continue;
-        prun[ev[i]] = cv[i] > 0 && fits ? run : -1;
-        if (ev[i] % P == p0) qr[ev[i] / P].x = fits ? run : 0;
-        run += cv[i];
-    }
-    __syncthreads();  // every query's first run is written
-    run = first;
-#pragma unroll
-    for (int i = 0; i < SG_PER; ++i) {
-        if (ev[i] < 0) continue;
-        run += cv[i];
-        if (ev[i] % P == p1 - 1) {
-            const int q = ev[i] / P;
-            qr[q].y = fits ? run - qr[q].x : 0;
-        }
-    }
-}
-
-// The same for at most SH_PAIRS pairs, two per thread, with the lists' counts
-// in a hash table in shared memory: the chain of global round trips (clear,
-// count, collect, read back) shrinks to the probes, the slab counts and the
-// stores.  9 us against 12 for 8 to 1,900 pairs, twice per search.
+// The whole grouping of a small launch (at most SH_PAIRS pairs, two per
+// thread) in one block: count the pairs of each touched list, cut the lists
+// into chunks, lay out the groups, the items and the output runs.  Pairs are
+// taken in query order, so that a scan over them gives every query one
+// contiguous block of runs; the lists' counts stand in a hash table in shared
+// memory, so that the chain of global round trips is the probes, the slab
+// counts and the stores.  It replaces a memset and three launches and looks
+// only at the lists the pairs touch: 9 to 15 us for 8 to 2,000 pairs.  More
+// pairs per thread are the slower way: 34 us for 7,000, the three kernels 20.
 constexpr int SH_PER = 2;
 constexpr int SH_PAIRS = 1024 * SH_PER;
 constexpr int SH_SLOTS = 2 * SH_PAIRS;  // a power of two, at most half full
@@ -1695,15 +1570,6 @@ void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_
                    pl.slabs_per_chunk, pl.ips, pl.item_cap, slab_bytes, s.lcnt, s.loff, s.nch,
                    s.items, s.qlist, s.prun, s.qrun, ix->ctl, pl.run_cap,
                    stats ? ix->stat : nullptr, ix->err);
-        prof_end(ix, tg, st);
-        return;
-    }
-    if (n <= SG_PAIRS) {
-        const int tg = prof_begin(ix, PROF_GROUP, 1, st);
-        launch_pdl(k_srch_small, 1, 1024, 0, st, probes, nq, P, p0, p1, L, dedupe,
-                   flagged ? s.prank : nullptr, ix->nslabs, ix->list_live, pl.tq, pl.ch, pl.slabs_per_chunk, pl.ips, pl.item_cap, slab_bytes,
-                   s.lcnt, s.touched, s.loff, s.nch, s.items, s.qlist, s.prun, s.qrun, ix->ctl,
-                   pl.run_cap, stats ? ix->stat : nullptr, ix->err);
         prof_end(ix, tg, st);
         return;
     }

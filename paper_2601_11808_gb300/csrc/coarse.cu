@@ -675,11 +675,11 @@ __global__ __launch_bounds__(CT_NT, 1) void k_coarse_tc(const float *__restrict_
 // ||x|| is bounded from the FP32 sum of squares s of the tile's rows
 // (relative error <= d u) as RU(sqrt(RU(s (1 + 4 d u)))).
 //
-// What bounds it: the epilogue's min/max and selects (4.6 half-rate
+// What bounds it: the epilogue's min/max and selects (4.3 half-rate
 // operations per list and row); a chunk's MMAs and its copy from L2 run
-// under it.  1,000,000 rows, 1,024 lists, d = 128: 560 us, 1,190 in launches
+// under it.  1,000,000 rows, 1,024 lists, d = 128: 526 us, 1,190 in launches
 // of one tile per CTA and two passes over the centroids; the split stage,
-// 200,000 rows: 142 us + 36 us to finish the undecided rows, 1,580 us when
+// 200,000 rows: 141 us + 36 us to finish the undecided rows, 1,580 us when
 // the matrix of distances was written and read back.
 constexpr int CF_CAP = 32;                  // lists of one undecided row's record
 constexpr int CF_SUB = 4;                   // threads per row
@@ -928,43 +928,41 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
                 if (j == nch - 1 && more && ok) store(par ^ 1);  // this tile's MMAs are done
                 if (ok) {
                     const uint32_t tad = tbase + b * CN + sub * 16 + ((uint32_t)(q * 32) << 16);
-                    float vv[2][16];
-                    tmem_ld16(tad, vv[0]);
 #pragma unroll
                     for (int k = 0; k < CN / 64; ++k) {
                         const int grp = j * (CN / 16) + sub + 4 * k;
                         const float4 *cv4 = reinterpret_cast<const float4 *>(scn + grp * 16);
-                        float (&v)[16] = vv[k & 1];
+                        float v[16];
+                        tmem_ld16(tad + k * 64, v);
                         tmem_ld_wait(v);
-                        if (k + 1 < CN / 64)  // the next group's load runs under this one
-                            tmem_ld16(tad + (k + 1) * 64, vv[(k + 1) & 1]);
-                        float lo[8], hi[8];
+                        // the smallest key of the group and its second: any other key
+                        // is in another row or another column of the 4 x 4 square, so
+                        // the second is the smaller second of the rows' and of the
+                        // columns' minima (30 operations, 37 by a tree of pairs)
+                        float key[16];
 #pragma unroll
                         for (int i4 = 0; i4 < 4; ++i4) {
                             const float4 cv = cv4[i4];
                             const float c4[4] = {cv.x, cv.y, cv.z, cv.w};
-                            float e[4];
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
                                 const float Dt = fmaf(-2.f, v[4 * i4 + i], c4[i]);
-                                e[i] = __uint_as_float((__float_as_uint(Dt) & ~15u) |
-                                                       (uint32_t)(4 * i4 + i));
+                                key[4 * i4 + i] = __uint_as_float((__float_as_uint(Dt) & ~15u) |
+                                                                  (uint32_t)(4 * i4 + i));
                             }
-                            lo[2 * i4] = fminf(e[0], e[1]);
-                            hi[2 * i4] = fmaxf(e[0], e[1]);
-                            lo[2 * i4 + 1] = fminf(e[2], e[3]);
-                            hi[2 * i4 + 1] = fmaxf(e[2], e[3]);
                         }
+                        float rw[4], cl[4];
 #pragma unroll
-                        for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-                            for (int i = 0; i < w; ++i) {
-                                const float mx = fmaxf(lo[2 * i], lo[2 * i + 1]);
-                                hi[i] = min3f(hi[2 * i], hi[2 * i + 1], mx);
-                                lo[i] = fminf(lo[2 * i], lo[2 * i + 1]);
-                            }
+                        for (int i = 0; i < 4; ++i) {
+                            rw[i] = min3f(key[4 * i], key[4 * i + 1], fminf(key[4 * i + 2], key[4 * i + 3]));
+                            cl[i] = min3f(key[i], key[4 + i], fminf(key[8 + i], key[12 + i]));
+                        }
+                        const float ra = fminf(rw[0], rw[1]), rb = fminf(rw[2], rw[3]);
+                        const float ca = fminf(cl[0], cl[1]), cb = fminf(cl[2], cl[3]);
+                        const float r2 = min3f(fmaxf(rw[0], rw[1]), fmaxf(rw[2], rw[3]), fmaxf(ra, rb));
+                        const float c2 = min3f(fmaxf(cl[0], cl[1]), fmaxf(cl[2], cl[3]), fmaxf(ca, cb));
                         // insert the group into the sorted three
-                        float mv = lo[0], ms = hi[0];
+                        float mv = fminf(ra, rb), ms = fminf(r2, c2);
                         int mg = grp;
 #pragma unroll
                         for (int i = 0; i < 3; ++i) {

@@ -156,8 +156,10 @@ __device__ __forceinline__ void drop_total(const IndexView &V, int n, bool count
 
 // one warp per list that lost a slab: stable compaction of the directory,
 // emptied slabs reset and pushed on the free stack.  RC_U x 32 entries and
-// their slabs' counts are in flight at once: a directory of 2,000 slabs
-// walked 32 at a time took 90 us, two dependent loads after each other.
+// their slabs' counts are in flight at once, and their emptied slabs take
+// their places on the stack together: a directory of 2,000 slabs walked 32 at
+// a time took 90 us, two dependent loads after each other, and with an atomic
+// on the stack's top per 32 entries still 61; 54 now.
 constexpr int RC_U = 8;
 __global__ void k_reclaim(IndexView V, const int32_t *__restrict__ affected)
 {
@@ -190,27 +192,32 @@ __global__ void k_reclaim(IndexView V, const int32_t *__restrict__ affected)
 #pragma unroll
             for (int u = 0; u < RC_U; ++u) live[u] = sv[u] >= 0 ? V.meta[sv[u]].live : 0;
             __syncwarp();  // the entries are read before any is overwritten
+            uint32_t dm[RC_U];
+            int nd = 0, t = 0;
 #pragma unroll
             for (int u = 0; u < RC_U; ++u) {
-                if (base + 32 * u >= n) break;  // warp-uniform
-                const int s = sv[u];
-                const bool keep = s >= 0 && live[u] > 0, drop = s >= 0 && !keep;
+                const bool keep = sv[u] >= 0 && live[u] > 0;
                 const uint32_t km = __ballot_sync(0xffffffffu, keep);
-                const uint32_t dm = __ballot_sync(0xffffffffu, drop);
-                if (keep) D[kept + __popc(km & lanemask_lt())] = s;
+                dm[u] = __ballot_sync(0xffffffffu, sv[u] >= 0 && !keep);
+                if (keep) D[kept + __popc(km & lanemask_lt())] = sv[u];
                 kept += __popc(km);
-                if (dm == 0u) continue;
-                int t = 0;
-                if (lane == 0) t = atomicAdd(V.free_top, __popc(dm));
-                t = __shfl_sync(0xffffffffu, t, 0) + __popc(dm & lanemask_lt());
-                if (drop) {
+                nd += __popc(dm[u]);
+            }
+            if (nd == 0) continue;
+            if (lane == 0) t = atomicAdd(V.free_top, nd);
+            t = __shfl_sync(0xffffffffu, t, 0);
+#pragma unroll
+            for (int u = 0; u < RC_U; ++u) {
+                if ((dm[u] >> lane) & 1u) {
+                    const int s = sv[u], p = t + __popc(dm[u] & lanemask_lt());
                     V.meta[s].list = -1;
                     V.meta[s].fill = 0;
                     V.meta[s].live = 0;
-                    if (t >= V.n_slabs) atomicOr(V.err, ERR_STACK);
-                    else V.free_list[t] = s;
+                    if (p >= V.n_slabs) atomicOr(V.err, ERR_STACK);
+                    else V.free_list[p] = s;
                     if (s == h) hfree = true;
                 }
+                t += __popc(dm[u]);
             }
         }
         hfree = __any_sync(0xffffffffu, hfree);

@@ -83,7 +83,9 @@ typedef struct {
     int64_t last_count;  /* vectors added / removed by that batch            */
     int64_t bytes_device;/* device memory held by the index                  */
     int64_t pairs_scanned;      /* (query, live vector) pairs the list scans
-                                   have scored since creation (FP32 path)    */
+                                   have scored since creation (FP32 path;
+                                   pairs of a query and a list ruled out by
+                                   their bound are not scanned nor counted)  */
     int64_t slab_bytes_scanned; /* slab bytes the list scans streamed since
                                    creation (payload, ids or norms, bitmap),
                                    one read per (list, query tile)           */
@@ -474,8 +476,8 @@ typedef struct {
     int32_t select_slabs;     /* SIVF_FP32, 0..8: the k-select buffer of
                                  each query row holds its best k plus room
                                  for this many slabs of candidates (0: the
-                                 built-in width, two slabs while that stays
-                                 within 256 entries).  Reduced dtypes,
+                                 built-in width, 64 entries while that stays
+                                 within 256 in all).  Reduced dtypes,
                                  vector-row scan, 0..3: room for this many
                                  128-row tiles of candidates beside the
                                  held 4k (0: two where shared memory keeps

@@ -8,10 +8,11 @@
 // through shared memory as 128-row A tiles (TMA 2-D loads, 128-byte
 // swizzle); the query tile, rounded to the same format, is the B operand;
 // tcgen05.mma accumulates the 128 x TN dot products in FP32 in tensor
-// memory (two accumulators, so the next tile's MMAs overlap the epilogue of
-// this one).  The epilogue forms the expanded distance
-// ||q||^2 + ||x||^2 - 2 s q.x (FP32 norms of the unrounded vectors, s the
-// dequantisation scale), and every query keeps its best K' (= 4k)
+// memory (all 512 columns: 8 or 16 accumulators, so the next tiles' MMAs
+// overlap the epilogue of this one, and the first tiles of an item can be
+// looked at for a bound before anything is appended).  The epilogue forms
+// the expanded distance ||q||^2 + ||x||^2 - 2 s q.x (FP32 norms of the
+// unrounded vectors, s the dequantisation scale), and every query keeps its best K' (= 4k)
 // (distance, slot) candidates.  A per-query shared bound (the K'-th
 // distance any item has found) prunes the rest.  A final pass recomputes
 // the K' survivors' distances exactly in FP32 from the FP32 payload and
@@ -25,16 +26,17 @@
 //   warp 0  (one lane) TMA loads of the A tiles, plus L2 prefetches of
 //           the payload rows and their ||x||^2 further ahead in the list;
 //   warp 1  (one lane) issues the MMAs; warp 2 also owns the TMEM;
-//   warps 4.. the epilogue: TN / 16 warps per TMEM lane quarter, 16
-//           query columns each; each thread reads its row's ||x||^2 from
+//   warps 4.. the epilogue: three warps per TMEM lane quarter, 16 query
+//           columns each (where TN has fewer blocks of columns, the quarter's
+//           warps share the tiles); each thread reads its row's ||x||^2 from
 //           global memory (L2) before it waits for the accumulator.
-// A tile's passing rows are appended to their query's buffer at positions
-// reserved by one shared atomic per (warp, query); a buffer is reduced to
-// its best K' (radix select, left unsorted) only after a tile that leaves
-// it too full for the next one, so most tiles end on a single barrier.
-// Each item writes its rows' best K' unsorted; a per-query merge selects
-// and sorts the best K' of all its items.  Every wait is bounded, and a
-// wait that gives up stops every role.
+// A tile's passing rows are appended to their query's buffer, each lane its
+// own, at a position taken by a shared atomic; a buffer is reduced to little more than its best K' (left unsorted) only after a
+// tile that leaves it too full for the next one, so most tiles end on a
+// single barrier.  Each item writes its rows' candidates unsorted with their
+// count; a per-query merge makes the exact selection of the best K' of all
+// its items.  Every wait is bounded, and a wait that gives up stops every
+// role.
 #include <cudaTypedefs.h>
 #include <math.h>
 
@@ -54,8 +56,7 @@ constexpr int TC_PF_BYTES = 192 * 1024;  // L2 prefetch distance per CTA
 
 // Query tiles: 48 queries for K' <= 64 (small enough candidate buffers for
 // three A stages), 32 for K' <= 128, 16 (and candidate buffers up to
-// K' = 512) for deeper re-ranks.  TN / 16 epilogue warps per TMEM lane
-// quarter, 16 query columns each.
+// K' = 512) for deeper re-ranks.
 template <int TN> struct TcShape {
     static constexpr int N = TN;                        // queries per tile (MMA N)
     // epilogue warps: three per TMEM lane quarter, also where TN has fewer
@@ -1364,7 +1365,7 @@ void merge_tc(sivf_index *ix, int64_t nq, int nphase, const SearchScratch &s, in
 // ---------------------------------------------------------------- re-rank
 // The per-query merge and the re-rank in one warp per query (K' <= 128):
 // merge_select leaves the query's best K' (distance, slot) entries in shared
-// memory, and the warp re-ranks those slots exactly as k_rerank does (eight
+// memory, and the warp computes those slots' FP32 direct-form distances (eight
 // lanes per candidate row, RK_UNR rounds of four, the query in registers),
 // so the candidate lists never go through global memory and nothing sorts
 // them by approximate distance.

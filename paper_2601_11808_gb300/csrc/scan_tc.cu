@@ -12,8 +12,8 @@
 // overlap the epilogue of this one, and the first tiles of an item can be
 // looked at for a bound before anything is appended).  The epilogue forms
 // the expanded distance ||q||^2 + ||x||^2 - 2 s q.x (FP32 norms of the
-// unrounded vectors, s the dequantisation scale), and every query keeps its best K' (= 4k)
-// (distance, slot) candidates.  A per-query shared bound (the K'-th
+// unrounded vectors, s the dequantisation scale), and every query keeps its
+// best K' (= 4k) (distance, slot) candidates.  A per-query shared bound (the K'-th
 // distance any item has found) prunes the rest.  A final pass recomputes
 // the K' survivors' distances exactly in FP32 from the FP32 payload and
 // keeps the best k by (distance, id).
@@ -31,9 +31,9 @@
 //           warps share the tiles); each thread reads its row's ||x||^2 from
 //           global memory (L2) before it waits for the accumulator.
 // A tile's passing rows are appended to their query's buffer, each lane its
-// own, at a position taken by a shared atomic; a buffer is reduced to little more than its best K' (left unsorted) only after a
-// tile that leaves it too full for the next one, so most tiles end on a
-// single barrier.  Each item writes its rows' candidates unsorted with their
+// own, at a position taken by a shared atomic; a buffer is reduced to little
+// more than its best K' (left unsorted) only after a tile that leaves it too
+// full for the next one, so most tiles end on a single barrier.  Each item writes its rows' candidates unsorted with their
 // count; a per-query merge makes the exact selection of the best K' of all
 // its items.  Every wait is bounded, and a wait that gives up stops every
 // role.

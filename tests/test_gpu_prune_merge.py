@@ -143,9 +143,9 @@ def test_merges_of_many_equal_distances(k):
 
 
 @pytest.mark.parametrize("nq,P", [(1, 1), (1, 64), (1024, 8), (1025, 8), (8192, 1), (8193, 1), (127, 64),
-                                  (129, 64)])
+                                  (129, 64), (1024, 2), (683, 3), (2048, 1), (2049, 1), (32, 64), (33, 64)])
 def test_grouping_in_one_block_and_in_three(nq, P):
-    """8,192 pairs group in one block, more in three launches."""
+    """2,048 pairs group in one block, more in three launches."""
     import torch
     rng = np.random.default_rng([nq, P])
     cent, x = _cloud(rng, 3000, 16, 70, 0.3)

@@ -171,6 +171,9 @@ struct SelArgs {
     const int *nhard;      // undecided, those with a record from the front, those to
     const int32_t *S;      // redo from the back (two counters, on the device), and
     int s_cap;             // the first kind's records (room for s_cap): [n, lists...]
+    float *Dw;             // refine_rows: the same distances, to be rewritten
+    float *gmin;           // [m, groups of 16 lists] the distances' group minima
+    const float *cmaxes;   // the largest ||c||^2 and ||c||
     int32_t *out;          // [m, P]
     uint32_t *err;
 };
@@ -218,6 +221,53 @@ __device__ __forceinline__ double exact_dist4(const float4 *a, const float4 *__r
     return acc;
 }
 
+// The same of n <= EX_FEW lists by a warp (d <= 128), the m-th list's in lane m:
+// each lane squares the differences of four coordinates of every list, then the
+// lanes 0 .. n-1 add up a list each, in the definition's order.  An FP64
+// instruction of a warp takes the same time for one lane as for 32: a list per
+// lane issues 640 of them at d = 128, this 176, which counts where several warps
+// of an SM are at it; the chain of additions (about 300 cycles each) is the same.
+constexpr int EX_FEW = 4;
+template <class Idx>
+__device__ __forceinline__ double exact_four(const float4 *x4, const float *__restrict__ cent, Idx list, int n,
+                                             int d, int lane)
+{
+    const int n4 = d >> 2;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 xv = lane < n4 ? x4[lane] : zero;
+    const double x[4] = {(double)xv.x, (double)xv.y, (double)xv.z, (double)xv.w};
+    double v[4][4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const float4 cv = m < n && lane < n4
+                              ? __ldg(reinterpret_cast<const float4 *>(cent + (size_t)list(m) * d) + lane)
+                              : zero;
+        const float c[4] = {cv.x, cv.y, cv.z, cv.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[m][k] = 0.0;
+            if (m < n) {
+                const double t = __dsub_rn(x[k], (double)c[k]);
+                v[m][k] = __dmul_rn(t, t);
+            }
+        }
+    }
+    double acc = 0.0;
+    for (int l = 0; l < n4; ++l)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            double t = __shfl_sync(0xffffffffu, v[0][k], l);
+#pragma unroll
+            for (int m = 1; m < 4; ++m)
+                if (m < n) {
+                    const double u = __shfl_sync(0xffffffffu, v[m][k], l);
+                    if (lane == m) t = u;
+                }
+            acc = __dadd_rn(acc, t);
+        }
+    return acc;
+}
+
 // Bound E of |Dt - Q|.  Written with explicit-rounding intrinsics so that
 // every evaluation for the same inputs gives the same bits (no contraction).
 __device__ __forceinline__ float bound_of(float Dt, float cnc, float cnrm, float xn,
@@ -239,7 +289,8 @@ __device__ __forceinline__ float norm_up(float ss, int d)
     return __fsqrt_ru(__fmul_ru(ss, 1.f + 4.f * (float)d * 5.9604645e-08f));
 }
 
-// block-wide helpers for SEL_NT threads
+// the smallest of a block of NT threads
+template <int NT>
 __device__ float block_min(float v, float *red)
 {
     for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -248,7 +299,7 @@ __device__ float block_min(float v, float *red)
     if (l == 0) red[w] = v;
     __syncthreads();
     if (w == 0) {
-        v = l < SEL_NT / 32 ? red[l] : INFINITY;
+        v = l < NT / 32 ? red[l] : INFINITY;
         for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
         if (l == 0) red[0] = v;
     }
@@ -258,22 +309,31 @@ __device__ float block_min(float v, float *red)
     return r;
 }
 
-// one row, by a block
-__device__ void select_row(const SelArgs &a, int row)
+// the tables of one row's selection
+struct SelTab {
+    double dx[SEL_SCAP];
+    float LB[SEL_SCAP], UB[SEL_SCAP], red[32];
+    int idx[SEL_SCAP], sel[kMaxK];
+    uint32_t hist[256], prefix, rank;
+    int ns, nsel;
+    unsigned char sure[SEL_SCAP];
+};
+
+// One row, by a block.  FRESH: the distances were written by this kernel (other
+// blocks of it, too), so they are read from L2.
+template <int NT, bool FRESH>
+__device__ void select_row(const SelArgs &a, int row, SelTab &tab)
 {
+    auto ld = [](const float *p) { return FRESH ? __ldcg(p) : *p; };
     const int tid = threadIdx.x;
     const float *Dr = a.D + (size_t)row * a.L;
     const float *xr = a.x + (size_t)row * a.d;
 
-    __shared__ float red[32];
-    __shared__ uint32_t hist[256];
-    __shared__ uint32_t s_prefix, s_rank;
-    __shared__ int s_ns, s_nsel;
-    __shared__ float sLB[SEL_SCAP], sUB[SEL_SCAP];
-    __shared__ int sIdx[SEL_SCAP];
-    __shared__ unsigned char sSure[SEL_SCAP];
-    __shared__ double sDx[SEL_SCAP];
-    __shared__ int sSel[kMaxK];
+    float *red = tab.red, *sLB = tab.LB, *sUB = tab.UB;
+    uint32_t *hist = tab.hist, &s_prefix = tab.prefix, &s_rank = tab.rank;
+    int &s_ns = tab.ns, &s_nsel = tab.nsel, *sIdx = tab.idx, *sSel = tab.sel;
+    unsigned char *sSure = tab.sure;
+    double *sDx = tab.dx;
 
     // every warp sums the row's squares for itself
     float part = 0.f;
@@ -286,11 +346,11 @@ __device__ void select_row(const SelArgs &a, int row)
     float T;
     if (a.P == 1) {
         float v = INFINITY;
-        for (int c = tid; c < a.L; c += SEL_NT) {
-            float Dt = Dr[c];
+        for (int c = tid; c < a.L; c += NT) {
+            float Dt = ld(Dr + c);
             v = fminf(v, upper_of(Dt, bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, gamma2)));
         }
-        T = block_min(v, red);
+        T = block_min<NT>(v, red);
     } else {
         if (tid == 0) {
             s_prefix = 0;
@@ -299,11 +359,11 @@ __device__ void select_row(const SelArgs &a, int row)
         uint32_t mask = 0;
         for (int pass = 0; pass < 4; ++pass) {
             const int shift = 24 - 8 * pass;
-            hist[tid] = 0;  // SEL_NT == 256 bins
+            for (int h = tid; h < 256; h += NT) hist[h] = 0;
             __syncthreads();
             const uint32_t prefix = s_prefix;
-            for (int c = tid; c < a.L; c += SEL_NT) {
-                float Dt = Dr[c];
+            for (int c = tid; c < a.L; c += NT) {
+                float Dt = ld(Dr + c);
                 uint32_t k = fkey(upper_of(Dt, bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, gamma2)));
                 if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
             }
@@ -346,8 +406,8 @@ __device__ void select_row(const SelArgs &a, int row)
         s_nsel = 0;
     }
     __syncthreads();
-    for (int c = tid; c < a.L; c += SEL_NT) {
-        float Dt = Dr[c];
+    for (int c = tid; c < a.L; c += NT) {
+        float Dt = ld(Dr + c);
         float E = bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, gamma2);
         if (lower_of(Dt, E) <= T) {
             int p = atomicAdd(&s_ns, 1);
@@ -364,7 +424,7 @@ __device__ void select_row(const SelArgs &a, int row)
 
     if (ns <= SEL_SCAP) {
         // sure members
-        for (int p = tid; p < ns; p += SEL_NT) {
+        for (int p = tid; p < ns; p += NT) {
             float ub = sUB[p];
             int cnt = 0;
             for (int q = 0; q < ns; ++q) cnt += (q != p && sLB[q] <= ub);
@@ -382,11 +442,11 @@ __device__ void select_row(const SelArgs &a, int row)
             // boundary members: exact FP64 distances, then rank among them
             const int nb = ns - nsure;
             if (nb > r) {
-                for (int p = tid; p < ns; p += SEL_NT)
+                for (int p = tid; p < ns; p += NT)
                     if (!sSure[p]) sDx[p] = exact_dist(xr, a.cent + (size_t)sIdx[p] * a.d, a.d);
                 __syncthreads();
             }
-            for (int p = tid; p < ns; p += SEL_NT) {
+            for (int p = tid; p < ns; p += NT) {
                 if (sSure[p]) continue;
                 bool take = true;
                 if (nb > r) {
@@ -413,7 +473,7 @@ __device__ void select_row(const SelArgs &a, int row)
         double *hd = sDx;  // P <= SEL_SCAP entries
         int n = 0;
         for (int c = 0; c < a.L; ++c) {
-            float Dt = Dr[c];
+            float Dt = ld(Dr + c);
             float E = bound_of(Dt, a.cn[c], a.cnrm_up[c], xn, gamma2);
             if (lower_of(Dt, E) > T) continue;
             double Dc = exact_dist(xr, a.cent + (size_t)c * a.d, a.d);
@@ -436,9 +496,9 @@ __device__ void select_row(const SelArgs &a, int row)
     // ties to the lower list index (the set itself is the exact one)
     const int nsel = min(s_nsel, a.P);
     if (s_nsel != a.P && tid == 0) atomicOr(a.err, ERR_SELECT);
-    for (int s = tid; s < nsel; s += SEL_NT) {  // their FP32 distances (P <= SEL_SCAP)
+    for (int s = tid; s < nsel; s += NT) {  // their FP32 distances (P <= SEL_SCAP)
         const int c = sSel[s];
-        float dc = Dr[c];
+        float dc = ld(Dr + c);
         if (a.two_level) {
             float dot = 0.f;
             for (int j = 0; j < a.d; ++j) dot = fmaf(xr[j], __ldg(a.cent + (size_t)c * a.d + j), dot);
@@ -447,7 +507,7 @@ __device__ void select_row(const SelArgs &a, int row)
         sLB[s] = dc;
     }
     __syncthreads();
-    for (int s = tid; s < a.P; s += SEL_NT) {
+    for (int s = tid; s < a.P; s += NT) {
         if (s >= nsel) {
             outr[s] = -1;
             continue;
@@ -467,9 +527,8 @@ __device__ void select_row(const SelArgs &a, int row)
 __global__ __launch_bounds__(SEL_NT) void k_coarse_select(SelArgs a)
 {
     pdl_begin();
-    // all rows, a block each; or the rows k_coarse_pick left (usually none)
-    const int nrows = a.hard ? *a.nhard : a.m;
-    for (int it = blockIdx.x; it < nrows; it += gridDim.x) select_row(a, a.hard ? a.hard[it] : it);
+    __shared__ SelTab tab;
+    for (int row = blockIdx.x; row < a.m; row += gridDim.x) select_row<SEL_NT, false>(a, row, tab);
 }
 
 // ------------------------------------------ BF16 tensor-core first stage
@@ -720,6 +779,15 @@ __device__ __forceinline__ float min3f(float a, float b, float c)
     float r;
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
+}
+
+// The largest split distance a list of the P nearest can have, from a value b
+// that P lists lie at or below: Dt - E <= T with T = b + Ebig needs Dt <= T +
+// Ebig + its roundings
+__device__ __forceinline__ float pick_limit(float b, float eb)
+{
+    const float T0 = __fadd_ru(b, eb);
+    return __fadd_ru(__fadd_ru(T0, eb), __fadd_ru(__fmul_ru(fabsf(T0), 1.2e-7f), 1e-30f));
 }
 
 // A tile of 128 rows held in registers by CF_EPI threads: fetched as FP32
@@ -1627,7 +1695,7 @@ __host__ __device__ constexpr int pk_ops(int d) { return 4 * ((d + 31) / 32) + 3
 // six times.  Their distances are recomputed in FP32 (PK_RG at a time, eight
 // lanes each) and decided as in the other selections: sure members
 // by their FP32 intervals, the rest by FP64 distance.  A row with more
-// candidates than `cap` is left to k_coarse_select (its number in `hard`).
+// candidates than `cap` is decided by the block (refine_rows).
 // 10,000 rows of 4,096 lists, P = 64: 165 us with k_coarse_dist against 580
 // (FP32 GEMM and block selection); 61 rows of 16,384 lists, P = 32: 43
 // against 118; 1,000 rows of 2,048 close lists, P = 64: 47 us, 121 when each
@@ -1641,21 +1709,35 @@ __host__ __device__ constexpr size_t pk_smem(int P)  // per warp: Dt, LB, UB, li
     return (size_t)pk_cap(P) * (4 + 4 + 4 + 4 + 8 + 4) + kMaxD * 4;
 }
 
-__global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const float *__restrict__ gmin,
-                                                              const float *__restrict__ cmaxes,
-                                                              int32_t *hard, int *nhard)
+// dot product of a row and a list's centroid, both spread over eight lanes
+__device__ __forceinline__ float pick_dot(const float4 (&xv)[4], const float4 (&cv)[4])
 {
-    pdl_begin();
-    extern __shared__ __align__(16) unsigned char pk[];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * CW_ROWS + w;
-    if (row >= a.m) return;  // whole warps
+    float dot = 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        dot = fmaf(xv[u].x, cv[u].x, dot);
+        dot = fmaf(xv[u].y, cv[u].y, dot);
+        dot = fmaf(xv[u].z, cv[u].z, dot);
+        dot = fmaf(xv[u].w, cv[u].w, dot);
+    }
+    dot += __shfl_xor_sync(0xffffffffu, dot, 4);
+    dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+    dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+    return dot;
+}
+
+// One row, by a warp (mem: pk_smem of it); false when it has more candidates than
+// the table holds.  FRESH: the distances are FP32 ones that this kernel has
+// written (other blocks of it, too), not to be computed again.
+template <bool FRESH>
+__device__ __forceinline__ bool pick_row(const SelArgs &a, int row, unsigned char *mem, int lane)
+{
+    auto ld = [](const float *p) { return FRESH ? __ldcg(p) : __ldg(p); };
     const int L = a.L, P = a.P, d = a.d, n4 = d >> 2, cap = pk_cap(P), G = (L + 15) / 16;
-    unsigned char *mem = pk + (size_t)w * pk_smem(P);
     double *sDx = reinterpret_cast<double *>(mem);
     float *sX = reinterpret_cast<float *>(sDx + cap), *sDt = sX + kMaxD, *sLB = sDt + cap, *sUB = sLB + cap;
     int *sIdx = reinterpret_cast<int *>(sUB + cap), *sSure = sIdx + cap;
-    const float *Dr = a.D + (size_t)row * L, *gr = gmin + (size_t)row * G;
+    const float *Dr = a.D + (size_t)row * L, *gr = a.gmin + (size_t)row * G;
     const float *xr = a.x + (size_t)row * d;
     float part = 0.f;
     for (int j = lane; j < d; j += 32) {
@@ -1664,13 +1746,12 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
         part = fmaf(v, v, part);
     }
     const float xn = norm_up(warp_sum(part), d);
-    const float b = kth_bound<32>([&](int i) { return i < G ? __ldg(gr + i) : INFINITY; },
+    const float b = kth_bound<32>([&](int i) { return i < G ? ld(gr + i) : INFINITY; },
                                   (G + 31) & ~31, P, lane);
-    const float cnmax = __ldg(cmaxes), cmax = __ldg(cmaxes + 1);
-    const float eb = bound_max(cnmax, abs_max(cnmax, xn, cmax), xn, cmax, a.gamma2_first);
-    // Dt - E <= T with T = b + Ebig needs Dt <= T + Ebig + its roundings
-    const float T0 = __fadd_ru(b, eb);
-    const float thr = __fadd_ru(__fadd_ru(T0, eb), __fadd_ru(__fmul_ru(fabsf(T0), 1.2e-7f), 1e-30f));
+    const float cnmax = __ldg(a.cmaxes), cmax = __ldg(a.cmaxes + 1);
+    const float eb = bound_max(cnmax, abs_max(cnmax, xn, cmax), xn, cmax,
+                               FRESH ? a.gamma2 : a.gamma2_first);
+    const float thr = pick_limit(b, eb);
     // the groups that can hold a candidate, then their lists: 4 lanes read a
     // group, 32 groups in flight
     int ng = 0, ns = 0;
@@ -1680,7 +1761,7 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int gi = g0 + 32 * u + lane;
-            v[u] = gi < G ? __ldg(gr + gi) : INFINITY;
+            v[u] = gi < G ? ld(gr + gi) : INFINITY;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -1701,14 +1782,15 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
             const int t = t0 + 8 * u + (lane >> 2);
             cl[u] = t < ng ? sGrp[t] * 16 + (lane & 3) * 4 : L;
             if (vec && cl[u] < L) {
-                const float4 f = __ldg(reinterpret_cast<const float4 *>(Dr + cl[u]));
+                const float4 *d4 = reinterpret_cast<const float4 *>(Dr + cl[u]);
+                const float4 f = FRESH ? __ldcg(d4) : __ldg(d4);
                 v[u][0] = f.x;
                 v[u][1] = f.y;
                 v[u][2] = f.z;
                 v[u][3] = f.w;
             } else {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) v[u][k] = cl[u] + k < L ? __ldg(Dr + cl[u] + k) : INFINITY;
+                for (int k = 0; k < 4; ++k) v[u][k] = cl[u] + k < L ? ld(Dr + cl[u] + k) : INFINITY;
             }
         }
 #pragma unroll
@@ -1723,17 +1805,21 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
             }
     }
     __syncwarp();
-    if (ng > cap || ns > cap || ns < P) {  // too many candidates (or no numbers): the block selection decides
-        if (lane == 0) hard[atomicAdd(nhard, 1)] = row;
-        return;
-    }
+    if (ng > cap || ns > cap || ns < P) return false;  // too many candidates (or no numbers)
     // FP32 distances and intervals: eight lanes a list, 16 lists in flight
     for (int p = lane; p < ns; p += 32) {
         sLB[p] = __ldg(a.cn + sIdx[p]);
         sUB[p] = __ldg(a.cnrm_up + sIdx[p]);
     }
     __syncwarp();
-    {
+    if (FRESH) {
+        for (int p = lane; p < ns; p += 32) {
+            const float Dt = ld(Dr + sIdx[p]), E = bound_of(Dt, sLB[p], sUB[p], xn, a.gamma2);
+            sDt[p] = Dt;
+            sLB[p] = lower_of(Dt, E);
+            sUB[p] = upper_of(Dt, E);
+        }
+    } else {
         const int g8 = lane >> 3, t8 = lane & 7;
         const float4 *x4 = reinterpret_cast<const float4 *>(sX);
         float4 xv[4];
@@ -1752,17 +1838,7 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
             }
 #pragma unroll
             for (int r = 0; r < PK_RG / 4; ++r) {
-                float dot = 0.f;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    dot = fmaf(xv[u].x, cv[r][u].x, dot);
-                    dot = fmaf(xv[u].y, cv[r][u].y, dot);
-                    dot = fmaf(xv[u].z, cv[r][u].z, dot);
-                    dot = fmaf(xv[u].w, cv[r][u].w, dot);
-                }
-                dot += __shfl_xor_sync(0xffffffffu, dot, 4);
-                dot += __shfl_xor_sync(0xffffffffu, dot, 2);
-                dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+                const float dot = pick_dot(xv, cv[r]);
                 const int p = p0 + 4 * r + g8;
                 if (t8 == 0 && p < ns) {
                     const float cnc = sLB[p], Dt = fmaf(-2.f, dot, cnc);
@@ -1810,7 +1886,12 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
             n += __popc(mk);
         }
         __syncwarp();
-        for (int t = lane; t < nb; t += 32) {
+        if (nb <= EX_FEW) {
+            const double D = exact_four(reinterpret_cast<const float4 *>(sX), a.cent,
+                                        [&](int m) { return sIdx[sBnd[m]]; }, nb, d, lane);
+            if (lane < nb) sDx[sBnd[lane]] = D;
+        }
+        for (int t = lane; t < nb && nb > EX_FEW; t += 32) {
             const int p = sBnd[t];
             sDx[p] = exact_dist4(reinterpret_cast<const float4 *>(sX),
                                  reinterpret_cast<const float4 *>(a.cent + (size_t)sIdx[p] * d), d);
@@ -1870,6 +1951,158 @@ __global__ __launch_bounds__(CW_ROWS * 32) void k_coarse_pick(SelArgs a, const f
         for (int q = 0; q < nsel; ++q) pos += (sDt[q] < dc) | ((sDt[q] == dc) & (sIdx[q] < c));  // no branches
         outr[pos] = c;
     }
+    return true;
+}
+
+// The rows of a block with more candidates than pick_row's table: the lists of a
+// row's cluster lie within the split's bound of its P-th by the hundred, but few
+// within FP32's.  Of the groups of 16 lists whose minimum is within that bound
+// for one of the rows, the distances and the minimum are written again in FP32
+// for all of them (the sums of k_coarse_gemm, bit for bit; the other groups'
+// lists cannot be chosen and keep theirs): a list per thread, the centroids
+// staged RF_K columns at a time.  pick_row then decides from them, a warp per
+// row, and the block rows that have more candidates even so (near-ties by the
+// hundred).  rows: the block's rows, -1 for the others.  10,000 rows of 2,048
+// lists in two clusters, P = 32: 0.73 ms, 11.8 by FP64 distances of all of them,
+// 0.98 by an FP32 matrix and a block per row.
+constexpr int PK_NT = CW_ROWS * 32;
+constexpr int RF_K = 16;           // columns staged at a time
+constexpr int RF_S = RF_K + 4;     // floats of a staged list: 16-byte reads without conflicts
+constexpr int RF_ST = 3;           // stages
+__host__ __device__ constexpr size_t pk_block_smem(int P, int G)
+{
+    const size_t stage = (size_t)RF_ST * PK_NT * RF_S * 4 + (size_t)G * 2, pick = (size_t)CW_ROWS * pk_smem(P);
+    const size_t most = stage > pick ? stage : pick;
+    return most > sizeof(SelTab) ? most : sizeof(SelTab);
+}
+__device__ __noinline__ void refine_rows(SelArgs a, const int *rows, int *left, unsigned char *mem)
+{
+    __shared__ __align__(16) float s_x[CW_ROWS][128];
+    __shared__ float s_thr[CW_ROWS];
+    __shared__ int s_ng;
+    float *sb = reinterpret_cast<float *>(mem);
+    uint16_t *grp = reinterpret_cast<uint16_t *>(sb + RF_ST * PK_NT * RF_S);  // the groups in reach
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int L = a.L, d = a.d, G = (L + 15) / 16;
+    a.two_level = 0;
+    {
+        float part = 0.f, thr = -INFINITY;
+        for (int j = lane; j < d; j += 32) {
+            const float v = rows[w] >= 0 ? a.x[(size_t)rows[w] * d + j] : 0.f;
+            s_x[w][j] = v;
+            part = fmaf(v, v, part);
+        }
+        if (rows[w] >= 0) {
+            const float *gr = a.gmin + (size_t)rows[w] * G;
+            const float xn = norm_up(warp_sum(part), d);
+            const float b = kth_bound<8>([&](int i) { return i < G ? __ldcg(gr + i) : INFINITY; },
+                                         (G + 31) & ~31, a.P, lane);
+            const float cnmax = __ldg(a.cmaxes), cmax = __ldg(a.cmaxes + 1);
+            thr = pick_limit(b, bound_max(cnmax, abs_max(cnmax, xn, cmax), xn, cmax, a.gamma2_first));
+        }
+        if (lane == 0) s_thr[w] = thr;
+        if (tid == 0) s_ng = 0;
+    }
+    __syncthreads();
+    for (int g0 = w * 32; g0 < G; g0 += PK_NT) {  // whole warps
+        const int g = g0 + lane;
+        bool on = false;
+        if (g < G)
+#pragma unroll
+            for (int r = 0; r < CW_ROWS; ++r)
+                if (rows[r] >= 0) on = on || !(__ldcg(a.gmin + (size_t)rows[r] * G + g) > s_thr[r]);
+        const uint32_t mk = __ballot_sync(0xffffffffu, on);
+        int at = 0;
+        if (lane == 0 && mk) at = atomicAdd(&s_ng, __popc(mk));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(mk & lanemask_lt());
+        if (on) grp[at] = (uint16_t)g;
+    }
+    __syncthreads();
+    const int ng = s_ng;
+    // steps of RF_K columns of PK_NT lists (eight groups), RF_ST - 1 in flight
+    int fi = 0, fk = 0, fs = 0;  // the next step to fetch: its first group, columns, stage
+    auto fetch = [&]() {
+        if (fi < ng) {
+            float *to = sb + fs * PK_NT * RF_S;
+#pragma unroll
+            for (int u = 0; u < RF_K / 4; ++u) {
+                const int r = (tid >> 2) + 32 * u, q = tid & 3;
+                const int c = min((int)grp[min(fi + (r >> 4), ng - 1)] * 16 + (r & 15), L - 1);
+                cp_async16_c(to + r * RF_S + 4 * q, a.cent + (size_t)c * d + fk + 4 * q, 16u);
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        fs = fs + 1 == RF_ST ? 0 : fs + 1;
+        fk += RF_K;
+        if (fk >= d) {
+            fk = 0;
+            fi += PK_NT / 16;
+        }
+    };
+#pragma unroll
+    for (int st = 0; st < RF_ST - 1; ++st) fetch();
+    int stage = 0;
+    for (int i = 0; i < ng; i += PK_NT / 16) {
+        float acc[CW_ROWS];
+#pragma unroll
+        for (int r = 0; r < CW_ROWS; ++r) acc[r] = 0.f;
+        for (int k0 = 0; k0 < d; k0 += RF_K) {
+            asm volatile("cp.async.wait_group %0;\n" ::"n"(RF_ST - 2) : "memory");
+            __syncthreads();  // this step has landed, the last one's stage has been read
+            fetch();
+            const float *sc = sb + (stage * PK_NT + tid) * RF_S;
+            stage = stage + 1 == RF_ST ? 0 : stage + 1;
+            float4 cv[RF_K / 4];
+#pragma unroll
+            for (int q = 0; q < RF_K / 4; ++q) cv[q] = *reinterpret_cast<const float4 *>(sc + 4 * q);
+#pragma unroll
+            for (int r = 0; r < CW_ROWS; ++r) {
+                if (rows[r] < 0) continue;
+#pragma unroll
+                for (int q = 0; q < RF_K / 4; ++q) {
+                    const float4 xv = *reinterpret_cast<const float4 *>(&s_x[r][k0 + 4 * q]);
+                    acc[r] = fmaf(xv.x, cv[q].x, acc[r]);
+                    acc[r] = fmaf(xv.y, cv[q].y, acc[r]);
+                    acc[r] = fmaf(xv.z, cv[q].z, acc[r]);
+                    acc[r] = fmaf(xv.w, cv[q].w, acc[r]);
+                }
+            }
+        }
+        const int at = i + (tid >> 4), g = at < ng ? grp[at] : 0, c = at < ng ? g * 16 + (tid & 15) : L;
+        const float cnc = c < L ? __ldg(a.cn + c) : 0.f;
+#pragma unroll
+        for (int r = 0; r < CW_ROWS; ++r) {
+            const float Dt = fmaf(-2.f, acc[r], cnc);
+            float mn = c < L ? Dt : INFINITY;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            if (rows[r] >= 0 && c < L) {
+                a.Dw[(size_t)rows[r] * L + c] = Dt;
+                if ((tid & 15) == 0) a.gmin[(size_t)rows[r] * G + g] = mn;
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();  // the rows are written; the stages have been read
+    bool ok = true;
+    if (rows[w] >= 0) ok = pick_row<true>(a, rows[w], mem + (size_t)w * pk_smem(a.P), lane);
+    if (lane == 0) left[w] = !ok;
+    __syncthreads();
+    for (int r = 0; r < CW_ROWS; ++r)
+        if (left[r]) select_row<PK_NT, true>(a, rows[r], *reinterpret_cast<SelTab *>(mem));
+}
+
+// rpb rows per block, a warp each (fewer rows: one, so that a block refines one)
+__global__ __launch_bounds__(PK_NT, 5) void k_coarse_pick(SelArgs a, int rpb)
+{
+    pdl_begin();
+    extern __shared__ __align__(16) unsigned char pk[];
+    __shared__ int s_rows[CW_ROWS], s_left[CW_ROWS];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row = w < rpb ? blockIdx.x * rpb + w : a.m;
+    const bool ok = row >= a.m || pick_row<false>(a, row, pk + (size_t)w * pk_smem(a.P), lane);
+    if (lane == 0) s_rows[w] = ok ? -1 : row;
+    if (__syncthreads_or(!ok)) refine_rows(a, s_rows, s_left, pk);
 }
 
 // Finishing selection of the rows the fused first stage left undecided (P =
@@ -2268,10 +2501,12 @@ int first_stage_split(const sivf_index *ix, int P)
 
 // Probe selection by k_coarse_dist and k_coarse_pick: P lists need twice as
 // many groups of 16 for the group minima to bound them well (L >= 32 P); the
-// warp's candidate table holds P <= 128.
+// warp's candidate table holds P <= 128.  Few short rows to select from are read
+// whole as fast (10,000 rows of 512 lists, d = 32, P = 2: 51 us, 60 by the pick).
 bool coarse_picks(const sivf_index *ix, int P)
 {
-    return P >= 2 && P <= PK_PMAX && ix->tmap_cent_ok && (int64_t)ix->nlist >= 32 * (int64_t)P;
+    if (P < 2 || P > PK_PMAX || !ix->tmap_cent_ok || (int64_t)ix->nlist < 32 * (int64_t)P) return false;
+    return P > CW_PMAX || (int64_t)ix->nlist * ix->d >= 32768;
 }
 
 // rows [0, m) of x -> out[m, P]; `Dbuf` holds at least `room` floats, L of
@@ -2283,8 +2518,8 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
     const double u = 5.9604644775390625e-08;
     const double gd = d * u / (1.0 - d * u);
     const bool warp_rows = P <= CW_PMAX && L <= CW_LMAX;
-    // row numbers, distances and group minima of at least one row
-    const int64_t pick_row = 1 + L + (L + 15) / 16;
+    // distances and group minima of at least one row
+    const int64_t pick_row = L + (L + 15) / 16;
     const bool pick = coarse_picks(ix, P) && room >= CF_HDR + pick_row;
     const int split = pick ? 3 : first_stage_split(ix, P);
     const bool two = split != 0;
@@ -2310,17 +2545,15 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
     for (int64_t r0 = 0; r0 < m; r0 += rows) {
         int mc = (int)std::min<int64_t>(rows, m - r0);
         const int cap = fused ? (int)std::min<int64_t>((room - CF_HDR - mc) / CF_STRIDE, mc) : 0;
-        const int tok = prof_begin(ix, PROF_COARSE, pick ? 3 : 2, st);
+        const int tok = prof_begin(ix, PROF_COARSE, 2, st);
         // the distance buffer of the fused stage: the number of undecided
-        // rows, those rows, the records; of the pick: the number of rows left
-        // to the block selection, the distances, the group minima, those rows
+        // rows, those rows, the records; of the pick: the distances and the
+        // group minima
         int32_t *nh = reinterpret_cast<int32_t *>(Dbuf), *rec = nh + CF_HDR + mc;
         float *Dm = pick ? Dbuf + CF_HDR : Dbuf, *gm = Dm + (size_t)mc * L;
-        int32_t *left = reinterpret_cast<int32_t *>(gm + (size_t)mc * ((L + 15) / 16));
         if (pick) {
             const int KC = d <= 64 ? 1 : 2;
             const size_t smem = coarse_fused_smem(KC, 2);
-            cudaMemsetAsync(nh, 0, sizeof(int32_t), st);
             const int nt = (mc + CT_M - 1) / CT_M, nch = (L + CF_CN - 1) / CF_CN;
             const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent);
             const CUtensorMap &tl = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent_lo);
@@ -2391,7 +2624,7 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         }
         SelArgs a;
         a.D = fused ? nullptr : Dm;
-        a.hard = fused ? nh + CF_HDR : pick ? left : nullptr;
+        a.hard = fused ? nh + CF_HDR : nullptr;
         a.nhard = nh;
         a.S = rec;
         a.s_cap = cap;
@@ -2409,13 +2642,15 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         const double gr = ro * u / (1.0 - ro * u);
         a.gamma2_re = (float)(2.0 * gr * (1.0 + 1e-6));
         a.two_level = two;
+        a.Dw = pick ? Dm : nullptr;
+        a.gmin = pick ? gm : nullptr;
+        a.cmaxes = ix->cmax;
         a.out = out + r0 * P;
         a.err = ix->err;
         if (pick) {
-            const size_t smem = CW_ROWS * pk_smem(P);  // 32 KB at P = 128
-            launch_pdl(k_coarse_pick, (unsigned)((mc + CW_ROWS - 1) / CW_ROWS), CW_ROWS * 32, smem, st,
-                       a, gm, ix->cmax, left, nh);
-            launch_pdl(k_coarse_select, std::min(mc, nsm), SEL_NT, 0, st, a);
+            const int rpb = mc <= 4 * nsm ? 1 : CW_ROWS;
+            launch_pdl(k_coarse_pick, (unsigned)((mc + rpb - 1) / rpb), PK_NT,
+                       pk_block_smem(P, (L + 15) / 16), st, a, rpb);
         } else if (warp_rows) {
             const unsigned gw = (unsigned)((mc + CW_ROWS - 1) / CW_ROWS);
             if (fused)  // loops over the undecided rows

@@ -167,10 +167,9 @@ struct SelArgs {
     float gamma2_first;    // the same factor for the first-stage distances D
     float gamma2_re;       // and for FP32 dot products summed across a warp (re_ops)
     int two_level;         // D is the BF16 tensor-core stage: recheck S in FP32
-    const int32_t *hard;   // k_coarse_finish: the rows the fused first stage left
-    const int *nhard;      // undecided, those with a record from the front, those to
-    const int32_t *S;      // redo from the back (two counters, on the device), and
-    int s_cap;             // the first kind's records (room for s_cap): [n, lists...]
+    const int *nhard;      // k_coarse_finish: how many records (on the device), and the
+    const int32_t *S;      // records [row, n, lists...] of the rows the fused first stage
+    int s_cap;             // left undecided (room for s_cap)
     float *Dw;             // refine_rows: the same distances, to be rewritten
     float *gmin;           // [m, groups of 16 lists] the distances' group minima
     const float *cmaxes;   // the largest ||c||^2 and ||c||
@@ -720,33 +719,43 @@ __global__ __launch_bounds__(CT_NT, 1) void k_coarse_tc(const float *__restrict_
 // Per group of 16 lists a thread takes the smallest and second smallest Dt,
 // the list's place in the group carried in the key's low four mantissa bits
 // (a relative change below 2^-19 of Dt), and keeps the best three groups and
-// the fourth's minimum.  With Amax >= |Dt| (max ||c||^2 + 2.04 ||x|| max ||c||: the parts' roundings included),
-// Ebig >= E_c for every c (the bound of the selection evaluated at max
-// ||c||^2, Amax and max ||c||, rounded up) and delta >= the key error,
-// T = min key + delta + Ebig is >= the smallest upper bound Dt_c + E_c, and
-// a list can belong to the selection's set S only if its key is at most
-// thr = T + Ebig + delta plus one unit in the last place of T (rounded up).
-// A row whose second smallest key is above thr has its argmin as the answer.
-// Any other row is appended to `hard` with a record of the lists that can
-// qualify (a group's 16 lists when its second is within thr), or, when they
-// are more than CF_CAP, a thread's fourth group is within thr or the records
-// are full, to the rows to redo from all lists (hard's end, downwards).
+// the fourth's minimum.  With Amax >= |Dt| (max ||c||^2 + 2.04 ||x|| max ||c||:
+// the parts' roundings included), Ebig >= E_c for every c (the bound of the
+// selection evaluated at max ||c||^2, Amax and max ||c||, rounded up) and delta
+// >= the key error, T = min key + delta + Ebig is >= the smallest upper bound
+// Dt_c + E_c, and a list can belong to the selection's set S only if its key is
+// at most thr = T + Ebig + delta plus one unit in the last place of T (rounded
+// up).  A row whose second smallest key is above thr has its argmin as the
+// answer.  Any other row gets a record of the lists that can qualify (a group's
+// 16 lists when its second is within thr) for k_coarse_finish, or, when they are
+// more than CF_CAP, a thread's fourth group is within thr or the records are
+// full, a place on its CTA's list of rows for the second pass.
 // ||x|| is bounded from the FP32 sum of squares s of the tile's rows
 // (relative error <= d u) as RU(sqrt(RU(s (1 + 4 d u)))).
+//
+// Second pass.  Several lists in one cluster are closer together than the
+// products' error, so that many lists in many groups can qualify: most rows of
+// the single product there, a tenth of the split's.  When its tiles are done,
+// the CTA gathers those rows into tiles of their own and lets the centroids
+// pass twice more, in the split form whichever form the first pass took: once
+// for the smallest Dt of each row, once for a bit per list within thr, which
+// k_coarse_finish decides from, however many they are.
 //
 // What bounds it: the epilogue's min/max and selects (4.3 half-rate
 // operations per list and row); a chunk's MMAs and its copy from L2 run
 // under it.  1,000,000 rows, 1,024 lists, d = 128: 526 us, 1,190 in launches
 // of one tile per CTA and two passes over the centroids; the split stage,
 // 200,000 rows: 141 us + 36 us to finish the undecided rows, 1,580 us when
-// the matrix of distances was written and read back.
+// the matrix of distances was written and read back.  With the second pass,
+// 200,000 rows of 512 trained lists in 16 clusters: 0.70 ms, 10.3 when the rows
+// without a record were recomputed from every list, 2.3 by the matrix.
 constexpr int CF_CAP = 32;                  // lists of one undecided row's record
 constexpr int CF_SUB = 4;                   // threads per row
-constexpr int CF_STRIDE = CF_CAP + 1;       // ints per record: n, lists
+constexpr int CF_STRIDE = CF_CAP + 2;       // ints per record: row, n, lists
 constexpr int CF_EPI = 128 * CF_SUB;        // epilogue threads
 constexpr int CF_NT = CF_EPI + 64;          // + the MMA warp and the copy warp
-constexpr int CF_HDR = 8;                   // ints (32 bytes) before the undecided rows: how many have
-                                            // a record, how many are to be redone
+constexpr int CF_HDR = 8;                   // ints (32 bytes) before the rows: how many records, how
+                                            // many rows with bits
 constexpr int CF_CN = 128;                  // centroids of a chunk (and of a TMA box)
 constexpr int CF_TB = 4;                    // TMEM buffers
 constexpr int CF_LMIN = 16;                 // fewer lists take the matrix form
@@ -754,10 +763,10 @@ constexpr int CF_LMIN = 16;                 // fewer lists take the matrix form
 constexpr int CW_LMAX = 4096;  // most lists of the fused stage and of one warp per row
 
 __host__ __device__ constexpr int cf_buffers(int parts) { return parts == 1 ? 4 : 2; }
-__host__ __device__ inline size_t coarse_fused_smem(int KC, int parts)
+__host__ __device__ inline size_t coarse_fused_smem(int KC)
 {
-    // A (parts), the chunk buffers (parts each), ||c||^2
-    return (size_t)KC * parts * (CT_M + cf_buffers(parts) * CF_CN) * 128 + CW_LMAX * 4 + 1024;
+    // both parts of A, two chunk buffers of both parts (or four of one), ||c||^2
+    return (size_t)KC * 2 * (CT_M + cf_buffers(2) * CF_CN) * 128 + CW_LMAX * 4 + 1024;
 }
 
 // Amax and Ebig: a bound of every |Dt| (the parts' roundings included), and
@@ -798,13 +807,15 @@ struct RowTile {
     static constexpr int W = KC * 8;              // 16-byte chunks of a row
     static constexpr int AU = CT_M * W / CF_EPI;  // chunks per thread: 2 KC
     float4 f0[AU], f1[AU];
-    __device__ __forceinline__ void fetch(const float *__restrict__ x, int row0, int m, int d, int tid)
+    // row_of(r): the row of x in the tile's place r, -1 for none
+    template <class R>
+    __device__ __forceinline__ void fetch(const float *__restrict__ x, R row_of, int d, int tid)
     {
 #pragma unroll
         for (int u = 0; u < AU; ++u) {
-            const int e = tid + u * CF_EPI, row = row0 + e / W, k0 = (e & (W - 1)) * 8;
+            const int e = tid + u * CF_EPI, row = row_of(e / W), k0 = (e & (W - 1)) * 8;
             f0[u] = f1[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row < m && k0 < d) {
+            if (row >= 0 && k0 < d) {
                 const float4 *xr = reinterpret_cast<const float4 *>(x + (size_t)row * d + k0);
                 f0[u] = __ldg(xr);
                 f1[u] = __ldg(xr + 1);
@@ -846,12 +857,296 @@ struct RowTile {
     }
 };
 
+// The nearest of a row's candidate lists (one warp; d <= 128: one float4 of the
+// row per lane).  The FP32 distances of up to ND_WIN lists at a time (ND_RG in
+// flight); those whose lower bound is at most the smallest upper bound so far
+// stay for the next window, and of the last that stay, when they are several,
+// the FP64 distances decide (ties to the lower index).  fill(at, w0) writes the
+// candidates' numbers from the w0-th on to tab[at, ND_WIN) and returns how many
+// there are in all.  tab, lbs: ND_WIN entries of the warp's shared memory.  -1
+// when no list qualifies.
+constexpr int ND_WIN = 64;
+constexpr int ND_RG = 8;
+struct NearArgs {
+    const float *cent, *cn, *cnrm_up;
+    float gamma_re;      // bound_of's factor of FP32 dot products summed across a warp
+};
+template <class Fill>
+__device__ __forceinline__ int decide_nearest(const NearArgs &a, Fill fill, int d, const float *xr,
+                                              float xn, int *tab, float *lbs, int lane)
+{
+    const int n4 = d >> 2;
+    const float4 *x4 = reinterpret_cast<const float4 *>(xr);
+    const float4 xv = lane < n4 ? __ldg(x4 + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+    double bd = INFINITY;  // the best by FP64 distance and index
+    int bc = 0x7fffffff;
+    bool exact = false;    // some were decided by FP64 distance
+    // the FP64 distances of the k lists in the table, next to each other: a pass
+    // costs the same for one as for 32
+    auto decide = [&](int k) {
+        auto take = [&](double D, int c) {
+            if (D < bd || (D == bd && c < bc)) {
+                bd = D;
+                bc = c;
+            }
+        };
+        if (k <= EX_FEW) {
+            const double D = exact_four(x4, a.cent, [&](int m) { return tab[m]; }, k, d, lane);
+            if (lane < k) take(D, tab[lane]);
+        } else {
+            for (int p = lane; p < k; p += 32)
+                take(exact_dist4(x4, reinterpret_cast<const float4 *>(a.cent + (size_t)tab[p] * d), d), tab[p]);
+        }
+        exact = true;
+        __syncwarp();
+    };
+    int total = fill(0, 0), k = 0;  // k: lists that stay
+    if (total == 0) return -1;
+    if (total == 1) return tab[0];
+    float T = INFINITY;
+    for (int w0 = 0; w0 < total;) {
+        const int n = k + min(total - w0, ND_WIN - k);
+        if (w0 > 0) fill(k, w0);
+        w0 += n - k;
+        for (int p0 = k; p0 < n; p0 += ND_RG) {
+            float s[ND_RG];
+#pragma unroll
+            for (int t = 0; t < ND_RG; ++t) {
+                const float4 *c4 = reinterpret_cast<const float4 *>(a.cent + (size_t)tab[min(p0 + t, n - 1)] * d);
+                const float4 cv = lane < n4 ? __ldg(c4 + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+                s[t] = fmaf(xv.w, cv.w, fmaf(xv.z, cv.z, fmaf(xv.y, cv.y, xv.x * cv.x)));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int t = 0; t < ND_RG; ++t) s[t] += __shfl_xor_sync(0xffffffffu, s[t], o);
+            float dot = s[0];
+#pragma unroll
+            for (int t = 1; t < ND_RG; ++t)
+                if (lane == t) dot = s[t];
+            if (lane < ND_RG && p0 + lane < n) {
+                const int c = tab[p0 + lane];
+                const float cnc = __ldg(a.cn + c), Dt = fmaf(-2.f, dot, cnc);
+                const float E = bound_of(Dt, cnc, __ldg(a.cnrm_up + c), xn, a.gamma_re);
+                lbs[p0 + lane] = lower_of(Dt, E);
+                T = fminf(T, upper_of(Dt, E));
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) T = fminf(T, __shfl_xor_sync(0xffffffffu, T, o));
+        __syncwarp();
+        k = 0;
+        for (int p0 = 0; p0 < n; p0 += 32) {  // every place is at most the one it is read from
+            const bool in = p0 + lane < n && lbs[p0 + lane] <= T;
+            const int c = in ? tab[p0 + lane] : 0;
+            const float lb = in ? lbs[p0 + lane] : 0.f;
+            const uint32_t mk = __ballot_sync(0xffffffffu, in);
+            __syncwarp();
+            if (in) {
+                tab[k + __popc(mk & lanemask_lt())] = c;
+                lbs[k + __popc(mk & lanemask_lt())] = lb;
+            }
+            k += __popc(mk);
+            __syncwarp();
+        }
+        if (k > ND_WIN / 2 && w0 < total) {  // room for the next window
+            decide(k);
+            k = 0;
+        }
+    }
+    if (!exact && k <= 1) return k == 1 ? tab[0] : -1;
+    if (k > 0) decide(k);
+    for (int o = 16; o > 0; o >>= 1) {
+        const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+        const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
+        if (od < bd || (od == bd && oc < bc)) {
+            bd = od;
+            bc = oc;
+        }
+    }
+    return bc;
+}
+
+// Second pass of the fused stage: arguments, barriers, the pass itself.
+struct SecondArgs {
+    int32_t *rows;       // [m] the rows of each CTA's list (second_place)
+    int32_t *list;       // [m] the places of those whose bits are written, and
+    int *n;              // how many
+    uint16_t *bits;      // [m / 128][groups of 16 lists][stride] lists within thr, by place
+    int stride;          // rows of a tile: 128, or all there are
+    float gamma;         // the split products' factor in bound_of
+};
+// where a CTA keeps the p-th row of its list: as far down its own tiles
+__device__ __forceinline__ int second_place(int p)
+{
+    return (int)(blockIdx.x + (uint32_t)(p >> 7) * gridDim.x) * CT_M + (p & 127);
+}
+struct SecondBars {
+    uint64_t fullb[2], freeb[2], mmab[CF_TB], tempty[CF_TB], afull;
+    __device__ void init()
+    {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&fullb[i], 1);
+            mbar_init(&freeb[i], 1);
+        }
+        for (int i = 0; i < CF_TB; ++i) {
+            mbar_init(&mmab[i], 1);
+            mbar_init(&tempty[i], CF_EPI / 32);
+        }
+        mbar_init(&afull, CF_EPI / 32);
+    }
+};
+
+template <int KC>
+__device__ __noinline__ void second_pass(const CUtensorMap &tmB, const CUtensorMap &tmBlo,
+                                         const float *__restrict__ x, int d, int L, int n,
+                                         const SecondArgs &a, int32_t *__restrict__ out1,
+                                         unsigned char *A, unsigned char *B, const float *scn,
+                                         const float *cmaxes, uint32_t tbase, SecondBars &bar,
+                                         volatile int *s_abort, float *sxn, float (*sMin)[CT_M],
+                                         int *srow, uint32_t *err)
+{
+    constexpr int CN = CF_CN, NB = 2, TB = CF_TB;
+    constexpr uint32_t PBYTES = KC * CN * 128, BBYTES = 2 * PBYTES, ABYTES = KC * CT_M * 128;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nch = (L + CN - 1) / CN, ntiles = (n + CT_M - 1) / CT_M, G = (L + 15) / 16;
+    const uint32_t steps = (uint32_t)ntiles * 2u * (uint32_t)nch;
+    if (warp == CF_EPI / 32 + 1) {
+        // ---- copies (one lane)
+        if (lane == 0) {
+            uint32_t g = 0;
+            for (; g < steps; ++g) {
+                const uint32_t b = g % NB, u = g / NB;
+                if (u >= 1 && !mbar_wait_ab(&bar.freeb[b], (u - 1) & 1, err, s_abort, kWaitNs)) break;
+                const int j = (int)(g % (uint32_t)nch);
+                mbar_arrive_expect_tx(&bar.fullb[b], BBYTES);
+#pragma unroll
+                for (int pp = 0; pp < 2; ++pp)
+#pragma unroll
+                    for (int kc = 0; kc < KC; ++kc)
+                        tma_load_2d(B + b * BBYTES + pp * PBYTES + (size_t)kc * CN * 128,
+                                    pp ? &tmBlo : &tmB, kc * 64, j * CN, &bar.fullb[b]);
+            }
+            for (uint32_t t = g > NB ? g - NB : 0; t < g; ++t)  // landed before exit
+                mbar_wait_bounded(&bar.fullb[t % NB], (t / NB) & 1, err);
+        }
+        __syncwarp();
+    } else if (warp == CF_EPI / 32) {
+        // ---- MMAs (one lane)
+        if (lane == 0) {
+            const uint32_t idesc = mma_idesc(1, 1, CT_M, CN), abase = smem_u32(A);
+            uint32_t g = 0;
+            for (; g < steps; ++g) {
+                const uint32_t b = g % NB, tb = g % TB, ut = g / TB;
+                bool ok = mbar_wait_ab(&bar.fullb[b], (g / NB) & 1, err, s_abort, kWaitNs);
+                if (ok && g % (2u * (uint32_t)nch) == 0)  // the tile's rows are stored
+                    ok = mbar_wait_ab(&bar.afull, (g / (2u * (uint32_t)nch)) & 1, err, s_abort, kWaitNs);
+                if (ok && ut >= 1) ok = mbar_wait_ab(&bar.tempty[tb], (ut - 1) & 1, err, s_abort, kWaitNs);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t bbase = smem_u32(B + b * BBYTES);
+#pragma unroll
+                for (int pr = 0; pr < 3; ++pr) {  // (x hi, c hi), (x hi, c lo), (x lo, c hi)
+                    const uint32_t ap = abase + (pr == 2 ? ABYTES : 0u);
+                    const uint32_t bp = bbase + (pr == 1 ? PBYTES : 0u);
+#pragma unroll
+                    for (int kc = 0; kc < KC; ++kc)
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_bf16(tbase + tb * CN,
+                                     smem_desc_sw128(ap + kc * CT_M * 128 + ks * 32, 1024),
+                                     smem_desc_sw128(bp + kc * CN * 128 + ks * 32, 1024), idesc,
+                                     (pr | kc | ks) != 0);
+                }
+                mma_commit(&bar.freeb[b]);
+                mma_commit(&bar.mmab[tb]);
+            }
+            if (g > 0) mbar_wait_bounded(&bar.mmab[(g - 1) % TB], ((g - 1) / TB) & 1, err);
+        }
+        __syncwarp();
+    } else {
+        // ---- rows in, epilogue
+        const int q = warp & 3, sub = warp >> 2, rloc = q * 32 + lane;
+        const float cnmax = __ldg(cmaxes), cmax = __ldg(cmaxes + 1);
+        uint32_t g = 0;
+        bool ok = true;
+        RowTile<KC, 2> rows;
+        for (int t = 0; t < ntiles; ++t) {
+            const int nrow = min(CT_M, n - t * CT_M), place = second_place(t * CT_M);
+            uint16_t *bits = a.bits + (size_t)(place >> 7) * G * a.stride;
+            if (tid < CT_M) srow[tid] = tid < nrow ? a.rows[second_place(t * CT_M + tid)] : -1;
+            named_bar_sync(1, CF_EPI);
+            rows.fetch(x, [&](int r) { return srow[r]; }, d, tid);
+            rows.store(A, ABYTES, d, tid, sxn);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar.afull);
+            float mn = INFINITY, thr = 0.f;
+            for (int pass = 0; pass < 2; ++pass) {
+                for (int j = 0; j < nch; ++j, ++g) {
+                    const uint32_t tb = g % TB;
+                    ok = __all_sync(0xffffffffu, ok && mbar_wait_ab(&bar.mmab[tb], (g / TB) & 1, err,
+                                                                    s_abort, kWaitNs));
+                    tc_fence_after();
+                    if (ok) {
+                        const uint32_t tad = tbase + tb * CN + sub * 16 + ((uint32_t)(q * 32) << 16);
+#pragma unroll
+                        for (int k = 0; k < CN / 64; ++k) {
+                            const int grp = j * (CN / 16) + sub + 4 * k;
+                            const float4 *cv4 = reinterpret_cast<const float4 *>(scn + grp * 16);
+                            float v[16];
+                            tmem_ld16(tad + k * 64, v);
+                            tmem_ld_wait(v);
+                            uint32_t within = 0u;
+#pragma unroll
+                            for (int i4 = 0; i4 < 4; ++i4) {
+                                const float4 cv = cv4[i4];
+                                const float c4[4] = {cv.x, cv.y, cv.z, cv.w};
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    const float Dt = fmaf(-2.f, v[4 * i4 + i], c4[i]);
+                                    if (pass == 0) mn = fminf(mn, Dt);
+                                    else if (Dt <= thr) within |= 1u << (4 * i4 + i);
+                                }
+                            }
+                            if (pass == 1 && grp < G && rloc < nrow) {
+                                if (L - grp * 16 < 16) within &= (1u << (L - grp * 16)) - 1u;
+                                bits[(size_t)grp * a.stride + rloc] = (uint16_t)within;
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar.tempty[tb]);
+                }
+                if (pass == 0) {
+                    sMin[sub][rloc] = mn;
+                    ok = named_bar_and(1, CF_EPI, ok && !*s_abort);
+                    if (!ok) break;
+                    mn = fminf(fminf(sMin[0][rloc], sMin[1][rloc]), fminf(sMin[2][rloc], sMin[3][rloc]));
+                    const float xn = sxn[rloc];
+                    const float eb = bound_max(cnmax, abs_max(cnmax, xn, cmax), xn, cmax, a.gamma);
+                    thr = pick_limit(mn, eb);
+                }
+            }
+            if (ok) ok = named_bar_and(1, CF_EPI, ok && !*s_abort);
+            if (!ok) {
+                // a wait ran out (the sticky error word is set): list 0 for the rows left
+                for (int p = t * CT_M + tid; p < n; p += CF_EPI) out1[a.rows[second_place(p)]] = 0;
+                break;
+            }
+            if (tid < nrow) a.list[atomicAdd(a.n, 1)] = place + tid;
+            named_bar_sync(1, CF_EPI);  // srow, sxn and sMin are reused
+        }
+    }
+}
+
 template <int KC, int PARTS>
 __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
     const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBlo,
     const float *__restrict__ x, int m, int d, const float *__restrict__ cn,
     const float *__restrict__ cmaxes, int L, float g1, int32_t *__restrict__ out1,
-    int32_t *__restrict__ outS, int cap, int32_t *__restrict__ hard, int *nhard, uint32_t *err)
+    int32_t *__restrict__ outS, int cap, int *nhard, const __grid_constant__ SecondArgs sp,
+    uint32_t *err)
 {
     pdl_begin();
     constexpr int CN = CF_CN, NB = cf_buffers(PARTS), TB = CF_TB;
@@ -860,14 +1155,15 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
     constexpr uint32_t ABYTES = KC * CT_M * 128;  // one part of the row tile
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-    unsigned char *A = smem;                               // PARTS x KC x 128 rows x 128 B
-    unsigned char *B = smem + PARTS * ABYTES;              // NB x PARTS x KC x CN rows x 128 B
+    unsigned char *A = smem;                               // 2 x KC x 128 rows x 128 B
+    unsigned char *B = smem + 2 * ABYTES;                  // NB x PARTS x KC x CN rows x 128 B
     float *scn = reinterpret_cast<float *>(B + NB * BBYTES);
     // chunk copied, chunk read (both per chunk buffer), products ready,
     // products read (per TMEM buffer), row tile stored
     __shared__ uint64_t fullb[NB], freeb[NB], mmab[TB], tempty[TB], afull;
+    __shared__ SecondBars bars2;
     __shared__ uint32_t tmem_base;
-    __shared__ int s_abort_;
+    __shared__ int s_abort_, s_second;  // s_second: rows left to the second pass
     volatile int *s_abort = &s_abort_;
     // by tile parity: the row's norm, and each thread's best key, its list,
     // the best key of its other lists, and its candidate count
@@ -884,8 +1180,10 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
             mbar_init(&tempty[i], CF_EPI / 32);
         }
         mbar_init(&afull, CF_EPI / 32);
+        bars2.init();
         fence_mbar_init();
         s_abort_ = 0;
+        s_second = 0;
     }
     if (warp == CF_EPI / 32) tmem_alloc(&tmem_base, TB * CN);
     tc_fence_before();
@@ -959,7 +1257,9 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
         // ---- rows in, epilogue
         const int q = warp & 3, sub = warp >> 2, rloc = q * 32 + lane;
         RowTile<KC, PARTS> rows;
-        auto fetch = [&](int tile) { rows.fetch(x, tile * CT_M, m, d, tid); };
+        auto fetch = [&](int tile) {
+            rows.fetch(x, [&](int r) { return tile * CT_M + r < m ? tile * CT_M + r : -1; }, d, tid);
+        };
         auto store = [&](int par) {
             rows.store(A, ABYTES, d, tid, sxn[par]);
             fence_proxy_async_smem();  // A (generic stores) is read by the MMAs
@@ -1115,10 +1415,10 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
                         if (redo) h = -1;
                     }
                     if (redo) {
-                        hard[m - 1 - atomicAdd(nhard + 1, 1)] = row;
+                        sp.rows[second_place(atomicAdd(&s_second, 1))] = row;
                     } else {
-                        hard[h] = row;
-                        outS[(size_t)h * CF_STRIDE] = total;
+                        outS[(size_t)h * CF_STRIDE] = row;
+                        outS[(size_t)h * CF_STRIDE + 1] = total;
                     }
                 }
             }
@@ -1127,7 +1427,7 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
             if (!decided && row < m) {
                 h = sArg[par][0][rloc];
                 if (h >= 0) {
-                    int32_t *o = outS + (size_t)h * CF_STRIDE + 1 + before;
+                    int32_t *o = outS + (size_t)h * CF_STRIDE + 2 + before;
 #pragma unroll
                     for (int i = 0; i < 3; ++i) {
                         const bool whole = sg[i] <= thr;
@@ -1137,6 +1437,16 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_fused(
                 }
             }
         }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const int nsecond = s_second;
+    if (nsecond > 0 && !s_abort_) {
+        second_pass<KC>(tmB, tmBlo, x, d, L, nsecond, sp, out1, A, B, scn, cmaxes, tbase, bars2,
+                        s_abort, sxn[0], sMin[0], &sn[0][0], err);
+    } else if (nsecond > 0 && tid < CF_EPI) {  // a wait ran out: list 0, as above
+        for (int p = tid; p < nsecond; p += CF_EPI) out1[sp.rows[second_place(p)]] = 0;
     }
     tc_fence_before();
     __syncthreads();
@@ -1256,7 +1566,10 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
             __syncwarp();
             if (lane == 0) mbar_arrive(&afull);
         };
-        rows.fetch(x, tile0 * CT_M, m, d, tid);
+        auto fetch = [&](int t) {
+            rows.fetch(x, [&](int r) { return t * CT_M + r < m ? t * CT_M + r : -1; }, d, tid);
+        };
+        fetch(tile0);
         store();
         const int G = (L + 15) / 16;
         // whole sectors where the rows are aligned to them
@@ -1269,7 +1582,7 @@ __global__ __launch_bounds__(CF_NT, 1) void k_coarse_dist(
             const int jn = j, row = tile * CT_M + q * 32 + lane;
             // the next tile's rows, if this CTA's range goes on into it
             const bool more = (uint32_t)(nch - j) < steps - g;
-            if (more && (g == 0 || j == 0)) rows.fetch(x, (tile + 1) * CT_M, m, d, tid);
+            if (more && (g == 0 || j == 0)) fetch(tile + 1);
             ok = __all_sync(0xffffffffu, ok && mbar_wait_ab(&mmab[tb], (g / TB) & 1, err, s_abort, kWaitNs));
             tc_fence_after();
             if (++j == nch) {
@@ -2105,94 +2418,100 @@ __global__ __launch_bounds__(PK_NT, 5) void k_coarse_pick(SelArgs a, int rpb)
     if (__syncthreads_or(!ok)) refine_rows(a, s_rows, s_left, pk);
 }
 
-// Finishing selection of the rows the fused first stage left undecided (P =
-// 1).  With a record, one warp per row: the FP32 distance of each candidate
-// list (CW_RG at a time, lanes over the coordinates), one list per lane; the
-// lists whose lower bound is at most the smallest upper bound remain, and if
-// they are several, their FP64 distances decide (ties to the lower index).
-// A row to redo takes a block: its warps read all lists' rows, FN_RG in
-// flight each, into one table of distances (a warp alone, list after list,
-// took 1.2 ms at 2,048 lists, the tail of the launch; four warps with eight
-// in flight 0.23 ms).
-constexpr int FN_RG = 16;
+// Assignment from k_coarse_dist's distances and group minima, a warp per row:
+// the lists within the split's bound of the smallest, of the groups whose
+// minimum is, decided by decide_nearest.  G <= 256 groups.
+constexpr int NR_GMAX = CW_LMAX / 16;
+__global__ __launch_bounds__(CW_ROWS * 32, 5) void k_coarse_near(SelArgs a, NearArgs near)
+{
+    pdl_begin();
+    __shared__ int s_tab[CW_ROWS][ND_WIN], s_grp[CW_ROWS][NR_GMAX];
+    __shared__ float s_lbs[CW_ROWS][ND_WIN];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row = blockIdx.x * CW_ROWS + w;
+    if (row >= a.m) return;  // whole warps
+    const int L = a.L, d = a.d, G = (L + 15) / 16;
+    const float *Dr = a.D + (size_t)row * L, *gr = a.gmin + (size_t)row * G;
+    const float *xr = a.x + (size_t)row * d;
+    float v[NR_GMAX / 32], b = INFINITY, part = 0.f;
+#pragma unroll
+    for (int u = 0; u < NR_GMAX / 32; ++u) {
+        v[u] = 32 * u + lane < G ? __ldg(gr + 32 * u + lane) : INFINITY;
+        b = fminf(b, v[u]);
+    }
+    for (int j = lane; j < d; j += 32) part = fmaf(xr[j], xr[j], part);
+    const float xn = norm_up(warp_sum(part), d);
+    for (int o = 16; o > 0; o >>= 1) b = fminf(b, __shfl_xor_sync(0xffffffffu, b, o));
+    const float cnmax = __ldg(a.cmaxes), cmax = __ldg(a.cmaxes + 1);
+    const float thr = pick_limit(b, bound_max(cnmax, abs_max(cnmax, xn, cmax), xn, cmax, a.gamma2_first));
+    int ng = 0;
+#pragma unroll
+    for (int u = 0; u < NR_GMAX / 32; ++u) {
+        const bool in = 32 * u + lane < G && v[u] <= thr;
+        const uint32_t mk = __ballot_sync(0xffffffffu, in);
+        if (in) s_grp[w][ng + __popc(mk & lanemask_lt())] = 32 * u + lane;
+        ng += __popc(mk);
+    }
+    __syncwarp();
+    auto fill = [&](int first, int w0) {  // two groups per load, eight in flight
+        int total = 0;
+        for (int t0 = 0; t0 < ng; t0 += 8) {
+            int c[4];
+            float e[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int t = t0 + 2 * u + (lane >> 4);
+                c[u] = t < ng ? s_grp[w][t] * 16 + (lane & 15) : L;
+                e[u] = c[u] < L ? __ldg(Dr + c[u]) : INFINITY;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = c[u] < L && e[u] <= thr;
+                const uint32_t mk = __ballot_sync(0xffffffffu, in);
+                const int at = first + total - w0 + __popc(mk & lanemask_lt());
+                if (in && at >= first && at < ND_WIN) s_tab[w][at] = c[u];
+                total += __popc(mk);
+            }
+        }
+        __syncwarp();
+        return total;
+    };
+    const int c = decide_nearest(near, fill, d, xr, xn, s_tab[w], s_lbs[w], lane);
+    if (lane == 0) {
+        if (c < 0 || c >= L) atomicOr(a.err, ERR_SELECT);
+        a.out[row] = c < 0 || c >= L ? -1 : c;
+    }
+}
+
+// Finishing selection of the rows that the fused first stage left undecided (P =
+// 1), a warp per row.  With a record: the FP32 distance of each candidate list
+// (CW_RG at a time, lanes over the coordinates), one list per lane; the lists
+// whose lower bound is at most the smallest upper bound remain, and if they are
+// several, their FP64 distances decide (ties to the lower index).  With the
+// second pass's bits: decide_nearest.
 constexpr int FN_ROWS = 8;     // warps per block
-__global__ __launch_bounds__(FN_ROWS * 32) void k_coarse_finish(SelArgs a)
+__global__ __launch_bounds__(FN_ROWS * 32, 2) void k_coarse_finish(SelArgs a, SecondArgs sp, NearArgs near)
 {
     pdl_begin();
     __shared__ __align__(16) float sX[FN_ROWS][kMaxD];
-    __shared__ float sD[CW_LMAX];
-    __shared__ float sT[FN_ROWS];
-    __shared__ double sB[FN_ROWS];
-    __shared__ int sC[FN_ROWS];
-    __shared__ int s_found, s_one;
+    __shared__ int s_tab[FN_ROWS][ND_WIN];
+    __shared__ float s_lbs[FN_ROWS][ND_WIN];
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const int L = a.L, d = a.d, n4 = d >> 2;
-    const int nrec = min(a.nhard[0], a.s_cap), nredo = a.nhard[1];
-    auto load_x = [&](const float *xr, float *to) {  // the row; its norm's bound
+    const int nrec = min(a.nhard[0], a.s_cap);
+    for (int it = blockIdx.x * FN_ROWS + w; it < nrec; it += gridDim.x * FN_ROWS) {  // whole warps
+        const int32_t *Sr = a.S + (size_t)it * CF_STRIDE;
+        const int row = Sr[0], n0 = min(Sr[1], CF_CAP);
+        const int c = lane < n0 ? Sr[2 + lane] : 0;
+        const float *xr = a.x + (size_t)row * d;
+        __syncwarp();  // the warp's sX is still read for its last row
         float part = 0.f;
         for (int j = lane; j < d; j += 32) {
             const float v = xr[j];
-            to[j] = v;
+            sX[w][j] = v;
             part = fmaf(v, v, part);
         }
-        return norm_up(warp_sum(part), d);
-    };
-    // partial dot product of list c's row with the row x4, this lane's share
-    auto share = [&](const float4 *x4, int c) {
-        const float4 *c4 = reinterpret_cast<const float4 *>(a.cent + (size_t)c * d);
-        float s = 0.f;
-#pragma unroll
-        for (int u = 0; u < kMaxD / 128; ++u) {
-            const int j4 = lane + 32 * u;
-            if (j4 >= n4) break;
-            const float4 xv = x4[j4], cv = __ldg(c4 + j4);
-            s = fmaf(xv.x, cv.x, s);
-            s = fmaf(xv.y, cv.y, s);
-            s = fmaf(xv.z, cv.z, s);
-            s = fmaf(xv.w, cv.w, s);
-        }
-        return s;
-    };
-    auto bounds = [&](int c, float Dt, float xn, float &lb, float &ub) {
-        const float E = bound_of(Dt, __ldg(a.cn + c), __ldg(a.cnrm_up + c), xn, a.gamma2_re);
-        lb = lower_of(Dt, E);
-        ub = upper_of(Dt, E);
-    };
-    auto fmin_warp = [&](float v) {
-        for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        return v;
-    };
-    double bd = INFINITY;  // the best of this thread's lists, by FP64 distance and index
-    int bc = 0x7fffffff;
-    auto better = [&](double D, int c) {
-        if (D < bd || (D == bd && c < bc)) {
-            bd = D;
-            bc = c;
-        }
-    };
-    auto best_warp = [&]() {
-        for (int o = 16; o > 0; o >>= 1) {
-            const double od = __shfl_xor_sync(0xffffffffu, bd, o);
-            const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
-            better(od, oc);
-        }
-    };
-    auto write = [&](int row, int c) {
-        if (c < 0 || c >= L) {
-            atomicOr(a.err, ERR_SELECT);
-            c = -1;
-        }
-        a.out[row] = c;
-    };
-
-    for (int it = blockIdx.x * FN_ROWS + w; it < nrec; it += gridDim.x * FN_ROWS) {  // whole warps
-        const int row = a.hard[it];
-        const int32_t *Sr = a.S + (size_t)it * CF_STRIDE;
-        const int n0 = min(Sr[0], CF_CAP);
-        const int c = lane < n0 ? Sr[1 + lane] : 0;
-        const float *xr = a.x + (size_t)row * d;
-        __syncwarp();  // the warp's sX is still read for its last row
-        const float xn = load_x(xr, sX[w]);
+        const float xn = norm_up(warp_sum(part), d);
         __syncwarp();
         const float4 *x4 = reinterpret_cast<const float4 *>(sX[w]);
         float dot = 0.f;
@@ -2201,7 +2520,15 @@ __global__ __launch_bounds__(FN_ROWS * 32) void k_coarse_finish(SelArgs a)
 #pragma unroll
             for (int t = 0; t < CW_RG; ++t) {
                 const int ct = __shfl_sync(0xffffffffu, c, p0 + t);
-                s[t] = p0 + t < n0 ? share(x4, ct) : 0.f;  // warp-uniform
+                const float4 *c4 = reinterpret_cast<const float4 *>(a.cent + (size_t)ct * d);
+                s[t] = 0.f;
+                if (p0 + t < n0 && lane < n4) {  // d <= 128
+                    const float4 xv = x4[lane], cv = __ldg(c4 + lane);
+                    s[t] = fmaf(xv.x, cv.x, s[t]);
+                    s[t] = fmaf(xv.y, cv.y, s[t]);
+                    s[t] = fmaf(xv.z, cv.z, s[t]);
+                    s[t] = fmaf(xv.w, cv.w, s[t]);
+                }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
@@ -2212,92 +2539,93 @@ __global__ __launch_bounds__(FN_ROWS * 32) void k_coarse_finish(SelArgs a)
                 if (lane == p0 + t) dot = s[t];
         }
         float lb = INFINITY, ub = INFINITY;
-        if (lane < n0) bounds(c, fmaf(-2.f, dot, __ldg(a.cn + c)), xn, lb, ub);
-        const float T = fmin_warp(ub);
+        if (lane < n0) {
+            const float cnc = __ldg(a.cn + c), Dt = fmaf(-2.f, dot, cnc);
+            const float E = bound_of(Dt, cnc, __ldg(a.cnrm_up + c), xn, a.gamma2_re);
+            lb = lower_of(Dt, E);
+            ub = upper_of(Dt, E);
+        }
+        float T = ub;
+        for (int o = 16; o > 0; o >>= 1) T = fminf(T, __shfl_xor_sync(0xffffffffu, T, o));
         const bool in = lane < n0 && lb <= T;
         const uint32_t mk = __ballot_sync(0xffffffffu, in);
         int chosen = -1;
         if (__popc(mk) == 1) {
             chosen = __shfl_sync(0xffffffffu, c, __ffs(mk) - 1);
         } else if (mk) {
-            bd = INFINITY;
-            bc = 0x7fffffff;
-            if (in) better(exact_dist4(x4, reinterpret_cast<const float4 *>(a.cent + (size_t)c * d), d), c);
-            best_warp();
+            double bd = INFINITY;
+            int bc = 0x7fffffff;
+            if (__popc(mk) <= EX_FEW) {
+                // the lanes that hold the lists, and their numbers
+                uint32_t todo = mk;
+                int cm[EX_FEW];
+#pragma unroll
+                for (int m = 0; m < EX_FEW; ++m) {
+                    cm[m] = __shfl_sync(0xffffffffu, c, todo ? __ffs(todo) - 1 : 0);
+                    todo &= todo - 1u;
+                }
+                auto pick = [&](int m) { return m == 0 ? cm[0] : m == 1 ? cm[1] : m == 2 ? cm[2] : cm[3]; };
+                const double D = exact_four(x4, a.cent, pick, __popc(mk), d, lane);
+                if (lane < __popc(mk)) {
+                    bd = D;
+                    bc = pick(lane);
+                }
+            } else if (in) {
+                bd = exact_dist4(x4, reinterpret_cast<const float4 *>(a.cent + (size_t)c * d), d);
+                bc = c;
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+                const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
+                if (od < bd || (od == bd && oc < bc)) {
+                    bd = od;
+                    bc = oc;
+                }
+            }
             chosen = bc;
         }
-        if (lane == 0) write(row, chosen);
+        if (lane == 0) {
+            if (chosen < 0 || chosen >= L) {
+                atomicOr(a.err, ERR_SELECT);
+                chosen = -1;
+            }
+            a.out[row] = chosen;
+        }
     }
 
-    for (int it = blockIdx.x; it < nredo; it += gridDim.x) {
-        const int row = a.hard[a.m - 1 - it];
+    const int nbits = *sp.n, G = (L + 15) / 16;
+    for (int it = blockIdx.x * FN_ROWS + w; it < nbits; it += gridDim.x * FN_ROWS) {  // whole warps
+        const int place = sp.list[it], row = sp.rows[place];
+        const uint16_t *bits = sp.bits + (size_t)(place >> 7) * G * sp.stride + (place & 127);
         const float *xr = a.x + (size_t)row * d;
-        __syncthreads();  // the tables are still read for the last row
-        const float xn = load_x(xr, sX[w]);
-        if (tid == 0) {
-            s_found = 0;
-            s_one = -1;
-        }
-        __syncwarp();
-        const float4 *x4 = reinterpret_cast<const float4 *>(sX[w]);
-        float T = INFINITY;
-        for (int c0 = w * FN_RG; c0 < L; c0 += FN_ROWS * FN_RG) {
-            float s[FN_RG];
-#pragma unroll
-            for (int t = 0; t < FN_RG; ++t) s[t] = share(x4, min(c0 + t, L - 1));
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int t = 0; t < FN_RG; ++t) s[t] += __shfl_xor_sync(0xffffffffu, s[t], o);
-            float dot = s[0];
-#pragma unroll
-            for (int t = 1; t < FN_RG; ++t)
-                if (lane == t) dot = s[t];
-            const int c = c0 + lane;
-            if (lane < FN_RG && c < L) {
-                const float Dt = fmaf(-2.f, dot, __ldg(a.cn + c));
-                float lb, ub;
-                bounds(c, Dt, xn, lb, ub);
-                sD[c] = Dt;
-                T = fminf(T, ub);
+        float part = 0.f;
+        for (int j = lane; j < d; j += 32) part = fmaf(xr[j], xr[j], part);
+        const float xn = norm_up(warp_sum(part), d);
+        auto fill = [&](int first, int w0) {
+            int total = 0;
+            for (int g0 = 0; g0 < G; g0 += 32) {
+                uint32_t mk = g0 + lane < G ? bits[(size_t)(g0 + lane) * sp.stride] : 0u;
+                const int k = __popc(mk);
+                int at = k;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, at, o);
+                    if (lane >= o) at += v;
+                }
+                const int all = __shfl_sync(0xffffffffu, at, 31);
+                at += first + total - k - w0;
+                for (; mk; mk &= mk - 1, ++at)
+                    if (at >= first && at < ND_WIN) s_tab[w][at] = (g0 + lane) * 16 + __ffs(mk) - 1;
+                total += all;
             }
-        }
-        T = fmin_warp(T);
-        if (lane == 0) sT[w] = T;
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < FN_ROWS; ++k) T = fminf(T, sT[k]);
-        for (int c = tid; c < L; c += FN_ROWS * 32) {
-            float lb, ub;
-            bounds(c, sD[c], xn, lb, ub);
-            if (lb <= T) {
-                atomicAdd(&s_found, 1);
-                s_one = c;
-            }
-        }
-        __syncthreads();
-        const int found = s_found;
-        if (found <= 1) {
-            if (tid == 0) write(row, s_one);
-            continue;
-        }
-        bd = INFINITY;
-        bc = 0x7fffffff;
-        for (int c = tid; c < L; c += FN_ROWS * 32) {
-            float lb, ub;
-            bounds(c, sD[c], xn, lb, ub);
-            if (lb <= T) better(exact_dist4(x4, reinterpret_cast<const float4 *>(a.cent + (size_t)c * d), d), c);
-        }
-        best_warp();
+            __syncwarp();
+            return total;
+        };
+        const int c = decide_nearest(near, fill, d, xr, xn, s_tab[w], s_lbs[w], lane);
         if (lane == 0) {
-            sB[w] = bd;
-            sC[w] = bc;
+            if (c < 0 || c >= L) atomicOr(a.err, ERR_SELECT);
+            a.out[row] = c < 0 || c >= L ? -1 : c;
         }
-        __syncthreads();
-        if (tid == 0) {
-            for (int k = 1; k < FN_ROWS; ++k) better(sB[k], sC[k]);
-            write(row, bc);
-        }
+        __syncwarp();  // the warp's tables are reused
     }
 }
 
@@ -2509,6 +2837,21 @@ bool coarse_picks(const sivf_index *ix, int P)
     return P > CW_PMAX || (int64_t)ix->nlist * ix->d >= 32768;
 }
 
+// Assignment of few rows: the fused stage gives 128 of them to a CTA, which
+// passes over every list, and over every list twice more for the rows that
+// need the second pass; k_coarse_dist deals its (tile, chunk) steps to all SMs.
+// Up to 40 tiles of close centroids, 20 of others: 301 rows of 2,048 trained
+// lists in 64 clusters take 34 us (host time included), 103 by the fused stage;
+// 5,000 rows 53 and 129, 10,000 rows 139 and 100.  2,500 rows of 527 lists in 32
+// clusters by the single product: 42 and 82; lists apart: the same to 2,500 rows,
+// then the fused stage (10,000 rows of 1,024 lists: 38 us, 53).
+static bool assign_near(const sivf_index *ix, int64_t m)
+{
+    const int L = ix->nlist;
+    if (!ix->tmap_cent_ok || L < CF_LMIN || L > CW_LMAX) return false;
+    return m <= (ix->assign_split ? 40 : 20) * CT_M;
+}
+
 // rows [0, m) of x -> out[m, P]; `Dbuf` holds at least `room` floats, L of
 // them at least.
 void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
@@ -2520,21 +2863,21 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
     const bool warp_rows = P <= CW_PMAX && L <= CW_LMAX;
     // distances and group minima of at least one row
     const int64_t pick_row = L + (L + 15) / 16;
-    const bool pick = coarse_picks(ix, P) && room >= CF_HDR + pick_row;
+    const bool near = P == 1 && assign_near(ix, m) && room >= CF_HDR + std::min<int64_t>(m, 8 * CT_M) * pick_row;
+    const bool pick = near || (coarse_picks(ix, P) && room >= CF_HDR + pick_row);
     const int split = pick ? 3 : first_stage_split(ix, P);
     const bool two = split != 0;
     const float gamma2_first = (float)(2.0 * first_stage_rel(d, split) * (1.0 + 1e-6));
+    const int ro = pick && !near ? pk_ops(d) : re_ops(d);
+    const float gamma2_re = (float)(2.0 * (ro * u / (1.0 - ro * u)) * (1.0 + 1e-6));
     // assignment (d <= 128) takes the fused first stage, which keeps only the
     // undecided rows and their candidate lists.  It needs far less room than
     // the matrix: a launch takes as many rows as leave records for half of
-    // them (958,000 where the matrix of L = 1024 lists takes 16,384); among
-    // close centroids about a third are undecided
-    const bool fused = P == 1 && two && ix->tmap_cent_ok && L >= CF_LMIN;
-    int64_t rows = std::min<int64_t>(std::max<int64_t>(room / L, 1), m);
-    if (fused)
-        rows = std::min<int64_t>(std::max<int64_t>((room - CF_HDR) * 2 / (2 + CF_STRIDE), 1), m);
-    else if (pick)
-        rows = std::min<int64_t>((room - CF_HDR) / pick_row, m);
+    // them beside the second pass's rows and bits (349,000 where the matrix of
+    // L = 1024 lists takes 16,384); among close centroids about a third are
+    // undecided
+    const bool fused = P == 1 && two && !pick && ix->tmap_cent_ok && L >= CF_LMIN;
+    const NearArgs na{ix->cent, ix->cnorm, ix->cnrm_up, gamma2_re};
     int nsm = 0;
     if (fused || pick) {
         int dev = 0;
@@ -2542,18 +2885,35 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         nsm = std::max(nsm, 1);
     }
+    // ints of the second pass's rows, their list and bits for r rows in one launch
+    const int64_t G = (L + 15) / 16;
+    auto second_ints = [&](int64_t r) {
+        return 2 * r + ((r + CT_M - 1) / CT_M * G * std::min<int64_t>(r, CT_M) + 1) / 2;
+    };
+    int64_t rows = std::min<int64_t>(std::max<int64_t>(room / L, 1), m);
+    if (fused) {
+        // with records for half of the rows, or what a tile can have
+        const int64_t most = room - CF_HDR, rec = CF_STRIDE / 2, row = 2 + (G + 1) / 2;
+        const int64_t many = (most - G * CT_M / 2) / (row + rec);
+        const int64_t tile = std::min<int64_t>(CT_M, most / (row + 4));
+        rows = std::min<int64_t>(std::max<int64_t>({many, tile, 1}), m);
+    } else if (pick) {
+        rows = std::min<int64_t>((room - CF_HDR) / pick_row, m);
+    }
     for (int64_t r0 = 0; r0 < m; r0 += rows) {
         int mc = (int)std::min<int64_t>(rows, m - r0);
-        const int cap = fused ? (int)std::min<int64_t>((room - CF_HDR - mc) / CF_STRIDE, mc) : 0;
+        const int64_t sec = fused ? second_ints(mc) : 0;
+        SecondArgs sa{};
+        const int cap = fused ? (int)std::max<int64_t>(0, std::min<int64_t>((room - CF_HDR - sec) / CF_STRIDE, mc)) : 0;
         const int tok = prof_begin(ix, PROF_COARSE, 2, st);
-        // the distance buffer of the fused stage: the number of undecided
-        // rows, those rows, the records; of the pick: the distances and the
-        // group minima
-        int32_t *nh = reinterpret_cast<int32_t *>(Dbuf), *rec = nh + CF_HDR + mc;
+        // the distance buffer of the fused stage: the numbers of records and of
+        // rows with bits, the second pass's rows, their list and bits, the
+        // records; of the pick: the distances and the group minima
+        int32_t *nh = reinterpret_cast<int32_t *>(Dbuf), *rec = nh + CF_HDR + sec;
         float *Dm = pick ? Dbuf + CF_HDR : Dbuf, *gm = Dm + (size_t)mc * L;
         if (pick) {
             const int KC = d <= 64 ? 1 : 2;
-            const size_t smem = coarse_fused_smem(KC, 2);
+            const size_t smem = coarse_fused_smem(KC);
             const int nt = (mc + CT_M - 1) / CT_M, nch = (L + CF_CN - 1) / CF_CN;
             const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent);
             const CUtensorMap &tl = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent_lo);
@@ -2571,7 +2931,13 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
             else go(k_coarse_dist<2>, 1);
         } else if (fused) {
             const int KC = d <= 64 ? 1 : 2, parts = split == 3 ? 2 : 1;
-            const size_t smem = coarse_fused_smem(KC, parts);
+            const size_t smem = coarse_fused_smem(KC);
+            sa.n = nh + 1;
+            sa.rows = nh + CF_HDR;
+            sa.list = sa.rows + mc;
+            sa.bits = reinterpret_cast<uint16_t *>(sa.list + mc);
+            sa.stride = std::min(mc, CT_M);
+            sa.gamma = (float)(2.0 * first_stage_rel(d, 3) * (1.0 + 1e-6));
             cudaMemsetAsync(nh, 0, 2 * sizeof(int32_t), st);
             const int nt = (mc + CT_M - 1) / CT_M;
             const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent);
@@ -2585,8 +2951,7 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
                     attr[i] = true;
                 }
                 launch_pdl(kern, std::min(nt, nsm), CF_NT, smem, st, tm, tl, x + r0 * d, mc, d,
-                           ix->cnorm, ix->cmax, L, gamma2_first, out + r0, rec, cap, nh + CF_HDR,
-                           nh, ix->err);
+                           ix->cnorm, ix->cmax, L, gamma2_first, out + r0, rec, cap, nh, sa, ix->err);
             };
             if (parts == 1) {
                 if (KC == 1) go(k_coarse_fused<1, 1>, 0);
@@ -2624,7 +2989,6 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         }
         SelArgs a;
         a.D = fused ? nullptr : Dm;
-        a.hard = fused ? nh + CF_HDR : nullptr;
         a.nhard = nh;
         a.S = rec;
         a.s_cap = cap;
@@ -2638,25 +3002,25 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         a.cnrm_up = ix->cnrm_up;
         a.gamma2 = (float)(2.0 * gd * (1.0 + 1e-6));
         a.gamma2_first = gamma2_first;
-        const int ro = pick ? pk_ops(d) : re_ops(d);
-        const double gr = ro * u / (1.0 - ro * u);
-        a.gamma2_re = (float)(2.0 * gr * (1.0 + 1e-6));
+        a.gamma2_re = gamma2_re;
         a.two_level = two;
         a.Dw = pick ? Dm : nullptr;
         a.gmin = pick ? gm : nullptr;
         a.cmaxes = ix->cmax;
         a.out = out + r0 * P;
         a.err = ix->err;
-        if (pick) {
+        if (near) {
+            launch_pdl(k_coarse_near, (unsigned)((mc + CW_ROWS - 1) / CW_ROWS), CW_ROWS * 32, 0, st, a, na);
+        } else if (pick) {
             const int rpb = mc <= 4 * nsm ? 1 : CW_ROWS;
             launch_pdl(k_coarse_pick, (unsigned)((mc + rpb - 1) / rpb), PK_NT,
                        pk_block_smem(P, (L + 15) / 16), st, a, rpb);
         } else if (warp_rows) {
             const unsigned gw = (unsigned)((mc + CW_ROWS - 1) / CW_ROWS);
-            if (fused)  // loops over the undecided rows
+            if (fused)  // loops over the records
                 launch_pdl(k_coarse_finish,
                            std::min<unsigned>((unsigned)((mc + FN_ROWS - 1) / FN_ROWS), 5u * (unsigned)nsm),
-                           FN_ROWS * 32, 0, st, a);
+                           FN_ROWS * 32, 0, st, a, sa, na);
             else if (P == 1) launch_pdl(k_coarse_select_w<1>, gw, CW_ROWS * 32, 0, st, a);
             else launch_pdl(k_coarse_select_w<CW_PMAX>, gw, CW_ROWS * 32, 0, st, a);
         } else {

@@ -165,7 +165,8 @@ struct SelArgs {
     const float *cnrm_up;  // [L]
     float gamma2;          // 2 * gamma_d
     float gamma2_first;    // the same factor for the first-stage distances D
-    float gamma2_re;       // and for FP32 dot products summed across a warp (re_ops)
+    float gamma2_re;       // and for FP32 dot products summed across a warp (re_ops) or, by
+    float gamma2_w;        // the pick, eight lanes of it (pk_ops); gamma2_w: across a warp
     int two_level;         // D is the BF16 tensor-core stage: recheck S in FP32
     const int *nhard;      // k_coarse_finish: how many records (on the device), and the
     const int32_t *S;      // records [row, n, lists...] of the rows the fused first stage
@@ -2250,7 +2251,13 @@ __device__ __forceinline__ bool pick_row(const SelArgs &a, int row, unsigned cha
     }
     if (nsel != P && lane == 0) atomicOr(a.err, ERR_SELECT);
     nsel = min(nsel, P);
-    // nearest first: ascending FP32 distance, ties to the lower list index
+    // Nearest first: ascending FP32 distance, ties to the lower list index.  The
+    // distances are those of the forms without group minima (k_coarse_gemm's sums;
+    // for P <= CW_PMAX of at most CW_LMAX lists k_coarse_select_w's), so that a
+    // list's place does not depend on the form: where two neighbours lie within
+    // the two sums' bounds of each other, that sum is formed for both.
+    __syncwarp();
+    int *sList = reinterpret_cast<int *>(sUB);
     int32_t *outr = a.out + (size_t)row * P;
     for (int s = lane; s < P; s += 32) {
         if (s >= nsel) {
@@ -2262,6 +2269,68 @@ __device__ __forceinline__ bool pick_row(const SelArgs &a, int row, unsigned cha
         int pos = 0;
 #pragma unroll 8
         for (int q = 0; q < nsel; ++q) pos += (sDt[q] < dc) | ((sDt[q] == dc) & (sIdx[q] < c));  // no branches
+        outr[pos] = c;
+        sLB[pos] = dc;
+        sList[pos] = c;
+    }
+    __syncwarp();
+    const bool sums = P > CW_PMAX || L > CW_LMAX;
+    bool close = false;
+    if (!(FRESH && sums)) {
+        const float ab = abs_max(cnmax, xn, cmax);
+        const float e1 = bound_max(cnmax, ab, xn, cmax, FRESH ? a.gamma2 : a.gamma2_re);
+        const float e2 = bound_max(cnmax, ab, xn, cmax, sums ? a.gamma2 : a.gamma2_w);
+        const float apart = __fmul_ru(2.0001f, __fadd_ru(e1, e2));
+        for (int i = lane; i < nsel; i += 32) {
+            const bool in = (i > 0 && !(sLB[i] - sLB[i - 1] > apart)) ||
+                            (i + 1 < nsel && !(sLB[i + 1] - sLB[i] > apart));
+            sSure[i] = in;
+            close = close || in;
+        }
+        close = __any_sync(0xffffffffu, close);
+        __syncwarp();
+    }
+    if (!close) return true;
+    const float4 *x4 = reinterpret_cast<const float4 *>(sX);
+    if (sums) {
+        for (int i = lane; i < nsel; i += 32) {
+            if (!sSure[i]) continue;
+            const float4 *c4 = reinterpret_cast<const float4 *>(a.cent + (size_t)sList[i] * d);
+            float dot = 0.f;
+#pragma unroll 4
+            for (int j = 0; j < n4; ++j) {
+                const float4 xv = x4[j], cv = __ldg(c4 + j);
+                dot = fmaf(xv.x, cv.x, dot);
+                dot = fmaf(xv.y, cv.y, dot);
+                dot = fmaf(xv.z, cv.z, dot);
+                dot = fmaf(xv.w, cv.w, dot);
+            }
+            sLB[i] = fmaf(-2.f, dot, __ldg(a.cn + sList[i]));
+        }
+    } else {
+        for (int i = 0; i < nsel; ++i) {
+            if (!sSure[i]) continue;  // warp-uniform
+            float dot = 0.f;
+            if (lane < n4) {
+                const float4 xv = x4[lane];
+                const float4 cv = __ldg(reinterpret_cast<const float4 *>(a.cent + (size_t)sList[i] * d) + lane);
+                dot = fmaf(xv.x, cv.x, dot);
+                dot = fmaf(xv.y, cv.y, dot);
+                dot = fmaf(xv.z, cv.z, dot);
+                dot = fmaf(xv.w, cv.w, dot);
+            }
+            dot = warp_sum(dot);
+            if (lane == 0) sLB[i] = fmaf(-2.f, dot, __ldg(a.cn + sList[i]));
+        }
+    }
+    __syncwarp();
+    for (int s = lane; s < nsel; s += 32) {
+        if (!sSure[s]) continue;  // alone in its place
+        const int c = sList[s];
+        const float dc = sLB[s];
+        int pos = s;  // its neighbours on both sides, as far as they are close
+        for (int q = s - 1; q >= 0 && sSure[q]; --q) pos -= (sLB[q] > dc) | ((sLB[q] == dc) & (sList[q] > c));
+        for (int q = s + 1; q < nsel && sSure[q]; ++q) pos += (sLB[q] < dc) | ((sLB[q] == dc) & (sList[q] < c));
         outr[pos] = c;
     }
     return true;
@@ -2869,7 +2938,8 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
     const bool two = split != 0;
     const float gamma2_first = (float)(2.0 * first_stage_rel(d, split) * (1.0 + 1e-6));
     const int ro = pick && !near ? pk_ops(d) : re_ops(d);
-    const float gamma2_re = (float)(2.0 * (ro * u / (1.0 - ro * u)) * (1.0 + 1e-6));
+    auto gamma_sum = [&](int ops) { return (float)(2.0 * (ops * u / (1.0 - ops * u)) * (1.0 + 1e-6)); };
+    const float gamma2_re = gamma_sum(ro);
     // assignment (d <= 128) takes the fused first stage, which keeps only the
     // undecided rows and their candidate lists.  It needs far less room than
     // the matrix: a launch takes as many rows as leave records for half of
@@ -3003,6 +3073,7 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
         a.gamma2 = (float)(2.0 * gd * (1.0 + 1e-6));
         a.gamma2_first = gamma2_first;
         a.gamma2_re = gamma2_re;
+        a.gamma2_w = gamma_sum(re_ops(d));
         a.two_level = two;
         a.Dw = pick ? Dm : nullptr;
         a.gmin = pick ? gm : nullptr;

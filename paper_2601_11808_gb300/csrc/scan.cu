@@ -767,7 +767,10 @@ __host__ __device__ constexpr int scan_buf_len(int K, int C)
 // of at least SCAN_BMIN rows' distances leaves room for two CTAs
 constexpr size_t SCAN_SMEM = 222 * 1024;
 constexpr size_t SCAN_HALF = 110 * 1024;
-constexpr int SCAN_BMIN = 256, SCAN_BMAX = 1024;
+constexpr int SCAN_BMIN = 256;
+// rows of a block at most: the few warps with a row of an 8-query tile keep 512
+// distances in registers for the selection, more they read again and again
+__host__ __device__ constexpr int scan_bmax(int TQ) { return TQ <= 8 ? 512 : 1024; }
 
 // shared memory carve-up, identical on host and device; nbs: slabs of a
 // block, whose distances the rows keep until they are selected from
@@ -789,11 +792,11 @@ __host__ __device__ inline ScanSmem scan_smem_at(int TQ, int C, int d, int M, in
     s.total = s.misc + 64 + (size_t)nbs * 4;
     return s;
 }
-// slabs of a block: the most rows up to SCAN_BMAX, two CTAs per SM for the
+// slabs of a block: the most rows up to scan_bmax, two CTAs per SM for the
 // tiles of at most 16 queries where SCAN_BMIN rows fit then
 __host__ __device__ inline int scan_block(int TQ, int C, int d, int M)
 {
-    const int most = SCAN_BMAX / C;
+    const int most = scan_bmax(TQ) / C;
     if (TQ <= 16)
         for (int n = most; n * C >= SCAN_BMIN; --n)
             if (scan_smem_at(TQ, C, d, M, n).total <= SCAN_HALF) return n;
@@ -936,7 +939,7 @@ __device__ __forceinline__ void dist_tile(float (&acc)[RQ][RX], const float *__r
         }
         return;
     }
-#pragma unroll 2
+#pragma unroll 4
     for (int j = 0; j < d; j += 4) {
         float4 qv[RQA], xv[RX];
 #pragma unroll
@@ -949,8 +952,11 @@ __device__ __forceinline__ void dist_tile(float (&acc)[RQ][RX], const float *__r
     }
 }
 
-template <int TQ, int C, bool XS>
-__global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(
+// ONE: shared memory leaves room for one CTA per SM, so that a thread may have
+// all the registers (at the 128 of two CTAs the small tiles spill: 12 queries of
+// 25 lists of 13,400 vectors, d = 192, 1,119 us, 785 so)
+template <int TQ, int C, bool XS, bool ONE>
+__global__ __launch_bounds__(SCAN_NT, ONE ? 1 : 2) void k_scan(
     const __grid_constant__ CUtensorMap tmap, ScanArgs a)
 {
     pdl_begin();
@@ -1055,16 +1061,25 @@ __global__ __launch_bounds__(SCAN_NT, TQ <= 16 ? 2 : 1) void k_scan(
         __syncwarp();
     };
 
-    // Select from the n distances of the block for row qr (one warp): while
-    // the row holds fewer than K, a value K of them lie at or below (kth_bound)
-    // is the bar, else its K-th; what is within it (ties included) goes to the
+    // Select from the n distances of the block for row qr (one warp): the row's
+    // K-th or the query's bound is the bar; while the row holds fewer than K and
+    // many lie within that, a value K of them lie at or below (kth_bound; always
+    // sought, it cost 780 queries of 11 lists among overlapping cells a quarter of
+    // their time: 1,354 us, 1,055 so); what is within it (ties included) goes to the
     // candidates, slots first, and is merged with its ids
     auto select_row = [&](int qr, int n) {
         const float *dr = DM + (size_t)qr * DS;
         float *bd = BD + (size_t)qr * M + K;
         int64_t *bi = BI + (size_t)qr * M + K;
         float bar = s_kd[qr];
-        if (s_nb[qr] < K)
+        bool many = s_nb[qr] < K;  // more within the bar than a merge takes cheaply
+        if (many && bar < 1e38f) {
+            int c = 0;
+#pragma unroll 8
+            for (int i = lane; i < n; i += 32) c += dr[i] <= bar;
+            many = __reduce_add_sync(0xffffffffu, c) > K + 16;
+        }
+        if (many)
             bar = fminf(bar, kth_bound<16>([&](int i) { return i < n ? dr[i] : INFINITY; },
                                            (n + 31) & ~31, K, lane));
         int cc = 0;
@@ -1356,14 +1371,14 @@ __global__ __launch_bounds__(MERGE_NT) void k_merge(const int2 *__restrict__ qru
 }
 
 // --------------------------------------------------------------- drivers
-template <int TQ, int C, bool SW>
+template <int TQ, int C, bool SW, bool ONE>
 static void launch_scan(sivf_index *ix, const ScanArgs &a, size_t smem, int grid,
                         cudaStream_t st)
 {
     if (SW) smem += 1024;  // base alignment slack
     static size_t attr = 48 * 1024;
     if (smem > attr) {
-        cudaFuncSetAttribute(k_scan<TQ, C, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_scan<TQ, C, SW, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
         attr = smem;
     }
@@ -1373,14 +1388,14 @@ static void launch_scan(sivf_index *ix, const ScanArgs &a, size_t smem, int grid
     static int occ = 1;
     if (smem != occ_smem) {
         int n = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_scan<TQ, C, SW>, SCAN_NT, smem) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_scan<TQ, C, SW, ONE>, SCAN_NT, smem) !=
             cudaSuccess)
             n = 1;
         occ = std::max(1, n);
         occ_smem = smem;
     }
     const int tok = prof_begin(ix, PROF_SCAN, 1, st);
-    launch_pdl(k_scan<TQ, C, SW>, grid * occ, SCAN_NT, smem, st,
+    launch_pdl(k_scan<TQ, C, SW, ONE>, grid * occ, SCAN_NT, smem, st,
                *reinterpret_cast<const CUtensorMap *>(ix->tmap_x32), a);
     prof_end(ix, tok, st);
 }
@@ -1597,10 +1612,15 @@ static void scan_launch(sivf_index *ix, int tq, ScanArgs a, cudaStream_t st)
     a.nbs = scan_block(tq, ix->C, ix->d, a.M);
     const size_t smem = scan_smem_at(tq, ix->C, ix->d, a.M, a.nbs).total;
     const int grid = 152;  // persistent: one CTA per SM
-#define SIVF_SCAN_CASE(TQ_, C_) \
-    if (tq == TQ_ && ix->C == C_)                                            \
-        return ix->tmap_x32_ok ? launch_scan<TQ_, C_, true>(ix, a, smem, grid, st) \
-                               : launch_scan<TQ_, C_, false>(ix, a, smem, grid, st);
+    const bool one = smem > SCAN_HALF;
+#define SIVF_SCAN_CASE(TQ_, C_)                                                                        \
+    if (tq == TQ_ && ix->C == C_) {                                                                    \
+        if (one || TQ_ > 16)                                                                           \
+            return ix->tmap_x32_ok ? launch_scan<TQ_, C_, true, true>(ix, a, smem, grid, st)           \
+                                   : launch_scan<TQ_, C_, false, true>(ix, a, smem, grid, st);         \
+        return ix->tmap_x32_ok ? launch_scan<TQ_, C_, true, (TQ_ > 16)>(ix, a, smem, grid, st)         \
+                               : launch_scan<TQ_, C_, false, (TQ_ > 16)>(ix, a, smem, grid, st);       \
+    }
     SIVF_SCAN_CASE(8, 32) SIVF_SCAN_CASE(16, 32) SIVF_SCAN_CASE(32, 32) SIVF_SCAN_CASE(64, 32)
     SIVF_SCAN_CASE(8, 64) SIVF_SCAN_CASE(16, 64) SIVF_SCAN_CASE(32, 64) SIVF_SCAN_CASE(64, 64)
     SIVF_SCAN_CASE(8, 128) SIVF_SCAN_CASE(16, 128) SIVF_SCAN_CASE(32, 128)

@@ -78,9 +78,13 @@ __global__ void k_centroid_norms(const float *__restrict__ cent, int L, int d,
         const float n2 = __double2float_rn(s), nu = __double2float_ru(sqrt(s) * (1.0 + 1e-12));
         cn[c] = n2;
         cnrm_up[c] = nu;
-        // the largest of each (not negative, so their bits order as integers)
-        atomicMax(reinterpret_cast<int *>(cmax), __float_as_int(n2));
-        atomicMax(reinterpret_cast<int *>(cmax) + 1, __float_as_int(nu));
+        // the largest of each (not negative, so their bits order as integers).
+        // A NaN's would be above all: its list is never chosen and counts for no
+        // bound, which a NaN would make undecidable for every other list
+        if (n2 == n2) {
+            atomicMax(reinterpret_cast<int *>(cmax), __float_as_int(n2));
+            atomicMax(reinterpret_cast<int *>(cmax) + 1, __float_as_int(nu));
+        }
     }
 }
 

@@ -398,6 +398,9 @@ __global__ __launch_bounds__(1024) void k_srch_hash(
 //   FP8: D = rq^2 + rx^2 - 2 s q^.x^ with ||q^|| <= rq + eq and ||x^|| <= rx +
 //     ex (E4M3 rounds to 2^-4 relative, 2^-10 of a code unit below the
 //     smallest normal; saturation only shortens x^), least at rx = R.
+// Sums of squares below FP32's range lose up to 2^-150 a term, 2e-43 in all (R
+// grows and the bound sinks by what covers it), and one beyond the range says
+// nothing of D: the pair stays.
 // One warp takes PR consecutive pairs of one query (8, or 4 for d > 128),
 // their centroid rows in flight together, and works out the bounds one pair
 // per lane (every lane for every pair: 324 against 82 us for 630,000 pairs);
@@ -498,11 +501,11 @@ __global__ __launch_bounds__(256) void k_pair_prune(PruneArgs a)
         const float u32 = 5.9604645e-08f;  // 2^-24
         const float up = 1.f + (2.f * d + 32.f) * u32, dn = 1.f - (2.f * d + 32.f) * u32;
         const float bound = __ldcg(a.thr + qi);
-        const float R = __fsqrt_ru(__ldg(a.lrad2 + l));
+        const float R = __fadd_ru(__fsqrt_ru(__ldg(a.lrad2 + l)), 2e-21f);
         const float rlo = __fsqrt_rd(__fmul_rd(s2, dn)), rhi = __fsqrt_ru(__fmul_ru(s2, up));
         const float gap = __fsub_rd(rlo, R);
         float lo = -INFINITY;  // lower bound of the scan's distances
-        if (gap > 0.f) {
+        if (gap > 0.f && rlo < INFINITY) {
             if (DT == SIVF_FP32) {
                 lo = __fmul_rd(__fmul_rd(gap, gap), dn);
             } else if (DT == SIVF_BF16) {
@@ -525,7 +528,7 @@ __global__ __launch_bounds__(256) void k_pair_prune(PruneArgs a)
                                err);
             }
         }
-        keep = !(lo > bound);
+        keep = !(__fsub_rd(lo, 1e-42f) > bound);
     }
     if (lane < np_here) {
         const int64_t e = qi * a.P + pb + lane;

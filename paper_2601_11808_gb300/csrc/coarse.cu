@@ -2991,13 +2991,9 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
             const int nt = (mc + CT_M - 1) / CT_M, nch = (L + CF_CN - 1) / CF_CN;
             const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent);
             const CUtensorMap &tl = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent_lo);
-            static bool attr[2] = {false, false};
+            static KernelSetup su[2];
             auto go = [&](auto kern, int i) {
-                if (!attr[i]) {
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-                    attr[i] = true;
-                }
+                opt_in_smem(su[i], kern, smem);
                 launch_pdl(kern, (unsigned)std::min<int64_t>((int64_t)nt * nch, nsm), CF_NT, smem, st,
                            tm, tl, x + r0 * d, mc, d, ix->cnorm, L, Dm, gm, ix->err);
             };
@@ -3016,14 +3012,9 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
             const int nt = (mc + CT_M - 1) / CT_M;
             const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent);
             const CUtensorMap &tl = *reinterpret_cast<const CUtensorMap *>(ix->tmap_cent_lo);
-            // shared memory opted in once per instantiation
-            static bool attr[4] = {false, false, false, false};
+            static KernelSetup su[4];
             auto go = [&](auto kern, int i) {
-                if (!attr[i]) {
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-                    attr[i] = true;
-                }
+                opt_in_smem(su[i], kern, smem);
                 launch_pdl(kern, std::min(nt, nsm), CF_NT, smem, st, tm, tl, x + r0 * d, mc, d,
                            ix->cnorm, ix->cmax, L, gamma2_first, out + r0, rec, cap, nh, sa, ix->err);
             };
@@ -3038,21 +3029,13 @@ void coarse_topP(sivf_index *ix, const float *x, int64_t m, int P, int32_t *out,
             const size_t smem = coarse_tc_smem(d, split);
             dim3 g((mc + CT_M - 1) / CT_M, (L + CT_N - 1) / CT_N);
             if (split == 1) {
-                static size_t attr = 0;
-                if (smem > attr) {
-                    cudaFuncSetAttribute(k_coarse_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-                    attr = smem;
-                }
+                static KernelSetup su;
+                opt_in_smem(su, k_coarse_tc<1>, smem);
                 launch_pdl(k_coarse_tc<1>, g, CT_NT, smem, st, x + r0 * d, mc, d, ix->cent_bf16,
                            nullptr, ix->cnorm, L, Dbuf, ix->err);
             } else {
-                static size_t attr = 0;
-                if (smem > attr) {
-                    cudaFuncSetAttribute(k_coarse_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-                    attr = smem;
-                }
+                static KernelSetup su;
+                opt_in_smem(su, k_coarse_tc<3>, smem);
                 launch_pdl(k_coarse_tc<3>, g, CT_NT, smem, st, x + r0 * d, mc, d, ix->cent_bf16,
                            ix->cent_lo, ix->cnorm, L, Dbuf, ix->err);
             }

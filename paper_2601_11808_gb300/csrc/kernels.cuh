@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <utility>
 
+#include "kernel_setup.cuh"
 #include "sivf_internal.cuh"
 
 namespace sivf {
@@ -50,6 +51,20 @@ inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
     // a failed launch is left in the runtime's last error, which every
     // caller checks after its launches
     (void)cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
+}
+
+// opts kernel `k` in to `smem` bytes of dynamic shared memory on the current
+// device; `su` is the kernel's own
+template <typename... P>
+inline void opt_in_smem(KernelSetup &su, void (*k)(P...), size_t smem)
+{
+    if (smem <= 48 * 1024) return;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    // a failure is left in the runtime's last error, as a failed launch is
+    su.opt_in(dev, smem, 48 * 1024, [&](size_t n) {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n) == cudaSuccess;
+    });
 }
 
 // ---- coarse quantizer (coarse.cu)

@@ -1379,24 +1379,19 @@ static void launch_scan(sivf_index *ix, const ScanArgs &a, size_t smem, int grid
                         cudaStream_t st)
 {
     if (SW) smem += 1024;  // base alignment slack
-    static size_t attr = 48 * 1024;
-    if (smem > attr) {
-        cudaFuncSetAttribute(k_scan<TQ, C, SW, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-        attr = smem;
-    }
+    static KernelSetup su;
+    opt_in_smem(su, k_scan<TQ, C, SW, ONE>, smem);
     // as many CTAs per SM as fit: the small tiles' shared memory leaves room
     // for two or more, which hide each other's barriers and load latency
-    static size_t occ_smem = 0;
-    static int occ = 1;
-    if (smem != occ_smem) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int occ = su.resident(dev, smem, [&] {
         int n = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_scan<TQ, C, SW, ONE>, SCAN_NT, smem) !=
             cudaSuccess)
             n = 1;
-        occ = std::max(1, n);
-        occ_smem = smem;
-    }
+        return std::max(1, n);
+    });
     const int tok = prof_begin(ix, PROF_SCAN, 1, st);
     launch_pdl(k_scan<TQ, C, SW, ONE>, grid * occ, SCAN_NT, smem, st,
                *reinterpret_cast<const CUtensorMap *>(ix->tmap_x32), a);
@@ -1576,12 +1571,8 @@ void group_pairs(sivf_index *ix, int64_t nq, int P, int p0, int p1, const int32_
     const int L = ix->nlist;
     const int64_t n = nq * (p1 - p0);
     if (n <= SH_PAIRS) {
-        static bool attr = false;
-        if (!attr) {
-            cudaFuncSetAttribute(k_srch_hash, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)SH_SMEM);
-            attr = true;
-        }
+        static KernelSetup su;
+        opt_in_smem(su, k_srch_hash, SH_SMEM);
         const int tg = prof_begin(ix, PROF_GROUP, 1, st);
         launch_pdl(k_srch_hash, 1, 1024, SH_SMEM, st, probes, nq, P, p0, p1, L, dedupe,
                    flagged ? s.prank : nullptr, ix->nslabs, ix->list_live, pl.tq, pl.ch,

@@ -949,11 +949,8 @@ bool qt_make_maps(sivf_index *ix, PFN_cuTensorMapEncodeTiled_v12000 enc)
 template <int DT>
 static void launch_qt(const unsigned char *tmap, const QtArgs &a, size_t smem, cudaStream_t st)
 {
-    static size_t attr = 0;
-    if (smem > attr) {
-        cudaFuncSetAttribute(k_scan_qt<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = smem;
-    }
+    static KernelSetup su;
+    opt_in_smem(su, k_scan_qt<DT>, smem);
     launch_pdl(k_scan_qt<DT>, 152, QT_NT, smem, st, *reinterpret_cast<const CUtensorMap *>(tmap),
                a);
 }

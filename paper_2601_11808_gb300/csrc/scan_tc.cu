@@ -2078,12 +2078,8 @@ static void launch_tc(const unsigned char *tmap, const unsigned char *tmap_t, Tc
 {
     a.nst = tc_stages<TN>(a.KC, a.M);
     const size_t smem = tc_smem<TN>(a.KC, a.M, a.nst).total;
-    static size_t attr = 0;
-    if (smem > attr) {
-        cudaFuncSetAttribute(k_scan_tc<DT, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-        attr = smem;
-    }
+    static KernelSetup su;
+    opt_in_smem(su, k_scan_tc<DT, TN>, smem);
     launch_pdl(k_scan_tc<DT, TN>, 152, TcShape<TN>::NT, smem, st,
                *reinterpret_cast<const CUtensorMap *>(tmap),
                *reinterpret_cast<const CUtensorMap *>(tmap_t), a);

@@ -1242,17 +1242,24 @@ __global__ __launch_bounds__(SCAN_NT, ONE ? 1 : 2) void k_scan(
 }
 
 // ------------------------------------------------------- per-query merge
-constexpr int MERGE_NT = 128;
+// threads of a block: two warps' tables of 1,024 entries take 40 KB
+__host__ __device__ constexpr int merge_nt(int E) { return E <= 16 ? 128 : 64; }
 constexpr int MERGE_RUNS_PER_LANE = 64;  // both phases' runs: at most 2,048 per query
+constexpr int MERGE_LONG = 32;           // entries of a run that a lane takes alone
 
 // One warp per query.  A query's runs of one scan phase (K entries each,
 // sorted, padded with (+inf, -1)) are contiguous, and at least k entries lie
-// at or below its shared bound after the scan: the warp streams them, gathers
-// those (usually little more than k) and sorts them in registers.  Only when
-// there are more than 32 E (ties, or k near 32 E) does it walk all runs, a
-// cursor per run, one result after the other.
+// at or below its shared bound after the scan: the warp gathers those (usually
+// little more than k) and sorts them in registers.  The bound is loose where
+// long lists were scanned in many chunks at once (few queries): a full table is
+// cut down to a value k of its entries lie at or below (kth_bound), which is the
+// bound from then on.  Short runs are streamed; of long ones a lane takes each
+// and leaves it at its first entry past the bound (14 queries, k = 100, 90
+// skewed lists: 137 us by streaming and then a cursor per run, 77 by cursors
+// alone).  Only where cutting leaves no room (ties, or k > 960) does it walk
+// all runs, a cursor per run, one result after the other.
 template <int E>
-__global__ __launch_bounds__(MERGE_NT) void k_merge(const int2 *__restrict__ qrun, int64_t nq,
+__global__ __launch_bounds__(merge_nt(E)) void k_merge(const int2 *__restrict__ qrun, int64_t nq,
                                                     int nphase, int K, int k,
                                                     const float *__restrict__ thr,
                                                     const float *__restrict__ part_d,
@@ -1262,41 +1269,85 @@ __global__ __launch_bounds__(MERGE_NT) void k_merge(const int2 *__restrict__ qru
 {
     pdl_begin();
     constexpr int MU = 8;  // loads in flight per lane
-    __shared__ float sd[MERGE_NT / 32][32 * E];
-    __shared__ int64_t si[MERGE_NT / 32][32 * E];
-    __shared__ uint64_t sk[MERGE_NT / 32][32 * E];
+    constexpr int NT = merge_nt(E);
+    __shared__ float sd[NT / 32][32 * E];
+    __shared__ int64_t si[NT / 32][32 * E];
+    __shared__ uint64_t sk[NT / 32][32 * E];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t q = (blockIdx.x * (int64_t)MERGE_NT + threadIdx.x) >> 5;
+    const int64_t q = (blockIdx.x * (int64_t)NT + threadIdx.x) >> 5;
     if (q >= nq) return;  // whole warps
     const int2 r0 = qrun[q];
     const int2 r1 = nphase > 1 ? qrun[nq + q] : make_int2(0, 0);
-    const float bound = thr[q];
+    float bound = thr[q];
     int have = 0;
-    for (int ph = 0; ph < 2 && k <= 32 * E; ++ph) {
+    bool room = k + k / 32 + 33 <= 32 * E;  // an append fits after a cut (kth_bound)
+    // the warp's entries v within the bound, at `e` of the runs
+    auto gather = [&](float v, int64_t e) {
+        uint32_t mk = __ballot_sync(0xffffffffu, v <= bound);  // pads are +inf
+        if (have + __popc(mk) > 32 * E) {
+            room = have >= k;
+            if (!room) return;
+            __syncwarp();
+            bound = fminf(bound, kth_bound<E>([&](int i) { return i < have ? sd[w][i] : INFINITY; },
+                                              32 * E, k, lane));
+            int n2 = 0;
+            for (int i0 = 0; i0 < have; i0 += 32) {
+                const int i = i0 + lane;
+                const float u = i < have ? sd[w][i] : INFINITY;
+                const int64_t id = i < have ? si[w][i] : -1;
+                const uint32_t keep = __ballot_sync(0xffffffffu, u <= bound);
+                if (u <= bound) {  // at or before i
+                    const int p = n2 + __popc(keep & lanemask_lt());
+                    sd[w][p] = u;
+                    si[w][p] = id;
+                }
+                n2 += __popc(keep);
+                __syncwarp();
+            }
+            have = n2;
+            mk = __ballot_sync(0xffffffffu, v <= bound);
+            room = have + __popc(mk) <= 32 * E;
+            if (!room) return;
+        }
+        if (v <= bound) {
+            const int p = have + __popc(mk & lanemask_lt());
+            sd[w][p] = v;
+            si[w][p] = part_i[e];
+        }
+        have += __popc(mk);
+    };
+    for (int ph = 0; ph < 2 && room; ++ph) {
         const int64_t b = (int64_t)(ph ? r1.x : r0.x) * K;
         const int64_t n = (int64_t)(ph ? r1.y : r0.y) * K;
-        for (int64_t i0 = lane; i0 - lane < n && have <= 32 * E; i0 += 32 * MU) {
+        if (K >= MERGE_LONG) {
+            for (int64_t g = 0; g < n && room; g += 32 * (int64_t)K) {
+                const int64_t e0 = g + (int64_t)lane * K;
+                bool on = e0 < n;
+                for (int j0 = 0; j0 < K && room && __any_sync(0xffffffffu, on); j0 += MU) {
+                    float v[MU];
+#pragma unroll
+                    for (int u = 0; u < MU; ++u)
+                        v[u] = on && j0 + u < K ? part_d[b + e0 + j0 + u] : INFINITY;
+#pragma unroll
+                    for (int u = 0; u < MU; ++u)
+                        if (room) gather(v[u], b + e0 + j0 + u);
+                    on &= v[MU - 1] <= bound;  // +inf past the run's end
+                }
+            }
+            continue;
+        }
+        for (int64_t i0 = lane; i0 - lane < n && room; i0 += 32 * MU) {
             float v[MU];
-            bool in[MU];
 #pragma unroll
             for (int u = 0; u < MU; ++u)
                 v[u] = i0 + 32 * u < n ? part_d[b + i0 + 32 * u] : INFINITY;
 #pragma unroll
-            for (int u = 0; u < MU; ++u) in[u] = v[u] <= bound;  // pads are +inf
-#pragma unroll
-            for (int u = 0; u < MU; ++u) {
-                const uint32_t mk = __ballot_sync(0xffffffffu, in[u]);
-                const int p = have + __popc(mk & lanemask_lt());
-                if (in[u] && p < 32 * E) {
-                    sd[w][p] = v[u];
-                    si[w][p] = part_i[b + i0 + 32 * u];
-                }
-                have += __popc(mk);
-            }
+            for (int u = 0; u < MU; ++u)
+                if (room) gather(v[u], b + i0 + 32 * u);
         }
     }
     __syncwarp();
-    if (k <= 32 * E && have <= 32 * E) {
+    if (room) {
         warp_order<E>(
             have, [&](int i) { return sd[w][i]; }, [&](int i) { return si[w][i]; },
             [&](int i, float v, int64_t id) {
@@ -1679,15 +1730,16 @@ void scan_lists(sivf_index *ix, const float *q, int64_t nq, int P, const int32_t
 void merge_topk(sivf_index *ix, int64_t nq, int P, const SearchPlan &pl,
                 const SearchScratch &s, int k, float *dist, int64_t *labels, cudaStream_t st)
 {
-    const unsigned blocks = (unsigned)((nq * 32 + MERGE_NT - 1) / MERGE_NT);
     const int nphase = fp32_two_phase(nq, P) ? 2 : 1;
     const int tok = prof_begin(ix, PROF_MERGE, 1, st);
 #define SIVF_MERGE(E_)                                                                            \
-    launch_pdl(k_merge<E_>, blocks, MERGE_NT, 0, st, s.qrun, nq, nphase, pl.K, k, s.thr, s.part_d, \
-               s.part_i, dist, labels)
+    launch_pdl(k_merge<E_>, (unsigned)((nq * 32 + merge_nt(E_) - 1) / merge_nt(E_)), merge_nt(E_), 0, st, \
+               s.qrun, nq, nphase, pl.K, k, s.thr, s.part_d, s.part_i, dist, labels)
     if (k <= 24) SIVF_MERGE(2);
     else if (k <= 72) SIVF_MERGE(4);
-    else SIVF_MERGE(8);
+    else if (k <= 160) SIVF_MERGE(8);
+    else if (k <= 448) SIVF_MERGE(16);
+    else SIVF_MERGE(32);
 #undef SIVF_MERGE
     prof_end(ix, tok, st);
 }

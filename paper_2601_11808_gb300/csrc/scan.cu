@@ -1070,7 +1070,7 @@ __global__ __launch_bounds__(SCAN_NT, ONE ? 1 : 2) void k_scan(
     // sought, it cost 780 queries of 11 lists among overlapping cells a quarter of
     // their time: 1,354 us, 1,055 so); what is within it (ties included) goes to the
     // candidates, slots first, and is merged with its ids
-    auto select_row = [&](int qr, int n) {
+    auto select_row = [&](int qr, int n, bool last) {
         const float *dr = DM + (size_t)qr * DS;
         float *bd = BD + (size_t)qr * M + K;
         int64_t *bi = BI + (size_t)qr * M + K;
@@ -1085,33 +1085,39 @@ __global__ __launch_bounds__(SCAN_NT, ONE ? 1 : 2) void k_scan(
         if (many)
             bar = fminf(bar, kth_bound<16>([&](int i) { return i < n ? dr[i] : INFINITY; },
                                            (n + 31) & ~31, K, lane));
-        int cc = 0;
-        auto merge = [&]() {
+        int cc = M > 256 ? s_cc[qr] : 0;  // those of earlier blocks have their ids
+        auto merge = [&](bool now) {
             __syncwarp();
             for (int e = lane; e < cc; e += 32) {
-                const int i = (int)bi[e];
-                bi[e] = __ldg(a.ids + (size_t)block_slab[i / C] * C + i % C);
+                const int i = ~(int)bi[e];
+                if (i >= 0) bi[e] = __ldg(a.ids + (size_t)block_slab[i / C] * C + i % C);
             }
             if (lane == 0) s_cc[qr] = cc;
             __syncwarp();
-            merge_row(qr);
-            bar = fminf(bar, s_kd[qr]);
-            cc = 0;
+            if (now) merge_row(qr);
         };
         for (int i0 = 0; i0 < n; i0 += 32) {
             const float v = dr[i0 + lane];  // n is a multiple of 32
             const bool in = v <= bar && v < INFINITY;
             const uint32_t mk = __ballot_sync(0xffffffffu, in);
             if (mk == 0u) continue;
-            if (cc + __popc(mk) > CB) merge();
+            if (cc + __popc(mk) > CB) {
+                merge(true);
+                bar = fminf(bar, s_kd[qr]);
+                cc = 0;
+            }
             if (in) {
                 const int p = cc + __popc(mk & lanemask_lt());
                 bd[p] = v;
-                bi[p] = i0 + lane;
+                bi[p] = ~(int64_t)(i0 + lane);  // its place in the block, negative
             }
             cc += __popc(mk);
         }
-        merge();
+        // more than 256 entries are sorted as a whole, whatever is new among them:
+        // they wait for a full buffer or the item's end (large K leaves room for
+        // blocks of one slab: K = 500, 1,000 queries of 16 of 90 skewed lists of a
+        // million vectors, 37.9 ms with a sort per block, 7.6 so)
+        merge(M <= 256 || last || s_nb[qr] + cc <= 256);
     };
 
     for (;;) {
@@ -1215,7 +1221,8 @@ __global__ __launch_bounds__(SCAN_NT, ONE ? 1 : 2) void k_scan(
                 ++g_issue;
             }
             if (idx % NBS == NBS - 1 || idx + 1 == ns) {
-                for (int qr = warp; qr < m; qr += SCAN_NT / 32) select_row(qr, (idx % NBS + 1) * C);
+                for (int qr = warp; qr < m; qr += SCAN_NT / 32)
+                    select_row(qr, (idx % NBS + 1) * C, idx + 1 == ns);
                 __syncthreads();
             }
         }

@@ -29,11 +29,14 @@
 // with the FP32 bound.  Lists outside S_b have exact distances above the
 // P-th smallest, so the result is the same set.
 //
-// The forms (d <= 128 except the last two):
-//   P = 1              k_coarse_fused, k_coarse_finish: no distance matrix
+// The forms (d % 16 == 0 and d <= 128 in the first three):
+//   P = 1, 16 <= L     k_coarse_fused, k_coarse_finish: no distance matrix;
+//     <= 4096            few rows: k_coarse_dist, k_coarse_near
 //   2 <= P <= 128 of   k_coarse_dist, k_coarse_pick: the matrix with group
-//   at least 32 P        minima, of which a row reads a few groups
-//   P <= 8, L <= 4096  k_coarse_tc, k_coarse_select_w
+//   at least 32 P        minima, of which a row reads a few groups (P <= 8
+//                        only where L d >= 32,768)
+//   P <= 8, L <= 4096  k_coarse_tc (k_coarse_gemm where d % 16), then
+//                        k_coarse_select_w
 //   else               k_coarse_gemm (FP32), k_coarse_select
 #include <float.h>
 #include <math.h>
@@ -233,8 +236,8 @@ __device__ __forceinline__ double exact_dist4(const float4 *a, const float4 *__r
 // of an SM are at it; the chain of additions (about 300 cycles each) is the same.
 constexpr int EX_FEW = 4;
 template <class Idx>
-__device__ __forceinline__ double exact_four(const float4 *x4, const float *__restrict__ cent, Idx list, int n,
-                                             int d, int lane)
+__device__ __forceinline__ double exact_four(const float4 *x4, const float *__restrict__ cent,
+                                             Idx list, int n, int d, int lane)
 {
     const int n4 = d >> 2;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -900,7 +903,8 @@ __device__ __forceinline__ int decide_nearest(const NearArgs &a, Fill fill, int 
             if (lane < k) take(D, tab[lane]);
         } else {
             for (int p = lane; p < k; p += 32)
-                take(exact_dist4(x4, reinterpret_cast<const float4 *>(a.cent + (size_t)tab[p] * d), d), tab[p]);
+                take(exact_dist4(x4, reinterpret_cast<const float4 *>(a.cent + (size_t)tab[p] * d), d),
+                     tab[p]);
         }
         exact = true;
         __syncwarp();

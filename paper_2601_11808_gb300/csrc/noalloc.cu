@@ -61,7 +61,7 @@ size_t need_bytes(const sivf_index *ix, int64_t nq, int P, const sivf::SearchPla
     add((size_t)nq * P * 4);          // probes
     add(L * 4);                       // lcnt
     add((L + 1) * 4);                 // loff
-    add((L + 1) * 4);                 // not used: batches are refused from the same size on
+    add((L + 1) * 4);                 // not carved: keeps the size from which batches are refused
     add(L * 4);                       // nch
     add((size_t)nq * P * 4);          // prank
     add((size_t)nq * P * 4);          // qlist

@@ -2023,11 +2023,12 @@ static size_t tc_total(int tn, int KC, int M, int nst)
 }
 
 // Entries of a row's candidate buffer.  A row folds its pending candidates
-// into its best K' once more than (room - 1) tiles of them wait (for
-// K' <= 128 also past 224), so with room for one tile any candidate at all
-// costs a fold per tile; the default takes room for three tiles (K' > 128)
-// or two where three A stages still fit beside it, else one.  sel > 0 asks
-// for sel tiles of room.
+// into its best K' once more than FT = room - step of them wait (for K' <= 128
+// at most 96), a step being what is appended between two checks: a round of TP
+// tiles, or a whole group of accumulators where an item runs without checks.
+// With room for one step any candidate at all costs a fold; the default takes
+// room for three tiles (K' > 128) or two where three A stages still fit beside
+// it, else one.  sel > 0 asks for sel tiles of room.
 int tc_buf_entries(const sivf_index *ix, int dtype, int Kc, int sel)
 {
     if (sel > 0) return tc_buf_len(Kc, sel);
